@@ -85,6 +85,11 @@ class TernaryNet:
         self.side_streams = [torch.cuda.Stream()]
         self.dw_stream = torch.cuda.Stream()     # weight gradients run beside the backward-for-data chain
         self.timed = None          # when a list: (kind, name, flops, start event, end event)
+        self._fwd = None           # calls of a forward pass, made on first use
+        self._bwd = None           # order and fusions of a backward pass, made on first use
+        self._pending_join = False
+        self._codes_ready = torch.cuda.Event()
+        self._dz_ready: dict[str, torch.cuda.Event] = {}
         H, W, C = in_shape
         self.act["input"] = torch.zeros((batch, H, W, C), dtype=torch.bfloat16, device="cuda")
         self._build()
@@ -177,12 +182,17 @@ class TernaryNet:
         self.act["input"].copy_(_bf16(bits).view(self.act["input"].shape))
 
     # ------------------------------------------------------------------ timing hooks
-    def _call(self, kind, name, flops, fn):
-        if self.timed is None:
-            fn()
+    def _call(self, kind, name, flops, entry, args, stream=None):
+        """Calls twn.<entry>(*args) on `stream` (None: the current one), between two events while timing.  The
+        stream is passed on instead of being made current: entering a stream context takes the host longer than
+        the call itself."""
+        fn = getattr(twn, entry)
+        if self.timed is None or kind is None:
+            fn(*args, stream=stream)
             return
-        e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-        e0.record(); fn(); e1.record()
+        with torch.cuda.stream(stream):
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            e0.record(); fn(*args); e1.record()
         self.timed.append((kind, name, flops, e0, e1))
 
     # ------------------------------------------------------------------ Algorithm 1, first loop
@@ -191,110 +201,92 @@ class TernaryNet:
         batched call (two launches per 32 layers) on the current stream.  The re-layouts of the codes
         for the backward pass follow as one batched launch on a side stream, beside the forward pass;
         the backward pass waits for its event."""
-        main = torch.cuda.current_stream()
         layers = list(self.layers.values())
+        entry = "ternarize_codes_batch" if self._delta_ready else "ternarize_batch"
         for i in range(0, len(layers), 32):
-            group = layers[i:i + 32]
             items = [(L.extra["W"], L.Cout, L.K, L.extra["stats"], L.extra["packed"], L.extra["ld"], None)
-                     for L in group]
-            if self._delta_ready:
-                # the thresholds were left behind by the previous step's update: coding sweep only
-                self._call("ternarize", f"layers {i}..{i + len(group) - 1}", 0,
-                           lambda: twn.ternarize_codes_batch(items, self.ws_tern))
-            else:
-                self._call("ternarize", f"layers {i}..{i + len(group) - 1}", 0,
-                           lambda: twn.ternarize_batch(items, self.delta_factor, self.ws_tern))
+                     for L in layers[i:i + 32]]
+            # with the thresholds left behind by the previous step's update only the coding sweep is needed
+            args = (items, self.ws_tern) if self._delta_ready else (items, self.delta_factor, self.ws_tern)
+            self._call("ternarize", f"layers {i}..{i + len(items) - 1}", 0, entry, args)
         for L in layers:
             if L.fold:
                 twn.fold_codes(L.desc, L.extra["packed"], L.extra["ld"], L.extra["packed_f"], L.fold[2])
         if self.train:
             # the re-layouts for the backward pass: one batched launch beside the forward pass
-            st = self.side_streams[0]
+            main, st = torch.cuda.current_stream(), self.side_streams[0]
             st.wait_stream(main)
             todo = [L for L in layers if "packed_b" in L.extra]
-            with torch.cuda.stream(st):
-                for i in range(0, len(todo), 32):
-                    twn.transpose_codes_batch([(L.extra["packed"], L.extra["ld"], L.desc, L.extra["packed_b"],
-                                                L.extra["ld_b"]) for L in todo[i:i + 32]])
-                ev = torch.cuda.Event()
-                ev.record(st)
-            for L in todo:
-                L.extra["ready_b"] = ev
+            for i in range(0, len(todo), 32):
+                twn.transpose_codes_batch([(L.extra["packed"], L.extra["ld"], L.desc, L.extra["packed_b"],
+                                            L.extra["ld_b"]) for L in todo[i:i + 32]], stream=st)
+            self._codes_ready.record(st)
             self._pending_join = True
         if join:
             self.join_side_streams()
 
-    def _wait_codes(self, L, key="ready"):
-        ev = L.extra.get(key)
-        if ev is not None:
-            torch.cuda.current_stream().wait_event(ev)
-
     def join_side_streams(self):
         """All side-stream work rejoins the current stream (required before a graph capture ends
         and before the master weights change)."""
-        if getattr(self, "_pending_join", False):
-            main = torch.cuda.current_stream()
-            main.wait_stream(self.side_streams[0])      # the only side stream ternarize_all forks
+        if self._pending_join:
+            torch.cuda.current_stream().wait_stream(self.side_streams[0])   # the only side stream ternarize_all forks
             self._pending_join = False
-            for L in self.layers.values():      # nothing left to wait for
-                L.extra.pop("ready", None)
-                L.extra.pop("ready_b", None)
 
     # ------------------------------------------------------------------ forward
-    def forward(self):
+    def _forward_calls(self):
+        """The calls of a forward pass, (kind, name, flops, entry point, arguments) each: a pass walks this list."""
+        calls = []
         for op in self.ops:
             kind = op[0]
             if kind == "layer":
                 L: Layer = op[1]
                 e = L.extra
                 x, y = self.act[L.src], self.act[L.name]
-                fl = 2 * L.macs
-                self._wait_codes(L)
+                row = ("tconv", L.name + ".fwd", 2 * L.macs)
                 if L.fold:
-                    twn.fold_input(L.desc, x, e["xf"])
-                    self._call("tconv", L.name + ".fwd", fl, lambda: twn.conv2d_fwd_folded(
-                        L.desc, e["xf"], e["packed_f"], L.fold[2], e["stats"], e["epi"], y, self.status))
+                    calls.append((None, "", 0, "fold_input", (L.desc, x, e["xf"])))
+                    calls.append((*row, "conv2d_fwd_folded", (L.desc, e["xf"], e["packed_f"], L.fold[2], e["stats"], e["epi"],
+                                                              y, self.status)))
                 elif L.small_cin:
-                    twn.im2col(L.desc, x, e["xcol"], L.ldk)
                     M = L.B * L.Ho * L.Wo
-                    self._call("tconv", L.name + ".fwd", fl, lambda: twn.gemm(
-                        e["xcol"], L.ldk, e["packed"], e["ld"], e["stats"], M, L.Cout, L.K, e["epi"], y,
-                        L.Cout, self.status))
+                    calls.append((None, "", 0, "im2col", (L.desc, x, e["xcol"], L.ldk)))
+                    calls.append((*row, "gemm", (e["xcol"], L.ldk, e["packed"], e["ld"], e["stats"], M, L.Cout, L.K, e["epi"],
+                                                 y, L.Cout, self.status)))
                 else:
-                    self._call("tconv", L.name + ".fwd", fl, lambda: twn.conv2d_fwd(
-                        L.desc, x, e["packed"], e["ld"], e["stats"], e["epi"], y, self.status))
+                    calls.append((*row, "conv2d_fwd", (L.desc, x, e["packed"], e["ld"], e["stats"], e["epi"], y, self.status)))
             elif kind == "maxpool":
                 _, name, src, k, s, p = op
                 x = self.act[src]
                 Bx, H, W, C = x.shape
-                twn.maxpool2d_fwd(x, Bx, H, W, C, k, s, p, self.act[name], self.aux.get(name))
+                calls.append((None, "", 0, "maxpool2d_fwd", (x, Bx, H, W, C, k, s, p, self.act[name], self.aux.get(name))))
             elif kind == "avgpool":
                 _, name, src = op
                 x = self.act[src]
                 Bx, H, W, C = x.shape
-                twn.avgpool_fwd(x, Bx, H * W, C, self.act[name])
+                calls.append((None, "", 0, "avgpool_fwd", (x, Bx, H * W, C, self.act[name])))
+        return calls
+
+    def forward(self):
+        if self._fwd is None or self._fwd[0] is not self.act["input"]:
+            self._fwd = (self.act["input"], self._forward_calls())
+        for call in self._fwd[1]:
+            self._call(*call)
         return self.act[self.ops[-1][1].name]
 
     # ------------------------------------------------------------------ backward
-    def backward(self, dlogits: torch.Tensor):
-        """dlogits: bf16 [B, classes], the gradient injected at the logits.  Fills extra['dW'] of
-        every layer.  An activation with two consumers (the input of a residual block) gets its
-        second contribution added through the residual input of the backward-for-data epilogue."""
-        assert self.train
+    def _backward_steps(self):
+        """The steps of a backward pass, in order, and the gradient of every activation.  A step is
+          ("call", entry point, arguments)          an untimed call
+          ("dw", layer, entry point, arguments)     a weight gradient, on its own stream
+          ("dx", layer, arguments before the epilogue, epilogue, output)
+        An argument that is None in place of dY stands for the gradient of the logits."""
         last: Layer = self.ops[-1][1]
-        acc: dict[str, torch.Tensor] = {last.name: dlogits.view(self.act[last.name].shape)}
+        acc: dict[str, torch.Tensor | None] = {last.name: None}
+        steps = []
 
         def emit_tensor(name, t):
             assert name not in acc, "a materialised gradient must be the first contribution"
             acc[name] = t
-
-        def emit(name, fn):
-            """fn(res, out): out = contribution (+ res).  The first contribution is written plainly."""
-            if name == "input":
-                return
-            out = self.grad[name]
-            fn(acc.get(name), out)
-            acc[name] = out
 
         # A layer P = relu(z * scale + shift) whose output feeds exactly one convolution gets its
         # dZ straight from that convolution's backward-for-data pass (the ReLU gate and the scale
@@ -334,8 +326,6 @@ class TernaryNet:
                 order.append(deferred.pop(op[1].src))
         order.extend(deferred.values())
 
-        main = torch.cuda.current_stream()
-        self.dw_stream.wait_stream(main)
         for op in order:
             kind = op[0]
             if kind == "layer":
@@ -343,7 +333,6 @@ class TernaryNet:
                 e = L.extra
                 dY = acc[L.name]
                 if dY is not FUSED:
-                    n = dY.numel()
                     y = self.act[L.name] if L.relu else None
                     dpre = None
                     if L.residual:
@@ -351,70 +340,91 @@ class TernaryNet:
                         dpre = e.get("dpre")
                         if dpre is None:
                             dpre = e["dpre"] = torch.zeros_like(e["dz"])
-                    twn.act_bwd(dY, y, e["scale"], n, L.Cout, e["dz"], dpre)
+                    steps.append(("call", "act_bwd", (dY, y, e["scale"], e["dz"].numel(), L.Cout, e["dz"], dpre)))
                     if L.residual:
                         emit_tensor(L.residual, dpre)
-                # dW needs only dz and the layer's input: it goes to its own stream (one after the
-                # other there, they share the workspace) and overlaps the dX chain of the layers below
-                dz_ready = torch.cuda.Event()
-                dz_ready.record(main)
-                with torch.cuda.stream(self.dw_stream):
-                    self.dw_stream.wait_event(dz_ready)
-                    if L.fold:
-                        self._call("dw", L.name + ".dW", 2 * L.macs, lambda: twn.conv2d_bwd_weight_folded(
-                            L.desc, e["xf"], e["dz"], e["dW"], self.ws_dw, self.status))
-                    else:
-                        x = e["xcol"] if L.small_cin else self.act[L.src]
-                        self._call("dw", L.name + ".dW", 2 * L.macs, lambda: twn.conv2d_bwd_weight(
-                            e["dw_desc"], x, e["dz"], e["dW"], self.ws_dw, self.status))
-                P = fused_producer(L) if L.src != "input" else None
+                if L.fold:
+                    steps.append(("dw", L, "conv2d_bwd_weight_folded", (L.desc, e["xf"], e["dz"], e["dW"], self.ws_dw, self.status)))
+                else:
+                    x = e["xcol"] if L.small_cin else self.act[L.src]
+                    steps.append(("dw", L, "conv2d_bwd_weight", (e["dw_desc"], x, e["dz"], e["dW"], self.ws_dw, self.status)))
+                if L.src == "input":
+                    continue
+                P = fused_producer(L)
                 if P is not None:
-                    self._wait_codes(L, "ready_b")
-                    epi = twn.epilogue(scale=P.extra["scale"], residual=self.act[P.name], out_dtype=twn.BF16,
-                                       residual_op=twn.RESIDUAL_GATE)
-                    self._call("tconv", L.name + ".dX", 2 * L.macs, lambda: twn.conv2d_bwd_data(
-                        L.desc, e["dz"], e["packed_b"], e["ld_b"], e["stats"], epi, P.extra["dz"], self.status))
+                    epi = dict(scale=P.extra["scale"], residual=self.act[P.name], out_dtype=twn.BF16, residual_op=twn.RESIDUAL_GATE)
+                    out = P.extra["dz"]
                     assert P.name not in acc
                     acc[P.name] = FUSED
-                elif L.src != "input":
-                    def bwd(res, out, L=L, e=e):
-                        self._wait_codes(L, "ready_b")
-                        epi = twn.epilogue(residual=res, out_dtype=twn.BF16)
-                        self._call("tconv", L.name + ".dX", 2 * L.macs, lambda: twn.conv2d_bwd_data(
-                            L.desc, e["dz"], e["packed_b"], e["ld_b"], e["stats"], epi, out, self.status))
-                    emit(L.src, bwd)
+                else:
+                    # a second contribution to a gradient adds to the first in place
+                    epi = dict(residual=acc.get(L.src), out_dtype=twn.BF16)
+                    out = acc[L.src] = self.grad[L.src]
+                steps.append(("dx", L, (L.desc, e["dz"], e["packed_b"], e["ld_b"], e["stats"]), epi, out))
             elif kind == "maxpool":
                 _, name, src, k, s, p = op
                 Bx, H, W, C = self.act[src].shape
                 dY = acc[name]
-
                 P = self.layers.get(src)
                 if P is not None and P.relu and not P.residual and consumers.get(src) == [name]:
                     # the pool is the only reader of a ReLU layer: its backward pass writes that
                     # layer's dZ (gate by the pooled value, folded batch-norm scale) in one sweep
-                    twn.maxpool2d_bwd_act(dY, self.aux[name], self.act[name], P.extra["scale"], Bx, H, W, C, k, s, p,
-                                          P.extra["dz"])
+                    steps.append(("call", "maxpool2d_bwd_act", (dY, self.aux[name], self.act[name], P.extra["scale"], Bx, H, W, C,
+                                                                k, s, p, P.extra["dz"])))
                     acc[src] = FUSED
-                    continue
-
-                def mp(res, out, dY=dY, name=name, Bx=Bx, H=H, W=W, C=C, k=k, s=s, p=p):
-                    assert res is None
-                    twn.maxpool2d_bwd(dY, self.aux[name], Bx, H, W, C, k, s, p, out)
-                emit(src, mp)
+                elif src != "input":
+                    emit_tensor(src, self.grad[src])
+                    steps.append(("call", "maxpool2d_bwd", (dY, self.aux[name], Bx, H, W, C, k, s, p, self.grad[src])))
             elif kind == "avgpool":
                 _, name, src = op
                 Bx, H, W, C = self.act[src].shape
-                dY = acc[name]
-
-                def ap(res, out, dY=dY, Bx=Bx, H=H, W=W, C=C):
-                    assert res is None
-                    twn.avgpool_bwd(dY, Bx, H * W, C, out)
-                emit(src, ap)
+                if src != "input":
+                    emit_tensor(src, self.grad[src])
+                    steps.append(("call", "avgpool_bwd", (acc[name], Bx, H * W, C, self.grad[src])))
             elif kind == "flatten":
                 _, name, src = op
                 emit_tensor(src, acc[name].view(self.act[src].shape))
-        main.wait_stream(self.dw_stream)
-        self.last_grads = acc
+        for st in steps:
+            if st[0] == "dw":
+                self._dz_ready[st[1].name] = torch.cuda.Event()
+        return steps, acc
+
+    def backward(self, dlogits: torch.Tensor):
+        """dlogits: bf16 [B, classes], the gradient injected at the logits.  Fills extra['dW'] of
+        every layer.  An activation with two consumers (the input of a residual block) gets its
+        second contribution added through the residual input of the backward-for-data epilogue."""
+        assert self.train
+        if self._bwd is None or self._bwd[0] is not self.act["input"]:
+            self._bwd = (self.act["input"], *self._backward_steps())
+        _, steps, acc = self._bwd
+        last: Layer = self.ops[-1][1]
+        dY = dlogits.view(self.act[last.name].shape)
+        main, side = torch.cuda.current_stream(), self.dw_stream
+        side.wait_stream(main)
+        wait_codes = self._pending_join
+        for st in steps:
+            kind = st[0]
+            if kind == "call":
+                args = st[2]
+                self._call(None, "", 0, st[1], args if args[0] is not None else (dY, *args[1:]), main)
+            elif kind == "dw":
+                # dW needs only dz and the layer's input: it goes to its own stream (one after the
+                # other there, they share the workspace) and overlaps the dX chain of the layers below
+                L = st[1]
+                ready = self._dz_ready[L.name]
+                ready.record(main)
+                side.wait_event(ready)
+                self._call("dw", L.name + ".dW", 2 * L.macs, st[2], st[3], side)
+            else:
+                _, L, args, epi, out = st
+                # Waited for before every one of these calls, not only the first: the second dependency keeps them
+                # from starting programmatically, early, on SMs that the weight gradients beside them can use
+                # (ResNet-18 step 1.332 ms, against 1.366 ms with one wait).
+                if wait_codes:
+                    main.wait_event(self._codes_ready)
+                self._call("tconv", L.name + ".dX", 2 * L.macs, "conv2d_bwd_data", (*args, twn.epilogue(**epi), out, self.status), main)
+        main.wait_stream(side)
+        self.last_grads = {**acc, last.name: dY}
 
     def sgd_step(self):
         """Algorithm 1, UpdateParameters: SGD with momentum and weight decay on every layer's master

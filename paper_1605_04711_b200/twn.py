@@ -1,6 +1,7 @@
-"""ctypes binding of libtwn.so: the same entry points as include/twn.h.
+"""Python binding of libtwn.so: the same entry points as include/twn.h.
 
-Argument marshalling only.  Tensors are torch tensors on the current CUDA
+Argument marshalling only: the compute calls go through the native module _twn (csrc/binding.cpp), the size
+queries and the status read-back through ctypes.  Tensors are torch tensors on the current CUDA
 device (torch provides memory and streams); every step of the computation runs
 in the library's kernels.  There is no fallback: if the library is missing or
 the device is not sm_100 the calls raise.
@@ -11,6 +12,18 @@ import ctypes as C
 import os
 
 import torch
+
+try:
+    from . import _twn as _C
+except ImportError as e:
+    class _Missing:
+        """Stands in for the native module where it is not built: every call says so."""
+        reason = str(e)
+
+        def __getattr__(self, name):
+            raise FileNotFoundError(f"the native binding does not load ({self.reason}): build it with "
+                                    "`python -m paper_1605_04711_b200.build`")
+    _C = _Missing()
 
 _PKG = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_PKG, "libtwn.so")
@@ -130,35 +143,23 @@ def ternarize(W: torch.Tensor, delta_factor: float, stats: torch.Tensor, packed:
     """twn_ternarize.  W fp32 [rows, cols] (or any shape with rows/cols given)."""
     if rows is None:
         rows, cols = (W.shape[0], W.numel() // W.shape[0]) if W.dim() > 1 else (1, W.numel())
-    _check(lib().twn_ternarize(_ptr(W), C.c_int64(rows), C.c_int64(cols), C.c_double(delta_factor),
-                               _ptr(stats), _ptr(packed), C.c_int64(ld_codes), _ptr(codes_i8),
-                               _ptr(workspace), C.c_size_t(workspace.numel() * workspace.element_size()),
-                               _stream(stream)), "twn_ternarize")
+    _check(_C.ternarize(W, rows, cols, delta_factor, stats, packed, ld_codes, codes_i8, workspace, stream),
+           "twn_ternarize")
 
 
 def sgd_update(W: torch.Tensor, dW: torch.Tensor, V: torch.Tensor, lr: float, momentum: float,
                weight_decay: float, delta_factor: float, stats_next, workspace: torch.Tensor, stream=None) -> None:
     """twn_sgd_update: in-place SGD step on the fp32 master weights; stats_next (optional) receives
     the threshold of the updated weights."""
-    _check(lib().twn_sgd_update(_ptr(W), _ptr(dW), _ptr(V), C.c_int64(W.numel()), C.c_float(lr),
-                                C.c_float(momentum), C.c_float(weight_decay), C.c_double(delta_factor),
-                                _ptr(stats_next), _ptr(workspace),
-                                C.c_size_t(workspace.numel() * workspace.element_size()), _stream(stream)),
+    _check(_C.sgd_update(W, dW, V, W.numel(), lr, momentum, weight_decay, delta_factor, stats_next, workspace, stream),
            "twn_sgd_update")
 
 
 def ternarize_codes(W: torch.Tensor, rows: int, cols: int, stats: torch.Tensor, packed: torch.Tensor,
                     ld_codes: int, codes_i8, workspace: torch.Tensor, stream=None) -> None:
     """twn_ternarize_codes: the coding sweep alone, against the threshold already in `stats`."""
-    _check(lib().twn_ternarize_codes(_ptr(W), C.c_int64(rows), C.c_int64(cols), _ptr(stats), _ptr(packed),
-                                     C.c_int64(ld_codes), _ptr(codes_i8), _ptr(workspace),
-                                     C.c_size_t(workspace.numel() * workspace.element_size()),
-                                     _stream(stream)), "twn_ternarize_codes")
-
-
-class TernarizeItem(C.Structure):
-    _fields_ = [("W", C.c_void_p), ("rows", C.c_int64), ("cols", C.c_int64), ("stats", C.c_void_p),
-                ("packed", C.c_void_p), ("ld_codes", C.c_int64), ("codes_i8", C.c_void_p)]
+    _check(_C.ternarize_codes(W, rows, cols, stats, packed, ld_codes, codes_i8, workspace, stream),
+           "twn_ternarize_codes")
 
 
 def ternarize_batch_workspace_bytes(count: int) -> int:
@@ -167,54 +168,24 @@ def ternarize_batch_workspace_bytes(count: int) -> int:
 
 def ternarize_batch(items, delta_factor: float, workspace: torch.Tensor, stream=None) -> None:
     """twn_ternarize_batch.  items: list of (W, rows, cols, stats, packed, ld_codes, codes_i8 or None)."""
-    arr = (TernarizeItem * max(len(items), 1))()
-    for i, (W, rows, cols, stats, packed, ld, codes) in enumerate(items):
-        arr[i] = TernarizeItem(_ptr(W).value, rows, cols, _ptr(stats).value, _ptr(packed).value, ld,
-                               _ptr(codes).value)
-    _check(lib().twn_ternarize_batch(arr, C.c_int(len(items)), C.c_double(delta_factor), _ptr(workspace),
-                                     C.c_size_t(workspace.numel() * workspace.element_size()),
-                                     _stream(stream)), "twn_ternarize_batch")
-
-
-class SgdItem(C.Structure):
-    _fields_ = [("W", C.c_void_p), ("dW", C.c_void_p), ("V", C.c_void_p), ("n", C.c_int64), ("stats_next", C.c_void_p)]
+    _check(_C.ternarize_batch(items, delta_factor, workspace, stream), "twn_ternarize_batch")
 
 
 def sgd_update_batch(items, lr: float, momentum: float, weight_decay: float, delta_factor: float,
                      workspace: torch.Tensor, stream=None) -> None:
     """twn_sgd_update_batch.  items: list of (W, dW, V, stats_next or None)."""
-    arr = (SgdItem * max(len(items), 1))()
-    for i, (W, dW, V, st) in enumerate(items):
-        assert dW.numel() == W.numel() == V.numel()
-        arr[i] = SgdItem(_ptr(W).value, _ptr(dW).value, _ptr(V).value, W.numel(), _ptr(st).value)
-    _check(lib().twn_sgd_update_batch(arr, C.c_int(len(items)), C.c_float(lr), C.c_float(momentum),
-                                      C.c_float(weight_decay), C.c_double(delta_factor), _ptr(workspace),
-                                      C.c_size_t(workspace.numel() * workspace.element_size()), _stream(stream)),
+    _check(_C.sgd_update_batch(items, lr, momentum, weight_decay, delta_factor, workspace, stream),
            "twn_sgd_update_batch")
 
 
 def ternarize_codes_batch(items, workspace: torch.Tensor, stream=None) -> None:
     """twn_ternarize_codes_batch.  items as for ternarize_batch; every stats holds its threshold already."""
-    arr = (TernarizeItem * max(len(items), 1))()
-    for i, (W, rows, cols, stats, packed, ld, codes) in enumerate(items):
-        arr[i] = TernarizeItem(_ptr(W).value, rows, cols, _ptr(stats).value, _ptr(packed).value, ld,
-                               _ptr(codes).value)
-    _check(lib().twn_ternarize_codes_batch(arr, C.c_int(len(items)), _ptr(workspace),
-                                           C.c_size_t(workspace.numel() * workspace.element_size()),
-                                           _stream(stream)), "twn_ternarize_codes_batch")
-
-
-class TransposeItem(C.Structure):
-    _fields_ = [("packed_fwd", C.c_void_p), ("ld_fwd", C.c_int64), ("desc", ConvDesc), ("packed_bwd", C.c_void_p),
-                ("ld_bwd", C.c_int64)]
+    _check(_C.ternarize_codes_batch(items, workspace, stream), "twn_ternarize_codes_batch")
 
 
 def transpose_codes_batch(items, stream=None) -> None:
     """twn_transpose_codes_batch.  items: list of (packed_fwd, ld_fwd, desc, packed_bwd, ld_bwd)."""
-    arr = (TransposeItem * max(len(items), 1))()
-    for i, (pf, ldf, desc, pb, ldb) in enumerate(items):
-        arr[i] = TransposeItem(_ptr(pf).value, ldf, desc, _ptr(pb).value, ldb)
-    _check(lib().twn_transpose_codes_batch(arr, C.c_int(len(items)), _stream(stream)), "twn_transpose_codes_batch")
+    _check(_C.transpose_codes_batch(items, stream), "twn_transpose_codes_batch")
 
 
 def ternarize_rows(W: torch.Tensor, delta_factor: float, stats: torch.Tensor, packed: torch.Tensor,
@@ -223,16 +194,14 @@ def ternarize_rows(W: torch.Tensor, delta_factor: float, stats: torch.Tensor, pa
     stats int64 [rows, 8] (one twn_stats_t per row)."""
     rows, cols = W.shape[0], W.numel() // max(W.shape[0], 1)
     assert stats.numel() * stats.element_size() >= 64 * rows
-    _check(lib().twn_ternarize_rows(_ptr(W), C.c_int64(rows), C.c_int64(cols), C.c_double(delta_factor),
-                                    _ptr(stats), _ptr(packed), C.c_int64(ld_codes), _ptr(codes_i8),
-                                    _stream(stream)), "twn_ternarize_rows")
+    _check(_C.ternarize_rows(W, rows, cols, delta_factor, stats, packed, ld_codes, codes_i8, stream),
+           "twn_ternarize_rows")
 
 
 def rows_scale(stats: torch.Tensor, rows: int, scale_in, scale_out: torch.Tensor, dev_status=None,
                stream=None) -> None:
     """twn_rows_scale: scale_out[r] = alpha_r * scale_in[r]."""
-    _check(lib().twn_rows_scale(_ptr(stats), C.c_int64(rows), _ptr(scale_in), _ptr(scale_out),
-                                _ptr(dev_status), _stream(stream)), "twn_rows_scale")
+    _check(_C.rows_scale(stats, rows, scale_in, scale_out, dev_status, stream), "twn_rows_scale")
 
 
 def new_stats_rows(rows: int, device="cuda") -> torch.Tensor:
@@ -259,29 +228,23 @@ def ternarize_static(W: torch.Tensor, delta_factor: float, stats: torch.Tensor, 
     for callers that cannot allocate device memory.  Calls on one device must not overlap."""
     if rows is None:
         rows, cols = (W.shape[0], W.numel() // W.shape[0]) if W.dim() > 1 else (1, W.numel())
-    _check(lib().twn_ternarize_static(_ptr(W), C.c_int64(rows), C.c_int64(cols),
-                                      C.c_double(delta_factor), _ptr(stats), _ptr(packed),
-                                      C.c_int64(ld_codes), _ptr(codes_i8), _stream(stream)),
+    _check(_C.ternarize_static(W, rows, cols, delta_factor, stats, packed, ld_codes, codes_i8, stream),
            "twn_ternarize_static")
 
 
 def pack(codes: torch.Tensor, rows: int, cols: int, packed: torch.Tensor, ld_codes: int,
          counts=None, stream=None) -> None:
-    _check(lib().twn_pack(_ptr(codes), C.c_int64(rows), C.c_int64(cols), _ptr(packed),
-                          C.c_int64(ld_codes), _ptr(counts), _stream(stream)), "twn_pack")
+    _check(_C.pack(codes, rows, cols, packed, ld_codes, counts, stream), "twn_pack")
 
 
 def unpack(packed: torch.Tensor, rows: int, cols: int, ld_codes: int, codes: torch.Tensor,
            dev_status=None, stream=None) -> None:
-    _check(lib().twn_unpack(_ptr(packed), C.c_int64(rows), C.c_int64(cols), C.c_int64(ld_codes),
-                            _ptr(codes), _ptr(dev_status), _stream(stream)), "twn_unpack")
+    _check(_C.unpack(packed, rows, cols, ld_codes, codes, dev_status, stream), "twn_unpack")
 
 
 def transpose_codes(packed_fwd: torch.Tensor, ld_fwd: int, desc: ConvDesc, packed_bwd: torch.Tensor,
                     ld_bwd: int, stream=None) -> None:
-    _check(lib().twn_transpose_codes(_ptr(packed_fwd), C.c_int64(ld_fwd), C.byref(desc),
-                                     _ptr(packed_bwd), C.c_int64(ld_bwd), _stream(stream)),
-           "twn_transpose_codes")
+    _check(_C.transpose_codes(packed_fwd, ld_fwd, desc, packed_bwd, ld_bwd, stream), "twn_transpose_codes")
 
 
 RESIDUAL_ADD, RESIDUAL_GATE = 0, 1
@@ -289,34 +252,20 @@ RESIDUAL_ADD, RESIDUAL_GATE = 0, 1
 
 def epilogue(scale=None, shift=None, residual=None, relu=False, out_dtype=F32, residual_op=RESIDUAL_ADD):
     """Builds a twn_epilogue_t; keeps no reference, the caller keeps the tensors alive."""
-    e = Epilogue()
-    e.scale = _ptr(scale).value or None
-    e.shift = _ptr(shift).value or None
-    e.residual = _ptr(residual).value or None
-    e.residual_dtype = BF16 if (residual is not None and residual.dtype == torch.bfloat16) else F32
-    e.relu = int(bool(relu))
-    e.out_dtype = out_dtype
-    e.residual_op = residual_op
+    e = Epilogue(_ptr(scale).value, _ptr(shift).value, _ptr(residual).value,
+                 BF16 if (residual is not None and residual.dtype == torch.bfloat16) else F32,
+                 int(bool(relu)), out_dtype, residual_op)
     return e
-
-
-def _alpha_stats(stats):
-    return _ptr(stats)
 
 
 def gemm(X: torch.Tensor, ldx: int, T_packed: torch.Tensor, ld_codes: int, stats, M: int, N: int,
          K: int, epi, Y: torch.Tensor, ldy: int, dev_status=None, stream=None) -> None:
-    _check(lib().twn_gemm(_ptr(X), C.c_int64(ldx), _ptr(T_packed), C.c_int64(ld_codes), _ptr(stats),
-                          C.c_int64(M), C.c_int64(N), C.c_int64(K),
-                          C.byref(epi) if epi is not None else None, _ptr(Y), C.c_int64(ldy),
-                          _ptr(dev_status), _stream(stream)), "twn_gemm")
+    _check(_C.gemm(X, ldx, T_packed, ld_codes, stats, M, N, K, epi, Y, ldy, dev_status, stream), "twn_gemm")
 
 
 def conv2d_fwd(desc: ConvDesc, X: torch.Tensor, T_fwd: torch.Tensor, ld_codes: int, stats, epi,
                Y: torch.Tensor, dev_status=None, stream=None) -> None:
-    _check(lib().twn_conv2d_fwd(C.byref(desc), _ptr(X), _ptr(T_fwd), C.c_int64(ld_codes), _ptr(stats),
-                                C.byref(epi) if epi is not None else None, _ptr(Y), _ptr(dev_status),
-                                _stream(stream)), "twn_conv2d_fwd")
+    _check(_C.conv2d_fwd(desc, X, T_fwd, ld_codes, stats, epi, Y, dev_status, stream), "twn_conv2d_fwd")
 
 
 def conv2d_fwd_bn_workspace_bytes(desc: ConvDesc) -> int:
@@ -326,24 +275,19 @@ def conv2d_fwd_bn_workspace_bytes(desc: ConvDesc) -> int:
 def conv2d_fwd_bn(desc: ConvDesc, X: torch.Tensor, T_fwd: torch.Tensor, ld_codes: int, stats, epi, Y: torch.Tensor,
                   bn_sum: torch.Tensor, bn_sumsq: torch.Tensor, workspace: torch.Tensor, dev_status=None,
                   stream=None) -> None:
-    _check(lib().twn_conv2d_fwd_bn(C.byref(desc), _ptr(X), _ptr(T_fwd), C.c_int64(ld_codes), _ptr(stats),
-                                   C.byref(epi) if epi is not None else None, _ptr(Y), _ptr(bn_sum), _ptr(bn_sumsq),
-                                   _ptr(workspace), C.c_size_t(workspace.numel()), _ptr(dev_status), _stream(stream)),
+    _check(_C.conv2d_fwd_bn(desc, X, T_fwd, ld_codes, stats, epi, Y, bn_sum, bn_sumsq, workspace, dev_status, stream),
            "twn_conv2d_fwd_bn")
 
 
 def bn_finalize(bn_sum: torch.Tensor, bn_sumsq: torch.Tensor, n: int, C_: int, gamma, beta, eps: float, scale, shift,
                 mean=None, var=None, stream=None) -> None:
-    _check(lib().twn_bn_finalize(_ptr(bn_sum), _ptr(bn_sumsq), C.c_int64(n), C.c_int64(C_), _ptr(gamma), _ptr(beta),
-                                 C.c_double(eps), _ptr(scale), _ptr(shift), _ptr(mean), _ptr(var), _stream(stream)),
+    _check(_C.bn_finalize(bn_sum, bn_sumsq, n, C_, gamma, beta, eps, scale, shift, mean, var, stream),
            "twn_bn_finalize")
 
 
 def conv2d_bwd_data(desc: ConvDesc, dZ: torch.Tensor, T_bwd: torch.Tensor, ld_codes: int, stats, epi,
                     dX: torch.Tensor, dev_status=None, stream=None) -> None:
-    _check(lib().twn_conv2d_bwd_data(C.byref(desc), _ptr(dZ), _ptr(T_bwd), C.c_int64(ld_codes),
-                                     _ptr(stats), C.byref(epi) if epi is not None else None, _ptr(dX),
-                                     _ptr(dev_status), _stream(stream)), "twn_conv2d_bwd_data")
+    _check(_C.conv2d_bwd_data(desc, dZ, T_bwd, ld_codes, stats, epi, dX, dev_status, stream), "twn_conv2d_bwd_data")
 
 
 # ---- binary precision weights: the same calls on 1-bit codes
@@ -360,46 +304,36 @@ def binarize(W: torch.Tensor, stats: torch.Tensor, packed: torch.Tensor, ld_code
              stream=None, rows: int | None = None, cols: int | None = None) -> None:
     if rows is None:
         rows, cols = (W.shape[0], W.numel() // W.shape[0]) if W.dim() > 1 else (1, W.numel())
-    _check(lib().twn_binarize(_ptr(W), C.c_int64(rows), C.c_int64(cols), _ptr(stats), _ptr(packed),
-                              C.c_int64(ld_codes), _ptr(workspace), C.c_size_t(workspace.numel()), _stream(stream)),
-           "twn_binarize")
+    _check(_C.binarize(W, rows, cols, stats, packed, ld_codes, workspace, stream), "twn_binarize")
 
 
 def unpack_b1(packed: torch.Tensor, rows: int, cols: int, ld_codes: int, codes: torch.Tensor, stream=None) -> None:
-    _check(lib().twn_unpack_b1(_ptr(packed), C.c_int64(rows), C.c_int64(cols), C.c_int64(ld_codes), _ptr(codes),
-                               _stream(stream)), "twn_unpack_b1")
+    _check(_C.unpack_b1(packed, rows, cols, ld_codes, codes, stream), "twn_unpack_b1")
 
 
 def transpose_codes_b1(packed_fwd: torch.Tensor, ld_fwd: int, desc: ConvDesc, packed_bwd: torch.Tensor, ld_bwd: int,
                        stream=None) -> None:
-    _check(lib().twn_transpose_codes_b1(_ptr(packed_fwd), C.c_int64(ld_fwd), C.byref(desc), _ptr(packed_bwd),
-                                        C.c_int64(ld_bwd), _stream(stream)), "twn_transpose_codes_b1")
+    _check(_C.transpose_codes_b1(packed_fwd, ld_fwd, desc, packed_bwd, ld_bwd, stream), "twn_transpose_codes_b1")
 
 
 def gemm_b1(X: torch.Tensor, ldx: int, B_packed: torch.Tensor, ld_codes: int, stats, M: int, N: int,
             K: int, epi, Y: torch.Tensor, ldy: int, dev_status=None, stream=None) -> None:
-    _check(lib().twn_gemm_b1(_ptr(X), C.c_int64(ldx), _ptr(B_packed), C.c_int64(ld_codes), _ptr(stats),
-                             C.c_int64(M), C.c_int64(N), C.c_int64(K),
-                             C.byref(epi) if epi is not None else None, _ptr(Y), C.c_int64(ldy),
-                             _ptr(dev_status), _stream(stream)), "twn_gemm_b1")
+    _check(_C.gemm_b1(X, ldx, B_packed, ld_codes, stats, M, N, K, epi, Y, ldy, dev_status, stream), "twn_gemm_b1")
 
 
 def conv2d_fwd_b1(desc: ConvDesc, X: torch.Tensor, B_fwd: torch.Tensor, ld_codes: int, stats, epi,
                   Y: torch.Tensor, dev_status=None, stream=None) -> None:
-    _check(lib().twn_conv2d_fwd_b1(C.byref(desc), _ptr(X), _ptr(B_fwd), C.c_int64(ld_codes), _ptr(stats),
-                                   C.byref(epi) if epi is not None else None, _ptr(Y), _ptr(dev_status),
-                                   _stream(stream)), "twn_conv2d_fwd_b1")
+    _check(_C.conv2d_fwd_b1(desc, X, B_fwd, ld_codes, stats, epi, Y, dev_status, stream), "twn_conv2d_fwd_b1")
 
 
 def conv2d_bwd_data_b1(desc: ConvDesc, dZ: torch.Tensor, B_bwd: torch.Tensor, ld_codes: int, stats, epi,
                        dX: torch.Tensor, dev_status=None, stream=None) -> None:
-    _check(lib().twn_conv2d_bwd_data_b1(C.byref(desc), _ptr(dZ), _ptr(B_bwd), C.c_int64(ld_codes),
-                                        _ptr(stats), C.byref(epi) if epi is not None else None, _ptr(dX),
-                                        _ptr(dev_status), _stream(stream)), "twn_conv2d_bwd_data_b1")
+    _check(_C.conv2d_bwd_data_b1(desc, dZ, B_bwd, ld_codes, stats, epi, dX, dev_status, stream),
+           "twn_conv2d_bwd_data_b1")
 
 
 def im2col(desc: ConvDesc, X: torch.Tensor, Xcol: torch.Tensor, ldk: int, stream=None) -> None:
-    _check(lib().twn_im2col(C.byref(desc), _ptr(X), _ptr(Xcol), C.c_int64(ldk), _stream(stream)), "twn_im2col")
+    _check(_C.im2col(desc, X, Xcol, ldk, stream), "twn_im2col")
 
 
 def fold_dims(desc: ConvDesc):
@@ -411,18 +345,15 @@ def fold_dims(desc: ConvDesc):
 
 
 def fold_input(desc: ConvDesc, X, Xf, stream=None) -> None:
-    _check(lib().twn_fold_input(C.byref(desc), _ptr(X), _ptr(Xf), _stream(stream)), "twn_fold_input")
+    _check(_C.fold_input(desc, X, Xf, stream), "twn_fold_input")
 
 
 def fold_codes(desc: ConvDesc, packed, ld_codes: int, packed_folded, ld_folded: int, stream=None) -> None:
-    _check(lib().twn_fold_codes(C.byref(desc), _ptr(packed), C.c_int64(ld_codes), _ptr(packed_folded),
-                                C.c_int64(ld_folded), _stream(stream)), "twn_fold_codes")
+    _check(_C.fold_codes(desc, packed, ld_codes, packed_folded, ld_folded, stream), "twn_fold_codes")
 
 
 def conv2d_fwd_folded(desc: ConvDesc, Xf, Tf, ld_folded: int, stats, epi, Y, dev_status=None, stream=None) -> None:
-    _check(lib().twn_conv2d_fwd_folded(C.byref(desc), _ptr(Xf), _ptr(Tf), C.c_int64(ld_folded), _ptr(stats),
-                                       C.byref(epi) if epi is not None else None, _ptr(Y), _ptr(dev_status),
-                                       _stream(stream)), "twn_conv2d_fwd_folded")
+    _check(_C.conv2d_fwd_folded(desc, Xf, Tf, ld_folded, stats, epi, Y, dev_status, stream), "twn_conv2d_fwd_folded")
 
 
 def conv2d_bwd_weight_folded_workspace_bytes(desc: ConvDesc) -> int:
@@ -430,42 +361,32 @@ def conv2d_bwd_weight_folded_workspace_bytes(desc: ConvDesc) -> int:
 
 
 def conv2d_bwd_weight_folded(desc: ConvDesc, Xf, dZ, dW, workspace, dev_status=None, stream=None) -> None:
-    _check(lib().twn_conv2d_bwd_weight_folded(C.byref(desc), _ptr(Xf), _ptr(dZ), _ptr(dW), _ptr(workspace),
-                                              C.c_size_t(workspace.numel() * workspace.element_size()),
-                                              _ptr(dev_status), _stream(stream)), "twn_conv2d_bwd_weight_folded")
+    _check(_C.conv2d_bwd_weight_folded(desc, Xf, dZ, dW, workspace, dev_status, stream), "twn_conv2d_bwd_weight_folded")
 
 
 def maxpool2d_fwd(X, B, H, W, Cc, k, stride, pad, Y, argmax=None, stream=None) -> None:
-    _check(lib().twn_maxpool2d_fwd(_ptr(X), C.c_int64(B), C.c_int64(H), C.c_int64(W), C.c_int64(Cc),
-                                   C.c_int(k), C.c_int(stride), C.c_int(pad), _ptr(Y), _ptr(argmax),
-                                   _stream(stream)), "twn_maxpool2d_fwd")
+    _check(_C.maxpool2d_fwd(X, B, H, W, Cc, k, stride, pad, Y, argmax, stream), "twn_maxpool2d_fwd")
 
 
 def maxpool2d_bwd(dY, argmax, B, H, W, Cc, k, stride, pad, dX, stream=None) -> None:
-    _check(lib().twn_maxpool2d_bwd(_ptr(dY), _ptr(argmax), C.c_int64(B), C.c_int64(H), C.c_int64(W),
-                                   C.c_int64(Cc), C.c_int(k), C.c_int(stride), C.c_int(pad), _ptr(dX),
-                                   _stream(stream)), "twn_maxpool2d_bwd")
+    _check(_C.maxpool2d_bwd(dY, argmax, B, H, W, Cc, k, stride, pad, dX, stream), "twn_maxpool2d_bwd")
 
 
 def maxpool2d_bwd_act(dY, argmax, pooled, scale, B, H, W, Cc, k, stride, pad, dZ, stream=None) -> None:
-    _check(lib().twn_maxpool2d_bwd_act(_ptr(dY), _ptr(argmax), _ptr(pooled), _ptr(scale), C.c_int64(B),
-                                       C.c_int64(H), C.c_int64(W), C.c_int64(Cc), C.c_int(k), C.c_int(stride),
-                                       C.c_int(pad), _ptr(dZ), _stream(stream)), "twn_maxpool2d_bwd_act")
+    _check(_C.maxpool2d_bwd_act(dY, argmax, pooled, scale, B, H, W, Cc, k, stride, pad, dZ, stream),
+           "twn_maxpool2d_bwd_act")
 
 
 def avgpool_fwd(X, B, HW, Cc, Y, stream=None) -> None:
-    _check(lib().twn_avgpool_fwd(_ptr(X), C.c_int64(B), C.c_int64(HW), C.c_int64(Cc), _ptr(Y),
-                                 _stream(stream)), "twn_avgpool_fwd")
+    _check(_C.avgpool_fwd(X, B, HW, Cc, Y, stream), "twn_avgpool_fwd")
 
 
 def avgpool_bwd(dY, B, HW, Cc, dX, stream=None) -> None:
-    _check(lib().twn_avgpool_bwd(_ptr(dY), C.c_int64(B), C.c_int64(HW), C.c_int64(Cc), _ptr(dX),
-                                 _stream(stream)), "twn_avgpool_bwd")
+    _check(_C.avgpool_bwd(dY, B, HW, Cc, dX, stream), "twn_avgpool_bwd")
 
 
 def act_bwd(dY, Y, scale, n, Cc, dZ, dPre=None, stream=None) -> None:
-    _check(lib().twn_act_bwd(_ptr(dY), _ptr(Y), _ptr(scale), C.c_int64(n), C.c_int64(Cc), _ptr(dZ),
-                             _ptr(dPre), _stream(stream)), "twn_act_bwd")
+    _check(_C.act_bwd(dY, Y, scale, n, Cc, dZ, dPre, stream), "twn_act_bwd")
 
 
 def conv2d_bwd_weight_workspace_bytes(desc: ConvDesc) -> int:
@@ -473,6 +394,4 @@ def conv2d_bwd_weight_workspace_bytes(desc: ConvDesc) -> int:
 
 
 def conv2d_bwd_weight(desc: ConvDesc, X, dZ, dW, workspace, dev_status=None, stream=None) -> None:
-    _check(lib().twn_conv2d_bwd_weight(C.byref(desc), _ptr(X), _ptr(dZ), _ptr(dW), _ptr(workspace),
-                                       C.c_size_t(workspace.numel() * workspace.element_size()),
-                                       _ptr(dev_status), _stream(stream)), "twn_conv2d_bwd_weight")
+    _check(_C.conv2d_bwd_weight(desc, X, dZ, dW, workspace, dev_status, stream), "twn_conv2d_bwd_weight")
