@@ -1,249 +1,129 @@
 // Threshold ternarization fused with 2-bit packing (Sec. 2.3: Eq. 3, Eq. 5 and the
-// threshold rule; Algorithm 1, first loop), plus the standalone pack / unpack /
+// threshold rule; Algorithm 1, first loop), the parameter update, plus the standalone pack / unpack /
 // re-layout kernels.
 //
-// Two sweeps over the fp32 master weights, both bound by HBM bandwidth:
-//   sweep 1  S = sum |W_i| in fp64  ->  delta = factor * S / n
-//   sweep 2  codes by Eq. 3, packed 16 per word; sum and count of the kept set
+// Ternarization is one launch of two phases, bound by HBM bandwidth:
+//   phase 1  S = sum |W_i| in fp64  ->  delta = factor * S / n
+//   phase 2  codes by Eq. 3, packed 16 per word; sum and count of the kept set
 //            ->  alpha (Eq. 5)
-// Sweep 2 walks the tensor back to front so that what sweep 1 read last is still
-// in L2.  Both reductions have a fixed order: per-thread strided partial sums,
-// a shuffle tree per warp, a shared-memory tree per block, one partial per block
-// in the workspace, and the block that finishes last folds the partials in index
-// order.  No floating-point atomics, no waiting on other blocks.
+// with a barrier of all blocks between them (grid-wide in a cooperative launch, a cluster's for small tensors).
+// Phase 2 walks every block's share back to front, so that what phase 1 read last comes from L1 and L2.
+//
+// All sums have a fixed order that depends on the shape of the tensor alone: a tensor is cut into at most
+// kMaxParts parts, every part is summed by one block in a fixed way (per-thread strided sums, shuffle tree per
+// warp, warps in order) and the parts are folded in a fixed way.  Which block takes a part does not matter, so a
+// tensor gets the same bits alone and in a batch, on any number of SMs.  No floating-point atomics.
+#include <cooperative_groups.h>
+
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace {
 
-constexpr int kThreads = 256;
+constexpr int kThreads = 256;       // pack, unpack, re-layouts
 constexpr int kWarps = kThreads / 32;
-constexpr int kMaxBlocks = 2048;
-// workspace: [0,256) tickets, then four arrays of kMaxBlocks 8-byte partials
-constexpr size_t kWorkspaceBytes = 256 + 4 * size_t(kMaxBlocks) * 8;
+constexpr int kSweepWarps = 16;
+constexpr int kSweepThreads = 32 * kSweepWarps;
+constexpr int kSweepBlocksPerSm = 2;                        // 64 registers; three blocks spill: 1e8 weights 131 -> 164 us
+constexpr unsigned int kMaxParts = kSweepBlocksPerSm * 148;  // one part per block of a full grid
+// A tensor of up to 8192 words (131072 weights) is "small": at most eight parts of up to 8 x 128 words, so that
+// one cluster of eight blocks holds it in registers, eight quarter-words per thread.
+constexpr int kSmallParts = 8, kSmallQuarters = 8, kQuarterWords = kSweepThreads / 4;
+constexpr unsigned long long kSmallWords = kSmallParts * kSmallQuarters * kQuarterWords;
+// workspace: [0,256) counters, then arrays of 8-byte partials
+constexpr size_t kWorkspaceBytes = 65792;
+static_assert(256 + 3 * kMaxParts * 8 <= kWorkspaceBytes, "the partial sums fit in the workspace");
+constexpr int kMaxBatch = 32;
 
 struct Workspace {
-    unsigned int *ticket1;
-    unsigned int *ticket2;
+    unsigned int *done;             // parts whose second sums are written
     double *part_sum;
     double *part_kept;
-    unsigned long long *part_pos;
-    unsigned long long *part_neg;
+    unsigned long long *part_cnt;   // negatives in the high half, positives in the low half
 };
 
-__host__ __device__ inline Workspace carve(void *ws)
+__host__ __device__ inline Workspace carve(void *ws, int t)
 {
-    char *b = static_cast<char *>(ws);
+    char *b = static_cast<char *>(ws) + (size_t)t * kWorkspaceBytes;
     Workspace w;
-    w.ticket1 = reinterpret_cast<unsigned int *>(b);
-    w.ticket2 = reinterpret_cast<unsigned int *>(b + 64);
+    w.done = reinterpret_cast<unsigned int *>(b);
     w.part_sum = reinterpret_cast<double *>(b + 256);
-    w.part_kept = w.part_sum + kMaxBlocks;
-    w.part_pos = reinterpret_cast<unsigned long long *>(w.part_kept + kMaxBlocks);
-    w.part_neg = w.part_pos + kMaxBlocks;
+    w.part_kept = w.part_sum + kMaxParts;
+    w.part_cnt = reinterpret_cast<unsigned long long *>(w.part_kept + kMaxParts);
     return w;
 }
 
-__device__ __forceinline__ double warp_sum(double v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    return v;
-}
-
-__device__ __forceinline__ unsigned long long warp_sum(unsigned long long v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    return v;
-}
-
-// Block-wide sum with a fixed order; the result is valid in thread 0.
 template <typename T>
-__device__ __forceinline__ T block_sum(T v, T *smem /* kWarps entries */)
+__device__ __forceinline__ T warp_sum(T v)
 {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    return v;
+}
+
+// Block-wide sums with a fixed order: a shuffle tree per warp, then every thread adds the sixteen warps' sums in
+// the same tree, so that one barrier does and nobody waits for a broadcast.  The buffers alternate from call to
+// call (`turn`): a buffer is written again two barriers later, when all have read it.
+struct Reduce {
+    double sum[2][kSweepWarps];
+    uint2 cnt[2][kSweepWarps];
+};
+__device__ __forceinline__ double tree16(const double *v)
+{
+    double t[kSweepWarps / 2];
+#pragma unroll
+    for (int i = 0; i < kSweepWarps / 2; ++i) t[i] = v[i] + v[i + kSweepWarps / 2];
+#pragma unroll
+    for (int o = kSweepWarps / 4; o > 0; o >>= 1)
+#pragma unroll
+        for (int i = 0; i < o; ++i) t[i] += t[i + o];
+    return t[0];
+}
+__device__ __forceinline__ double sweep_sum(double v, Reduce &red, unsigned int &turn)
+{
+    double *buf = red.sum[turn & 1];
+    ++turn;
     v = warp_sum(v);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if ((threadIdx.x & 31) == 0) buf[threadIdx.x >> 5] = v;
     __syncthreads();
-    if (lane == 0) smem[warp] = v;
+    return tree16(buf);
+}
+// The same for a sum and two counts of the block (below 2^32).
+__device__ __forceinline__ double sweep_sum(double v, unsigned int &pos, unsigned int &neg, Reduce &red, unsigned int &turn)
+{
+    double *buf = red.sum[turn & 1];
+    uint2 *cnt = red.cnt[turn & 1];
+    ++turn;
+    v = warp_sum(v);
+    const unsigned int p = __reduce_add_sync(0xffffffffu, pos), q = __reduce_add_sync(0xffffffffu, neg);
+    if ((threadIdx.x & 31) == 0) { buf[threadIdx.x >> 5] = v; cnt[threadIdx.x >> 5] = make_uint2(p, q); }
     __syncthreads();
-    T r = T(0);
-    if (warp == 0) {
-        r = lane < kWarps ? smem[lane] : T(0);
-        r = warp_sum(r);
-    }
-    return r;
+    pos = neg = 0;
+#pragma unroll
+    for (int i = 0; i < kSweepWarps; ++i) { pos += cnt[i].x; neg += cnt[i].y; }
+    return tree16(buf);
 }
 
-// Returns true in every thread of the block that took the last of `grid` tickets.
-__device__ __forceinline__ bool last_block(unsigned int *ticket, unsigned int grid)
-{
-    __shared__ bool is_last;
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) is_last = (atomicAdd(ticket, 1u) == grid - 1);
-    __syncthreads();
-    return is_last;
-}
-
-// ---- sweep 1 -------------------------------------------------------------
-// `vb` of `vg`: this block's index and the number of blocks that work on this tensor (the whole
-// grid for a single tensor, a slice of it when several tensors share one launch).
-__device__ __forceinline__ void sum_abs_body(const float *__restrict__ W, long long n, double factor, const Workspace ws,
-                                             twn_stats_t *__restrict__ stats, unsigned int vb, unsigned int vg)
-{
-    __shared__ double red[kWarps];
-    const long long n4 = n >> 2;
-    const float4 *W4 = reinterpret_cast<const float4 *>(W);
-    const long long stride = (long long)vg * kThreads;
-    long long i = (long long)vb * kThreads + threadIdx.x;
-
-    double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-    for (; i + 3 * stride < n4; i += 4 * stride) {
-        const float4 v0 = __ldg(W4 + i);
-        const float4 v1 = __ldg(W4 + i + stride);
-        const float4 v2 = __ldg(W4 + i + 2 * stride);
-        const float4 v3 = __ldg(W4 + i + 3 * stride);
-        a0 += (double)fabsf(v0.x); a1 += (double)fabsf(v0.y); a2 += (double)fabsf(v0.z); a3 += (double)fabsf(v0.w);
-        a0 += (double)fabsf(v1.x); a1 += (double)fabsf(v1.y); a2 += (double)fabsf(v1.z); a3 += (double)fabsf(v1.w);
-        a0 += (double)fabsf(v2.x); a1 += (double)fabsf(v2.y); a2 += (double)fabsf(v2.z); a3 += (double)fabsf(v2.w);
-        a0 += (double)fabsf(v3.x); a1 += (double)fabsf(v3.y); a2 += (double)fabsf(v3.z); a3 += (double)fabsf(v3.w);
-    }
-    for (; i < n4; i += stride) {
-        const float4 v = __ldg(W4 + i);
-        a0 += (double)fabsf(v.x); a1 += (double)fabsf(v.y); a2 += (double)fabsf(v.z); a3 += (double)fabsf(v.w);
-    }
-    // scalar tail (n % 4 elements), by the first threads of block 0
-    if (vb == 0) {
-        const long long t = (n4 << 2) + threadIdx.x;
-        if (t < n) a0 += (double)fabsf(__ldg(W + t));
-    }
-    const double bsum = block_sum((a0 + a1) + (a2 + a3), red);
-    if (threadIdx.x == 0) ws.part_sum[vb] = bsum;
-
-    if (last_block(ws.ticket1, vg)) {
-        double s = 0.0;
-        for (int b = threadIdx.x; b < (int)vg; b += kThreads) s += __ldcg(ws.part_sum + b);
-        s = block_sum(s, red);
-        if (threadIdx.x == 0) {
-            const double delta = n > 0 ? factor * (s / (double)n) : 0.0;
-            stats->sum_abs = s;
-            stats->delta = delta;
-            stats->status = isfinite(s) ? TWN_OK : TWN_ERR_NONFINITE;
-            stats->reserved = 0;
-            *ws.ticket1 = 0u;
-        }
-    }
-}
-
-__global__ void __launch_bounds__(kThreads)
-sum_abs_kernel(const float *__restrict__ W, long long n, double factor, void *ws_raw,
-               twn_stats_t *__restrict__ stats)
-{
-    sum_abs_body(W, n, factor, carve(ws_raw), stats, blockIdx.x, gridDim.x);
-}
-
-// ---- parameter update fused with sweep 1 of the next iteration -------------
-// Last step of Algorithm 1 (UpdateParameters: SGD with momentum and L2 weight decay on the fp32
-// master weights, Sec. 3):
-//     g = dW + wd * W;   V' = mu * V + g;   W' = W - lr * V'
-// every operation a separately rounded fp32 operation in this order (no fused multiply-add), so
-// the result is defined to the bit.  The next iteration starts by ternarizing W', whose
-// threshold needs sum |W'|: it is accumulated here while W' is still in registers, which saves
-// the first sweep of that ternarization (one read of the weights).
-__device__ __forceinline__ float sgd_one(float w, float g, float &v, float lr, float mu, float wd)
-{
-    const float grad = __fadd_rn(g, __fmul_rn(wd, w));
-    v = __fadd_rn(__fmul_rn(mu, v), grad);
-    return __fsub_rn(w, __fmul_rn(lr, v));
-}
-
-// `vb` of `vg`: this block's index among the blocks that work on this tensor.
-__device__ __forceinline__ void sgd_update_body(float *__restrict__ W, const float *__restrict__ dW, float *__restrict__ V,
-                                                long long n, float lr, float mu, float wd, double factor,
-                                                const Workspace ws, twn_stats_t *__restrict__ stats, unsigned int vb,
-                                                unsigned int vg)
-{
-    __shared__ double red[kWarps];
-    const long long n4 = n >> 2;
-    float4 *W4 = reinterpret_cast<float4 *>(W);
-    float4 *V4 = reinterpret_cast<float4 *>(V);
-    const float4 *G4 = reinterpret_cast<const float4 *>(dW);
-    const long long stride = (long long)vg * kThreads;
-    double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-#pragma unroll 2
-    for (long long i = (long long)vb * kThreads + threadIdx.x; i < n4; i += stride) {
-        float4 w = W4[i], v = V4[i];
-        const float4 g = __ldg(G4 + i);
-        w.x = sgd_one(w.x, g.x, v.x, lr, mu, wd);
-        w.y = sgd_one(w.y, g.y, v.y, lr, mu, wd);
-        w.z = sgd_one(w.z, g.z, v.z, lr, mu, wd);
-        w.w = sgd_one(w.w, g.w, v.w, lr, mu, wd);
-        W4[i] = w;
-        V4[i] = v;
-        a0 += (double)fabsf(w.x); a1 += (double)fabsf(w.y); a2 += (double)fabsf(w.z); a3 += (double)fabsf(w.w);
-    }
-    if (vb == 0) {
-        const long long t = (n4 << 2) + threadIdx.x;
-        if (t < n) {
-            float v = V[t];
-            const float w = sgd_one(W[t], __ldg(dW + t), v, lr, mu, wd);
-            W[t] = w;
-            V[t] = v;
-            a0 += (double)fabsf(w);
-        }
-    }
-    const double bsum = block_sum((a0 + a1) + (a2 + a3), red);
-    if (threadIdx.x == 0) ws.part_sum[vb] = bsum;
-    if (last_block(ws.ticket1, vg)) {
-        double s = 0.0;
-        for (int b = threadIdx.x; b < (int)vg; b += kThreads) s += __ldcg(ws.part_sum + b);
-        s = block_sum(s, red);
-        if (threadIdx.x == 0) {
-            if (stats) {
-                stats->sum_abs = s;
-                stats->delta = n > 0 ? factor * (s / (double)n) : 0.0;
-                stats->status = isfinite(s) ? TWN_OK : TWN_ERR_NONFINITE;
-                stats->reserved = 0;
-            }
-            *ws.ticket1 = 0u;
-        }
-    }
-}
-
-__global__ void __launch_bounds__(kThreads)
-sgd_update_kernel(float *__restrict__ W, const float *__restrict__ dW, float *__restrict__ V, long long n,
-                  float lr, float mu, float wd, double factor, void *ws_raw, twn_stats_t *__restrict__ stats)
-{
-    sgd_update_body(W, dW, V, n, lr, mu, wd, factor, carve(ws_raw), stats, blockIdx.x, gridDim.x);
-}
-
-// ---- sweep 2 -------------------------------------------------------------
-// 2-bit field of one weight: bit 0 = kept, bit 1 = negative  (00 / 01 / 11).
-__device__ __forceinline__ uint32_t code2(float w, float thr, double &kept_sum)
-{
-    const float a = fabsf(w);
-    const bool keep = a > thr;
-    if (keep) kept_sum += (double)a;
-    return keep ? (w < 0.0f ? 3u : 1u) : 0u;
-}
-
+// ---- the codes --------------------------------------------------------------
 // Bit position of element e (0..15) inside its word: even elements fill the low
 // half-word, odd elements the high half-word, each from the top down, so that a left
 // shift by 2*(e/2) brings the element's field to the top two bits of its half-word.
 __host__ __device__ __forceinline__ int field_pos(int e) { return 14 - 2 * (e >> 1) + 16 * (e & 1); }
 
-// Four consecutive weights -> one byte: low nibble = fields of elements 0 (upper) and 2,
-// high nibble = fields of elements 1 (upper) and 3.
-__device__ __forceinline__ uint32_t code8(const float4 v, float thr, double &k0, double &k1)
+// A "quarter byte" holds the 2-bit fields (bit 0 = kept, bit 1 = negative: 00 / 01 / 11) of four consecutive
+// weights: low nibble = elements 0 (upper) and 2, high nibble = elements 1 (upper) and 3.
+//
+// Bits 0..15 of x -> the even bits of the result.
+__device__ __forceinline__ uint32_t spread16(uint32_t x)
 {
-    uint32_t c = code2(v.x, thr, k0) << 2;
-    c |= code2(v.z, thr, k0);
-    c |= code2(v.y, thr, k1) << 6;
-    c |= code2(v.w, thr, k1) << 4;
-    return c;
+    x = (x | (x << 8)) & 0x00FF00FFu;
+    x = (x | (x << 4)) & 0x0F0F0F0Fu;
+    x = (x | (x << 2)) & 0x33333333u;
+    return (x | (x << 1)) & 0x55555555u;
 }
 
-// Bytes B0..B3 (as produced by code8 for four consecutive float4) -> the word of
+// Quarter bytes B0..B3 of sixteen consecutive weights -> the word of
 // those 16 elements: low half = low nibbles, high half = high nibbles, B0's on top.
 __device__ __forceinline__ uint32_t bytes_to_word(uint32_t r)
 {
@@ -267,7 +147,7 @@ __device__ __forceinline__ uint32_t word_to_bytes(uint32_t w)
     return __byte_perm(lo | (hi << 4), 0u, 0x0123);
 }
 
-// int8 image of the four fields of a code8 byte, in element order:
+// int8 image of the four fields of a quarter byte, in element order:
 // 00 -> 0x00, 01 -> 0x01, 11 -> 0xFF
 __device__ __forceinline__ uint32_t fields_to_i8x4(uint32_t c8)
 {
@@ -281,207 +161,663 @@ __device__ __forceinline__ uint32_t fields_to_i8x4(uint32_t c8)
     return r;
 }
 
-// Fast path geometry: a "unit" is 512 consecutive weights = 128 float4 = 32 words,
-// handled by one warp: lane l loads float4 (unit*128 + j*32 + l) for j = 0..3, so
-// every load instruction covers 512 contiguous bytes.  A 4x4 byte transpose inside
-// each group of four lanes then leaves lane l with the four bytes of word
-// unit*32 + (l%4)*8 + l/4, and the warp stores one contiguous 128-byte line.
-__device__ __forceinline__ void code_pack_body(const float *__restrict__ W, long long rows, long long cols,
-                                               long long ld_codes, long long fast_units, uint32_t *__restrict__ packed,
-                                               int8_t *__restrict__ codes_i8, const Workspace ws,
-                                               twn_stats_t *__restrict__ stats, unsigned int vb, unsigned int vg)
-{
-    __shared__ double red[kWarps];
-    __shared__ unsigned long long redu[kWarps];
-    const long long n = rows * cols;
-    // delta rounded toward -inf: for any float w,  w > delta  <=>  w > thr
-    const float thr = __double2float_rd(stats->delta);
-
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    double k0 = 0.0, k1 = 0.0;
-    unsigned long long npos = 0, nneg = 0;
-
-    // -- fast units, back to front
-    const long long gwarps = (long long)vg * kWarps;
-    const float4 *W4 = reinterpret_cast<const float4 *>(W);
-    for (long long u = fast_units - 1 - ((long long)vb * kWarps + warp); u >= 0; u -= gwarps) {
-        const long long f0 = u * 128 + lane;
-        const float4 v0 = __ldg(W4 + f0);
-        const float4 v1 = __ldg(W4 + f0 + 32);
-        const float4 v2 = __ldg(W4 + f0 + 64);
-        const float4 v3 = __ldg(W4 + f0 + 96);
-        const uint32_t c0 = code8(v0, thr, k0, k1);
-        const uint32_t c1 = code8(v1, thr, k0, k1);
-        const uint32_t c2 = code8(v2, thr, k0, k1);
-        const uint32_t c3 = code8(v3, thr, k0, k1);
-        uint32_t r = c0 | (c1 << 8) | (c2 << 16) | (c3 << 24);
-        const uint32_t neg = __popc((r >> 1) & 0x55555555u);
-        nneg += neg;
-        npos += __popc(r & 0x55555555u) - neg;
-        if (codes_i8) {
-            uint32_t *o = reinterpret_cast<uint32_t *>(codes_i8) + f0;
-            o[0] = fields_to_i8x4(c0);
-            o[32] = fields_to_i8x4(c1);
-            o[64] = fields_to_i8x4(c2);
-            o[96] = fields_to_i8x4(c3);
-        }
-        // 4x4 byte transpose across lanes l^2 then l^1
-        const uint32_t y = __shfl_xor_sync(0xffffffffu, r, 2);
-        r = __byte_perm(r, y, (lane & 2) ? 0x3276 : 0x5410);
-        const uint32_t z = __shfl_xor_sync(0xffffffffu, r, 1);
-        r = __byte_perm(r, z, (lane & 1) ? 0x3715 : 0x6240);
-        packed[u * 32 + (lane & 3) * 8 + (lane >> 2)] = bytes_to_word(r);
-    }
-
-    // -- everything else, one thread per word: the tail of a flat tensor, ragged rows, padding
-    const long long wpr = ld_codes >> 4;
-    const long long total_words = rows * wpr;
-    const long long first_word = fast_units * 32;
-    for (long long w = first_word + (long long)vb * kThreads + threadIdx.x; w < total_words;
-         w += (long long)vg * kThreads) {
-        const long long r = w / wpr;
-        const long long j0 = (w - r * wpr) << 4;
-        uint32_t word = 0;
-#pragma unroll 4
-        for (int e = 0; e < 16; ++e) {
-            const long long j = j0 + e;
-            if (j < cols) {
-                const float v = __ldg(W + r * cols + j);
-                const uint32_t c = code2(v, thr, k0);
-                word |= c << field_pos(e);
-                if (codes_i8) codes_i8[r * cols + j] = (int8_t)((c & 1u) ? ((c & 2u) ? -1 : 1) : 0);
-            }
-        }
-        const uint32_t neg = __popc((word >> 1) & 0x55555555u);
-        nneg += neg;
-        npos += __popc(word & 0x55555555u) - neg;
-        packed[w] = word;
-    }
-
-    const double bk = block_sum(k0 + k1, red);
-    const unsigned long long bp = block_sum(npos, redu);
-    const unsigned long long bn = block_sum(nneg, redu);
-    if (threadIdx.x == 0) {
-        ws.part_kept[vb] = bk;
-        ws.part_pos[vb] = bp;
-        ws.part_neg[vb] = bn;
-    }
-    if (last_block(ws.ticket2, vg)) {
-        double s = 0.0;
-        unsigned long long p = 0, q = 0;
-        for (int b = threadIdx.x; b < (int)vg; b += kThreads) {
-            s += __ldcg(ws.part_kept + b);
-            p += __ldcg(ws.part_pos + b);
-            q += __ldcg(ws.part_neg + b);
-        }
-        s = block_sum(s, red);
-        p = block_sum(p, redu);
-        q = block_sum(q, redu);
-        if (threadIdx.x == 0) {
-            const unsigned long long kept = p + q;
-            stats->sum_abs_kept = s;
-            stats->alpha = kept > 0 ? s / (double)kept : 0.0;
-            stats->n_pos = p;
-            stats->n_neg = q;
-            stats->n_zero = (unsigned long long)n - kept;
-            *ws.ticket2 = 0u;
-        }
-    }
-}
-
-__global__ void __launch_bounds__(kThreads)
-code_pack_kernel(const float *__restrict__ W, long long rows, long long cols, long long ld_codes,
-                 long long fast_units, uint32_t *__restrict__ packed, int8_t *__restrict__ codes_i8,
-                 void *ws_raw, twn_stats_t *__restrict__ stats)
-{
-    code_pack_body(W, rows, cols, ld_codes, fast_units, packed, codes_i8, carve(ws_raw), stats, blockIdx.x, gridDim.x);
-}
-
-// ---- several tensors in one launch ------------------------------------------
-// A training step ternarizes every layer (Algorithm 1, first loop).  One launch per sweep for
-// all of them: the blocks of the grid are dealt out to the tensors in proportion to their size,
-// and each tensor keeps its own tickets and partials, so its results are bit-identical to those
-// of a call of its own.
-constexpr int kMaxBatch = 32;
-struct BatchItem {
+// ---- parts ------------------------------------------------------------------
+// A part is a run of consecutive packed words that hold codes (the padding words of a row belong to none); the
+// weights of consecutive words follow one another in memory, so a part is a contiguous range of weights as well,
+// whatever the row length.
+struct Item {
     const float *W;
-    long long rows, cols, ld_codes, fast_units;
+    twn_stats_t *stats;
     uint32_t *packed;
     int8_t *codes_i8;
-    twn_stats_t *stats;
-};
-struct BatchParams {
-    int count;
-    unsigned int first_block[kMaxBatch + 1];   // blocks [first_block[t], first_block[t+1]) work on tensor t
-    BatchItem item[kMaxBatch];
+    unsigned long long n, words;     // weights; words that hold codes
+    long long rows, cols, wpr;
+    unsigned int wpr_used;           // words of a row that hold codes
+    unsigned int wpr_magic;          // floor(2^32 / wpr_used) + 1, 0 for one word per row
+    unsigned int parts, part_words;
+    unsigned int first_part;         // of this tensor, among the parts of the launch
+    unsigned int first_pass;         // weights of a part that phase 1 reads without keeping them in L2
+    bool small;
+    bool vec4;                       // every word starts on a 16-byte boundary
+    bool dense;                      // word w of the packed matrix holds weights 16 w ..
 };
 
-// Slice t of a batch workspace: the tickets of all tensors come first (256 bytes each, so that one
-// small memset clears them), then the partials.
-__host__ __device__ inline Workspace carve_batch(void *ws, int t, int count)
+template <int N>
+struct Launch {
+    int count;
+    unsigned int parts;              // of all tensors
+    double factor;
+    Item item[N];
+};
+
+struct PartRange {
+    unsigned long long w0, f0;       // first word, first weight
+    unsigned long long out0;         // packed word of the first word's row
+    unsigned int j0, words, len;     // the first word's position in its row; words, weights
+};
+
+__device__ __forceinline__ void row_of(const Item &it, unsigned long long w, unsigned long long &row, unsigned int &j)
 {
-    char *b = static_cast<char *>(ws);
-    Workspace w;
-    w.ticket1 = reinterpret_cast<unsigned int *>(b + (size_t)t * 256);
-    w.ticket2 = reinterpret_cast<unsigned int *>(b + (size_t)t * 256 + 64);
-    char *p = b + (size_t)count * 256 + (size_t)t * (4 * size_t(kMaxBlocks) * 8);
-    w.part_sum = reinterpret_cast<double *>(p);
-    w.part_kept = w.part_sum + kMaxBlocks;
-    w.part_pos = reinterpret_cast<unsigned long long *>(w.part_kept + kMaxBlocks);
-    w.part_neg = w.part_pos + kMaxBlocks;
-    return w;
+    if (w >> 32) { row = w / it.wpr_used; j = (unsigned int)(w - row * it.wpr_used); }
+    else { row = (unsigned int)w / it.wpr_used; j = (unsigned int)w - (unsigned int)row * it.wpr_used; }
 }
 
-__device__ __forceinline__ int batch_tensor_of(const BatchParams &P, unsigned int block)
+__device__ __forceinline__ PartRange part_range(const Item &it, unsigned int part)
+{
+    PartRange r;
+    r.w0 = (unsigned long long)part * it.part_words;
+    const unsigned long long left = it.words > r.w0 ? it.words - r.w0 : 0;
+    r.words = left < it.part_words ? (unsigned int)left : it.part_words;
+    r.out0 = 0; r.j0 = 0; r.f0 = 0; r.len = 0;
+    if (r.words == 0) return r;
+    unsigned long long row, row1;
+    unsigned int j1;
+    row_of(it, r.w0, row, r.j0);
+    row_of(it, r.w0 + r.words, row1, j1);
+    r.out0 = row * (unsigned long long)it.wpr;
+    r.f0 = row * (unsigned long long)it.cols + 16ull * r.j0;
+    const unsigned long long f1 = row1 * (unsigned long long)it.cols + 16ull * j1;
+    r.len = (unsigned int)((f1 < it.n ? f1 : it.n) - r.f0);
+    return r;
+}
+
+// Word `wl` of a part: its index in the packed matrix, its first weight (counted from the part's) and how many
+// weights it holds.
+struct Place {
+    unsigned long long out;
+    unsigned int f, valid;
+};
+__device__ __forceinline__ Place place_word(const Item &it, const PartRange &r, unsigned int wl)
+{
+    Place p;
+    if (it.dense) {
+        p.out = r.w0 + wl;
+        p.f = 16 * wl;
+        p.valid = min(16u, r.len - p.f);
+    } else {
+        const unsigned int jj = r.j0 + wl;
+        // jj / wpr_used: the multiplication is at most one too high
+        unsigned int ro = it.wpr_magic ? __umulhi(jj, it.wpr_magic) : jj;
+        if (ro * it.wpr_used > jj) --ro;
+        const unsigned int j = jj - ro * it.wpr_used, cols = (unsigned int)it.cols;
+        p.out = r.out0 + (unsigned long long)ro * (unsigned long long)it.wpr + j;
+        p.f = ro * cols + 16 * j - 16 * r.j0;
+        p.valid = min(16u, cols - 16 * j);
+    }
+    return p;
+}
+
+// Quarter `q` (four weights) of a part, zeros where there is no weight.
+__device__ __forceinline__ float4 load_quarter(const Item &it, const PartRange &r, unsigned int q)
+{
+    float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    const unsigned int wl = q >> 2, e = 4 * (q & 3);
+    if (wl < r.words) {
+        const Place p = place_word(it, r, wl);
+        if (p.valid > e) {
+            const unsigned int left = p.valid - e;
+            const float *w = it.W + r.f0 + (p.f + e);
+            if (it.vec4 && left >= 4) {
+                v = __ldg(reinterpret_cast<const float4 *>(w));
+            } else {
+                v.x = __ldg(w);
+                if (left > 1) v.y = __ldg(w + 1);
+                if (left > 2) v.z = __ldg(w + 2);
+                if (left > 3) v.w = __ldg(w + 3);
+            }
+        }
+    }
+    return v;
+}
+
+// A 16-byte load of weights that need not stay in L2.
+__device__ __forceinline__ float4 ld_stream(const float4 *p, unsigned long long policy)
+{
+    float4 v;
+    asm("ld.global.nc.L2::cache_hint.v4.f32 {%0, %1, %2, %3}, [%4], %5;" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p), "l"(policy));
+    return v;
+}
+__device__ __forceinline__ unsigned long long evict_first_policy()
+{
+    unsigned long long p;
+    asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
+    return p;
+}
+
+// The four quarters that a thread has in a group of 512 words.  All loads of a thread are issued before any is used
+// and none sits behind a branch of its own (with load_quarter's branches 96 million weights in rows of 8001 took
+// 208 us, half of it waiting for one load at a time).  Rows that start off the 16-byte boundaries are read by two
+// aligned vectors and shifted.
+__device__ __forceinline__ void load_group(const Item &it, const PartRange &r, unsigned int w_grp, float4 (&v)[4])
+{
+    const unsigned int tid = threadIdx.x;
+    const float *W = it.W + r.f0;
+    if (it.dense && w_grp + 512 <= r.words && (w_grp + 512ull) * 16 <= r.len) {
+        const float4 *v4 = reinterpret_cast<const float4 *>(W) + (size_t)w_grp * 4 + tid;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[k] = it.first_pass ? ld_stream(v4 + k * kSweepThreads, evict_first_policy()) : __ldg(v4 + k * kSweepThreads);
+        return;
+    }
+    // what the branch-free paths may read: up to the end of the group's last word, and seven weights more
+    const Place last = place_word(it, r, min(w_grp + 511, r.words - 1));
+    if (r.f0 + last.f + 24 > it.n || it.dense) {
+#pragma unroll 1
+        for (int k = 0; k < 4; ++k) {
+            const float4 x = load_quarter(it, r, w_grp * 4 + k * kSweepThreads + tid);
+            if (k == 0) v[0] = x; else if (k == 1) v[1] = x; else if (k == 2) v[2] = x; else v[3] = x;
+        }
+        return;
+    }
+    unsigned int f[4], left[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const unsigned int q = w_grp * 4 + k * kSweepThreads + tid, wl = q >> 2, e = 4 * (q & 3);
+        const Place p = place_word(it, r, min(wl, r.words - 1));
+        left[k] = wl < r.words && p.valid > e ? p.valid - e : 0;
+        f[k] = left[k] ? p.f + e : p.f;
+    }
+    if (it.vec4) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[k] = __ldg(reinterpret_cast<const float4 *>(W + f[k]));
+    } else {
+        float4 a[4], b[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const float4 *w4 = reinterpret_cast<const float4 *>(W + f[k] - ((r.f0 + f[k]) & 3));
+            a[k] = __ldg(w4);
+            b[k] = __ldg(w4 + 1);
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const unsigned int mis = (unsigned int)(r.f0 + f[k]);
+            const bool one = mis & 1, two = mis & 2;
+            const float s0 = one ? a[k].y : a[k].x, s1 = one ? a[k].z : a[k].y, s2 = one ? a[k].w : a[k].z,
+                        s3 = one ? b[k].x : a[k].w, s4 = one ? b[k].y : b[k].x, s5 = one ? b[k].z : b[k].y;
+            v[k] = make_float4(two ? s2 : s0, two ? s3 : s1, two ? s4 : s2, two ? s5 : s3);
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        if (left[k] < 1) v[k].x = 0.0f;
+        if (left[k] < 2) v[k].y = 0.0f;
+        if (left[k] < 3) v[k].z = 0.0f;
+        if (left[k] < 4) v[k].w = 0.0f;
+    }
+}
+
+struct AbsSum {
+    double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
+    __device__ __forceinline__ void add(const float4 v)
+    {
+        a0 += (double)fabsf(v.x); a1 += (double)fabsf(v.y); a2 += (double)fabsf(v.z); a3 += (double)fabsf(v.w);
+    }
+    __device__ __forceinline__ double total() const { return (a0 + a1) + (a2 + a3); }
+};
+
+// The kept weights of a part: per-thread sums and counts, and the codes of one group of 512 words.  A thread codes
+// quarter-word q = k * 512 + tid of the group for k = 0..3, so a warp covers 512 consecutive bytes of weights at a
+// time; each byte of `bytes` is one quarter.
+struct Coder {
+    double k[4] = {0.0, 0.0, 0.0, 0.0};
+    unsigned int pos = 0, neg = 0;
+    __device__ __forceinline__ double kept() const { return (k[0] + k[1]) + (k[2] + k[3]); }
+    __device__ __forceinline__ void group(const Item &it, const PartRange &r, unsigned int w_grp, const float4 (&v)[4], float thr)
+    {
+        const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+        // Bound by instruction issue, above all by the half-rate integer pipe: a comparison, a select, three shifts
+        // and two merges per weight took 29 us for 20 million weights that are in L2.  Here a weight costs that pipe
+        // two instructions, the comparison (as 1.0 or 0.0) and a funnel shift that collects the signs; the masking
+        // and the collection of the kept bits are multiplications.
+        float kept_bits = 0.0f;          // below 2^16, exact
+        uint32_t sign_bits = 0;
+#pragma unroll
+        for (int i = 3; i >= 0; --i) {
+            const float w4[4] = {v[i].y, v[i].w, v[i].x, v[i].z};
+#pragma unroll
+            for (int x = 0; x < 4; ++x) {
+                float keep;
+                asm("set.gt.f32.f32 %0, %1, %2;" : "=f"(keep) : "f"(fabsf(w4[x])), "f"(thr));
+                k[x] += (double)(fabsf(w4[x]) * keep);
+                kept_bits = fmaf(kept_bits, 2.0f, keep);
+                sign_bits = __funnelshift_l(__float_as_uint(w4[x]), sign_bits, 1);
+            }
+        }
+        const uint32_t kb = (uint32_t)kept_bits, nb = sign_bits & kb;
+        const unsigned int n_neg = __popc(nb);
+        neg += n_neg;
+        pos += __popc(kb) - n_neg;
+        uint32_t bytes = spread16(kb) | (spread16(nb) << 1);
+        if (it.codes_i8) {
+#pragma unroll 1
+            for (int i = 0; i < 4; ++i) {
+                const unsigned int q = i * kSweepThreads + tid, wl = w_grp + (q >> 2), e = 4 * (q & 3);
+                if (wl >= r.words) continue;
+                const Place p = place_word(it, r, wl);
+                const uint32_t c4 = fields_to_i8x4((bytes >> (8 * i)) & 0xFFu);
+                for (unsigned int x = 0; x < 4 && e + x < p.valid; ++x) it.codes_i8[r.f0 + p.f + e + x] = (int8_t)(c4 >> (8 * x));
+            }
+        }
+        // a word's four quarters sit in the bytes of four neighbouring lanes: a 4x4 byte transpose (lanes
+        // l^2, then l^1) leaves lane l with word l/4 of its warp's share of quarter-row l%4
+        const uint32_t y = __shfl_xor_sync(0xffffffffu, bytes, 2);
+        bytes = __byte_perm(bytes, y, (lane & 2) ? 0x3276 : 0x5410);
+        const uint32_t z = __shfl_xor_sync(0xffffffffu, bytes, 1);
+        bytes = __byte_perm(bytes, z, (lane & 1) ? 0x3715 : 0x6240);
+        const unsigned int wl = w_grp + (lane & 3) * kQuarterWords + warp * 8 + (lane >> 2);
+        if (wl < r.words) it.packed[it.dense ? r.w0 + wl : place_word(it, r, wl).out] = bytes_to_word(bytes);
+    }
+};
+
+__device__ __forceinline__ double threshold(const Item &it, double s, double factor)
+{
+    return it.n > 0 ? factor * (s / (double)it.n) : 0.0;
+}
+__device__ __forceinline__ void write_threshold(const Item &it, double s, double delta)
+{
+    it.stats->sum_abs = s;
+    it.stats->delta = delta;
+    it.stats->status = isfinite(s) ? TWN_OK : TWN_ERR_NONFINITE;
+    it.stats->reserved = 0;
+}
+__device__ __forceinline__ void write_kept(const Item &it, double kept, unsigned long long pos, unsigned long long neg)
+{
+    const unsigned long long n_kept = pos + neg;
+    it.stats->sum_abs_kept = kept;
+    it.stats->alpha = n_kept > 0 ? kept / (double)n_kept : 0.0;
+    it.stats->n_pos = pos;
+    it.stats->n_neg = neg;
+    it.stats->n_zero = it.n - n_kept;
+}
+
+// padding words of the rows
+__device__ __forceinline__ void write_padding(const Item &it, unsigned int b, unsigned int G)
+{
+    const unsigned int pad = (unsigned int)(it.wpr - it.wpr_used);
+    if (pad == 0 || !it.packed) return;
+    const unsigned long long total = (unsigned long long)it.rows * pad;
+    for (unsigned long long i = (unsigned long long)b * kSweepThreads + threadIdx.x; i < total; i += (unsigned long long)G * kSweepThreads) {
+        const unsigned long long r = i >> 32 ? i / pad : (unsigned int)i / pad;
+        it.packed[r * it.wpr + it.wpr_used + (i - r * pad)] = 0u;
+    }
+}
+
+// ---- small tensors: one cluster -------------------------------------------------
+// Latency is all there is (50 thousand weights: 14.3 us as two sweeps over memory with a cleared ticket, 12 of them
+// waiting for memory and launches).  A block keeps its part in registers between the phases, the sums travel through
+// distributed shared memory, and the cluster's barrier (0.2 us) stands where larger tensors need the grid's.
+__device__ __forceinline__ uint32_t peer_smem(const void *p, uint32_t rank)
+{
+    uint32_t a;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+    return a;
+}
+__device__ __forceinline__ void st_peer(uint32_t addr, unsigned long long v)
+{
+    asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(addr), "l"(v) : "memory");
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.aligned;" ::: "memory"); }
+
+// Eight values in the order of the shuffle tree that folds the parts of a larger tensor.
+__device__ __forceinline__ double tree8(const double *p)
+{
+    return ((p[0] + p[4]) + (p[2] + p[6])) + ((p[1] + p[5]) + (p[3] + p[7]));
+}
+
+template <int Q, bool SUMS>      // quarter-words per thread; false: the coding sweep alone
+__global__ void __launch_bounds__(kSweepThreads, 1)
+ternarize_small_kernel(const __grid_constant__ Launch<1> P)
+{
+    __shared__ Reduce red;
+    __shared__ double sum_s[kSmallParts], kept_s[kSmallParts];
+    __shared__ unsigned long long cnt_s[kSmallParts];
+    const Item &it = P.item[0];
+    const unsigned int b = blockIdx.x, G = gridDim.x, tid = threadIdx.x;
+    unsigned int turn = 0;
+    if (tid < kSmallParts) { sum_s[tid] = 0.0; kept_s[tid] = 0.0; cnt_s[tid] = 0ull; }
+    cluster_arrive();                    // from here on other blocks may write this block's sums
+    PartRange r = part_range(it, b);
+    float4 v[Q < 4 ? 4 : Q];
+#pragma unroll
+    for (int k = 0; k < (Q < 4 ? 4 : Q); ++k)
+        v[k] = k < Q ? load_quarter(it, r, k * kSweepThreads + tid) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    write_padding(it, b, G);
+    double delta;
+    if (SUMS) {
+        AbsSum a;
+#pragma unroll
+        for (int k = 0; k < Q; ++k) a.add(v[k]);
+        const double part = sweep_sum(a.total(), red, turn);
+        cluster_wait();
+        if (tid < G) st_peer(peer_smem(&sum_s[b], tid), __double_as_longlong(part));
+        cluster_arrive();
+        cluster_wait();
+        const double s = tree8(sum_s);
+        delta = threshold(it, s, P.factor);
+        if (b == 0 && tid == 0) write_threshold(it, s, delta);
+    } else {
+        cluster_wait();
+        delta = __ldcg(&it.stats->delta);
+    }
+    // delta rounded toward -inf: for any float w,  w > delta  <=>  w > thr
+    const float thr = __double2float_rd(delta);
+    Coder c;
+#pragma unroll
+    for (int g = (Q + 3) / 4; g-- > 0;) {
+        const float4 four[4] = {v[4 * g], v[4 * g + 1], v[4 * g + 2], v[4 * g + 3]};
+        c.group(it, r, g * 512, four, thr);
+    }
+    const double kept = sweep_sum(c.kept(), c.pos, c.neg, red, turn);
+    if (tid == 0) {
+        st_peer(peer_smem(&kept_s[b], 0), __double_as_longlong(kept));
+        st_peer(peer_smem(&cnt_s[b], 0), ((unsigned long long)c.neg << 32) + c.pos);
+    }
+    cluster_arrive();
+    cluster_wait();
+    if (b == 0 && tid == 0) {
+        unsigned long long pos = 0, neg = 0;
+#pragma unroll
+        for (int i = 0; i < kSmallParts; ++i) { pos += cnt_s[i] & 0xFFFFFFFFull; neg += cnt_s[i] >> 32; }
+        write_kept(it, tree8(kept_s), pos, neg);
+    }
+}
+
+// ---- any tensor: a cooperative launch -------------------------------------------
+template <int N> __device__ __forceinline__ int item_of_part(const Launch<N> &P, unsigned int g)
 {
     int t = 0;
-    while (t + 1 < P.count && block >= P.first_block[t + 1]) ++t;
+    if (N > 1)
+        while (t + 1 < P.count && g >= P.item[t + 1].first_part) ++t;
     return t;
 }
 
-__global__ void __launch_bounds__(kThreads)
-sum_abs_batch_kernel(const __grid_constant__ BatchParams P, double factor, void *ws_raw)
+// sum |W| over the weights of a part: whole 16-byte vectors from the boundary below its first weight on, and by
+// plain loads the weights before the first and after the last whole vector (small tensors: by quarter-words, as the
+// kernel above adds them).
+__device__ __forceinline__ double part_abs_sum(const Item &it, const PartRange &r)
 {
-    const int t = batch_tensor_of(P, blockIdx.x);
-    const BatchItem &it = P.item[t];
-    sum_abs_body(it.W, it.rows * it.cols, factor, carve_batch(ws_raw, t, P.count), it.stats,
-                 blockIdx.x - P.first_block[t], P.first_block[t + 1] - P.first_block[t]);
+    AbsSum a;
+    if (it.small) {
+#pragma unroll 1
+        for (unsigned int q = threadIdx.x; q < 4 * r.words; q += kSweepThreads) a.add(load_quarter(it, r, q));
+        return a.total();
+    }
+    const unsigned int head = (unsigned int)(r.f0 & 3ull);
+    const float4 *v4 = reinterpret_cast<const float4 *>(it.W + (r.f0 - head));
+    const unsigned long long end = (unsigned long long)head + r.len;
+    const unsigned long long first = head ? 1 : 0, last = end >> 2;     // vectors [first, last) lie inside the part
+    unsigned long long i = first + threadIdx.x;
+    // a tensor larger than L2: what phase 2 reads last is not kept, so that what it reads first still is
+    const unsigned long long pol = evict_first_policy();
+    for (const unsigned long long end1 = min((unsigned long long)(it.first_pass >> 2), last); i + 3 * kSweepThreads < end1; i += 4 * kSweepThreads) {
+        const float4 v0 = ld_stream(v4 + i, pol), v1 = ld_stream(v4 + i + kSweepThreads, pol),
+                     v2 = ld_stream(v4 + i + 2 * kSweepThreads, pol), v3 = ld_stream(v4 + i + 3 * kSweepThreads, pol);
+        a.add(v0); a.add(v1); a.add(v2); a.add(v3);
+    }
+    for (; i + 3 * kSweepThreads < last; i += 4 * kSweepThreads) {
+        const float4 v0 = __ldg(v4 + i), v1 = __ldg(v4 + i + kSweepThreads), v2 = __ldg(v4 + i + 2 * kSweepThreads),
+                     v3 = __ldg(v4 + i + 3 * kSweepThreads);
+        a.add(v0); a.add(v1); a.add(v2); a.add(v3);
+    }
+    for (; i < last; i += kSweepThreads) a.add(__ldg(v4 + i));
+    if (threadIdx.x < 8) {
+        const unsigned int x = threadIdx.x & 3;
+        const unsigned long long e = threadIdx.x < 4 ? x : 4 * last + x;
+        const bool inside = e < end && (threadIdx.x < 4 ? (first && x >= head) : last >= first);
+        if (inside) a.a0 += (double)fabsf(__ldg(reinterpret_cast<const float *>(v4) + e));
+    }
+    return a.total();
 }
 
-__global__ void __launch_bounds__(kThreads)
-code_pack_batch_kernel(const __grid_constant__ BatchParams P, void *ws_raw)
+// Folds `parts` partial sums in a fixed order; the result is valid in every thread.
+__device__ __forceinline__ double fold_parts(const double *p, unsigned int parts, Reduce &red, unsigned int &turn)
 {
-    const int t = batch_tensor_of(P, blockIdx.x);
-    const BatchItem &it = P.item[t];
-    code_pack_body(it.W, it.rows, it.cols, it.ld_codes, it.fast_units, it.packed, it.codes_i8,
-                   carve_batch(ws_raw, t, P.count), it.stats, blockIdx.x - P.first_block[t],
-                   P.first_block[t + 1] - P.first_block[t]);
+    double s = 0.0;
+    for (unsigned int i = threadIdx.x; i < parts; i += kSweepThreads) s += __ldcg(p + i);
+    return sweep_sum(s, red, turn);
 }
 
+// N: tensors of the launch (1, or up to kMaxBatch).  SUMS: false for the coding sweep alone, against the
+// threshold that is in the stats.
+template <int N, bool SUMS>
+__global__ void __launch_bounds__(kSweepThreads, kSweepBlocksPerSm)
+ternarize_kernel(const __grid_constant__ Launch<N> P, void *ws_raw)
+{
+    __shared__ Reduce red;
+    __shared__ unsigned long long red_cnt64[2][kSweepWarps];
+    __shared__ unsigned int last_mask;
+    const int tid = threadIdx.x;
+    const unsigned int b = blockIdx.x, G = gridDim.x;
+    unsigned int turn = 0;
+
+    if (tid == 0) last_mask = 0;
+    if (b == 0 && tid < P.count) *carve(ws_raw, tid).done = 0u;
+
+    // ---- phase 1
+    if (SUMS) {
+        for (unsigned int g = b; g < P.parts; g += G) {
+            const int ti = item_of_part(P, g);
+            const Item &it = P.item[ti];
+            const double sum = sweep_sum(part_abs_sum(it, part_range(it, g - it.first_part)), red, turn);
+            if (tid == 0) carve(ws_raw, ti).part_sum[g - it.first_part] = sum;
+        }
+    }
+#pragma unroll 1
+    for (int t = 0; t < P.count; ++t) write_padding(P.item[t], b, G);
+
+    cooperative_groups::this_grid().sync();
+
+    double delta = 0.0;
+    if (SUMS) {
+        if (N == 1) {
+            // every block folds for itself
+            const double s = fold_parts(carve(ws_raw, 0).part_sum, P.item[0].parts, red, turn);
+            delta = threshold(P.item[0], s, P.factor);
+            if (b == 0 && tid == 0) write_threshold(P.item[0], s, delta);
+        } else {
+            for (int t = (int)b; t < P.count; t += (int)G) {
+                const double s = fold_parts(carve(ws_raw, t).part_sum, P.item[t].parts, red, turn);
+                if (tid == 0) write_threshold(P.item[t], s, threshold(P.item[t], s, P.factor));
+            }
+            cooperative_groups::this_grid().sync();
+        }
+    }
+
+    // ---- phase 2, back to front
+    const unsigned int mine = b < P.parts ? (P.parts - 1 - b) / G + 1 : 0;
+    for (unsigned int i = mine; i-- > 0;) {
+        const unsigned int g = b + i * G;
+        const int ti = item_of_part(P, g);
+        const Item &it = P.item[ti];
+        const PartRange r = part_range(it, g - it.first_part);
+        // delta rounded toward -inf: for any float w,  w > delta  <=>  w > thr
+        const float thr = __double2float_rd(N == 1 && SUMS ? delta : __ldcg(&it.stats->delta));
+        Coder c;
+        for (unsigned int grp = (r.words + 511) >> 9; grp-- > 0;) {
+            float4 v[4];
+            load_group(it, r, grp << 9, v);
+            c.group(it, r, grp << 9, v, thr);
+        }
+        const double kept = sweep_sum(c.kept(), c.pos, c.neg, red, turn);
+        if (tid == 0) {
+            const Workspace ws = carve(ws_raw, ti);
+            ws.part_kept[g - it.first_part] = kept;
+            ws.part_cnt[g - it.first_part] = ((unsigned long long)c.neg << 32) + c.pos;
+            unsigned int old;
+            asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(old) : "l"(ws.done) : "memory");
+            if (old == it.parts - 1) last_mask |= 1u << ti;
+        }
+    }
+    // the block that wrote the last part of a tensor folds its second sums
+    __syncthreads();
+    for (unsigned int mask = last_mask; mask; mask &= mask - 1) {
+        const int ti = __ffs(mask) - 1;
+        const Item &it = P.item[ti];
+        const Workspace ws = carve(ws_raw, ti);
+        double s = 0.0;
+        unsigned long long pos = 0, neg = 0;
+        for (unsigned int i = tid; i < it.parts; i += kSweepThreads) {
+            s += __ldcg(ws.part_kept + i);
+            const unsigned long long c = __ldcg(ws.part_cnt + i);
+            pos += c & 0xFFFFFFFFull;
+            neg += c >> 32;
+        }
+        const double kept = sweep_sum(s, red, turn);
+        pos = warp_sum(pos);
+        neg = warp_sum(neg);
+        if ((tid & 31) == 0) { red_cnt64[0][tid >> 5] = pos; red_cnt64[1][tid >> 5] = neg; }
+        __syncthreads();
+        if (tid == 0) {
+            pos = neg = 0;
+            for (int w = 0; w < kSweepWarps; ++w) { pos += red_cnt64[0][w]; neg += red_cnt64[1][w]; }
+            write_kept(it, kept, pos, neg);
+        }
+        __syncthreads();
+    }
+}
+
+// ---- parameter update fused with the sums of the next iteration ----------------
+// Last step of Algorithm 1 (UpdateParameters: SGD with momentum and L2 weight decay on the fp32
+// master weights, Sec. 3):
+//     g = dW + wd * W;   V' = mu * V + g;   W' = W - lr * V'
+// every operation a separately rounded fp32 operation in this order (no fused multiply-add), so
+// the result is defined to the bit.  The next iteration starts by ternarizing W', whose
+// threshold needs sum |W'|: it is accumulated here while W' is still in registers, which saves
+// the first phase of that ternarization (one read of the weights).
 struct SgdItem {
     float *W;
     const float *dW;
     float *V;
     long long n;
     twn_stats_t *stats;
+    unsigned int first_block;        // blocks [first_block, first_block of the next item) work on this tensor
 };
-struct SgdBatch {
+template <int N>
+struct SgdLaunch {
     int count;
-    unsigned int first_block[kMaxBatch + 1];
-    SgdItem item[kMaxBatch];
+    unsigned int blocks;
+    float lr, mu, wd;
+    double factor;
+    SgdItem item[N];
 };
 
-__global__ void __launch_bounds__(kThreads)
-sgd_update_batch_kernel(const __grid_constant__ SgdBatch P, float lr, float mu, float wd, double factor, void *ws_raw)
+__device__ __forceinline__ float sgd_one(float w, float g, float &v, float lr, float mu, float wd)
 {
-    int t = 0;
-    while (t + 1 < P.count && blockIdx.x >= P.first_block[t + 1]) ++t;
-    const SgdItem &it = P.item[t];
-    sgd_update_body(it.W, it.dW, it.V, it.n, lr, mu, wd, factor, carve_batch(ws_raw, t, P.count), it.stats,
-                    blockIdx.x - P.first_block[t], P.first_block[t + 1] - P.first_block[t]);
+    const float grad = __fadd_rn(g, __fmul_rn(wd, w));
+    v = __fadd_rn(__fmul_rn(mu, v), grad);
+    return __fsub_rn(w, __fmul_rn(lr, v));
+}
+
+__device__ __forceinline__ void sgd_four(float4 &w, const float4 g, float4 &v, float lr, float mu, float wd, double &a0, double &a1)
+{
+    w.x = sgd_one(w.x, g.x, v.x, lr, mu, wd);
+    w.y = sgd_one(w.y, g.y, v.y, lr, mu, wd);
+    w.z = sgd_one(w.z, g.z, v.z, lr, mu, wd);
+    w.w = sgd_one(w.w, g.w, v.w, lr, mu, wd);
+    a0 += (double)fabsf(w.x); a1 += (double)fabsf(w.y); a0 += (double)fabsf(w.z); a1 += (double)fabsf(w.w);
+}
+
+// The blocks' sums meet as in the ternarization kernels: through distributed shared memory where one cluster of at
+// most eight blocks does, else through the workspace and a grid-wide barrier (1.2 us; a ticket in the workspace has to
+// be cleared first, by a memset that costs its own launch: 3 us).
+template <int N, bool CLUSTER>
+__global__ void __launch_bounds__(kSweepThreads, kSweepBlocksPerSm)
+sgd_update_kernel(const __grid_constant__ SgdLaunch<N> P, void *ws_raw)
+{
+    static_assert(!CLUSTER || N == 1, "a batch meets grid-wide");
+    __shared__ Reduce red;
+    __shared__ double sum_s[kSmallParts];
+    unsigned int turn = 0;
+    double own = 0.0;
+    if (CLUSTER) {
+        if (threadIdx.x < kSmallParts) sum_s[threadIdx.x] = 0.0;
+        cluster_arrive();
+    }
+    for (unsigned int g = blockIdx.x; g < P.blocks; g += gridDim.x) {
+        int t = 0;
+        if (N > 1)
+            while (t + 1 < P.count && g >= P.item[t + 1].first_block) ++t;
+        const SgdItem &it = P.item[t];
+        const unsigned int vb = g - it.first_block;
+        const unsigned int vg = (t + 1 < P.count ? P.item[t + 1 < N ? t + 1 : 0].first_block : P.blocks) - it.first_block;
+        const long long n4 = it.n >> 2;
+        float4 *W4 = reinterpret_cast<float4 *>(it.W);
+        float4 *V4 = reinterpret_cast<float4 *>(it.V);
+        const float4 *G4 = reinterpret_cast<const float4 *>(it.dW);
+        const long long stride = (long long)vg * kSweepThreads;
+        double a0 = 0.0, a1 = 0.0;
+        long long i = (long long)vb * kSweepThreads + threadIdx.x;
+        // two iterations in flight: six 16-byte loads per thread, 1024 threads per SM
+        for (; i + stride < n4; i += 2 * stride) {
+            float4 w = W4[i], v = V4[i], w2 = W4[i + stride], v2 = V4[i + stride];
+            const float4 d = __ldg(G4 + i), d2 = __ldg(G4 + i + stride);
+            sgd_four(w, d, v, P.lr, P.mu, P.wd, a0, a1);
+            W4[i] = w;
+            V4[i] = v;
+            sgd_four(w2, d2, v2, P.lr, P.mu, P.wd, a0, a1);
+            W4[i + stride] = w2;
+            V4[i + stride] = v2;
+        }
+        if (i < n4) {
+            float4 w = W4[i], v = V4[i];
+            sgd_four(w, __ldg(G4 + i), v, P.lr, P.mu, P.wd, a0, a1);
+            W4[i] = w;
+            V4[i] = v;
+        }
+        if (vb == 0) {
+            const long long e = (n4 << 2) + threadIdx.x;
+            if (e < it.n) {
+                float v = it.V[e];
+                const float w = sgd_one(it.W[e], __ldg(it.dW + e), v, P.lr, P.mu, P.wd);
+                it.W[e] = w;
+                it.V[e] = v;
+                a0 += (double)fabsf(w);
+            }
+        }
+        const double s = sweep_sum(a0 + a1, red, turn);
+        if (CLUSTER) own = s;
+        else if (threadIdx.x == 0) carve(ws_raw, t).part_sum[vb] = s;
+    }
+    auto finish = [&](const SgdItem &it, double s) {
+        it.stats->sum_abs = s;
+        it.stats->delta = it.n > 0 ? P.factor * (s / (double)it.n) : 0.0;
+        it.stats->status = isfinite(s) ? TWN_OK : TWN_ERR_NONFINITE;
+        it.stats->reserved = 0;
+    };
+    if (CLUSTER) {
+        // a block has at most one share
+        cluster_wait();
+        if (threadIdx.x == 0) st_peer(peer_smem(&sum_s[blockIdx.x], 0), __double_as_longlong(own));
+        cluster_arrive();
+        cluster_wait();
+        if (blockIdx.x == 0 && threadIdx.x == 0 && P.item[0].stats) finish(P.item[0], tree8(sum_s));
+    } else {
+        cooperative_groups::this_grid().sync();
+        for (int t = (int)blockIdx.x; t < P.count; t += (int)gridDim.x) {
+            const SgdItem &it = P.item[t];
+            if (!it.stats) continue;
+            const unsigned int vg = (t + 1 < P.count ? P.item[t + 1 < N ? t + 1 : 0].first_block : P.blocks) - it.first_block;
+            const double s = fold_parts(carve(ws_raw, t).part_sum, vg, red, turn);
+            if (threadIdx.x == 0) finish(it, s);
+        }
+    }
 }
 
 // ---- standalone pack / unpack / re-layout ----------------------------------
+// Block-wide sum with a fixed order; the result is valid in thread 0.
+template <typename T>
+__device__ __forceinline__ T block_sum(T v, T *smem /* kWarps entries */)
+{
+    v = warp_sum(v);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    __syncthreads();
+    if (lane == 0) smem[warp] = v;
+    __syncthreads();
+    T r = T(0);
+    if (warp == 0) r = warp_sum(lane < kWarps ? smem[lane] : T(0));
+    return r;
+}
+
 __device__ __forceinline__ uint32_t i8x4_to_fields(uint32_t x, uint32_t &bad)
 {
     // a byte is valid iff (byte + 1) mod 256 <= 2
@@ -725,52 +1061,199 @@ fold_codes_kernel(const uint32_t *__restrict__ in, int ld_in, int Cout, int Cin,
 int grid_for(long long items_per_thread_units, int sm_count)
 {
     long long blocks = (items_per_thread_units + kThreads - 1) / kThreads;
-    const long long cap = (long long)sm_count * 8 < kMaxBlocks ? (long long)sm_count * 8 : kMaxBlocks;
+    const long long cap = (long long)sm_count * 8;
     if (blocks > cap) blocks = cap;
     if (blocks < 1) blocks = 1;
     return (int)blocks;
+}
+
+// What phase 1 reads last and phase 2 first is marked to stay in L2, the rest of a tensor larger than this to go first:
+// of 134 MB (8192 x 4096 weights, three tensors in turn) 53.4 us without marks, 50.3 / 49.3 / 50.0 / 50.7 / 51.4 us with 1 /
+// 40 / 60 / 80 / 100 MB kept; of 403 MB 136.9 us without, 131.4 us with 40 MB.
+constexpr unsigned long long kKeptBytes = 40000000ull;
+
+// A tensor as the sweeps see it; false if an argument is not acceptable (*rc says why).
+bool make_item(const float *W, int64_t rows, int64_t cols, twn_stats_t *stats, uint32_t *packed, int64_t ld_codes,
+               int8_t *codes_i8, Item *it, int *rc)
+{
+    const long long n = (long long)rows * cols;
+    *rc = TWN_ERR_INVALID_ARG;
+    if (rows < 0 || cols < 0 || !stats || ld_codes < cols || ld_codes % 64 != 0) return false;
+    if (n != 0 && (!W || !packed)) return false;
+    *rc = TWN_ERR_MISALIGNED;
+    if (!twn_aligned(W, 16) || !twn_aligned(packed, 16) || !twn_aligned(stats, 8) || !twn_aligned(codes_i8, 16)) return false;
+    it->W = W; it->stats = stats; it->packed = packed; it->codes_i8 = codes_i8;
+    it->rows = rows; it->cols = cols; it->wpr = ld_codes / 16;
+    it->n = (unsigned long long)n;
+    const unsigned long long used = (unsigned long long)(cols + 15) / 16;
+    it->words = (unsigned long long)rows * used;
+    // One part per block of a full grid, of at least 8192 weights: below that the fixed cost of a part (its
+    // reduction) would show in a batch.  Small tensors: at most eight parts, of whole quarter-word rounds.
+    it->small = it->words <= kSmallWords;
+    const unsigned long long most = it->small ? kSmallParts : kMaxParts, step = it->small ? kQuarterWords : 512;
+    unsigned long long part = (it->words + most - 1) / most;
+    part = std::max(1ull, (part + step - 1) / step) * step;
+    *rc = TWN_ERR_TOO_LARGE;
+    if (used > 0xFFFFFFFFull || part > 0x08000000ull) return false;
+    it->wpr_used = (unsigned int)used;
+    it->wpr_magic = used > 1 ? (unsigned int)((1ull << 32) / used + 1) : 0;
+    it->part_words = (unsigned int)part;
+    it->parts = (unsigned int)std::max(1ull, (it->words + part - 1) / part);
+    it->vec4 = rows == 1 || cols % 4 == 0;
+    it->dense = rows == 1 || ld_codes == cols;
+    it->first_pass = 4ull * n > kKeptBytes ? (unsigned int)(16 * part - 16 * part * kKeptBytes / (4ull * n)) : 0;
+    it->first_part = 0;
+    *rc = TWN_OK;
+    return true;
+}
+
+// cudaLaunchKernelEx with one attribute.
+template <typename K, typename... A>
+int launch_with(K kernel, unsigned int grid, cudaLaunchAttributeID id, cudaLaunchAttributeValue val, cudaStream_t s, const A &...args)
+{
+    cudaLaunchAttribute attr[1];
+    attr[0].id = id;
+    attr[0].val = val;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(kSweepThreads);
+    cfg.stream = s;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    TWN_CUDA_OK(cudaLaunchKernelEx(&cfg, kernel, args...));
+    return TWN_OK;
+}
+
+template <int N, bool SUMS>
+int launch_sweeps(Launch<N> &P, double factor, void *ws, cudaStream_t s)
+{
+    twn_device_info dev;
+    const int rc = twn_current_device(&dev);
+    if (rc != TWN_OK) return rc;
+    P.factor = factor;
+    P.parts = 0;
+    for (int t = 0; t < P.count; ++t) {
+        P.item[t].first_part = P.parts;
+        P.parts += P.item[t].parts;
+    }
+    cudaLaunchAttributeValue val = {};
+    if constexpr (N == 1) {
+        if (P.item[0].small) {
+            unsigned int grid = 1;
+            while (grid < P.parts) grid *= 2;
+            val.clusterDim.x = grid;
+            val.clusterDim.y = val.clusterDim.z = 1;
+            const unsigned int q = P.item[0].part_words / kQuarterWords;
+            auto kernel = q <= 1 ? ternarize_small_kernel<1, SUMS> : q <= 2 ? ternarize_small_kernel<2, SUMS>
+                        : q <= 4 ? ternarize_small_kernel<4, SUMS> : ternarize_small_kernel<8, SUMS>;
+            return launch_with(kernel, grid, cudaLaunchAttributeClusterDimension, val, s, P);
+        }
+    }
+    val.cooperative = 1;
+    return launch_with(ternarize_kernel<N, SUMS>, std::min(P.parts, (unsigned int)(dev.sm_count * kSweepBlocksPerSm)),
+                       cudaLaunchAttributeCooperative, val, s, P, ws);
+}
+
+bool batch_items(const twn_ternarize_item_t *items, int count, Launch<kMaxBatch> &P, int *rc)
+{
+    P.count = count;
+    for (int t = 0; t < count; ++t) {
+        const twn_ternarize_item_t &it = items[t];
+        if (!make_item(it.W, it.rows, it.cols, it.stats, it.packed, it.ld_codes, it.codes_i8, &P.item[t], rc)) return false;
+    }
+    return true;
+}
+
+template <int N>
+int launch_sgd(SgdLaunch<N> &P, void *ws, cudaStream_t s)
+{
+    twn_device_info dev;
+    const int rc = twn_current_device(&dev);
+    if (rc != TWN_OK) return rc;
+    // per tensor, as many blocks as run at once or fewer: the same number alone and in a batch, so the same sums
+    P.blocks = 0;
+    for (int t = 0; t < P.count; ++t) {
+        const long long want = (P.item[t].n / 4 + kSweepThreads - 1) / kSweepThreads;
+        P.item[t].first_block = P.blocks;
+        P.blocks += (unsigned int)std::max(1ll, std::min((long long)kMaxParts, want));
+    }
+    cudaLaunchAttributeValue val = {};
+    if constexpr (N == 1) {
+        if (P.blocks <= kSmallParts) {
+            unsigned int grid = 1;
+            while (grid < P.blocks) grid *= 2;
+            val.clusterDim.x = grid;
+            val.clusterDim.y = val.clusterDim.z = 1;
+            return launch_with(sgd_update_kernel<N, true>, grid, cudaLaunchAttributeClusterDimension, val, s, P, ws);
+        }
+    }
+    val.cooperative = 1;
+    return launch_with(sgd_update_kernel<N, false>, std::min(P.blocks, (unsigned int)(dev.sm_count * kSweepBlocksPerSm)),
+                       cudaLaunchAttributeCooperative, val, s, P, ws);
 }
 
 }  // namespace
 
 extern "C" size_t twn_ternarize_workspace_bytes(void) { return kWorkspaceBytes; }
 
+extern "C" size_t twn_ternarize_batch_workspace_bytes(int count) { return count > 0 ? (size_t)count * kWorkspaceBytes : 0; }
+
 extern "C" int twn_ternarize(const float *W, int64_t rows, int64_t cols, double delta_factor,
                              twn_stats_t *stats, uint32_t *packed, int64_t ld_codes,
                              int8_t *codes_i8, void *workspace, size_t workspace_bytes,
                              twn_stream_t stream)
 {
-    TWN_REQUIRE(rows >= 0 && cols >= 0, TWN_ERR_INVALID_ARG);
-    TWN_REQUIRE(stats != nullptr && workspace != nullptr, TWN_ERR_INVALID_ARG);
-    TWN_REQUIRE(delta_factor >= 0.0 && delta_factor == delta_factor, TWN_ERR_INVALID_ARG);
-    TWN_REQUIRE(ld_codes >= cols && ld_codes % 64 == 0, TWN_ERR_INVALID_ARG);
-    const long long n = (long long)rows * cols;
-    TWN_REQUIRE(n == 0 || (W != nullptr && packed != nullptr), TWN_ERR_INVALID_ARG);
+    int rc;
+    Launch<1> P;
+    P.count = 1;
+    TWN_REQUIRE(workspace != nullptr && delta_factor >= 0.0 && delta_factor == delta_factor, TWN_ERR_INVALID_ARG);
+    if (!make_item(W, rows, cols, stats, packed, ld_codes, codes_i8, &P.item[0], &rc)) return rc;
     TWN_REQUIRE(workspace_bytes >= kWorkspaceBytes, TWN_ERR_WORKSPACE);
-    TWN_REQUIRE(twn_aligned(W, 16) && twn_aligned(packed, 16) && twn_aligned(stats, 8) &&
-                    twn_aligned(workspace, 256) && twn_aligned(codes_i8, 16), TWN_ERR_MISALIGNED);
-    twn_device_info dev;
-    const int rc = twn_current_device(&dev);
-    if (rc != TWN_OK) return rc;
-    cudaStream_t s = twn_cu(stream);
+    TWN_REQUIRE(twn_aligned(workspace, 256), TWN_ERR_MISALIGNED);
+    return launch_sweeps<1, true>(P, delta_factor, workspace, twn_cu(stream));
+}
 
-    // the two tickets must start at zero
-    TWN_CUDA_OK(cudaMemsetAsync(workspace, 0, 128, s));
+extern "C" int twn_ternarize_codes(const float *W, int64_t rows, int64_t cols, twn_stats_t *stats, uint32_t *packed,
+                                   int64_t ld_codes, int8_t *codes_i8, void *workspace, size_t workspace_bytes,
+                                   twn_stream_t stream)
+{
+    int rc;
+    Launch<1> P;
+    P.count = 1;
+    TWN_REQUIRE(workspace != nullptr, TWN_ERR_INVALID_ARG);
+    if (!make_item(W, rows, cols, stats, packed, ld_codes, codes_i8, &P.item[0], &rc)) return rc;
+    TWN_REQUIRE(workspace_bytes >= kWorkspaceBytes, TWN_ERR_WORKSPACE);
+    TWN_REQUIRE(twn_aligned(workspace, 256), TWN_ERR_MISALIGNED);
+    return launch_sweeps<1, false>(P, 0.0, workspace, twn_cu(stream));
+}
 
-    const int g1 = grid_for((n / 4 + 3) / 4, dev.sm_count);
-    sum_abs_kernel<<<g1, kThreads, 0, s>>>(W, n, delta_factor, workspace, stats);
+extern "C" int twn_ternarize_batch(const twn_ternarize_item_t *items, int count, double delta_factor,
+                                   void *workspace, size_t workspace_bytes, twn_stream_t stream)
+{
+    TWN_REQUIRE(count >= 0 && count <= kMaxBatch, TWN_ERR_INVALID_ARG);
+    if (count == 0) return TWN_OK;
+    TWN_REQUIRE(items != nullptr && workspace != nullptr, TWN_ERR_INVALID_ARG);
+    TWN_REQUIRE(delta_factor >= 0.0 && delta_factor == delta_factor, TWN_ERR_INVALID_ARG);
+    TWN_REQUIRE(workspace_bytes >= twn_ternarize_batch_workspace_bytes(count), TWN_ERR_WORKSPACE);
+    TWN_REQUIRE(twn_aligned(workspace, 256), TWN_ERR_MISALIGNED);
+    int rc;
+    Launch<kMaxBatch> P;
+    if (!batch_items(items, count, P, &rc)) return rc;
+    return launch_sweeps<kMaxBatch, true>(P, delta_factor, workspace, twn_cu(stream));
+}
 
-    // a flat run of whole 512-weight units exists when rows are stored back to back
-    const bool flat = (rows <= 1) || (ld_codes == cols);
-    const long long fast_units = flat ? n / 512 : 0;
-    const long long rest_words = (long long)rows * (ld_codes / 16) - fast_units * 32;
-    long long work = fast_units * 32 / 4;  // threads: each warp-iteration covers one unit
-    if (rest_words > work) work = rest_words;
-    const int g2 = grid_for(work, dev.sm_count);
-    code_pack_kernel<<<g2, kThreads, 0, s>>>(W, rows, cols, ld_codes, fast_units, packed, codes_i8,
-                                             workspace, stats);
-    TWN_CUDA_OK(cudaGetLastError());
-    return TWN_OK;
+extern "C" int twn_ternarize_codes_batch(const twn_ternarize_item_t *items, int count, void *workspace,
+                                         size_t workspace_bytes, twn_stream_t stream)
+{
+    TWN_REQUIRE(count >= 0 && count <= kMaxBatch, TWN_ERR_INVALID_ARG);
+    if (count == 0) return TWN_OK;
+    TWN_REQUIRE(items != nullptr && workspace != nullptr, TWN_ERR_INVALID_ARG);
+    TWN_REQUIRE(workspace_bytes >= twn_ternarize_batch_workspace_bytes(count), TWN_ERR_WORKSPACE);
+    TWN_REQUIRE(twn_aligned(workspace, 256), TWN_ERR_MISALIGNED);
+    int rc;
+    Launch<kMaxBatch> P;
+    if (!batch_items(items, count, P, &rc)) return rc;
+    return launch_sweeps<kMaxBatch, false>(P, 0.0, workspace, twn_cu(stream));
 }
 
 extern "C" int twn_sgd_update(float *W, const float *dW, float *V, int64_t n, float lr, float momentum,
@@ -785,15 +1268,11 @@ extern "C" int twn_sgd_update(float *W, const float *dW, float *V, int64_t n, fl
     TWN_REQUIRE(workspace_bytes >= kWorkspaceBytes, TWN_ERR_WORKSPACE);
     TWN_REQUIRE(twn_aligned(W, 16) && twn_aligned(dW, 16) && twn_aligned(V, 16) && twn_aligned(stats_next, 8) &&
                     twn_aligned(workspace, 256), TWN_ERR_MISALIGNED);
-    twn_device_info dev;
-    const int rc = twn_current_device(&dev);
-    if (rc != TWN_OK) return rc;
-    cudaStream_t s = twn_cu(stream);
-    TWN_CUDA_OK(cudaMemsetAsync(workspace, 0, 128, s));
-    const int g = grid_for((n / 4 + 1) / 2, dev.sm_count);
-    sgd_update_kernel<<<g, kThreads, 0, s>>>(W, dW, V, n, lr, momentum, weight_decay, delta_factor, workspace, stats_next);
-    TWN_CUDA_OK(cudaGetLastError());
-    return TWN_OK;
+    SgdLaunch<1> P;
+    P.count = 1;
+    P.lr = lr; P.mu = momentum; P.wd = weight_decay; P.factor = delta_factor;
+    P.item[0] = SgdItem{W, dW, V, n, stats_next, 0};
+    return launch_sgd(P, workspace, twn_cu(stream));
 }
 
 extern "C" int twn_sgd_update_batch(const twn_sgd_item_t *items, int count, float lr, float momentum,
@@ -807,153 +1286,17 @@ extern "C" int twn_sgd_update_batch(const twn_sgd_item_t *items, int count, floa
     TWN_REQUIRE(delta_factor >= 0.0 && delta_factor == delta_factor, TWN_ERR_INVALID_ARG);
     TWN_REQUIRE(workspace_bytes >= twn_ternarize_batch_workspace_bytes(count), TWN_ERR_WORKSPACE);
     TWN_REQUIRE(twn_aligned(workspace, 256), TWN_ERR_MISALIGNED);
-    twn_device_info dev;
-    const int rc = twn_current_device(&dev);
-    if (rc != TWN_OK) return rc;
-    SgdBatch P;
+    SgdLaunch<kMaxBatch> P;
     P.count = count;
-    unsigned int g = 0;
+    P.lr = lr; P.mu = momentum; P.wd = weight_decay; P.factor = delta_factor;
     for (int t = 0; t < count; ++t) {
         const twn_sgd_item_t &it = items[t];
         TWN_REQUIRE(it.n >= 0 && (it.n == 0 || (it.W && it.dW && it.V)), TWN_ERR_INVALID_ARG);
         TWN_REQUIRE(twn_aligned(it.W, 16) && twn_aligned(it.dW, 16) && twn_aligned(it.V, 16) &&
                         twn_aligned(it.stats_next, 8), TWN_ERR_MISALIGNED);
-        SgdItem si;
-        si.W = it.W; si.dW = it.dW; si.V = it.V; si.n = it.n; si.stats = it.stats_next;
-        P.item[t] = si;
-        P.first_block[t] = g;
-        g += (unsigned int)grid_for((it.n / 4 + 1) / 2, dev.sm_count);     // the grid of a call of its own
+        P.item[t] = SgdItem{it.W, it.dW, it.V, it.n, it.stats_next, 0};
     }
-    P.first_block[count] = g;
-    cudaStream_t s = twn_cu(stream);
-    TWN_CUDA_OK(cudaMemsetAsync(workspace, 0, (size_t)count * 256, s));
-    sgd_update_batch_kernel<<<g, kThreads, 0, s>>>(P, lr, momentum, weight_decay, delta_factor, workspace);
-    TWN_CUDA_OK(cudaGetLastError());
-    return TWN_OK;
-}
-
-extern "C" int twn_ternarize_codes_batch(const twn_ternarize_item_t *items, int count, void *workspace,
-                                         size_t workspace_bytes, twn_stream_t stream)
-{
-    TWN_REQUIRE(count >= 0 && count <= kMaxBatch, TWN_ERR_INVALID_ARG);
-    if (count == 0) return TWN_OK;
-    TWN_REQUIRE(items != nullptr && workspace != nullptr, TWN_ERR_INVALID_ARG);
-    TWN_REQUIRE(workspace_bytes >= twn_ternarize_batch_workspace_bytes(count), TWN_ERR_WORKSPACE);
-    TWN_REQUIRE(twn_aligned(workspace, 256), TWN_ERR_MISALIGNED);
-    twn_device_info dev;
-    const int rc = twn_current_device(&dev);
-    if (rc != TWN_OK) return rc;
-    BatchParams B;
-    B.count = count;
-    unsigned int gb = 0;
-    for (int t = 0; t < count; ++t) {
-        const twn_ternarize_item_t &it = items[t];
-        TWN_REQUIRE(it.rows >= 0 && it.cols >= 0 && it.stats != nullptr, TWN_ERR_INVALID_ARG);
-        TWN_REQUIRE(it.ld_codes >= it.cols && it.ld_codes % 64 == 0, TWN_ERR_INVALID_ARG);
-        const long long n = (long long)it.rows * it.cols;
-        TWN_REQUIRE(n == 0 || (it.W != nullptr && it.packed != nullptr), TWN_ERR_INVALID_ARG);
-        TWN_REQUIRE(twn_aligned(it.W, 16) && twn_aligned(it.packed, 16) && twn_aligned(it.stats, 8) &&
-                        twn_aligned(it.codes_i8, 16), TWN_ERR_MISALIGNED);
-        const bool flat = (it.rows <= 1) || (it.ld_codes == it.cols);
-        const long long fast_units = flat ? n / 512 : 0;
-        const long long rest_words = (long long)it.rows * (it.ld_codes / 16) - fast_units * 32;
-        long long work = fast_units * 32 / 4;
-        if (rest_words > work) work = rest_words;
-        BatchItem bi;
-        bi.W = it.W; bi.rows = it.rows; bi.cols = it.cols; bi.ld_codes = it.ld_codes; bi.fast_units = fast_units;
-        bi.packed = it.packed; bi.codes_i8 = it.codes_i8; bi.stats = it.stats;
-        B.item[t] = bi;
-        B.first_block[t] = gb;
-        gb += (unsigned int)grid_for(work, dev.sm_count);
-    }
-    B.first_block[count] = gb;
-    cudaStream_t s = twn_cu(stream);
-    TWN_CUDA_OK(cudaMemsetAsync(workspace, 0, (size_t)count * 256, s));
-    code_pack_batch_kernel<<<gb, kThreads, 0, s>>>(B, workspace);
-    TWN_CUDA_OK(cudaGetLastError());
-    return TWN_OK;
-}
-
-extern "C" int twn_ternarize_codes(const float *W, int64_t rows, int64_t cols, twn_stats_t *stats, uint32_t *packed,
-                                   int64_t ld_codes, int8_t *codes_i8, void *workspace, size_t workspace_bytes,
-                                   twn_stream_t stream)
-{
-    TWN_REQUIRE(rows >= 0 && cols >= 0, TWN_ERR_INVALID_ARG);
-    TWN_REQUIRE(stats != nullptr && workspace != nullptr, TWN_ERR_INVALID_ARG);
-    TWN_REQUIRE(ld_codes >= cols && ld_codes % 64 == 0, TWN_ERR_INVALID_ARG);
-    const long long n = (long long)rows * cols;
-    TWN_REQUIRE(n == 0 || (W != nullptr && packed != nullptr), TWN_ERR_INVALID_ARG);
-    TWN_REQUIRE(workspace_bytes >= kWorkspaceBytes, TWN_ERR_WORKSPACE);
-    TWN_REQUIRE(twn_aligned(W, 16) && twn_aligned(packed, 16) && twn_aligned(stats, 8) &&
-                    twn_aligned(workspace, 256) && twn_aligned(codes_i8, 16), TWN_ERR_MISALIGNED);
-    twn_device_info dev;
-    const int rc = twn_current_device(&dev);
-    if (rc != TWN_OK) return rc;
-    cudaStream_t s = twn_cu(stream);
-    TWN_CUDA_OK(cudaMemsetAsync(workspace, 0, 128, s));
-    const bool flat = (rows <= 1) || (ld_codes == cols);
-    const long long fast_units = flat ? n / 512 : 0;
-    const long long rest_words = (long long)rows * (ld_codes / 16) - fast_units * 32;
-    long long work = fast_units * 32 / 4;
-    if (rest_words > work) work = rest_words;
-    code_pack_kernel<<<grid_for(work, dev.sm_count), kThreads, 0, s>>>(W, rows, cols, ld_codes, fast_units, packed,
-                                                                       codes_i8, workspace, stats);
-    TWN_CUDA_OK(cudaGetLastError());
-    return TWN_OK;
-}
-
-extern "C" size_t twn_ternarize_batch_workspace_bytes(int count)
-{
-    return count > 0 ? (size_t)count * (256 + 4 * size_t(kMaxBlocks) * 8) : 0;
-}
-
-extern "C" int twn_ternarize_batch(const twn_ternarize_item_t *items, int count, double delta_factor,
-                                   void *workspace, size_t workspace_bytes, twn_stream_t stream)
-{
-    TWN_REQUIRE(count >= 0 && count <= kMaxBatch, TWN_ERR_INVALID_ARG);
-    if (count == 0) return TWN_OK;
-    TWN_REQUIRE(items != nullptr && workspace != nullptr, TWN_ERR_INVALID_ARG);
-    TWN_REQUIRE(delta_factor >= 0.0 && delta_factor == delta_factor, TWN_ERR_INVALID_ARG);
-    TWN_REQUIRE(workspace_bytes >= twn_ternarize_batch_workspace_bytes(count), TWN_ERR_WORKSPACE);
-    TWN_REQUIRE(twn_aligned(workspace, 256), TWN_ERR_MISALIGNED);
-    twn_device_info dev;
-    const int rc = twn_current_device(&dev);
-    if (rc != TWN_OK) return rc;
-
-    BatchParams A, B;
-    A.count = B.count = count;
-    unsigned int ga = 0, gb = 0;
-    for (int t = 0; t < count; ++t) {
-        const twn_ternarize_item_t &it = items[t];
-        TWN_REQUIRE(it.rows >= 0 && it.cols >= 0 && it.stats != nullptr, TWN_ERR_INVALID_ARG);
-        TWN_REQUIRE(it.ld_codes >= it.cols && it.ld_codes % 64 == 0, TWN_ERR_INVALID_ARG);
-        const long long n = (long long)it.rows * it.cols;
-        TWN_REQUIRE(n == 0 || (it.W != nullptr && it.packed != nullptr), TWN_ERR_INVALID_ARG);
-        TWN_REQUIRE(twn_aligned(it.W, 16) && twn_aligned(it.packed, 16) && twn_aligned(it.stats, 8) &&
-                        twn_aligned(it.codes_i8, 16), TWN_ERR_MISALIGNED);
-        // the same grids and the same split into fast units and rest as a call of its own
-        const bool flat = (it.rows <= 1) || (it.ld_codes == it.cols);
-        const long long fast_units = flat ? n / 512 : 0;
-        const long long rest_words = (long long)it.rows * (it.ld_codes / 16) - fast_units * 32;
-        long long work = fast_units * 32 / 4;
-        if (rest_words > work) work = rest_words;
-        BatchItem bi;
-        bi.W = it.W; bi.rows = it.rows; bi.cols = it.cols; bi.ld_codes = it.ld_codes; bi.fast_units = fast_units;
-        bi.packed = it.packed; bi.codes_i8 = it.codes_i8; bi.stats = it.stats;
-        A.item[t] = B.item[t] = bi;
-        A.first_block[t] = ga;
-        B.first_block[t] = gb;
-        ga += (unsigned int)grid_for((n / 4 + 3) / 4, dev.sm_count);
-        gb += (unsigned int)grid_for(work, dev.sm_count);
-    }
-    A.first_block[count] = ga;
-    B.first_block[count] = gb;
-    cudaStream_t s = twn_cu(stream);
-    TWN_CUDA_OK(cudaMemsetAsync(workspace, 0, (size_t)count * 256, s));     // the tickets start at zero
-    sum_abs_batch_kernel<<<ga, kThreads, 0, s>>>(A, delta_factor, workspace);
-    code_pack_batch_kernel<<<gb, kThreads, 0, s>>>(B, workspace);
-    TWN_CUDA_OK(cudaGetLastError());
-    return TWN_OK;
+    return launch_sgd(P, workspace, twn_cu(stream));
 }
 
 // ---- the variant that allocates nothing ------------------------------------------------
@@ -983,39 +1326,19 @@ extern "C" int twn_ternarize_static(const float *W, int64_t rows, int64_t cols, 
                                     int8_t *codes_i8, twn_stream_t stream)
 {
     TWN_REQUIRE(rows >= 0 && cols >= 0, TWN_ERR_INVALID_ARG);
-    TWN_REQUIRE(stats != nullptr, TWN_ERR_INVALID_ARG);
     TWN_REQUIRE(delta_factor >= 0.0 && delta_factor == delta_factor, TWN_ERR_INVALID_ARG);
-    TWN_REQUIRE(ld_codes >= cols && ld_codes % 64 == 0, TWN_ERR_INVALID_ARG);
     TWN_REQUIRE(cols == 0 || rows <= TWN_TERNARIZE_STATIC_MAX_WEIGHTS / cols, TWN_ERR_TOO_LARGE);
-    const long long n = (long long)rows * cols;
-    TWN_REQUIRE(n <= TWN_TERNARIZE_STATIC_MAX_WEIGHTS, TWN_ERR_TOO_LARGE);
-    TWN_REQUIRE(n == 0 || (W != nullptr && packed != nullptr), TWN_ERR_INVALID_ARG);
-    TWN_REQUIRE(twn_aligned(W, 16) && twn_aligned(packed, 16) && twn_aligned(stats, 8) &&
-                    twn_aligned(codes_i8, 16), TWN_ERR_MISALIGNED);
+    int rc;
+    Launch<1> P;
+    P.count = 1;
+    if (!make_item(W, rows, cols, stats, packed, ld_codes, codes_i8, &P.item[0], &rc)) return rc;
     twn_device_info dev;
-    int rc = twn_current_device(&dev);
+    rc = twn_current_device(&dev);
     if (rc != TWN_OK) return rc;
     void *scratch = nullptr;
     rc = static_scratch_ptr(dev.ordinal, &scratch);
     if (rc != TWN_OK) return rc;
-    cudaStream_t s = twn_cu(stream);
-
-    // the array still holds the previous call's partials; only the two tickets must start at zero
-    TWN_CUDA_OK(cudaMemsetAsync(scratch, 0, 128, s));
-
-    const int g1 = grid_for((n / 4 + 3) / 4, dev.sm_count);
-    sum_abs_kernel<<<g1, kThreads, 0, s>>>(W, n, delta_factor, scratch, stats);
-
-    const bool flat = (rows <= 1) || (ld_codes == cols);
-    const long long fast_units = flat ? n / 512 : 0;
-    const long long rest_words = (long long)rows * (ld_codes / 16) - fast_units * 32;
-    long long work = fast_units * 32 / 4;
-    if (rest_words > work) work = rest_words;
-    const int g2 = grid_for(work, dev.sm_count);
-    code_pack_kernel<<<g2, kThreads, 0, s>>>(W, rows, cols, ld_codes, fast_units, packed, codes_i8,
-                                             scratch, stats);
-    TWN_CUDA_OK(cudaGetLastError());
-    return TWN_OK;
+    return launch_sweeps<1, true>(P, delta_factor, scratch, twn_cu(stream));
 }
 
 extern "C" int twn_pack(const int8_t *codes, int64_t rows, int64_t cols, uint32_t *packed,
