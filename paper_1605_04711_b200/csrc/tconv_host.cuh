@@ -88,8 +88,19 @@ struct EpilogueArgs {
 // Contraction with the layer's decoded weights resident in shared memory (tconv_res.cu).  Launches
 // and returns TWN_OK with *handled = true when the launch fits that kernel (at most 64 output
 // channels, unit input stride, decoded weights that fit in shared memory, outputs that TMA can
-// store); otherwise *handled = false and nothing has been launched.
+// store) and should not take longer than `rival_us`; otherwise *handled = false and nothing has been launched.
 int launch_conv_resident(const Geometry &g, const void *X, const uint32_t *T, const EpilogueArgs &epi, void *Y,
-                         int32_t *dev_status, const twn_device_info &dev, cudaStream_t s, bool *handled);
+                         int32_t *dev_status, const twn_device_info &dev, cudaStream_t s, double rival_us, bool *handled);
+
+// Contraction for problems that do not fill the GPU (tconv_split.cu): tiles of 128 channels x `pix` pixels (32, 64, 128
+// or 256), the reduction of each split over a cluster of `splits` blocks (1, 2, 4 or 8; 256 pixels: 1 or 2).  Takes every
+// geometry but batch statistics and reductions of more than 512 k-blocks per block.
+struct SplitPlan {
+    int pix, splits;
+    double us;        // what the launch should take
+};
+SplitPlan plan_conv_split(const Geometry &g, int sm_count);
+int launch_conv_split(const Geometry &g, const void *X, const uint32_t *T, const EpilogueArgs &epi, void *Y,
+                      int32_t *dev_status, const twn_device_info &dev, cudaStream_t s, const SplitPlan &plan);
 
 }  // namespace twn_detail

@@ -511,7 +511,7 @@ tconv_res_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
 
 int twn_detail::launch_conv_resident(const Geometry &g, const void *X, const uint32_t *T, const EpilogueArgs &epi,
                                      void *Y, int32_t *dev_status, const twn_device_info &dev, cudaStream_t s,
-                                     bool *handled)
+                                     double rival_us, bool *handled)
 {
     *handled = false;
     if (g.sw != 1 || g.sh != 1 || g.Cout > kNMax || g.Cout < 1) return TWN_OK;
@@ -572,6 +572,11 @@ int twn_detail::launch_conv_resident(const Geometry &g, const void *X, const uin
     // large problems whose tiles would be mostly empty stay with the general kernel
     const long long pixels = (long long)g.Bv * g.Hv * g.Wv;
     if (pixels > 65536 && total * kPix > 3 * pixels) return TWN_OK;
+
+    // Fitted to measured launches (1 to 13 tiles per block): set-up with the decoding of the weights, then the tiles.
+    const double per_tile = 0.13 * P.kbpt * (g.Cin < kBlockK ? (double)g.Cin / kBlockK : 1.0);
+    const long long per_block = (total + dev.sm_count - 1) / dev.sm_count;
+    if (4.3 + 0.26 * P.kbpt + (per_block - 1) * (per_tile > 0.5 ? per_tile : 0.5) > rival_us) return TWN_OK;
 
     P.w_lo = w_lo; P.h_lo = h_lo;
     const int row_pix = BW + hw;
