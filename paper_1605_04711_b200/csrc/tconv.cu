@@ -44,6 +44,9 @@
 #include <cstddef>
 
 #include <mutex>
+#ifndef MARGIN
+#define MARGIN 0.9
+#endif
 
 #include "common.cuh"
 #include "tc_ptx.cuh"
@@ -775,7 +778,7 @@ int launch_conv(const Geometry &g, const void *X, const uint32_t *T, const twn_s
     ea.relu = epi ? epi->relu : 0;
     ea.out_dtype = epi ? epi->out_dtype : out_dtype_default;
     // problems that do not fill the GPU: small tiles, the reduction split over a cluster
-    const SplitPlan split = plan_conv_split(g, dev.sm_count);
+    const SplitPlan split = plan_conv_split(g, dev.sm_count / (g.beside > 1 ? g.beside : 1));
     // narrow layers: the kernel that decodes the layer's codes once per block
     bool handled = false;
     rc = launch_conv_resident(g, X, T, ea, Y, dev_status, dev, s, split.us, &handled);
@@ -831,7 +834,7 @@ int launch_conv(const Geometry &g, const void *X, const uint32_t *T, const twn_s
     if (c192 < (choice ? c256 : c128)) choice = 2;
     // the model counts cycles of the rounds; a launch as a whole takes (fitted to 65 measured launches, mean error 6 %)
     const double us = 3.9 + 0.454e-3 * (double)(choice == 0 ? c128 : choice == 1 ? c256 : c192);
-    if (split.us < us) return launch_conv_split(g, X, T, ea, Y, dev_status, dev, s, split);
+    if (split.us < MARGIN * us) return launch_conv_split(g, X, T, ea, Y, dev_status, dev, s, split);
     P.dsets = (choice != 1 && two) ? 2 : 1;
     if (g.code_bits == 1) {
         if (choice == 1) return launch_conv_t<256, 1, 1>(g, P, X, dev, enc, s);
@@ -1141,6 +1144,7 @@ int conv_bwd_data_impl(const twn_conv_desc_t *d, const void *dZ, const uint32_t 
                 }
             }
             g.code_bits = bits;
+            g.beside = pool ? (d->stride_h * d->stride_w < 4 ? d->stride_h * d->stride_w : 4) : 1;
             // A residue class no tap reaches gets epilogue(0); when the epilogue only adds a second gradient
             // branch that already lives in dX (in place), that leaves the class as it is: nothing to launch.
             if (g.n_taps == 0 && epi && epi->residual == dX && epi->residual_op == TWN_RESIDUAL_ADD && !epi->scale &&

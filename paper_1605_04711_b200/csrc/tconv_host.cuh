@@ -55,6 +55,7 @@ struct Geometry {
     int n_taps;
     Tap taps[kMaxTaps];
     long long Cin;   // channels per tap
+    int beside;      // launches that run at the same time as this one (0 or 1: none)
 };
 
 // Picks the pixel-tile shape BW x BH x BB (BW and BH powers of two, product `pix`) that needs the
