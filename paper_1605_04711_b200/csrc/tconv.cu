@@ -44,9 +44,6 @@
 #include <cstddef>
 
 #include <mutex>
-#ifndef MARGIN
-#define MARGIN 0.9
-#endif
 
 #include "common.cuh"
 #include "tc_ptx.cuh"
@@ -834,7 +831,11 @@ int launch_conv(const Geometry &g, const void *X, const uint32_t *T, const twn_s
     if (c192 < (choice ? c256 : c128)) choice = 2;
     // the model counts cycles of the rounds; a launch as a whole takes (fitted to 65 measured launches, mean error 6 %)
     const double us = 3.9 + 0.454e-3 * (double)(choice == 0 ? c128 : choice == 1 ? c256 : c192);
-    if (split.us < MARGIN * us) return launch_conv_split(g, X, T, ea, Y, dev_status, dev, s, split);
+    // The more SMs the general kernel fills by itself, the clearer the gain has to be: beside the weight gradients of a
+    // training step a split launch takes SMs that would not have been idle (ResNet-18 at batch 64).
+    const long long tiles = choice == 0 ? t128 : choice == 1 ? t256 : t192;
+    const double fill = tiles < sms ? (double)tiles / (double)sms : 1.0;
+    if (split.us < (1.0 - 0.25 * fill) * us) return launch_conv_split(g, X, T, ea, Y, dev_status, dev, s, split);
     P.dsets = (choice != 1 && two) ? 2 : 1;
     if (g.code_bits == 1) {
         if (choice == 1) return launch_conv_t<256, 1, 1>(g, P, X, dev, enc, s);
