@@ -4,6 +4,8 @@
 // 16-byte accesses along the channel dimension where the channel count allows it.
 #include <cuda_bf16.h>
 
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace {
@@ -53,39 +55,39 @@ im2col_kernel(const __nv_bfloat16 *__restrict__ X, twn_conv_desc_t d, I Ho, I Wo
     }
 }
 
-// Patch variant for short rows (small Cin): a block takes 64 consecutive output pixels of one
-// output row.  The input window they read (kh rows of (63*stride_w + kw) pixels) is copied to
-// shared memory with zeros outside the image; the shared-memory offset of every patch column is
-// tabulated once; then each warp writes whole patch rows, one 16-byte chunk per lane, so that a
-// store instruction covers a contiguous run of the output.
-constexpr int kPatchPix = 64;
-constexpr int kPatchMaxElems = 12288;   // window elements (24 KB)
-constexpr int kPatchMaxCols = 1024;     // ldk
+// Tile variant (small Cin, where the kernel above is bound by its index arithmetic and its 2-byte loads): a block
+// takes several whole output rows of an image.  The input rows they read are copied to shared memory with zeros outside
+// the image and the shared-memory offset of every patch column is tabulated; a thread then keeps one 16-byte column chunk
+// and steps over the pixels, so it holds its eight offsets in registers and consecutive threads store consecutive chunks.
+// (With one block per 64 pixels of a row and a warp per patch row, 28x28x1 at batch 100 left 28 of 32 lanes idle: 11.7 us.)
+constexpr int kTileMaxElems = 24 * 1024;   // window elements (48 KB)
+constexpr int kTileMaxCols = 1024;         // ldk
 
 __global__ void __launch_bounds__(kT)
-im2col_patch_kernel(const __nv_bfloat16 *__restrict__ X, twn_conv_desc_t d, int Ho, int Wo, int wseg,
-                    __nv_bfloat16 *__restrict__ out, int ldk, int win_w)
+im2col_tile_kernel(const __nv_bfloat16 *__restrict__ X, twn_conv_desc_t d, int Ho, int Wo, int rows, int row_groups,
+                   __nv_bfloat16 *__restrict__ out, int ldk)
 {
-    extern __shared__ __align__(16) unsigned char smem_patch[];
-    __nv_bfloat16 *win = reinterpret_cast<__nv_bfloat16 *>(smem_patch);       // [kh][win_w * Cin] (+1 zero at the end)
-    int *tab = reinterpret_cast<int *>(smem_patch + ((size_t)(d.kh * win_w * (int)d.Cin + 1) * 2 + 15) / 16 * 16);
-    const int Cin = (int)d.Cin, K = d.kh * d.kw * Cin, row_el = win_w * Cin, zero_at = d.kh * row_el;
-    int blk = blockIdx.x;
-    const int seg = blk % wseg; blk /= wseg;
-    const int ho = blk % Ho, b = blk / Ho;
-    const int wo0 = seg * kPatchPix;
-    const int h0 = ho * d.stride_h - d.pad_h, w0 = wo0 * d.stride_w - d.pad_w;
-    const int H = (int)d.H, W = (int)d.W;
-    for (int i = threadIdx.x; i < zero_at + 1; i += kT) {
-        const int r = i / row_el, j = i - r * row_el;
-        const int w = w0 + j / Cin, h = h0 + r;
-        __nv_bfloat16 x = __float2bfloat16_rn(0.0f);
-        if (i < zero_at && h >= 0 && h < H && w >= 0 && w < W)
-            x = X[(((long long)b * H + h) * W + w0) * Cin + j];
-        win[i] = x;
+    pdl_begin();
+    extern __shared__ __align__(16) unsigned char smem_tile[];
+    const int Cin = (int)d.Cin, K = d.kh * d.kw * Cin, H = (int)d.H, W = (int)d.W;
+    const int win_w = (Wo - 1) * d.stride_w + d.kw, row_el = win_w * Cin;
+    const int win_h = (rows - 1) * d.stride_h + d.kh, zero_at = win_h * row_el;
+    int *tab = reinterpret_cast<int *>(smem_tile);                               // [ldk]
+    uint16_t *win = reinterpret_cast<uint16_t *>(smem_tile + (size_t)ldk * 4);   // [win_h][row_el], then a zero
+    const int b = blockIdx.x / row_groups, ho0 = (blockIdx.x - b * row_groups) * rows;
+    const int h0 = ho0 * d.stride_h - d.pad_h;
+    const uint16_t *src = reinterpret_cast<const uint16_t *>(X) + (size_t)b * H * W * Cin;
+    const int in_el = W * Cin, lead = d.pad_w * Cin;       // elements of an input row; the window starts `lead` before it
+    for (int r = threadIdx.x >> 5; r < win_h; r += kT / 32) {
+        const int h = h0 + r;
+        for (int j = threadIdx.x & 31; j < row_el; j += 32) {
+            const int e = j - lead;
+            win[r * row_el + j] = h >= 0 && h < H && e >= 0 && e < in_el ? __ldg(src + (size_t)h * in_el + e) : (uint16_t)0;
+        }
     }
+    if (threadIdx.x == 0) win[zero_at] = 0;
     for (int k = threadIdx.x; k < ldk; k += kT) {
-        int off = zero_at;                       // columns K..ldk-1 read the zero
+        int off = -1;                            // columns K..ldk-1 are zero
         if (k < K) {
             const int t = k / Cin, c = k - t * Cin, r = t / d.kw, sx = t - r * d.kw;
             off = r * row_el + sx * Cin + c;
@@ -93,21 +95,41 @@ im2col_patch_kernel(const __nv_bfloat16 *__restrict__ X, twn_conv_desc_t d, int 
         tab[k] = off;
     }
     __syncthreads();
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int chunks = ldk >> 3;
-    const int step = d.stride_w * Cin;           // window elements between neighbouring output pixels
-    const int npix = Wo - wo0 < kPatchPix ? Wo - wo0 : kPatchPix;
-    __nv_bfloat16 *const orow = out + (((long long)b * Ho + ho) * Wo + wo0) * ldk;
-    for (int ch = lane; ch < chunks; ch += 32) {
-        int o[8];
+    const int chunks = ldk >> 3, lanes = kT / chunks * chunks;      // threads that work: whole pixels' worth
+    if (chunks > kT) {
+        // wider than the block: the chunks go round
+        const int n = min(rows, Ho - ho0) * Wo * chunks;
+        for (int i = threadIdx.x; i < n; i += kT) {
+            const int p = i / chunks, ch = i - p * chunks, ho = p / Wo, wo = p - ho * Wo;
+            const int base = ho * d.stride_h * row_el + wo * d.stride_w * Cin;
+            uint32_t v[4];
 #pragma unroll
-        for (int e = 0; e < 8; ++e) o[e] = tab[ch * 8 + e];
-        for (int p = warp; p < npix; p += kT / 32) {
-            __align__(16) __nv_bfloat16 v[8];
-#pragma unroll
-            for (int e = 0; e < 8; ++e) v[e] = win[o[e] == zero_at ? zero_at : o[e] + p * step];
-            *reinterpret_cast<uint4 *>(orow + (long long)p * ldk + ch * 8) = *reinterpret_cast<const uint4 *>(v);
+            for (int e = 0; e < 4; ++e) {
+                const int o0 = tab[ch * 8 + 2 * e], o1 = tab[ch * 8 + 2 * e + 1];
+                v[e] = (uint32_t)win[o0 < 0 ? zero_at : base + o0] | ((uint32_t)win[o1 < 0 ? zero_at : base + o1] << 16);
+            }
+            *reinterpret_cast<uint4 *>(out + ((size_t)(b * Ho + ho0) * Wo + p) * ldk + ch * 8) = make_uint4(v[0], v[1], v[2], v[3]);
         }
+        return;
+    }
+    if (threadIdx.x >= lanes) return;
+    const int ch = threadIdx.x % chunks, step = lanes / chunks;     // this thread's chunk; pixels between its items
+    int o[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) o[e] = tab[ch * 8 + e];
+    const int n_pix = min(rows, Ho - ho0) * Wo;
+    int p = threadIdx.x / chunks, ho = p / Wo, wo = p - ho * Wo;
+    __nv_bfloat16 *dst = out + ((size_t)(b * Ho + ho0) * Wo + p) * ldk + ch * 8;
+    for (; p < n_pix; p += step, dst += (size_t)step * ldk) {
+        const int base = ho * d.stride_h * row_el + wo * d.stride_w * Cin;
+        uint32_t v[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+            v[e] = (uint32_t)win[o[2 * e] < 0 ? zero_at : base + o[2 * e]] |
+                   ((uint32_t)win[o[2 * e + 1] < 0 ? zero_at : base + o[2 * e + 1]] << 16);
+        *reinterpret_cast<uint4 *>(dst) = make_uint4(v[0], v[1], v[2], v[3]);
+        wo += step;
+        while (wo >= Wo) { wo -= Wo; ++ho; }
     }
 }
 
@@ -267,6 +289,7 @@ __global__ void __launch_bounds__(kT)
 maxpool_fwd_vec_kernel(const __nv_bfloat16 *__restrict__ X, int B, int H, int W, int C, int k, int stride, int pad,
                         int Ho, int Wo, __nv_bfloat16 *__restrict__ Y, uint8_t *__restrict__ idx)
 {
+    pdl_begin();
     const int Cv = C >> 3, per_row = Wo * Cv, total = B * Ho * per_row;
     // one window (8 channels) per thread over the flat index: every block has the same work
     for (int it = blockIdx.x * kT + threadIdx.x; it < total; it += gridDim.x * kT) {
@@ -684,6 +707,7 @@ __global__ void __launch_bounds__(kT)
 act_bwd_vec_kernel(const uint4 *__restrict__ dY, const uint4 *__restrict__ Y, const float *__restrict__ scale,
                    long long n8, int C8, uint4 *__restrict__ dZ, uint4 *__restrict__ dPre)
 {
+    pdl_begin();
     for (long long i = (long long)blockIdx.x * kT + threadIdx.x; i < n8; i += (long long)gridDim.x * kT) {
         float g[8];
         unpack8(__ldg(dY + i), g);
@@ -726,13 +750,21 @@ extern "C" int twn_im2col(const twn_conv_desc_t *d, const void *X, void *Xcol, i
     TWN_REQUIRE(Ho > 0 && Wo > 0, TWN_ERR_INVALID_ARG);
     const long long items = d->B * Ho * Wo * (ldk / 8);
     const bool small = items * 8 < 0x7fffffffLL && d->B * d->H * d->W * d->Cin < 0x7fffffffLL;
-    const long long win_w = (long long)(kPatchPix - 1) * d->stride_w + d->kw;
-    const long long wseg = (Wo + kPatchPix - 1) / kPatchPix;
-    if (d->kh * win_w * d->Cin <= kPatchMaxElems && ldk <= kPatchMaxCols && d->B * Ho * wseg < 0x7fffffffLL) {
-        const size_t smem = ((size_t)(d->kh * win_w * d->Cin + 1) * 2 + 15) / 16 * 16 + (size_t)ldk * sizeof(int);
-        im2col_patch_kernel<<<(int)(d->B * Ho * wseg), kT, smem, twn_cu(stream)>>>(
-            static_cast<const __nv_bfloat16 *>(X), *d, (int)Ho, (int)Wo, (int)wseg, static_cast<__nv_bfloat16 *>(Xcol),
-            (int)ldk, (int)win_w);
+    // output rows per block: about 256 pixels, fewer while that leaves SMs without a block, and what fits in shared memory
+    const long long row_el = ((Wo - 1) * d->stride_w + d->kw) * d->Cin;
+    long long rows = std::min(Ho, std::max(1ll, 256 / Wo));
+    while (rows > 1 && (d->B * ((Ho + rows - 1) / rows) < 2 * dev.sm_count || ((rows - 1) * d->stride_h + d->kh) * row_el > kTileMaxElems)) --rows;
+    const long long elems = ((rows - 1) * d->stride_h + d->kh) * row_el, groups = (Ho + rows - 1) / rows;
+    if (elems <= kTileMaxElems && ldk <= kTileMaxCols && d->B * groups < 0x7fffffffLL && d->H * d->W * d->Cin < 0x7fffffffLL) {
+        const size_t smem = (size_t)ldk * 4 + (size_t)(elems + 1) * 2;
+        static bool attr_set[64] = {false};
+        if (!attr_set[dev.ordinal]) {
+            TWN_CUDA_OK(cudaFuncSetAttribute(im2col_tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTileMaxCols * 4 + (kTileMaxElems + 1) * 2));
+            attr_set[dev.ordinal] = true;
+        }
+        TWN_CUDA_OK(twn_launch_small(im2col_tile_kernel, (int)(d->B * groups), kT, smem, twn_cu(stream),
+                                     static_cast<const __nv_bfloat16 *>(X), *d, (int)Ho, (int)Wo, (int)rows, (int)groups,
+                                     static_cast<__nv_bfloat16 *>(Xcol), (int)ldk));
     } else if (small)
         im2col_kernel<int><<<blocks_for(items, dev.sm_count), kT, 0, twn_cu(stream)>>>(
             static_cast<const __nv_bfloat16 *>(X), *d, (int)Ho, (int)Wo, static_cast<__nv_bfloat16 *>(Xcol), (int)ldk);
@@ -800,8 +832,8 @@ extern "C" int twn_maxpool2d_fwd(const void *X, int64_t B, int64_t H, int64_t W,
     const bool vec = C % 8 == 0 && twn_aligned(X, 16) && twn_aligned(Y, 16) && twn_aligned(argmax, 8);
     cudaStream_t s = twn_cu(stream);
     if (vec && small) {
-        maxpool_fwd_vec_kernel<<<blocks_for(B * Ho * Wo * (C / 8), dev.sm_count * 4), kT, 0, s>>>(x, (int)B, (int)H, (int)W, (int)C, k, stride, pad, (int)Ho, (int)Wo,
-                                                    y, argmax);
+        TWN_CUDA_OK(twn_launch_small(maxpool_fwd_vec_kernel, blocks_for(B * Ho * Wo * (C / 8), dev.sm_count * 4), kT, 0, s, x, (int)B, (int)H,
+                                     (int)W, (int)C, k, stride, pad, (int)Ho, (int)Wo, y, argmax));
     }
     else if (vec)
         maxpool_fwd_kernel<long long, 8><<<blocks_for(B * Ho * Wo * C / 8, dev.sm_count), kT, 0, s>>>(
@@ -917,9 +949,9 @@ extern "C" int twn_act_bwd(const void *dY, const void *Y, const float *scale, in
     const bool vec = C % 8 == 0 && n % 8 == 0 && twn_aligned(dY, 16) && twn_aligned(Y, 16) && twn_aligned(dZ, 16) &&
                      twn_aligned(dPre, 16) && twn_aligned(scale, 16);
     if (vec)
-        act_bwd_vec_kernel<<<blocks_for(n / 8, dev.sm_count), kT, 0, twn_cu(stream)>>>(
-            static_cast<const uint4 *>(dY), static_cast<const uint4 *>(Y), scale, n / 8, (int)(C / 8),
-            static_cast<uint4 *>(dZ), static_cast<uint4 *>(dPre));
+        TWN_CUDA_OK(twn_launch_small(act_bwd_vec_kernel, blocks_for(n / 8, dev.sm_count), kT, 0, twn_cu(stream),
+                                     static_cast<const uint4 *>(dY), static_cast<const uint4 *>(Y), scale, n / 8, (int)(C / 8),
+                                     static_cast<uint4 *>(dZ), static_cast<uint4 *>(dPre)));
     else
         act_bwd_kernel<<<blocks_for(n, dev.sm_count), kT, 0, twn_cu(stream)>>>(
             static_cast<const __nv_bfloat16 *>(dY), static_cast<const __nv_bfloat16 *>(Y), scale, n, C,

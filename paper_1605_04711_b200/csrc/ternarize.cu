@@ -21,8 +21,9 @@
 
 namespace {
 
-constexpr int kThreads = 256;       // pack, unpack, re-layouts
+constexpr int kThreads = 256;       // pack, unpack
 constexpr int kWarps = kThreads / 32;
+constexpr int kTrThreads = 128;     // re-layouts
 constexpr int kSweepWarps = 16;
 constexpr int kSweepThreads = 32 * kSweepWarps;
 constexpr int kSweepBlocksPerSm = 2;                        // 64 registers; three blocks spill: 1e8 weights 131 -> 164 us
@@ -984,7 +985,7 @@ __device__ __forceinline__ void transpose_codes_body(const uint32_t *__restrict_
     const int wpr_out = ld_out >> 4, wpr_in = ld_in >> 4;
     const int total = Cin * wpr_out;
     const int cols_out = taps * Cout;
-    for (int w = vb * kThreads + threadIdx.x; w < total; w += vg * kThreads) {
+    for (int w = vb * kTrThreads + threadIdx.x; w < total; w += vg * kTrThreads) {
         const int c = w / wpr_out;
         const int j0 = (w - c * wpr_out) << 4;
         int t = j0 / Cout, o = j0 - t * Cout;
@@ -1003,58 +1004,89 @@ __device__ __forceinline__ void transpose_codes_body(const uint32_t *__restrict_
 }
 
 // The same re-layout for filter banks whose taps start on word boundaries on both sides (Cin % 16 == 0, and
-// Cout % 16 == 0 or a single tap): a thread takes one tap, 64 output channels and 16 input channels, i.e. 64 input words (word
-// column (t*Cin + c0)/16 of rows o0 .. o0+63, read coalesced across the threads of a warp, which take consecutive
-// c0) and transposes four 16 x 16 blocks of codes in registers into the 16 runs of four output words
-// (rows c0 .. c0+15, word columns (t*Cout + o0)/16 ..).  One load per output word instead of sixteen.
-constexpr int kFastRows = 64;
+// Cout % 16 == 0 or a single tap): a thread transposes one 16 x 16 block of codes, from words of 16 rows into words of
+// 16 rows, in registers.  A warp takes 4 blocks along the input channels and 8 along the output channels of a tap, so
+// that its loads cover 16-byte and its stores 32-byte runs.  What bounds it is latency (a bank has a few thousand
+// blocks): one round of loads per thread and a transpose in four exchange steps, 96 instructions; with four blocks per
+// thread, one after the other, and 768 instructions each, 192 -> 384 channels 3x3 took 10 us.
 __host__ __device__ __forceinline__ bool transpose_fast_ok(int Cout, int Cin, int taps)
 {
     return Cin % 16 == 0 && (Cout % 16 == 0 || taps == 1);
 }
-__host__ __device__ __forceinline__ int transpose_fast_groups(int Cout) { return (Cout + kFastRows - 1) / kFastRows; }
+__host__ __device__ __forceinline__ int transpose_fast_warps(int Cout, int Cin, int taps)
+{
+    return taps * (((Cin >> 4) + 3) / 4) * (((Cout + 15) / 16 + 7) / 8);
+}
+// 16 words of 16 two-bit fields each, transposed.  Row e of the block and element e of a word sit at position
+// field_pos(e) / 2, for rows and elements alike, so in the order of positions this is a plain bit-matrix transpose.
+__device__ __forceinline__ void transpose16(uint32_t (&w)[16])
+{
+    auto at = [](int k) { return k < 8 ? 2 * (7 - k) : 2 * (15 - k) + 1; };      // the row at position k
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        uint32_t &a = w[at(k)], &b = w[at(k + 8)];
+        const uint32_t x = __byte_perm(a, b, 0x5410), y = __byte_perm(a, b, 0x7632);
+        a = x; b = y;
+    }
+#pragma unroll
+    for (int k = 0; k < 16; ++k)
+        if (!(k & 4)) {
+            uint32_t &a = w[at(k)], &b = w[at(k + 4)];
+            const uint32_t x = __byte_perm(a, b, 0x6240), y = __byte_perm(a, b, 0x7351);
+            a = x; b = y;
+        }
+#pragma unroll
+    for (int k = 0; k < 16; ++k)
+        if (!(k & 2)) {
+            uint32_t &a = w[at(k)], &b = w[at(k + 2)];
+            const uint32_t t = ((a >> 4) ^ b) & 0x0F0F0F0Fu;
+            b ^= t; a ^= t << 4;
+        }
+#pragma unroll
+    for (int k = 0; k < 16; ++k)
+        if (!(k & 1)) {
+            uint32_t &a = w[at(k)], &b = w[at(k + 1)];
+            const uint32_t t = ((a >> 2) ^ b) & 0x33333333u;
+            b ^= t; a ^= t << 2;
+        }
+}
 __device__ __forceinline__ void transpose_codes_fast_body(const uint32_t *__restrict__ in, int ld_in, int Cout, int Cin,
                                                           int taps, uint32_t *__restrict__ out, int ld_out,
                                                           unsigned int vb, unsigned int vg)
 {
     const int wpr_out = ld_out >> 4, wpr_in = ld_in >> 4;
-    const int cgs = Cin >> 4, ogs = transpose_fast_groups(Cout);
-    const int units = taps * ogs * cgs;
-    for (int u = vb * kThreads + threadIdx.x; u < units; u += vg * kThreads) {
-        const int cg = u % cgs;
-        const int og = (u / cgs) % ogs;
-        const int t = u / (cgs * ogs);
-        const int o0 = og * kFastRows, c0 = cg << 4;
+    const int cgs = Cin >> 4, ogs = (Cout + 15) / 16;
+    const int cts = (cgs + 3) / 4, ots = (ogs + 7) / 8, total = taps * cts * ots;
+    const int lane = threadIdx.x & 31;
+    for (int u = vb * (kTrThreads / 32) + (threadIdx.x >> 5); u < total; u += vg * (kTrThreads / 32)) {
+        const int ct = u % cts, ot = (u / cts) % ots, t = u / (cts * ots);
+        const int cg = ct * 4 + (lane & 3), og = ot * 8 + (lane >> 2);
+        if (cg >= cgs || og >= ogs) continue;
+        const int c0 = cg << 4, o0 = og << 4;
         const uint32_t *src = in + (size_t)o0 * wpr_in + ((t * Cin + c0) >> 4);
+        // rows past Cout (the last block of a bank whose Cout is no multiple of 16) read as zero codes
+        uint32_t w[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) w[i] = o0 + i < Cout ? __ldg(src + (size_t)i * wpr_in) : 0u;
+        transpose16(w);
         uint32_t *dst = out + (size_t)c0 * wpr_out + ((t * Cout + o0) >> 4);
-#pragma unroll 1
-        for (int q = 0; q < kFastRows / 16 && o0 + q * 16 < Cout; ++q) {
-            // rows past Cout (the last group of a bank whose Cout is no multiple of 16) read as zero codes
-            uint32_t w[16];
 #pragma unroll
-            for (int i = 0; i < 16; ++i) w[i] = o0 + q * 16 + i < Cout ? __ldg(src + (size_t)(q * 16 + i) * wpr_in) : 0u;
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                uint32_t word = 0;
-#pragma unroll
-                for (int i = 0; i < 16; ++i) word |= ((w[i] >> field_pos(j)) & 3u) << field_pos(i);
-                dst[(size_t)j * wpr_out + q] = word;
-            }
-        }
+        for (int j = 0; j < 16; ++j) dst[(size_t)j * wpr_out] = w[j];
     }
     // columns past the last tap (a row pitch larger than taps * Cout) read as zero codes
     const int used = (taps * Cout + 15) >> 4;
     if (used < wpr_out) {
         const int pad = wpr_out - used;
-        for (int i = vb * kThreads + threadIdx.x; i < Cin * pad; i += vg * kThreads)
+        for (int i = vb * kTrThreads + threadIdx.x; i < Cin * pad; i += vg * kTrThreads)
             out[(size_t)(i / pad) * wpr_out + used + i % pad] = 0u;
     }
 }
 
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kTrThreads)
 transpose_codes_kernel(const uint32_t *__restrict__ in, int ld_in, int Cout, int Cin,
                        int taps, uint32_t *__restrict__ out, int ld_out)
 {
+    pdl_begin();
     if (transpose_fast_ok(Cout, Cin, taps)) transpose_codes_fast_body(in, ld_in, Cout, Cin, taps, out, ld_out, blockIdx.x, gridDim.x);
     else transpose_codes_body(in, ld_in, Cout, Cin, taps, out, ld_out, blockIdx.x, gridDim.x);
 }
@@ -1071,7 +1103,7 @@ struct TransposeBatch {
     TransposeItem item[kMaxBatch];
 };
 
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kTrThreads)
 transpose_codes_batch_kernel(const __grid_constant__ TransposeBatch P)
 {
     int t = 0;
@@ -1125,6 +1157,12 @@ int grid_for(long long items_per_thread_units, int sm_count)
 // of 134 MB (8192 x 4096 weights, three tensors in turn) 53.4 us without marks, 50.3 / 49.3 / 50.0 / 50.7 / 51.4 us with 1 /
 // 40 / 60 / 80 / 100 MB kept; of 403 MB 136.9 us without, 131.4 us with 40 MB.
 constexpr unsigned long long kKeptBytes = 40000000ull;
+
+int transpose_blocks(int Cout, int Cin, int taps, long long words, int sm_count)
+{
+    const long long threads = transpose_fast_ok(Cout, Cin, taps) ? 32ll * transpose_fast_warps(Cout, Cin, taps) : words;
+    return (int)std::max(1ll, std::min((threads + kTrThreads - 1) / kTrThreads, (long long)sm_count * 16));
+}
 
 // A tensor as the sweeps see it; false if an argument is not acceptable (*rc says why).
 bool make_item(const float *W, int64_t rows, int64_t cols, twn_stats_t *stats, uint32_t *packed, int64_t ld_codes,
@@ -1456,10 +1494,9 @@ extern "C" int twn_transpose_codes(const uint32_t *packed_fwd, int64_t ld_fwd,
     const long long words = d->Cin * (ld_bwd / 16);
     TWN_REQUIRE(words < 0x7fffffffLL && d->Cout * (ld_fwd / 16) < 0x7fffffffLL && ld_fwd < 0x7fffffffLL &&
                     ld_bwd < 0x7fffffffLL, TWN_ERR_INVALID_ARG);
-    // threads' worth of work: one output word each, or one tap x 64 x 16 block of codes each
-    const long long work = transpose_fast_ok((int)d->Cout, (int)d->Cin, (int)taps) ? taps * transpose_fast_groups((int)d->Cout) * (d->Cin / 16) : words;
-    transpose_codes_kernel<<<grid_for(work, dev.sm_count), kThreads, 0, twn_cu(stream)>>>(
-        packed_fwd, (int)ld_fwd, (int)d->Cout, (int)d->Cin, (int)taps, packed_bwd, (int)ld_bwd);
+    TWN_CUDA_OK(twn_launch_small(transpose_codes_kernel, transpose_blocks((int)d->Cout, (int)d->Cin, (int)taps, words, dev.sm_count),
+                                 kTrThreads, 0, twn_cu(stream), packed_fwd, (int)ld_fwd, (int)d->Cout, (int)d->Cin, (int)taps,
+                                 packed_bwd, (int)ld_bwd));
     TWN_CUDA_OK(cudaGetLastError());
     return TWN_OK;
 }
@@ -1492,11 +1529,10 @@ extern "C" int twn_transpose_codes_batch(const twn_transpose_item_t *items, int 
         ti.Cout = (int)d->Cout; ti.Cin = (int)d->Cin; ti.taps = (int)taps;
         P.item[t] = ti;
         P.first_block[t] = g;
-        const long long work = transpose_fast_ok(ti.Cout, ti.Cin, ti.taps) ? taps * transpose_fast_groups(ti.Cout) * (d->Cin / 16) : words;
-        g += (unsigned int)grid_for(work, dev.sm_count);
+        g += (unsigned int)transpose_blocks(ti.Cout, ti.Cin, ti.taps, words, dev.sm_count);
     }
     P.first_block[count] = g;
-    transpose_codes_batch_kernel<<<g, kThreads, 0, twn_cu(stream)>>>(P);
+    transpose_codes_batch_kernel<<<g, kTrThreads, 0, twn_cu(stream)>>>(P);
     TWN_CUDA_OK(cudaGetLastError());
     return TWN_OK;
 }
