@@ -43,6 +43,7 @@
 
 #include <cstddef>
 
+#include <algorithm>
 #include <mutex>
 
 #include "common.cuh"
@@ -754,6 +755,20 @@ int launch_conv_t(const Geometry &g, ConvParams &P, const void *X, const twn_dev
     return TWN_OK;
 }
 
+EpilogueArgs epilogue_args(const twn_stats_t *stats, const twn_epilogue_t *epi, int out_dtype_default)
+{
+    EpilogueArgs ea;
+    ea.alpha = stats ? &stats->alpha : nullptr;
+    ea.scale = epi ? epi->scale : nullptr;
+    ea.shift = epi ? epi->shift : nullptr;
+    ea.residual = epi ? epi->residual : nullptr;
+    ea.res_dtype = epi ? epi->residual_dtype : TWN_F32;
+    ea.res_gate = (epi && epi->residual) ? epi->residual_op : 0;
+    ea.relu = epi ? epi->relu : 0;
+    ea.out_dtype = epi ? epi->out_dtype : out_dtype_default;
+    return ea;
+}
+
 int launch_conv(const Geometry &g, const void *X, const uint32_t *T, const twn_stats_t *stats,
                 const twn_epilogue_t *epi, void *Y, int out_dtype_default, int32_t *dev_status, cudaStream_t s)
 {
@@ -765,15 +780,7 @@ int launch_conv(const Geometry &g, const void *X, const uint32_t *T, const twn_s
 
     // the epilogue keeps output offsets in 32 bits
     if ((long long)g.Bv * g.OH * g.OW * g.ldy >= 0xFFFFFFFFLL) return TWN_ERR_INVALID_ARG;
-    EpilogueArgs ea;
-    ea.alpha = stats ? &stats->alpha : nullptr;
-    ea.scale = epi ? epi->scale : nullptr;
-    ea.shift = epi ? epi->shift : nullptr;
-    ea.residual = epi ? epi->residual : nullptr;
-    ea.res_dtype = epi ? epi->residual_dtype : TWN_F32;
-    ea.res_gate = (epi && epi->residual) ? epi->residual_op : 0;
-    ea.relu = epi ? epi->relu : 0;
-    ea.out_dtype = epi ? epi->out_dtype : out_dtype_default;
+    const EpilogueArgs ea = epilogue_args(stats, epi, out_dtype_default);
     // problems that do not fill the GPU: small tiles, the reduction split over a cluster
     const SplitPlan split = plan_conv_split(g, dev.sm_count / (g.beside > 1 ? g.beside : 1));
     // narrow layers: the kernel that decodes the layer's codes once per block
@@ -1095,67 +1102,93 @@ int conv_bwd_data_impl(const twn_conv_desc_t *d, const void *dZ, const uint32_t 
     if (rc != TWN_OK) return rc;
     const long long Ho = (d->H + 2 * d->pad_h - d->kh) / d->stride_h + 1;
     const long long Wo = (d->W + 2 * d->pad_w - d->kw) / d->stride_w + 1;
-    // One launch per residue class (ph, pw) of the input pixel modulo the stride: inside a
+    // One residue class (ph, pw) of the input pixel modulo the stride at a time: inside a
     // class the adjoint is a stride-1 sum over the taps r with (ph + pad - r) divisible by
-    // the stride, reading dZ at ho = h' + (ph + pad - r)/stride.  The classes write disjoint
-    // pixels, so with more than one class they run side by side on helper streams.
-    cudaStream_t user = twn_cu(stream);
-    ForkPool *pool = nullptr;
-    std::unique_lock<std::mutex> lock(g_fork_mutex, std::defer_lock);
-    if (d->stride_h * d->stride_w > 1) {
-        twn_device_info dev;
-        rc = twn_current_device(&dev);
-        if (rc != TWN_OK) return rc;
-        lock.lock();
-        pool = fork_pool(dev.ordinal);
-        if (pool) {
-            TWN_CUDA_OK(cudaEventRecord(pool->fork, user));
-            for (int i = 0; i < 3; ++i) TWN_CUDA_OK(cudaStreamWaitEvent(pool->side[i], pool->fork, 0));
-        }
-    }
-    int cls = 0;
-    int first_error = TWN_OK;
+    // the stride, reading dZ at ho = h' + (ph + pad - r)/stride.  The classes write disjoint pixels.
+    Geometry all;
+    memset(&all, 0, sizeof all);
+    all.XB = d->B; all.XH = Ho; all.XW = Wo; all.XC = d->Cout; all.ldx = d->Cout;
+    all.Bv = (int)d->B;
+    all.OH = (int)d->H; all.OW = (int)d->W;
+    all.osh = d->stride_h; all.osw = d->stride_w;
+    all.ldy = d->Cin;
+    all.sh = all.sw = 1;
+    all.Cout = (int)d->Cin; all.ld_codes = ld_codes; all.code_cols = taps * d->Cout;
+    all.Cin = d->Cout;
+    all.code_bits = bits;
+    TapClass cls[64];
+    int n_cls = 0;
+    // A residue class no tap reaches gets epilogue(0); when the epilogue only adds a second gradient
+    // branch that already lives in dX (in place), that leaves the class as it is: nothing to launch.
+    const bool skip_empty = epi && epi->residual == dX && epi->residual_op == TWN_RESIDUAL_ADD && !epi->scale && !epi->shift &&
+                            !epi->relu && epi->residual_dtype == epi->out_dtype;
     for (int ph = 0; ph < d->stride_h; ++ph)
         for (int pw = 0; pw < d->stride_w; ++pw) {
             if (ph >= d->H || pw >= d->W) continue;
-            cudaStream_t s = (pool && cls % 4 != 0) ? pool->side[cls % 4 - 1] : user;
-            ++cls;
-            Geometry g;
-            memset(&g, 0, sizeof g);
-            g.XB = d->B; g.XH = Ho; g.XW = Wo; g.XC = d->Cout; g.ldx = d->Cout;
-            g.Bv = (int)d->B;
-            g.Hv = (int)((d->H - ph + d->stride_h - 1) / d->stride_h);
-            g.Wv = (int)((d->W - pw + d->stride_w - 1) / d->stride_w);
-            g.OH = (int)d->H; g.OW = (int)d->W;
-            g.osh = d->stride_h; g.osw = d->stride_w; g.ooh = ph; g.oow = pw;
-            g.ldy = d->Cin;
-            g.sh = g.sw = 1;
-            g.Cout = (int)d->Cin; g.ld_codes = ld_codes; g.code_cols = taps * d->Cout;
-            g.Cin = d->Cout;
+            TapClass c;
+            c.Hv = (int)((d->H - ph + d->stride_h - 1) / d->stride_h);
+            c.Wv = (int)((d->W - pw + d->stride_w - 1) / d->stride_w);
+            c.ooh = ph; c.oow = pw;
+            c.tap0 = all.n_taps;
             for (int r = 0; r < d->kh; ++r) {
                 const int xh = ph + d->pad_h - r;
                 if (((xh % d->stride_h) + d->stride_h) % d->stride_h != 0) continue;
                 for (int s = 0; s < d->kw; ++s) {
                     const int xw = pw + d->pad_w - s;
                     if (((xw % d->stride_w) + d->stride_w) % d->stride_w != 0) continue;
-                    Tap &t = g.taps[g.n_taps++];
+                    Tap &t = all.taps[all.n_taps++];
                     t.dh = (int16_t)(xh / d->stride_h);
                     t.dw = (int16_t)(xw / d->stride_w);
                     t.koff = (int32_t)((r * d->kw + s) * d->Cout);
                 }
             }
-            g.code_bits = bits;
-            g.beside = pool ? (d->stride_h * d->stride_w < 4 ? d->stride_h * d->stride_w : 4) : 1;
-            // A residue class no tap reaches gets epilogue(0); when the epilogue only adds a second gradient
-            // branch that already lives in dX (in place), that leaves the class as it is: nothing to launch.
-            if (g.n_taps == 0 && epi && epi->residual == dX && epi->residual_op == TWN_RESIDUAL_ADD && !epi->scale &&
-                !epi->shift && !epi->relu && epi->residual_dtype == epi->out_dtype) {
-                --cls;              // the class takes no stream slot
-                continue;
-            }
-            rc = launch_conv(g, dZ, T_bwd, stats, epi, dX, TWN_F32, dev_status, s);
-            if (rc != TWN_OK && first_error == TWN_OK) first_error = rc;
+            c.n_taps = all.n_taps - c.tap0;
+            if (c.n_taps == 0 && skip_empty) continue;
+            cls[n_cls++] = c;
         }
+    auto one_class = [&](const TapClass &c, int beside) {
+        Geometry g = all;
+        g.Hv = c.Hv; g.Wv = c.Wv; g.ooh = c.ooh; g.oow = c.oow;
+        g.n_taps = c.n_taps;
+        for (int t = 0; t < c.n_taps; ++t) g.taps[t] = all.taps[c.tap0 + t];
+        g.beside = beside;
+        return g;
+    };
+    cudaStream_t user = twn_cu(stream);
+    if (n_cls <= 1) return n_cls == 0 ? TWN_OK : launch_conv(one_class(cls[0], 1), dZ, T_bwd, stats, epi, dX, TWN_F32, dev_status, user);
+    twn_device_info dev;
+    rc = twn_current_device(&dev);
+    if (rc != TWN_OK) return rc;
+    if (n_cls <= kMaxClasses && encode_fn()) {
+        // all classes in one launch
+        if ((long long)all.Bv * all.OH * all.OW * all.ldy >= 0xFFFFFFFFLL) return TWN_ERR_INVALID_ARG;
+        Geometry g = all;
+        g.Hv = cls[0].Hv; g.Wv = cls[0].Wv;
+        g.n_classes = n_cls;
+        for (int c = 0; c < n_cls; ++c) g.cls[c] = cls[c];
+        // The launches of the classes share the SMs, so together they take what the longest takes on its share.
+        // Narrow gradients of many pixels stay with them: the kernel of narrow layers is the faster one there (64 images
+        // of 56x56x64 <- 128: 27 us, 40 us in one launch; 20 images 21 and 18 us).
+        const SplitPlan plan = plan_conv_split(g, dev.sm_count);
+        double apart = 0.0;
+        for (int c = 0; c < n_cls; ++c) apart = std::max(apart, 1.5 + plan_conv_split(one_class(cls[c], 1), dev.sm_count / n_cls).us);
+        const long long pixels = (long long)all.Bv * all.OH * all.OW;
+        if (plan.pix && plan.us < apart && !(all.Cout <= 96 && pixels > 1000 * 128))
+            return launch_conv_split(g, dZ, T_bwd, epilogue_args(stats, epi, TWN_F32), dX, dev_status, dev, user, plan);
+    }
+    // A launch per class, side by side on helper streams.
+    std::unique_lock<std::mutex> lock(g_fork_mutex);
+    ForkPool *pool = fork_pool(dev.ordinal);
+    if (pool) {
+        TWN_CUDA_OK(cudaEventRecord(pool->fork, user));
+        for (int i = 0; i < 3; ++i) TWN_CUDA_OK(cudaStreamWaitEvent(pool->side[i], pool->fork, 0));
+    }
+    int first_error = TWN_OK;
+    for (int c = 0; c < n_cls; ++c) {
+        cudaStream_t s = (pool && c % 4 != 0) ? pool->side[c % 4 - 1] : user;
+        rc = launch_conv(one_class(cls[c], pool ? std::min(n_cls, 4) : 1), dZ, T_bwd, stats, epi, dX, TWN_F32, dev_status, s);
+        if (rc != TWN_OK && first_error == TWN_OK) first_error = rc;
+    }
     if (pool) {
         // always rejoin, also after a failed launch: the caller's stream must not be left forked
         for (int i = 0; i < 3; ++i) {

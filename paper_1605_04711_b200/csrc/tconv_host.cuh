@@ -37,6 +37,13 @@ inline EncodeTiledFn encode_fn()
     return fn;
 }
 
+// Part of a virtual output grid that is contracted with its own taps: a residue class of a strided
+// backward-for-data pass.
+constexpr int kMaxClasses = 4;
+struct TapClass {
+    int Hv, Wv, ooh, oow, tap0, n_taps;
+};
+
 struct Geometry {
     // input tensor X: NHWC [XB, XH, XW, XC] with pixel pitch ldx (elements)
     long long XB, XH, XW, XC, ldx;
@@ -56,6 +63,9 @@ struct Geometry {
     Tap taps[kMaxTaps];
     long long Cin;   // channels per tap
     int beside;      // launches that run at the same time as this one (0 or 1: none)
+    // 0: one class, described by the fields above; else all of them in one launch (launch_conv_split only)
+    int n_classes;
+    TapClass cls[kMaxClasses];
 };
 
 // Picks the pixel-tile shape BW x BH x BB (BW and BH powers of two, product `pix`) that needs the

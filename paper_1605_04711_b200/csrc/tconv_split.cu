@@ -52,16 +52,18 @@ template <> struct Cfg<128> { static constexpr int kStages = 4, kTmem = 256; };
 template <> struct Cfg<256> { static constexpr int kStages = 4, kTmem = 512; };
 
 struct SplitParams {
-    int n_tiles, tw, th;              // channel tiles; pixel tiles per row and column (the images follow)
+    int n_tiles;                      // channel tiles
     int lgBW, lgBH;                   // pixel tile = BW x BH x BB, product PIX
-    int kb, kb_per_block;             // k-blocks of the reduction, per block of the cluster
     int n_cblk;                       // k-blocks per tap
     int codes_aligned;
     const uint32_t *T;
     long long wpr;
     int sw, sh;
-    int Bv, Hv, Wv;                   // virtual output grid and its embedding in the output tensor
-    int OH, OW, osh, osw, ooh, oow;
+    int Bv, OH, OW, osh, osw;         // images; embedding of the virtual output grid in the output tensor
+    // The classes of the output grid, one for all but strided backward passes.  Their tiles follow one another, and
+    // each has its own run of taps, so their reductions differ in length.
+    int n_classes;
+    struct { int tile0, tw, th, Hv, Wv, ooh, oow, tap0, kb, kb_per_block; } cls[kMaxClasses];
     long long ldy;
     int Cout;
     const double *alpha;
@@ -199,13 +201,16 @@ tconv_split_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
 
     // a cluster's blocks are consecutive: rank = block mod splits
     const int tile = (int)blockIdx.x / splits, rank = (int)blockIdx.x - tile * splits;
-    const int nt = tile % P.n_tiles;
-    int pt = tile / P.n_tiles;
-    const int twi = pt % P.tw; pt /= P.tw;
-    const int thi = pt % P.th, tbi = pt / P.th;
+    int ci = 0;
+    while (ci + 1 < P.n_classes && tile >= P.cls[ci + 1].tile0) ++ci;
+    const auto &C = P.cls[ci];
+    const int nt = (tile - C.tile0) % P.n_tiles;
+    int pt = (tile - C.tile0) / P.n_tiles;
+    const int twi = pt % C.tw; pt /= C.tw;
+    const int thi = pt % C.th, tbi = pt / C.th;
     const int w0 = twi << P.lgBW, h0 = thi << P.lgBH, b0 = tbi * (PIX >> (P.lgBW + P.lgBH));
-    const int k0 = rank * P.kb_per_block;
-    const int k1 = k0 + P.kb_per_block < P.kb ? k0 + P.kb_per_block : P.kb;
+    const int k0 = rank * C.kb_per_block;
+    const int k1 = k0 + C.kb_per_block < C.kb ? k0 + C.kb_per_block : C.kb;
     const int n_kb = k1 > k0 ? k1 - k0 : 0;
     const int per = PIX / splits;                    // pixels that this block finishes
     const uint32_t share_bytes = (uint32_t)(per * kPitch * 4);
@@ -221,12 +226,12 @@ tconv_split_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
     }
     for (int i = tid; i < n_kb; i += kThreads) {
         const int t = (k0 + i) / P.n_cblk, cb = k0 + i - t * P.n_cblk;
-        sm->kword[i] = (uint32_t)(P.taps[t].koff / kCodesPerWord) + cb * kWordsPerBlock;
+        sm->kword[i] = (uint32_t)(P.taps[C.tap0 + t].koff / kCodesPerWord) + cb * kWordsPerBlock;
     }
     for (int p = tid; p < PIX; p += kThreads) {
         const int wv = w0 + (p & ((1 << P.lgBW) - 1)), hv = h0 + ((p >> P.lgBW) & ((1 << P.lgBH) - 1)), bv = b0 + (p >> (P.lgBW + P.lgBH));
-        sm->off[p] = wv < P.Wv && hv < P.Hv && bv < P.Bv
-                         ? (uint32_t)((((long long)bv * P.OH + (hv * P.osh + P.ooh)) * P.OW + (wv * P.osw + P.oow)) * P.ldy)
+        sm->off[p] = wv < C.Wv && hv < C.Hv && bv < P.Bv
+                         ? (uint32_t)((((long long)bv * P.OH + (hv * P.osh + C.ooh)) * P.OW + (wv * P.osw + C.oow)) * P.ldy)
                          : 0xFFFFFFFFu;
     }
     if (warp == 1) {
@@ -247,7 +252,7 @@ tconv_split_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
                 const int s = i % kStages;
                 if (i >= kStages && !mbar_wait(&sm->empty[s], ((i / kStages) & 1) ^ 1, abort_flag, P.status)) break;
                 mbar_expect_tx(&sm->full[s], L::kXBytes);
-                const Tap tap = P.taps[t];
+                const Tap tap = P.taps[C.tap0 + t];
                 tma_load_4d(sm->x[s], &map_x, &sm->full[s], cb * kBlockK, w0 * P.sw + tap.dw, h0 * P.sh + tap.dh, b0);
                 if (++cb == P.n_cblk) { cb = 0; ++t; }
             }
@@ -393,12 +398,19 @@ int launch_t(const Geometry &g, SplitParams &P, const void *X, int splits, const
         TWN_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost));
         attr_set[dev.ordinal] = true;
     }
-    const long long tiles = pick_tile(g, PIX, &P.lgBW, &P.lgBH) * P.n_tiles;
+    pick_tile(g, PIX, &P.lgBW, &P.lgBH);
     const int BW = 1 << P.lgBW, BH = 1 << P.lgBH, BB = PIX >> (P.lgBW + P.lgBH);
-    P.tw = (g.Wv + BW - 1) / BW;
-    P.th = (g.Hv + BH - 1) / BH;
+    long long tiles = 0;
+    for (int c = 0; c < P.n_classes; ++c) {
+        auto &C = P.cls[c];
+        C.tile0 = (int)tiles;
+        C.tw = (C.Wv + BW - 1) / BW;
+        C.th = (C.Hv + BH - 1) / BH;
+        C.kb_per_block = (C.kb + splits - 1) / splits;
+        tiles += (long long)P.n_tiles * C.tw * C.th * ((g.Bv + BB - 1) / BB);
+        if (tiles > 0x7fffffffLL) return TWN_ERR_INVALID_ARG;
+    }
     if (tiles <= 0 || tiles * splits > 0x7fffffffLL) return TWN_ERR_INVALID_ARG;
-    P.kb_per_block = (P.kb + splits - 1) / splits;
     CUtensorMap map_x;
     cuuint64_t dims[4] = {(cuuint64_t)g.XC, (cuuint64_t)g.XW, (cuuint64_t)g.XH, (cuuint64_t)g.XB};
     const long long rowp = g.x_row_pitch ? g.x_row_pitch : g.XW * g.ldx;
@@ -444,7 +456,12 @@ SplitPlan plan_conv_split(const Geometry &g, int sm_count)
     static const double E[4] = {3.89, 4.47, 5.51, 7.73}, R[4] = {0.241, 0.249, 0.255, 0.275};
     SplitPlan best = {0, 0, 1e30};
     if (g.bn_partial) return best;
-    const long long kb = (long long)g.n_taps * ((g.Cin + kBlockK - 1) / kBlockK);
+    // with classes: as many tiles as the largest has each (it comes first), the longest reduction and the mean one
+    const int classes = g.n_classes > 0 ? g.n_classes : 1;
+    const long long cblk = (g.Cin + kBlockK - 1) / kBlockK;
+    long long kb = g.n_classes > 0 ? 0 : g.n_taps * cblk;
+    for (int c = 0; c < g.n_classes; ++c) kb = std::max(kb, g.cls[c].n_taps * cblk);
+    const double mean = g.n_classes > 0 && kb > 0 ? (double)g.n_taps * cblk / classes / kb : 1.0;
     const int n_tiles = (g.Cout + kChan - 1) / kChan;
     for (int i = 0; i < 4; ++i) {
         int a, b;
@@ -453,13 +470,14 @@ SplitPlan plan_conv_split(const Geometry &g, int sm_count)
         for (int splits = 1; splits <= (pix == 256 ? 2 : 8); splits *= 2) {
             const long long n = (kb + splits - 1) / splits;
             if ((splits > 1 && splits > kb) || n > kMaxBlocks) continue;
-            const double ctas = (double)tiles * splits, L = ctas / sm_count;
+            const double ctas = (double)tiles * classes * splits, L = ctas / sm_count;
             const bool alone = pix == 256 || (pix == 128 && splits >= 4);
             // clusters of 4 and 8 fill 128 and 112 of 148 SMs
             const double slots = sm_count * (splits == 8 ? 112.0 / 148 : splits == 4 ? 128.0 / 148 : splits == 2 ? 144.0 / 148 : 1.0);
             const double rounds = alone ? std::ceil(ctas / slots) : std::max(1.0, 0.607 * L + 0.428);
             const double x = splits > 1 ? 0.58 + pix * (0.0004 + 0.0008 * splits) : 0.0;
-            const double us = -1.0 + rounds * (E[i] + n * R[i] * (1.0 + 0.25 * std::min(1.0, L))) + x * (alone ? rounds : 1.0);
+            const double r = n * R[i] * (1.0 + 0.25 * std::min(1.0, L));
+            const double us = -1.0 + std::max(E[i] + r, rounds * (E[i] + mean * r)) + x * (alone ? rounds : 1.0);
             if (us < best.us) best = SplitPlan{pix, splits, us};
         }
     }
@@ -472,7 +490,13 @@ int launch_conv_split(const Geometry &g, const void *X, const uint32_t *T, const
     SplitParams P;
     P.n_tiles = (g.Cout + kChan - 1) / kChan;
     P.n_cblk = (int)((g.Cin + kBlockK - 1) / kBlockK);
-    P.kb = g.n_taps * P.n_cblk;
+    P.n_classes = g.n_classes > 0 ? g.n_classes : 1;
+    for (int c = 0; c < P.n_classes; ++c) {
+        const TapClass k = g.n_classes > 0 ? g.cls[c] : TapClass{g.Hv, g.Wv, g.ooh, g.oow, 0, g.n_taps};
+        P.cls[c].Hv = k.Hv; P.cls[c].Wv = k.Wv; P.cls[c].ooh = k.ooh; P.cls[c].oow = k.oow;
+        P.cls[c].tap0 = k.tap0;
+        P.cls[c].kb = k.n_taps * P.n_cblk;
+    }
     P.codes_aligned = 1;
     for (int t = 0; t < g.n_taps; ++t) {
         P.taps[t] = g.taps[t];
@@ -481,8 +505,8 @@ int launch_conv_split(const Geometry &g, const void *X, const uint32_t *T, const
     P.T = T;
     P.wpr = g.ld_codes / (g.code_bits == 1 ? 32 : 16);
     P.sw = g.sw; P.sh = g.sh;
-    P.Bv = g.Bv; P.Hv = g.Hv; P.Wv = g.Wv;
-    P.OH = g.OH; P.OW = g.OW; P.osh = g.osh; P.osw = g.osw; P.ooh = g.ooh; P.oow = g.oow;
+    P.Bv = g.Bv;
+    P.OH = g.OH; P.OW = g.OW; P.osh = g.osh; P.osw = g.osw;
     P.ldy = g.ldy;
     P.Cout = g.Cout;
     P.alpha = epi.alpha; P.scale = epi.scale; P.shift = epi.shift;
