@@ -77,8 +77,12 @@ typedef struct {
  * a ReLU fused into the backward-for-data pass of the layer above it: with `residual` = the
  * lower layer's output and `scale` = its folded batch-norm scale, twn_conv2d_bwd_data writes
  * the lower layer's dZ directly (Algorithm 1, TernaryBackward, followed by the chain rule
- * through y = relu(z * scale + shift)). */
-enum { TWN_RESIDUAL_ADD = 0, TWN_RESIDUAL_GATE = 1 };
+ * through y = relu(z * scale + shift)).
+ * TWN_SUM_IN_ORDER, or-ed in, keeps a launch that would not fill the GPU from splitting the reduction over several
+ * thread blocks: every sum then runs over the taps and channels in order, and an output has the same bits whatever
+ * the batch and the launch shape.  Forward passes of a training step want that: a ReLU gate that a differently rounded
+ * sum flips changes the gradient there by all of its value, not by a rounding. */
+enum { TWN_RESIDUAL_ADD = 0, TWN_RESIDUAL_GATE = 1, TWN_SUM_IN_ORDER = 2 };
 typedef struct {
     const float *scale;    /* fp32 [N] or NULL (folded batch-norm scale)            */
     const float *shift;    /* fp32 [N] or NULL                                      */
@@ -86,7 +90,7 @@ typedef struct {
     int32_t residual_dtype;/* TWN_F32 | TWN_BF16                                    */
     int32_t relu;          /* 0 | 1                                                 */
     int32_t out_dtype;     /* TWN_F32 | TWN_BF16 (round to nearest even)            */
-    int32_t residual_op;   /* TWN_RESIDUAL_ADD (0) | TWN_RESIDUAL_GATE              */
+    int32_t residual_op;   /* TWN_RESIDUAL_ADD or _GATE, | TWN_SUM_IN_ORDER          */
 } twn_epilogue_t;
 
 /* ---- library ---------------------------------------------------------- */

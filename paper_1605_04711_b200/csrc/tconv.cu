@@ -763,7 +763,8 @@ EpilogueArgs epilogue_args(const twn_stats_t *stats, const twn_epilogue_t *epi, 
     ea.shift = epi ? epi->shift : nullptr;
     ea.residual = epi ? epi->residual : nullptr;
     ea.res_dtype = epi ? epi->residual_dtype : TWN_F32;
-    ea.res_gate = (epi && epi->residual) ? epi->residual_op : 0;
+    ea.res_gate = (epi && epi->residual) ? epi->residual_op & TWN_RESIDUAL_GATE : 0;
+    ea.in_order = epi && (epi->residual_op & TWN_SUM_IN_ORDER);
     ea.relu = epi ? epi->relu : 0;
     ea.out_dtype = epi ? epi->out_dtype : out_dtype_default;
     return ea;
@@ -782,7 +783,7 @@ int launch_conv(const Geometry &g, const void *X, const uint32_t *T, const twn_s
     if ((long long)g.Bv * g.OH * g.OW * g.ldy >= 0xFFFFFFFFLL) return TWN_ERR_INVALID_ARG;
     const EpilogueArgs ea = epilogue_args(stats, epi, out_dtype_default);
     // problems that do not fill the GPU: small tiles, the reduction split over a cluster
-    const SplitPlan split = plan_conv_split(g, dev.sm_count / (g.beside > 1 ? g.beside : 1));
+    const SplitPlan split = plan_conv_split(g, dev.sm_count / (g.beside > 1 ? g.beside : 1), ea.in_order);
     // narrow layers: the kernel that decodes the layer's codes once per block
     bool handled = false;
     rc = launch_conv_resident(g, X, T, ea, Y, dev_status, dev, s, split.us, &handled);
@@ -888,7 +889,7 @@ int check_epilogue(const twn_epilogue_t *e)
     TWN_REQUIRE(e->out_dtype == TWN_F32 || e->out_dtype == TWN_BF16, TWN_ERR_INVALID_ARG);
     TWN_REQUIRE(e->residual_dtype == TWN_F32 || e->residual_dtype == TWN_BF16, TWN_ERR_INVALID_ARG);
     TWN_REQUIRE(e->relu == 0 || e->relu == 1, TWN_ERR_INVALID_ARG);
-    TWN_REQUIRE(e->residual_op == TWN_RESIDUAL_ADD || e->residual_op == TWN_RESIDUAL_GATE, TWN_ERR_INVALID_ARG);
+    TWN_REQUIRE(e->residual_op >= 0 && e->residual_op <= (TWN_RESIDUAL_GATE | TWN_SUM_IN_ORDER), TWN_ERR_INVALID_ARG);
     TWN_REQUIRE(twn_aligned(e->scale, 4) && twn_aligned(e->shift, 4) && twn_aligned(e->residual, 4), TWN_ERR_MISALIGNED);
     return TWN_OK;
 }
@@ -1120,7 +1121,7 @@ int conv_bwd_data_impl(const twn_conv_desc_t *d, const void *dZ, const uint32_t 
     int n_cls = 0;
     // A residue class no tap reaches gets epilogue(0); when the epilogue only adds a second gradient
     // branch that already lives in dX (in place), that leaves the class as it is: nothing to launch.
-    const bool skip_empty = epi && epi->residual == dX && epi->residual_op == TWN_RESIDUAL_ADD && !epi->scale && !epi->shift &&
+    const bool skip_empty = epi && epi->residual == dX && !(epi->residual_op & TWN_RESIDUAL_GATE) && !epi->scale && !epi->shift &&
                             !epi->relu && epi->residual_dtype == epi->out_dtype;
     for (int ph = 0; ph < d->stride_h; ++ph)
         for (int pw = 0; pw < d->stride_w; ++pw) {
@@ -1169,12 +1170,13 @@ int conv_bwd_data_impl(const twn_conv_desc_t *d, const void *dZ, const uint32_t 
         // The launches of the classes share the SMs, so together they take what the longest takes on its share.
         // Narrow gradients of many pixels stay with them: the kernel of narrow layers is the faster one there (64 images
         // of 56x56x64 <- 128: 27 us, 40 us in one launch; 20 images 21 and 18 us).
-        const SplitPlan plan = plan_conv_split(g, dev.sm_count);
+        const EpilogueArgs ea = epilogue_args(stats, epi, TWN_F32);
+        const SplitPlan plan = plan_conv_split(g, dev.sm_count, ea.in_order);
         double apart = 0.0;
-        for (int c = 0; c < n_cls; ++c) apart = std::max(apart, 1.5 + plan_conv_split(one_class(cls[c], 1), dev.sm_count / n_cls).us);
+        for (int c = 0; c < n_cls; ++c) apart = std::max(apart, 1.5 + plan_conv_split(one_class(cls[c], 1), dev.sm_count / n_cls, ea.in_order).us);
         const long long pixels = (long long)all.Bv * all.OH * all.OW;
         if (plan.pix && plan.us < apart && !(all.Cout <= 96 && pixels > 1000 * 128))
-            return launch_conv_split(g, dZ, T_bwd, epilogue_args(stats, epi, TWN_F32), dX, dev_status, dev, user, plan);
+            return launch_conv_split(g, dZ, T_bwd, ea, dX, dev_status, dev, user, plan);
     }
     // A launch per class, side by side on helper streams.
     std::unique_lock<std::mutex> lock(g_fork_mutex);

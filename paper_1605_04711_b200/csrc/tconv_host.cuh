@@ -94,6 +94,7 @@ struct EpilogueArgs {
     const float *scale, *shift;
     const void *residual;
     int res_dtype, res_gate, relu, out_dtype;
+    bool in_order;                // the reduction is not split (TWN_SUM_IN_ORDER)
 };
 
 // Contraction with the layer's decoded weights resident in shared memory (tconv_res.cu).  Launches
@@ -110,7 +111,7 @@ struct SplitPlan {
     int pix, splits;
     double us;        // what the launch should take
 };
-SplitPlan plan_conv_split(const Geometry &g, int sm_count);
+SplitPlan plan_conv_split(const Geometry &g, int sm_count, bool in_order);
 int launch_conv_split(const Geometry &g, const void *X, const uint32_t *T, const EpilogueArgs &epi, void *Y,
                       int32_t *dev_status, const twn_device_info &dev, cudaStream_t s, const SplitPlan &plan);
 

@@ -450,7 +450,7 @@ namespace twn_detail {
 // for blocks that have an SM to themselves the number of rounds, where clusters do not fill every SM; E and R what a
 // block and a k-block take (few pixels make a k-block hardly cheaper: its decoding and its issue stay); X the exchange.
 // What it picks takes 3 % longer on average than the best of what was measured, and a third less than without this kernel.
-SplitPlan plan_conv_split(const Geometry &g, int sm_count)
+SplitPlan plan_conv_split(const Geometry &g, int sm_count, bool in_order)
 {
     static const int pixels[4] = {32, 64, 128, 256};
     static const double E[4] = {3.89, 4.47, 5.51, 7.73}, R[4] = {0.241, 0.249, 0.255, 0.275};
@@ -467,7 +467,7 @@ SplitPlan plan_conv_split(const Geometry &g, int sm_count)
         int a, b;
         const int pix = pixels[i];
         const long long tiles = pick_tile(g, pix, &a, &b) * n_tiles;
-        for (int splits = 1; splits <= (pix == 256 ? 2 : 8); splits *= 2) {
+        for (int splits = 1; splits <= (in_order ? 1 : pix == 256 ? 2 : 8); splits *= 2) {
             const long long n = (kb + splits - 1) / splits;
             if ((splits > 1 && splits > kb) || n > kMaxBlocks) continue;
             const double ctas = (double)tiles * classes * splits, L = ctas / sm_count;

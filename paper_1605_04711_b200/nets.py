@@ -132,7 +132,9 @@ class TernaryNet:
                 self.act[L.name] = torch.zeros((B, L.Ho, L.Wo, L.Cout), dtype=out_dtype, device="cuda")
                 res = self.act[L.residual] if L.residual else None
                 e["epi"] = twn.epilogue(e["scale"], e["shift"], res, relu=L.relu,
-                                        out_dtype=twn.F32 if L.out_f32 else twn.BF16)
+                                        out_dtype=twn.F32 if L.out_f32 else twn.BF16,
+                                        # the backward pass goes through the gates of these very bits
+                                        residual_op=twn.SUM_IN_ORDER if self.train else twn.RESIDUAL_ADD)
                 if self.optimizer:
                     if L.small_cin and not L.fold:
                         raise NotImplementedError("the update needs a weight gradient in the layout of the weights")

@@ -248,6 +248,7 @@ def transpose_codes(packed_fwd: torch.Tensor, ld_fwd: int, desc: ConvDesc, packe
 
 
 RESIDUAL_ADD, RESIDUAL_GATE = 0, 1
+SUM_IN_ORDER = 2          # or-ed into residual_op
 
 
 def epilogue(scale=None, shift=None, residual=None, relu=False, out_dtype=F32, residual_op=RESIDUAL_ADD):
