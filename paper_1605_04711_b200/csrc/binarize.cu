@@ -5,139 +5,209 @@
 //   B_i = +1 if W_i >= 0, -1 if W_i < 0;      alpha = (1/n) sum |W_i|
 //
 // Neither needs a threshold, so one sweep over the fp32 master weights does both: 4 bytes read and
-// 1/32 byte written per weight, bound by HBM bandwidth.  A warp works on one word of 32 codes at a
-// time: lane l loads the element whose bit it owns in the packed word (a permutation inside one
-// 128-byte line, so the load is fully coalesced), and a warp vote on "negative" IS the packed word.
-// sum |W| has a fixed order: per-lane fp64 partial sums, shuffle tree, block tree, one partial per
-// block, folded in index order by the block that finishes last.
-#include "common.cuh"
+// 1/32 byte written per weight, bound by HBM bandwidth.  A thread holds eight quarters of four weights; their 32 signs
+// are collected by funnel shifts, and an 8x8 transpose of 4-bit groups among eight lanes leaves every lane with one
+// whole word.  (A warp vote per word of 32 costs a 4-byte load, a vote and a select per weight of a lane, and rows that
+// are no whole words were voted one word at a time.)
+// sum |W| has a fixed order: per-thread fp64 sums, the trees of sweep.cuh, one part per block.  The blocks meet through
+// the workspace and a grid-wide barrier, those of a small tensor as one cluster through distributed shared memory.
+#include <algorithm>
+
+#include "sweep.cuh"
 
 namespace {
 
-constexpr int kThreads = 256;
-constexpr int kWarps = kThreads / 32;
-constexpr int kMaxBlocks = 2048;
-// workspace: [0,256) ticket, then kMaxBlocks fp64 partial sums and kMaxBlocks 8-byte negative counts
-constexpr size_t kBinWorkspaceBytes = 256 + 2 * size_t(kMaxBlocks) * 8;
+constexpr int kThreads = 256;            // the helpers below
+constexpr int kGroupWords = 512;         // words of a group: eight quarter-words per thread
+// workspace: kMaxParts fp64 sums, then kMaxParts negative counts (the size is that of an earlier layout)
+constexpr size_t kBinWorkspaceBytes = 256 + 2 * size_t(2048) * 8;
 
-// element of a 32-code group whose bit is bit l of the word: even elements fill the low half-word from
-// bit 15 down, odd elements the high half-word from bit 31 down
-__device__ __forceinline__ int element_of_bit(int l) { return l < 16 ? 2 * (15 - l) : 2 * (31 - l) + 1; }
 __host__ __device__ inline int bit_of_element(int e) { return 15 - (e >> 1) + 16 * (e & 1); }
 
-__device__ __forceinline__ double warp_sum_d(double v)
+struct BinParams {
+    const float *W;
+    uint32_t *packed;
+    twn_stats_t *stats;
+    double *part_sum;
+    unsigned long long *part_neg;
+    unsigned long long n, words;         // weights; words that hold codes
+    long long rows, cols, wpr;
+    unsigned int wpr_used, parts, part_words;
+    bool vec4, dense;                    // quarters start on 16-byte boundaries; word w holds weights 32 w ..
+};
+
+// Word w: its index in the packed matrix, its first weight and how many weights it holds.
+struct BinPlace {
+    unsigned long long out, f;
+    unsigned int valid;
+};
+__device__ __forceinline__ BinPlace bin_place(const BinParams &P, unsigned long long w)
 {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    return v;
+    BinPlace p;
+    if (P.dense) {
+        p.out = w;
+        p.f = 32ull * w;
+        p.valid = (unsigned int)min(32ull, P.n - p.f);
+    } else {
+        const unsigned long long row = w >> 32 ? w / P.wpr_used : (unsigned int)w / P.wpr_used;
+        const unsigned long long j = w - row * P.wpr_used;
+        p.out = row * P.wpr + j;
+        p.f = row * P.cols + 32 * j;
+        p.valid = (unsigned int)min(32ull, (unsigned long long)P.cols - 32 * j);
+    }
+    return p;
 }
-__device__ __forceinline__ unsigned long long warp_sum_u(unsigned long long v)
+
+// Eight nibbles of x, exchanged among the lanes of an aligned group of eight: lane l gets nibble l of every lane.
+__device__ __forceinline__ uint32_t exchange_nibbles(uint32_t x)
 {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    return v;
+    const int lane = threadIdx.x;
+    uint32_t y = __shfl_xor_sync(0xffffffffu, x, 4);
+    x = __byte_perm(x, y, (lane & 4) ? 0x3276 : 0x5410);
+    y = __shfl_xor_sync(0xffffffffu, x, 2);
+    x = __byte_perm(x, y, (lane & 2) ? 0x3715 : 0x6240);
+    y = __shfl_xor_sync(0xffffffffu, x, 1);
+    return (lane & 1) ? ((x & 0xF0F0F0F0u) | ((y >> 4) & 0x0F0F0F0Fu)) : ((x & 0x0F0F0F0Fu) | ((y << 4) & 0xF0F0F0F0u));
 }
 
-__global__ void __launch_bounds__(kThreads)
-binarize_kernel(const float *__restrict__ W, long long rows, long long cols, long long ld_codes,
-                uint32_t *__restrict__ packed, void *ws_raw, twn_stats_t *__restrict__ stats)
+template <bool CLUSTER>
+__global__ void __launch_bounds__(kSweepThreads, kSweepBlocksPerSm)
+binarize_kernel(const __grid_constant__ BinParams P)
 {
-    __shared__ double red_s[kWarps];
-    __shared__ unsigned long long red_n[kWarps];
-    __shared__ bool is_last;
-    unsigned int *ticket = reinterpret_cast<unsigned int *>(ws_raw);
-    double *part_sum = reinterpret_cast<double *>(static_cast<char *>(ws_raw) + 256);
-    unsigned long long *part_neg = reinterpret_cast<unsigned long long *>(part_sum + kMaxBlocks);
-
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int e = element_of_bit(lane);
-    const long long wpr = ld_codes >> 5;                       // words per packed row
-    const long long total_words = rows * wpr;
-    const long long warp_id = (long long)blockIdx.x * kWarps + warp, n_warps = (long long)gridDim.x * kWarps;
-    // a contiguous matrix whose rows are whole words is one long row
-    const bool flat = (ld_codes == cols);
-    const long long n = rows * cols;
-
-    double acc = 0.0;
-    unsigned long long negs = 0;
-    if (flat) {
-        // sixteen words per warp and iteration, their loads issued before any is used: the sweep is bound by the
-        // bytes a warp keeps in flight
-        constexpr int kU = 16;
-        double a1 = 0.0;
-        for (long long w0 = warp_id * kU; w0 < total_words; w0 += n_warps * kU) {
-            float x[kU];
+    __shared__ Reduce red;
+    __shared__ double sum_s[kSmallParts];
+    __shared__ unsigned long long neg_s[kSmallParts];
+    const unsigned int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, b = blockIdx.x, G = gridDim.x;
+    unsigned int turn = 0;
+    if (CLUSTER) {
+        if (tid < kSmallParts) { sum_s[tid] = 0.0; neg_s[tid] = 0ull; }
+        cluster_arrive();
+    }
+    // padding words of the rows
+    const unsigned int pad = (unsigned int)(P.wpr - P.wpr_used);
+    if (pad && P.packed)
+        for (unsigned long long i = (unsigned long long)b * kSweepThreads + tid; i < (unsigned long long)P.rows * pad; i += (unsigned long long)G * kSweepThreads) {
+            const unsigned long long r = i >> 32 ? i / pad : (unsigned int)i / pad;
+            P.packed[r * P.wpr + P.wpr_used + (i - r * pad)] = 0u;
+        }
+    double own = 0.0;
+    unsigned long long own_neg = 0;
+    for (unsigned int part = b; part < P.parts; part += G) {
+        const unsigned long long w0 = (unsigned long long)part * P.part_words;
+        const unsigned long long w1 = min(w0 + P.part_words, P.words);
+        double a[4] = {0.0, 0.0, 0.0, 0.0};
+        unsigned int neg = 0, none = 0;
+        for (unsigned long long wg = w0; wg < w1; wg += kGroupWords) {
+            float4 v[8];
+            if (P.dense && P.vec4 && wg + kGroupWords <= w1 && (wg + kGroupWords) * 32 <= P.n) {
+                const float4 *v4 = reinterpret_cast<const float4 *>(P.W) + wg * 8 + tid;
 #pragma unroll
-            for (int u = 0; u < kU; ++u) x[u] = (w0 + u < total_words) ? __ldg(W + ((w0 + u) << 5) + e) : 0.0f;
+                for (int k = 0; k < 8; ++k) v[k] = __ldg(v4 + k * kSweepThreads);
+            } else {
+                // quarter-words that are not whole are masked; addresses stay inside the part
+                unsigned long long f[8];
+                unsigned int left[8];
 #pragma unroll
-            for (int u = 0; u < kU; ++u) {
-                if (u & 1) a1 += (double)fabsf(x[u]); else acc += (double)fabsf(x[u]);
-                const unsigned int word = __ballot_sync(0xffffffffu, x[u] < 0.0f);     // -0.0 and NaN vote "not negative"
-                if (lane == u && w0 + u < total_words) {
-                    packed[w0 + u] = word;
-                    negs += (unsigned long long)__popc(word);
+                for (int k = 0; k < 8; ++k) {
+                    const unsigned long long w = wg + (k * kSweepThreads + tid) / 8;
+                    const unsigned int e = 4 * (tid & 7);
+                    const BinPlace p = bin_place(P, min(w, w1 - 1));
+                    left[k] = w < w1 && p.valid > e ? p.valid - e : 0;
+                    f[k] = left[k] ? p.f + e : p.f;
+                }
+                if (P.vec4 && !P.dense) {
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) v[k] = __ldg(reinterpret_cast<const float4 *>(P.W + f[k]));
+                } else {
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) {
+                        v[k].x = left[k] > 0 ? __ldg(P.W + f[k]) : 0.0f;
+                        v[k].y = left[k] > 1 ? __ldg(P.W + f[k] + 1) : 0.0f;
+                        v[k].z = left[k] > 2 ? __ldg(P.W + f[k] + 2) : 0.0f;
+                        v[k].w = left[k] > 3 ? __ldg(P.W + f[k] + 3) : 0.0f;
+                    }
+                }
+#pragma unroll
+                for (int k = 0; k < 8; ++k)
+                    if (left[k] < 4) {
+                        if (left[k] < 1) v[k].x = 0.0f;
+                        if (left[k] < 2) v[k].y = 0.0f;
+                        if (left[k] < 3) v[k].z = 0.0f;
+                        v[k].w = 0.0f;
+                    }
+            }
+            // nibble k of `signs`: elements 0, 2, 1, 3 of quarter k, the first on the left
+            uint32_t signs = 0;
+#pragma unroll
+            for (int k = 7; k >= 0; --k) {
+                const float x4[4] = {v[k].x, v[k].z, v[k].y, v[k].w};
+#pragma unroll
+                for (int x = 0; x < 4; ++x) {
+                    a[x] += (double)fabsf(x4[x]);
+                    // "negative" is w < 0, which -0.0 is not: adding zero makes it +0.0
+                    signs = __funnelshift_l(__float_as_uint(__fadd_rn(x4[x], 0.0f)), signs, 1);
                 }
             }
+            neg += __popc(signs);
+            // Lane l now has word l % 8 of the eight that its group shares, a quarter per nibble, the first on the right:
+            // reverse the nibbles, then even elements to the low half and odd ones to the high half.
+            uint32_t x = __byte_perm(exchange_nibbles(signs), 0u, 0x0123);
+            x = ((x >> 4) & 0x0F0F0F0Fu) | ((x << 4) & 0xF0F0F0F0u);
+            uint32_t even = (x >> 2) & 0x33333333u, odd = x & 0x33333333u;
+            even = (even | (even >> 2)) & 0x0F0F0F0Fu; odd = (odd | (odd >> 2)) & 0x0F0F0F0Fu;
+            even = (even | (even >> 4)) & 0x00FF00FFu; odd = (odd | (odd >> 4)) & 0x00FF00FFu;
+            even = (even | (even >> 8)) & 0x0000FFFFu; odd = (odd | (odd >> 8)) & 0x0000FFFFu;
+            const unsigned long long w = wg + (lane & 7) * (kSweepThreads / 8) + warp * 4 + (lane >> 3);
+            if (w < w1) P.packed[P.dense ? w : bin_place(P, w).out] = even | (odd << 16);
         }
-        acc += a1;
-    } else {
-        for (long long w = warp_id; w < total_words; w += n_warps) {
-            const long long r = w / wpr, c = ((w - r * wpr) << 5) + e;
-            const bool valid = c < cols;
-            const float x = valid ? __ldg(W + r * cols + c) : 0.0f;
-            acc += (double)fabsf(x);
-            const unsigned int word = __ballot_sync(0xffffffffu, x < 0.0f);
-            if (lane == 0) {
-                packed[w] = word;
-                negs += (unsigned long long)__popc(word);
-            }
+        const double s = sweep_sum((a[0] + a[1]) + (a[2] + a[3]), neg, none, red, turn);
+        if (CLUSTER) {
+            own = s;                     // a block of the cluster has at most one part
+            own_neg = neg;
+        } else if (tid == 0) {
+            P.part_sum[part] = s;
+            P.part_neg[part] = neg;
         }
     }
-    // block partials
-    acc = warp_sum_d(acc);
-    negs = warp_sum_u(negs);
-    if (lane == 0) { red_s[warp] = acc; red_n[warp] = negs; }
-    __syncthreads();
-    if (warp == 0) {
-        double s = lane < kWarps ? red_s[lane] : 0.0;
-        unsigned long long c = lane < kWarps ? red_n[lane] : 0ull;
-        s = warp_sum_d(s);
-        c = warp_sum_u(c);
-        if (lane == 0) { part_sum[blockIdx.x] = s; part_neg[blockIdx.x] = c; }
-    }
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) is_last = (atomicAdd(ticket, 1u) == gridDim.x - 1);
-    __syncthreads();
-    if (!is_last) return;
-    // the last block folds the partials in index order
     double s = 0.0;
     unsigned long long c = 0;
-    for (int b = threadIdx.x; b < (int)gridDim.x; b += kThreads) { s += __ldcg(part_sum + b); c += __ldcg(part_neg + b); }
-    s = warp_sum_d(s);
-    c = warp_sum_u(c);
-    __syncthreads();
-    if (lane == 0) { red_s[warp] = s; red_n[warp] = c; }
-    __syncthreads();
-    if (warp == 0) {
-        s = lane < kWarps ? red_s[lane] : 0.0;
-        c = lane < kWarps ? red_n[lane] : 0ull;
-        s = warp_sum_d(s);
-        c = warp_sum_u(c);
-        if (lane == 0) {
-            stats->delta = 0.0;
-            stats->alpha = n > 0 ? s / (double)n : 0.0;
-            stats->sum_abs = s;
-            stats->sum_abs_kept = s;
-            stats->n_neg = c;
-            stats->n_zero = 0;
-            stats->n_pos = (unsigned long long)n - c;
-            stats->status = isfinite(s) ? TWN_OK : TWN_ERR_NONFINITE;
-            stats->reserved = 0;
-            *ticket = 0u;
+    if (CLUSTER) {
+        cluster_wait();
+        if (tid == 0) {
+            st_peer(peer_smem(&sum_s[b], 0), __double_as_longlong(own));
+            st_peer(peer_smem(&neg_s[b], 0), own_neg);
         }
+        cluster_arrive();
+        cluster_wait();
+        if (b != 0) return;
+        s = tree8(sum_s);
+        for (int i = 0; i < kSmallParts; ++i) c += neg_s[i];
+    } else {
+        cooperative_groups::this_grid().sync();
+        if (b != 0) return;
+        unsigned int lo = 0, hi = 0;     // of at most kMaxParts counts below 2^32: no carry gets lost
+        for (unsigned int i = tid; i < P.parts; i += kSweepThreads) {
+            s += __ldcg(P.part_sum + i);
+            const unsigned long long k = __ldcg(P.part_neg + i);
+            lo += (unsigned int)(k & 0xFFFFFull);
+            hi += (unsigned int)(k >> 20);
+        }
+        s = sweep_sum(s, lo, hi, red, turn);
+        c = lo + ((unsigned long long)hi << 20);
+    }
+    if (tid == 0) {
+        P.stats->delta = 0.0;
+        P.stats->alpha = P.n > 0 ? s / (double)P.n : 0.0;
+        P.stats->sum_abs = s;
+        P.stats->sum_abs_kept = s;
+        P.stats->n_neg = c;
+        P.stats->n_zero = 0;
+        P.stats->n_pos = P.n - c;
+        P.stats->status = isfinite(s) ? TWN_OK : TWN_ERR_NONFINITE;
+        P.stats->reserved = 0;
     }
 }
+
 
 __global__ void __launch_bounds__(kThreads)
 unpack_b1_kernel(const uint32_t *__restrict__ packed, long long rows, long long cols, long long ld_codes,
@@ -175,7 +245,7 @@ transpose_b1_kernel(const uint32_t *__restrict__ in, long long ld_in, int Cout, 
 int grid_for_words(long long work, int sms)
 {
     long long g = (work + kThreads - 1) / kThreads;
-    const long long cap = (long long)sms * 8 < kMaxBlocks ? (long long)sms * 8 : kMaxBlocks;
+    const long long cap = (long long)sms * 8;
     if (g > cap) g = cap;
     if (g < 1) g = 1;
     return (int)g;
@@ -199,14 +269,33 @@ extern "C" int twn_binarize(const float *W, int64_t rows, int64_t cols, twn_stat
     twn_device_info dev;
     const int rc = twn_current_device(&dev);
     if (rc != TWN_OK) return rc;
-    cudaStream_t s = twn_cu(stream);
-    TWN_CUDA_OK(cudaMemsetAsync(workspace, 0, 64, s));           // the ticket
-    const long long words = (long long)rows * (ld_codes / 32);
-    // a warp takes one word per iteration
-    const int grid = grid_for_words(words * 32, dev.sm_count);
-    binarize_kernel<<<grid, kThreads, 0, s>>>(W, rows, cols, ld_codes, packed, workspace, stats);
-    TWN_CUDA_OK(cudaGetLastError());
-    return TWN_OK;
+    BinParams P;
+    P.W = W; P.packed = packed; P.stats = stats;
+    P.part_sum = static_cast<double *>(workspace);
+    P.part_neg = reinterpret_cast<unsigned long long *>(P.part_sum + kMaxParts);
+    P.n = (unsigned long long)n;
+    P.rows = rows; P.cols = cols; P.wpr = ld_codes / 32;
+    const unsigned long long used = (unsigned long long)(cols + 31) / 32;
+    P.words = (unsigned long long)rows * used;
+    // whole groups per part, at most one part per block of a full grid
+    const unsigned long long part = std::max(1ull, ((P.words + kMaxParts - 1) / kMaxParts + kGroupWords - 1) / kGroupWords) * kGroupWords;
+    TWN_REQUIRE(used <= 0xFFFFFFFFull && part <= 0x04000000ull, TWN_ERR_TOO_LARGE);
+    P.wpr_used = (unsigned int)used;
+    P.part_words = (unsigned int)part;
+    P.parts = (unsigned int)std::max(1ull, (P.words + part - 1) / part);
+    P.vec4 = twn_aligned(W, 16) && (rows == 1 || cols % 4 == 0);
+    P.dense = rows == 1 || ld_codes == cols;
+    cudaLaunchAttributeValue val = {};
+    if (P.parts <= (unsigned int)kSmallParts) {
+        unsigned int grid = 1;
+        while (grid < P.parts) grid *= 2;
+        val.clusterDim.x = grid;
+        val.clusterDim.y = val.clusterDim.z = 1;
+        return launch_with(binarize_kernel<true>, grid, cudaLaunchAttributeClusterDimension, val, twn_cu(stream), P);
+    }
+    val.cooperative = 1;
+    return launch_with(binarize_kernel<false>, std::min(P.parts, (unsigned int)(dev.sm_count * kSweepBlocksPerSm)),
+                       cudaLaunchAttributeCooperative, val, twn_cu(stream), P);
 }
 
 extern "C" int twn_unpack_b1(const uint32_t *packed, int64_t rows, int64_t cols, int64_t ld_codes, int8_t *codes,

@@ -13,24 +13,18 @@
 // kMaxParts parts, every part is summed by one block in a fixed way (per-thread strided sums, shuffle tree per
 // warp, warps in order) and the parts are folded in a fixed way.  Which block takes a part does not matter, so a
 // tensor gets the same bits alone and in a batch, on any number of SMs.  No floating-point atomics.
-#include <cooperative_groups.h>
-
 #include <algorithm>
 
-#include "common.cuh"
+#include "sweep.cuh"
 
 namespace {
 
 constexpr int kThreads = 256;       // pack, unpack
 constexpr int kWarps = kThreads / 32;
 constexpr int kTrThreads = 128;     // re-layouts
-constexpr int kSweepWarps = 16;
-constexpr int kSweepThreads = 32 * kSweepWarps;
-constexpr int kSweepBlocksPerSm = 2;                        // 64 registers; three blocks spill: 1e8 weights 131 -> 164 us
-constexpr unsigned int kMaxParts = kSweepBlocksPerSm * 148;  // one part per block of a full grid
 // A tensor of up to 8192 words (131072 weights) is "small": at most eight parts of up to 8 x 128 words, so that
 // one cluster of eight blocks holds it in registers, eight quarter-words per thread.
-constexpr int kSmallParts = 8, kSmallQuarters = 8, kQuarterWords = kSweepThreads / 4;
+constexpr int kSmallQuarters = 8, kQuarterWords = kSweepThreads / 4;
 constexpr unsigned long long kSmallWords = kSmallParts * kSmallQuarters * kQuarterWords;
 // workspace: [0,256) counters, then arrays of 8-byte partials
 constexpr size_t kWorkspaceBytes = 65792;
@@ -53,57 +47,6 @@ __host__ __device__ inline Workspace carve(void *ws, int t)
     w.part_kept = w.part_sum + kMaxParts;
     w.part_cnt = reinterpret_cast<unsigned long long *>(w.part_kept + kMaxParts);
     return w;
-}
-
-template <typename T>
-__device__ __forceinline__ T warp_sum(T v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    return v;
-}
-
-// Block-wide sums with a fixed order: a shuffle tree per warp, then every thread adds the sixteen warps' sums in
-// the same tree, so that one barrier does and nobody waits for a broadcast.  The buffers alternate from call to
-// call (`turn`): a buffer is written again two barriers later, when all have read it.
-struct Reduce {
-    double sum[2][kSweepWarps];
-    uint2 cnt[2][kSweepWarps];
-};
-__device__ __forceinline__ double tree16(const double *v)
-{
-    double t[kSweepWarps / 2];
-#pragma unroll
-    for (int i = 0; i < kSweepWarps / 2; ++i) t[i] = v[i] + v[i + kSweepWarps / 2];
-#pragma unroll
-    for (int o = kSweepWarps / 4; o > 0; o >>= 1)
-#pragma unroll
-        for (int i = 0; i < o; ++i) t[i] += t[i + o];
-    return t[0];
-}
-__device__ __forceinline__ double sweep_sum(double v, Reduce &red, unsigned int &turn)
-{
-    double *buf = red.sum[turn & 1];
-    ++turn;
-    v = warp_sum(v);
-    if ((threadIdx.x & 31) == 0) buf[threadIdx.x >> 5] = v;
-    __syncthreads();
-    return tree16(buf);
-}
-// The same for a sum and two counts of the block (below 2^32).
-__device__ __forceinline__ double sweep_sum(double v, unsigned int &pos, unsigned int &neg, Reduce &red, unsigned int &turn)
-{
-    double *buf = red.sum[turn & 1];
-    uint2 *cnt = red.cnt[turn & 1];
-    ++turn;
-    v = warp_sum(v);
-    const unsigned int p = __reduce_add_sync(0xffffffffu, pos), q = __reduce_add_sync(0xffffffffu, neg);
-    if ((threadIdx.x & 31) == 0) { buf[threadIdx.x >> 5] = v; cnt[threadIdx.x >> 5] = make_uint2(p, q); }
-    __syncthreads();
-    pos = neg = 0;
-#pragma unroll
-    for (int i = 0; i < kSweepWarps; ++i) { pos += cnt[i].x; neg += cnt[i].y; }
-    return tree16(buf);
 }
 
 // ---- the codes --------------------------------------------------------------
@@ -451,25 +394,6 @@ __device__ __forceinline__ void write_padding(const Item &it, unsigned int b, un
 // Latency is all there is (50 thousand weights: 14.3 us as two sweeps over memory with a cleared ticket, 12 of them
 // waiting for memory and launches).  A block keeps its part in registers between the phases, the sums travel through
 // distributed shared memory, and the cluster's barrier (0.2 us) stands where larger tensors need the grid's.
-__device__ __forceinline__ uint32_t peer_smem(const void *p, uint32_t rank)
-{
-    uint32_t a;
-    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
-    return a;
-}
-__device__ __forceinline__ void st_peer(uint32_t addr, unsigned long long v)
-{
-    asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(addr), "l"(v) : "memory");
-}
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.aligned;" ::: "memory"); }
-
-// Eight values in the order of the shuffle tree that folds the parts of a larger tensor.
-__device__ __forceinline__ double tree8(const double *p)
-{
-    return ((p[0] + p[4]) + (p[2] + p[6])) + ((p[1] + p[5]) + (p[3] + p[7]));
-}
-
 template <int Q, bool SUMS>      // quarter-words per thread; false: the coding sweep alone
 __global__ void __launch_bounds__(kSweepThreads, 1)
 ternarize_small_kernel(const __grid_constant__ Launch<1> P)
@@ -1197,23 +1121,6 @@ bool make_item(const float *W, int64_t rows, int64_t cols, twn_stats_t *stats, u
     it->first_part = 0;
     *rc = TWN_OK;
     return true;
-}
-
-// cudaLaunchKernelEx with one attribute.
-template <typename K, typename... A>
-int launch_with(K kernel, unsigned int grid, cudaLaunchAttributeID id, cudaLaunchAttributeValue val, cudaStream_t s, const A &...args)
-{
-    cudaLaunchAttribute attr[1];
-    attr[0].id = id;
-    attr[0].val = val;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(kSweepThreads);
-    cfg.stream = s;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    TWN_CUDA_OK(cudaLaunchKernelEx(&cfg, kernel, args...));
-    return TWN_OK;
 }
 
 template <int N, bool SUMS>
