@@ -50,36 +50,6 @@ __host__ __device__ inline Workspace carve(void *ws, int t)
 }
 
 // ---- the codes --------------------------------------------------------------
-// Bit position of element e (0..15) inside its word: even elements fill the low
-// half-word, odd elements the high half-word, each from the top down, so that a left
-// shift by 2*(e/2) brings the element's field to the top two bits of its half-word.
-__host__ __device__ __forceinline__ int field_pos(int e) { return 14 - 2 * (e >> 1) + 16 * (e & 1); }
-
-// A "quarter byte" holds the 2-bit fields (bit 0 = kept, bit 1 = negative: 00 / 01 / 11) of four consecutive
-// weights: low nibble = elements 0 (upper) and 2, high nibble = elements 1 (upper) and 3.
-//
-// Bits 0..15 of x -> the even bits of the result.
-__device__ __forceinline__ uint32_t spread16(uint32_t x)
-{
-    x = (x | (x << 8)) & 0x00FF00FFu;
-    x = (x | (x << 4)) & 0x0F0F0F0Fu;
-    x = (x | (x << 2)) & 0x33333333u;
-    return (x | (x << 1)) & 0x55555555u;
-}
-
-// Quarter bytes B0..B3 of sixteen consecutive weights -> the word of
-// those 16 elements: low half = low nibbles, high half = high nibbles, B0's on top.
-__device__ __forceinline__ uint32_t bytes_to_word(uint32_t r)
-{
-    r = __byte_perm(r, 0u, 0x0123);
-    uint32_t lo = r & 0x0F0F0F0Fu, hi = (r >> 4) & 0x0F0F0F0Fu;
-    lo = (lo | (lo >> 4)) & 0x00FF00FFu;
-    lo = (lo | (lo >> 8)) & 0x0000FFFFu;
-    hi = (hi | (hi >> 4)) & 0x00FF00FFu;
-    hi = (hi | (hi >> 8)) & 0x0000FFFFu;
-    return lo | (hi << 16);
-}
-
 // inverse: word -> bytes B0..B3
 __device__ __forceinline__ uint32_t word_to_bytes(uint32_t w)
 {
@@ -89,20 +59,6 @@ __device__ __forceinline__ uint32_t word_to_bytes(uint32_t w)
     hi = (hi | (hi << 8)) & 0x00FF00FFu;
     hi = (hi | (hi << 4)) & 0x0F0F0F0Fu;
     return __byte_perm(lo | (hi << 4), 0u, 0x0123);
-}
-
-// int8 image of the four fields of a quarter byte, in element order:
-// 00 -> 0x00, 01 -> 0x01, 11 -> 0xFF
-__device__ __forceinline__ uint32_t fields_to_i8x4(uint32_t c8)
-{
-    uint32_t r = 0;
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-        const uint32_t f = (c8 >> (2 - 2 * (e >> 1) + 4 * (e & 1))) & 3u;
-        const uint32_t b = (f & 1u) ? ((f & 2u) ? 0xFFu : 0x01u) : 0u;
-        r |= b << (8 * e);
-    }
-    return r;
 }
 
 // ---- parts ------------------------------------------------------------------
@@ -313,29 +269,7 @@ struct Coder {
     __device__ __forceinline__ void group(const Item &it, const PartRange &r, unsigned int w_grp, const float4 (&v)[4], float thr)
     {
         const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-        // Bound by instruction issue, above all by the half-rate integer pipe: a comparison, a select, three shifts
-        // and two merges per weight took 29 us for 20 million weights that are in L2.  Here a weight costs that pipe
-        // two instructions, the comparison (as 1.0 or 0.0) and a funnel shift that collects the signs; the masking
-        // and the collection of the kept bits are multiplications.
-        float kept_bits = 0.0f;          // below 2^16, exact
-        uint32_t sign_bits = 0;
-#pragma unroll
-        for (int i = 3; i >= 0; --i) {
-            const float w4[4] = {v[i].y, v[i].w, v[i].x, v[i].z};
-#pragma unroll
-            for (int x = 0; x < 4; ++x) {
-                float keep;
-                asm("set.gt.f32.f32 %0, %1, %2;" : "=f"(keep) : "f"(fabsf(w4[x])), "f"(thr));
-                k[x] += (double)(fabsf(w4[x]) * keep);
-                kept_bits = fmaf(kept_bits, 2.0f, keep);
-                sign_bits = __funnelshift_l(__float_as_uint(w4[x]), sign_bits, 1);
-            }
-        }
-        const uint32_t kb = (uint32_t)kept_bits, nb = sign_bits & kb;
-        const unsigned int n_neg = __popc(nb);
-        neg += n_neg;
-        pos += __popc(kb) - n_neg;
-        uint32_t bytes = spread16(kb) | (spread16(nb) << 1);
+        const uint32_t bytes = code_quarters(v, thr, k, pos, neg);
         if (it.codes_i8) {
 #pragma unroll 1
             for (int i = 0; i < 4; ++i) {
@@ -346,14 +280,9 @@ struct Coder {
                 for (unsigned int x = 0; x < 4 && e + x < p.valid; ++x) it.codes_i8[r.f0 + p.f + e + x] = (int8_t)(c4 >> (8 * x));
             }
         }
-        // a word's four quarters sit in the bytes of four neighbouring lanes: a 4x4 byte transpose (lanes
-        // l^2, then l^1) leaves lane l with word l/4 of its warp's share of quarter-row l%4
-        const uint32_t y = __shfl_xor_sync(0xffffffffu, bytes, 2);
-        bytes = __byte_perm(bytes, y, (lane & 2) ? 0x3276 : 0x5410);
-        const uint32_t z = __shfl_xor_sync(0xffffffffu, bytes, 1);
-        bytes = __byte_perm(bytes, z, (lane & 1) ? 0x3715 : 0x6240);
+        const uint32_t word = exchange_quarters(bytes);
         const unsigned int wl = w_grp + (lane & 3) * kQuarterWords + warp * 8 + (lane >> 2);
-        if (wl < r.words) it.packed[it.dense ? r.w0 + wl : place_word(it, r, wl).out] = bytes_to_word(bytes);
+        if (wl < r.words) it.packed[it.dense ? r.w0 + wl : place_word(it, r, wl).out] = word;
     }
 };
 

@@ -3,192 +3,156 @@
 // gets its own threshold delta_r = factor * mean |W_r| (Sec. 2.3), its own codes (Eq. 3) and
 // its own scale alpha_r = mean of |W_r,i| over |W_r,i| > delta_r (Eq. 5).
 //
-// One thread block per filter.  The threshold needs the whole filter before any code can be
-// written, but a filter is small (25 ... 8192 weights in the networks of the paper), so the
-// block keeps it in shared memory between the two steps: each weight crosses HBM once
-// (4 bytes read, 0.25 bytes written), against two reads for the per-layer rule.  Several
-// blocks share an SM, so the loads of one filter overlap the coding of another.  Filters
-// longer than the shared-memory budget, or whose rows are not 16-byte aligned, are read a
-// second time (from L2, as a rule).  Both sums are fp64 with a fixed order (per-thread
-// partials, shuffle tree, shared-memory tree): same inputs, same bits.  No scratch memory.
-#include "common.cuh"
+// A team of threads per filter: a warp for filters of up to 1024 weights (12000 filters of 64 weights took 31 us with a
+// block each, most of it blocks starting and joining), a block beyond.  The threshold needs the whole filter before any
+// code can be written, but a filter is small (25 ... 8192 weights in the networks of the paper), so the team keeps it in
+// registers between the two steps, up to sixteen 16-byte vectors per thread: each weight crosses HBM once (4 bytes read,
+// 0.25 bytes written), against two reads for the per-layer rule.  Longer filters are read a second time, back to front
+// (from L2, as a rule).  Filters that start off the 16-byte boundaries are read by two aligned vectors and shifted (with
+// 4-byte loads, twice over, 4000 filters of 5001 weights took 62 us).  Both sums are fp64 with a fixed order (per-thread
+// sums, shuffle tree, warps in order): same inputs, same bits.  No scratch memory.
+#include "sweep.cuh"
 
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kWarps = kThreads / 32;
-constexpr long long kSmemCols = 16384;                      // longest filter kept in shared memory (64 KB)
 
-__device__ __forceinline__ double warp_sum(double v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    return v;
-}
-__device__ __forceinline__ unsigned long long warp_sum(unsigned long long v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    return v;
-}
-
-// Block-wide sums with a fixed order: a shuffle tree per warp, one partial per warp in shared
-// memory, and after a single barrier every thread adds the kWarps partials in index order.
-__device__ __forceinline__ double block_sum_all(double v, double *part /* kWarps entries, not in use by a slower warp */)
-{
-    v = warp_sum(v);
-    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = v;
-    __syncthreads();
-    double r = 0.0;
-#pragma unroll
-    for (int w = 0; w < kWarps; ++w) r += part[w];
-    return r;
-}
-// The same for a floating-point and an integer quantity at once (one barrier for both).
-__device__ __forceinline__ void block_sum_all2(double &a, unsigned long long &b, double *part_a, unsigned long long *part_b)
-{
-    a = warp_sum(a);
-    b = warp_sum(b);
-    if ((threadIdx.x & 31) == 0) { part_a[threadIdx.x >> 5] = a; part_b[threadIdx.x >> 5] = b; }
-    __syncthreads();
-    double ra = 0.0;
-    unsigned long long rb = 0ull;
-#pragma unroll
-    for (int w = 0; w < kWarps; ++w) { ra += part_a[w]; rb += part_b[w]; }
-    a = ra;
-    b = rb;
-}
-
-// Bit position of element e (0..15) inside its packed word (the layout of twn_ternarize): even
-// elements fill the low half-word, odd elements the high one, each from its top bits down.
-__device__ __forceinline__ int field_pos(int e) { return 14 - 2 * (e >> 1) + 16 * (e & 1); }
-
-// 2-bit field of one weight against the threshold: 00 = 0, 01 = +1, 11 = -1 (Eq. 3; a weight
-// equal to the threshold is 0).  Kept magnitudes are summed in fp64.  Branch-free and short: the
-// coding sweep is bound by instruction issue, not by memory.
-__device__ __forceinline__ uint32_t field_of(float w, float thr, double &kept)
-{
-    const bool keep = fabsf(w) > thr;
-    kept += (double)(keep ? fabsf(w) : 0.0f);
-    return keep ? ((__float_as_uint(w) >> 31) * 2u + 1u) : 0u;
-}
-
-__device__ __forceinline__ int8_t code_of(uint32_t f) { return (f & 1u) ? ((f & 2u) ? (int8_t)-1 : (int8_t)1) : (int8_t)0; }
-
-// MODE 0: any alignment, scalar loads, the filter is read twice.
-// MODE 1: rows 16-byte aligned and cols % 4 == 0, filter longer than the shared-memory budget: read twice.
-// MODE 2: as 1, and the filter (cols * 4 bytes of dynamic shared memory) stays on chip between the steps.
-template <int MODE>
-__global__ void __launch_bounds__(kThreads, 6)      // six blocks of 32 KB filters per SM: at most 40 registers
+// T threads per filter (32 or kThreads), R vectors of four weights per thread and chunk.
+template <int T, int R>
+__global__ void __launch_bounds__(kThreads, R >= 12 ? 2 : R >= 6 ? 4 : 5)
 ternarize_rows_kernel(const float *__restrict__ W, long long rows, long long cols, double factor,
                       twn_stats_t *__restrict__ stats, uint32_t *__restrict__ packed, long long wpr,
-                      int8_t *__restrict__ codes_i8)
+                      int8_t *__restrict__ codes_i8, int vec4)
 {
-    extern __shared__ float4 rowbuf[];
-    __shared__ double red_s[kWarps], red_k[kWarps];      // partials of the two sweeps: separate, so that a warp
-    __shared__ unsigned long long red_u[kWarps];         // ahead of the others never overwrites what they still read
-    const int tid = threadIdx.x, lane = tid & 31;
-    const long long words = (cols + 15) >> 4;         // words that hold codes; the rest of a row is padding
-    const int n4 = (int)(cols >> 2);
+    constexpr int kTeams = kThreads / T, kV = (R + 3) / 4 * 4, kWarps = T / 32;
+    __shared__ double part_a[T == 32 ? 1 : kWarps], part_b[T == 32 ? 1 : kWarps];
+    __shared__ uint2 part_c[T == 32 ? 1 : kWarps];
+    const int t = threadIdx.x % T, lane = threadIdx.x & 31, warp = t >> 5;
+    const long long row = (long long)blockIdx.x * kTeams + threadIdx.x / T;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");      // as pdl_begin, at any grid: the launch stands alone
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (row >= rows) return;             // a whole team
+    const long long f_row = row * cols, n = rows * cols;
+    const float *Wr = W + f_row;
+    const int n4 = (int)((cols + 3) >> 2), words = (int)((cols + 15) >> 4);
+    const int chunks = (n4 + T * R - 1) / (T * R);
+    const unsigned int mis = (unsigned int)(reinterpret_cast<uintptr_t>(Wr) >> 2) & 3u;      // of every quarter of the filter
+    // the vectors that its quarters reach into lie inside the matrix
+    const bool shifted = f_row + (long long)n4 * 4 + 4 <= n && f_row >= (long long)mis;
 
-    for (long long row = blockIdx.x; row < rows; row += gridDim.x) {
-        const float *Wr = W + row * cols;
-        uint32_t *Pr = packed + row * wpr;
-        int8_t *Cr = codes_i8 ? codes_i8 + row * cols : nullptr;
-
-        // ---- step 1: S = sum |W_r,i|  ->  delta_r
-        double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-        if (MODE >= 1) {
-            const float4 *W4 = reinterpret_cast<const float4 *>(Wr);
-#pragma unroll 8
-            for (int i = tid; i < n4; i += kThreads) {
-                const float4 x = __ldg(W4 + i);
-                if (MODE == 2) rowbuf[i] = x;
-                a0 += (double)fabsf(x.x); a1 += (double)fabsf(x.y); a2 += (double)fabsf(x.z); a3 += (double)fabsf(x.w);
-            }
-        } else {
-            for (long long i = tid; i < cols; i += kThreads) a0 += (double)fabsf(__ldg(Wr + i));
-        }
-        const double S = block_sum_all((a0 + a1) + (a2 + a3), red_s);
-        const double delta = cols > 0 ? factor * (S / (double)cols) : 0.0;
-        // a float w satisfies |w| > delta exactly when |w| > the largest float <= delta
-        const float thr = __double2float_rd(delta);
-
-        // ---- step 2: codes, packed 16 per word; sum and counts of the kept set
-        double k0 = 0.0, k1 = 0.0;
-        unsigned int nz = 0u, ng = 0u;             // kept, negative (a filter has fewer than 2^31 weights)
-        if (MODE == 2) {
-            // float4 i holds elements 4i..4i+3: a quarter of word i/4, whose other quarters sit in
-            // the neighbouring lanes of the same group of four; every thread reads back what it wrote.
-            // Elements 0 and 2 of the quarter go to the low half-word, 1 and 3 to the high one, the
-            // first of each pair two bits above the second.
-            const int sh = 12 - 4 * (lane & 3);    // field_pos of element 2 of this lane's quarter
-            auto quarter = [&](const int i, const float4 x, const bool in_row) {
-                const uint32_t f0 = field_of(x.x, thr, k0), f1 = field_of(x.y, thr, k1);
-                const uint32_t f2 = field_of(x.z, thr, k0), f3 = field_of(x.w, thr, k1);
-                uint32_t part = ((f0 * 4u + f2) | ((f1 * 4u + f3) << 16)) << sh;
-                nz += __popc(part & 0x55555555u);
-                ng += __popc(part & 0xAAAAAAAAu);
-                if (Cr && in_row) {
-                    // cols % 4 == 0 and the matrix is aligned: the four codes are one aligned word
-                    const uint32_t c4 = (uint32_t)(uint8_t)code_of(f0) | ((uint32_t)(uint8_t)code_of(f1) << 8) |
-                                        ((uint32_t)(uint8_t)code_of(f2) << 16) | ((uint32_t)(uint8_t)code_of(f3) << 24);
-                    *reinterpret_cast<uint32_t *>(Cr + 4 * (long long)i) = c4;
-                }
-                part |= __shfl_xor_sync(0xffffffffu, part, 1);
-                part |= __shfl_xor_sync(0xffffffffu, part, 2);
-                if ((lane & 3) == 0 && in_row) Pr[i >> 2] = part;
-            };
-            // whole sweeps of the block first (no bounds to check), then one ragged sweep
-            const int full = n4 / kThreads;
-#pragma unroll 4
-            for (int it = 0; it < full; ++it) {
-                const int i = it * kThreads + tid;
-                quarter(i, rowbuf[i], true);
-            }
-            if (full * kThreads < n4) {
-                const int i = full * kThreads + tid;
-                quarter(i, i < n4 ? rowbuf[i] : make_float4(0.0f, 0.0f, 0.0f, 0.0f), i < n4);
-            }
-        } else {
-            for (long long j = tid; j < words; j += kThreads) {
-                uint32_t word = 0u;
+    float4 v[kV];
 #pragma unroll
-                for (int e = 0; e < 16; ++e) {
-                    const long long c = 16 * j + e;
-                    if (c < cols) {
-                        const uint32_t f = field_of(__ldg(Wr + c), thr, k0);
-                        word |= f << field_pos(e);
-                        if (Cr) Cr[c] = code_of(f);
-                    }
-                }
-                nz += __popc(word & 0x55555555u);
-                ng += __popc(word & 0xAAAAAAAAu);
-                Pr[j] = word;
+    for (int k = R; k < kV; ++k) v[k] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    auto load = [&](int chunk) {
+        const int q0 = chunk * (T * R) + t;
+        if (vec4) {
+#pragma unroll
+            for (int k = 0; k < R; ++k)
+                v[k] = q0 + k * T < n4 ? __ldg(reinterpret_cast<const float4 *>(Wr) + q0 + k * T) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            return;
+        }
+#pragma unroll
+        for (int k = 0; k < R; ++k) {
+            const int q = q0 + k * T;
+            const long long e = 4ll * q;
+            const int left = q < n4 ? (cols - e < 4 ? (int)(cols - e) : 4) : 0;
+            float4 x = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            if (shifted) {
+                const float4 *p = reinterpret_cast<const float4 *>(Wr + (left ? e : 0) - mis);
+                const float4 a = __ldg(p), b = __ldg(p + 1);
+                const bool one = mis & 1, two = mis & 2;
+                const float s0 = one ? a.y : a.x, s1 = one ? a.z : a.y, s2 = one ? a.w : a.z, s3 = one ? b.x : a.w,
+                            s4 = one ? b.y : b.x, s5 = one ? b.z : b.y;
+                x = make_float4(two ? s2 : s0, two ? s3 : s1, two ? s4 : s2, two ? s5 : s3);
+                if (left < 1) x.x = 0.0f;
+                if (left < 2) x.y = 0.0f;
+                if (left < 3) x.z = 0.0f;
+                if (left < 4) x.w = 0.0f;
+            } else {
+                if (left > 0) x.x = __ldg(Wr + e);
+                if (left > 1) x.y = __ldg(Wr + e + 1);
+                if (left > 2) x.z = __ldg(Wr + e + 2);
+                if (left > 3) x.w = __ldg(Wr + e + 3);
             }
+            v[k] = x;
         }
-        // padding words of the row
-        for (long long j = words + tid; j < wpr; j += kThreads) Pr[j] = 0u;
+    };
+    // sums over the team, the same in all its threads
+    auto team_sum = [&](double x, double *part) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+        if (T == 32) return x;
+        if (lane == 0) part[warp] = x;
+        __syncthreads();
+        x = 0.0;
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) x += part[w];
+        return x;
+    };
 
-        double K = k0 + k1;
-        // positives in the low, negatives in the high half
-        unsigned long long c2 = (unsigned long long)(nz - ng) + ((unsigned long long)ng << 32);
-        block_sum_all2(K, c2, red_k, red_u);
-        if (tid == 0) {
-            const unsigned long long n_pos = c2 & 0xFFFFFFFFull, n_neg = c2 >> 32;
-            twn_stats_t st;
-            st.delta = delta;
-            st.alpha = (n_pos + n_neg) > 0 ? K / (double)(n_pos + n_neg) : 0.0;
-            st.sum_abs = S;
-            st.sum_abs_kept = K;
-            st.n_neg = n_neg;
-            st.n_pos = n_pos;
-            st.n_zero = (unsigned long long)cols - n_pos - n_neg;
-            st.status = isfinite(S) ? TWN_OK : TWN_ERR_NONFINITE;
-            st.reserved = 0;
-            stats[row] = st;
+    // ---- step 1: S = sum |W_r,i|  ->  delta_r
+    double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
+    for (int c = 0; c < chunks; ++c) {
+        load(c);
+#pragma unroll
+        for (int k = 0; k < R; ++k) {
+            a0 += (double)fabsf(v[k].x); a1 += (double)fabsf(v[k].y); a2 += (double)fabsf(v[k].z); a3 += (double)fabsf(v[k].w);
         }
-        __syncthreads();       // the partials are free for the next filter of this block
+    }
+    const double S = team_sum((a0 + a1) + (a2 + a3), part_a);
+    const double delta = cols > 0 ? factor * (S / (double)cols) : 0.0;
+    // a float w satisfies |w| > delta exactly when |w| > the largest float <= delta
+    const float thr = __double2float_rd(delta);
+
+    // ---- step 2: codes, packed 16 per word; sum and counts of the kept set
+    uint32_t *Pr = packed + row * wpr;
+    double kept[4] = {0.0, 0.0, 0.0, 0.0};
+    unsigned int pos = 0, neg = 0;
+    for (int c = chunks - 1; c >= 0; --c) {
+        if (c < chunks - 1) load(c);     // the last chunk is still in registers
+#pragma unroll
+        for (int g = 0; g < kV / 4; ++g) {
+            const float4 four[4] = {v[4 * g], v[4 * g + 1], v[4 * g + 2], v[4 * g + 3]};
+            const uint32_t bytes = code_quarters(four, thr, kept, pos, neg);
+            const int q0 = c * (T * R) + 4 * g * T;          // first quarter of these four rounds
+            if (codes_i8) {
+#pragma unroll 1
+                for (int k = 0; k < 4; ++k) {
+                    const long long e = 4ll * (q0 + k * T + t);
+                    const uint32_t c4 = fields_to_i8x4((bytes >> (8 * k)) & 0xFFu);
+                    if (4 * g + k < R)
+                        for (int x = 0; x < 4 && e + x < cols; ++x) codes_i8[f_row + e + x] = (int8_t)(c4 >> (8 * x));
+                }
+            }
+            const uint32_t word = exchange_quarters(bytes);
+            const int w = q0 / 4 + (lane & 3) * (T / 4) + (t >> 2);
+            if (w < words && 4 * g + (lane & 3) < R) Pr[w] = word;
+        }
+    }
+    // padding words of the row
+    for (long long j = words + t; j < wpr; j += T) Pr[j] = 0u;
+
+    const double K = team_sum((kept[0] + kept[1]) + (kept[2] + kept[3]), part_b);
+    unsigned int p = __reduce_add_sync(0xffffffffu, pos), q = __reduce_add_sync(0xffffffffu, neg);
+    if (T > 32) {
+        if (lane == 0) part_c[warp] = make_uint2(p, q);
+        __syncthreads();
+        p = q = 0;
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) { p += part_c[w].x; q += part_c[w].y; }
+    }
+    if (t == 0) {
+        twn_stats_t st;
+        st.delta = delta;
+        st.alpha = (p | q) ? K / (double)((unsigned long long)p + q) : 0.0;
+        st.sum_abs = S;
+        st.sum_abs_kept = K;
+        st.n_neg = q;
+        st.n_pos = p;
+        st.n_zero = (unsigned long long)cols - p - q;
+        st.status = isfinite(S) ? TWN_OK : TWN_ERR_NONFINITE;
+        st.reserved = 0;
+        stats[row] = st;
     }
 }
 
@@ -219,28 +183,27 @@ extern "C" int twn_ternarize_rows(const float *W, int64_t rows, int64_t cols, do
     twn_device_info dev;
     const int rc = twn_current_device(&dev);
     if (rc != TWN_OK) return rc;
-    // one block per filter: blocks are scheduled as others retire, so filters of any number spread
-    // evenly over the SMs (the row loop of the kernel only serves more than 2^31 - 1 filters)
-    const int grid = (int)(rows < 0x7fffffffLL ? rows : 0x7fffffffLL);
-    const bool vec = twn_aligned(W, 16) && cols % 4 == 0 && twn_aligned(codes_i8, 4);
-    if (vec && cols <= kSmemCols) {
-        static bool attr_set[64] = {false};
-        if (!attr_set[dev.ordinal]) {
-            TWN_CUDA_OK(cudaFuncSetAttribute(ternarize_rows_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)(kSmemCols * 4)));
-            attr_set[dev.ordinal] = true;
-        }
-        ternarize_rows_kernel<2><<<grid, kThreads, (size_t)cols * 4, twn_cu(stream)>>>(
-            W, rows, cols, delta_factor, stats, packed, ld_codes / 16, codes_i8);
-    } else if (vec) {
-        ternarize_rows_kernel<1><<<grid, kThreads, 0, twn_cu(stream)>>>(W, rows, cols, delta_factor, stats, packed,
-                                                                      ld_codes / 16, codes_i8);
-    } else {
-        ternarize_rows_kernel<0><<<grid, kThreads, 0, twn_cu(stream)>>>(W, rows, cols, delta_factor, stats, packed,
-                                                                      ld_codes / 16, codes_i8);
-    }
-    TWN_CUDA_OK(cudaGetLastError());
-    return TWN_OK;
+    // the smallest team and vector count that hold a filter; longer ones go round in chunks of 8192 weights
+    const bool vec = twn_aligned(W, 16) && cols % 4 == 0;
+    auto launch = [&](auto kernel, int teams) -> int {
+        const long long grid = (rows + teams - 1) / teams;
+        TWN_REQUIRE(grid < 0x7fffffffLL, TWN_ERR_TOO_LARGE);
+        TWN_CUDA_OK(twn_launch_pdl(true, kernel, (int)grid, kThreads, 0, twn_cu(stream), W, (long long)rows, (long long)cols, delta_factor,
+                                     stats, packed, (long long)(ld_codes / 16), codes_i8, (int)vec));
+        return TWN_OK;
+    };
+    constexpr int kWarpTeams = kThreads / 32;
+    if (cols <= 128) return launch(ternarize_rows_kernel<32, 1>, kWarpTeams);
+    if (cols <= 256) return launch(ternarize_rows_kernel<32, 2>, kWarpTeams);
+    if (cols <= 512) return launch(ternarize_rows_kernel<32, 4>, kWarpTeams);
+    if (cols <= 1024) return launch(ternarize_rows_kernel<32, 8>, kWarpTeams);
+    if (cols <= 2048) return launch(ternarize_rows_kernel<kThreads, 2>, 1);
+    if (cols <= 3072) return launch(ternarize_rows_kernel<kThreads, 3>, 1);
+    if (cols <= 4096) return launch(ternarize_rows_kernel<kThreads, 4>, 1);
+    if (cols <= 6144) return launch(ternarize_rows_kernel<kThreads, 6>, 1);
+    if (cols <= 8192 || cols > 16384) return launch(ternarize_rows_kernel<kThreads, 8>, 1);      // fewer registers: more blocks on an SM
+    if (cols <= 12288) return launch(ternarize_rows_kernel<kThreads, 12>, 1);
+    return launch(ternarize_rows_kernel<kThreads, 16>, 1);
 }
 
 extern "C" int twn_rows_scale(const twn_stats_t *stats, int64_t rows, const float *scale_in, float *scale_out,

@@ -34,3 +34,44 @@ def test_codes_and_sums(rows, cols, extra):
         assert abs(st["delta"] - ref.delta) <= 1e-12 * ref.delta and abs(st["alpha"] - ref.alpha) <= 1e-12 * ref.alpha
         assert (st["n_neg"], st["n_zero"], st["n_pos"]) == (ref.n_neg, ref.n_zero, ref.n_pos)
         assert np.array_equal(host_u32(packed), want)
+
+
+@pytest.mark.parametrize("rows,cols,offset", [
+    (1, 3, 0), (9, 127, 0), (33, 129, 0), (17, 257, 0), (70, 513, 1), (70, 1023, 0), (5, 1025, 0), (3, 2049, 3), (7, 4097, 0),
+    (4, 8190, 0), (3, 16385, 0), (2, 40003, 2), (3, 33024, 0)])
+def test_filters(rows, cols, offset):
+    """Teams of a warp and of a block, every vector count, chunked filters, matrices off the 16-byte boundaries."""
+    W = dg.draw(6, f"filters{rows}x{cols}", rows * cols, "laplace").reshape(rows, cols)
+    buf = torch.zeros(rows * cols + 8, dtype=torch.float32, device="cuda")
+    Wd = buf[offset:offset + rows * cols].view(rows, cols)
+    Wd.copy_(dev_f32(W))
+    ld = twn.ld_for(cols) + (64 if rows == 7 else 0)
+    stats = twn.new_stats_rows(rows)
+    packed = torch.full((rows, ld // 16), -1, dtype=torch.int32, device="cuda")
+    codes = torch.full((rows, cols), 7, dtype=torch.int8, device="cuda")
+    twn.ternarize_rows(Wd, 0.7, stats, packed, ld, codes)
+    got, words = twn.stats_rows_to_host(stats), host_u32(packed)
+    for r in range(rows):
+        ref, want = oracle.ternarize(W[r:r + 1], 0.7)
+        assert got[r]["status"] == 0 and abs(got[r]["delta"] - ref.delta) <= 1e-12 * ref.delta
+        assert abs(got[r]["alpha"] - ref.alpha) <= 1e-12 * ref.alpha
+        assert (got[r]["n_neg"], got[r]["n_zero"], got[r]["n_pos"]) == (ref.n_neg, ref.n_zero, ref.n_pos)
+        assert np.array_equal(words[r:r + 1], oracle.pack(want.reshape(1, cols), ld))
+        assert np.array_equal(codes[r].cpu().numpy(), want.reshape(-1))
+
+
+@pytest.mark.parametrize("rows,cols,offset", [(1, 1, 0), (1, 131, 0), (3, 33, 0), (31, 3784, 0), (129, 1030, 0), (64, 2048, 2),
+                                              (9, 16416, 0), (300, 1027, 1), (1, 16384 * 9 + 5, 0)])
+def test_signs(rows, cols, offset):
+    W = dg.draw(7, f"signs{rows}x{cols}", rows * cols, "normal").reshape(rows, cols)
+    W[0, 0] = -0.0
+    buf = torch.zeros(rows * cols + 8, dtype=torch.float32, device="cuda")
+    Wd = buf[offset:offset + rows * cols].view(rows, cols)
+    Wd.copy_(dev_f32(W))
+    ld = twn.ld_for_b1(cols)
+    stats = twn.new_stats()
+    packed = torch.full((rows, ld // 32), -1, dtype=torch.int32, device="cuda")
+    twn.binarize(Wd, stats, packed, ld, workspace(twn.binarize_workspace_bytes()))
+    st, (ref, codes) = twn.stats_to_host(stats), oracle.binarize(W)
+    assert st["status"] == 0 and abs(st["alpha"] - ref.alpha) <= 1e-12 * ref.alpha and st["n_neg"] == int((W < 0).sum())
+    assert np.array_equal(host_u32(packed), oracle.pack1(codes.reshape(rows, cols), ld))
