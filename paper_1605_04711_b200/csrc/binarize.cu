@@ -81,6 +81,7 @@ binarize_kernel(const __grid_constant__ BinParams P)
     unsigned int turn = 0;
     if (CLUSTER) {
         if (tid < kSmallParts) { sum_s[tid] = 0.0; neg_s[tid] = 0ull; }
+        pdl_begin();
         cluster_arrive();
     }
     // padding words of the rows
@@ -285,17 +286,12 @@ extern "C" int twn_binarize(const float *W, int64_t rows, int64_t cols, twn_stat
     P.parts = (unsigned int)std::max(1ull, (P.words + part - 1) / part);
     P.vec4 = twn_aligned(W, 16) && (rows == 1 || cols % 4 == 0);
     P.dense = rows == 1 || ld_codes == cols;
-    cudaLaunchAttributeValue val = {};
     if (P.parts <= (unsigned int)kSmallParts) {
         unsigned int grid = 1;
         while (grid < P.parts) grid *= 2;
-        val.clusterDim.x = grid;
-        val.clusterDim.y = val.clusterDim.z = 1;
-        return launch_with(binarize_kernel<true>, grid, cudaLaunchAttributeClusterDimension, val, twn_cu(stream), P);
+        return launch_cluster(binarize_kernel<true>, grid, twn_cu(stream), P);
     }
-    val.cooperative = 1;
-    return launch_with(binarize_kernel<false>, std::min(P.parts, (unsigned int)(dev.sm_count * kSweepBlocksPerSm)),
-                       cudaLaunchAttributeCooperative, val, twn_cu(stream), P);
+    return launch_cooperative(binarize_kernel<false>, std::min(P.parts, (unsigned int)(dev.sm_count * kSweepBlocksPerSm)), twn_cu(stream), P);
 }
 
 extern "C" int twn_unpack_b1(const uint32_t *packed, int64_t rows, int64_t cols, int64_t ld_codes, int8_t *codes,

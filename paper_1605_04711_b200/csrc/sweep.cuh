@@ -84,13 +84,33 @@ __device__ __forceinline__ double tree8(const double *p)
     return ((p[0] + p[4]) + (p[2] + p[6])) + ((p[1] + p[5]) + (p[3] + p[7]));
 }
 
-// cudaLaunchKernelEx with one attribute.
+// A cluster of `grid` blocks.  It may start while the kernel before it drains (its blocks wait in pdl_begin), as the
+// small kernels around it do: 6.2 -> 4.6 us per call for a stream of small ternarizations.
 template <typename K, typename... A>
-int launch_with(K kernel, unsigned int grid, cudaLaunchAttributeID id, cudaLaunchAttributeValue val, cudaStream_t s, const A &...args)
+int launch_cluster(K kernel, unsigned int grid, cudaStream_t s, const A &...args)
+{
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = grid;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(kSweepThreads);
+    cfg.stream = s;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    TWN_CUDA_OK(cudaLaunchKernelEx(&cfg, kernel, args...));
+    return TWN_OK;
+}
+// A grid whose blocks all run at once and may wait for one another.
+template <typename K, typename... A>
+int launch_cooperative(K kernel, unsigned int grid, cudaStream_t s, const A &...args)
 {
     cudaLaunchAttribute attr[1];
-    attr[0].id = id;
-    attr[0].val = val;
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(kSweepThreads);

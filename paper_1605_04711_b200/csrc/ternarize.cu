@@ -334,6 +334,7 @@ ternarize_small_kernel(const __grid_constant__ Launch<1> P)
     const unsigned int b = blockIdx.x, G = gridDim.x, tid = threadIdx.x;
     unsigned int turn = 0;
     if (tid < kSmallParts) { sum_s[tid] = 0.0; kept_s[tid] = 0.0; cnt_s[tid] = 0ull; }
+    pdl_begin();
     cluster_arrive();                    // from here on other blocks may write this block's sums
     PartRange r = part_range(it, b);
     float4 v[Q < 4 ? 4 : Q];
@@ -639,6 +640,7 @@ sgd_update_kernel(const __grid_constant__ SgdLaunch<N> P, void *ws_raw)
     double own = 0.0;
     if (CLUSTER) {
         if (threadIdx.x < kSmallParts) sum_s[threadIdx.x] = 0.0;
+        pdl_begin();
         cluster_arrive();
     }
     for (unsigned int g = blockIdx.x; g < P.blocks; g += gridDim.x) {
@@ -1064,22 +1066,17 @@ int launch_sweeps(Launch<N> &P, double factor, void *ws, cudaStream_t s)
         P.item[t].first_part = P.parts;
         P.parts += P.item[t].parts;
     }
-    cudaLaunchAttributeValue val = {};
     if constexpr (N == 1) {
         if (P.item[0].small) {
             unsigned int grid = 1;
             while (grid < P.parts) grid *= 2;
-            val.clusterDim.x = grid;
-            val.clusterDim.y = val.clusterDim.z = 1;
             const unsigned int q = P.item[0].part_words / kQuarterWords;
             auto kernel = q <= 1 ? ternarize_small_kernel<1, SUMS> : q <= 2 ? ternarize_small_kernel<2, SUMS>
                         : q <= 4 ? ternarize_small_kernel<4, SUMS> : ternarize_small_kernel<8, SUMS>;
-            return launch_with(kernel, grid, cudaLaunchAttributeClusterDimension, val, s, P);
+            return launch_cluster(kernel, grid, s, P);
         }
     }
-    val.cooperative = 1;
-    return launch_with(ternarize_kernel<N, SUMS>, std::min(P.parts, (unsigned int)(dev.sm_count * kSweepBlocksPerSm)),
-                       cudaLaunchAttributeCooperative, val, s, P, ws);
+    return launch_cooperative(ternarize_kernel<N, SUMS>, std::min(P.parts, (unsigned int)(dev.sm_count * kSweepBlocksPerSm)), s, P, ws);
 }
 
 bool batch_items(const twn_ternarize_item_t *items, int count, Launch<kMaxBatch> &P, int *rc)
@@ -1105,19 +1102,14 @@ int launch_sgd(SgdLaunch<N> &P, void *ws, cudaStream_t s)
         P.item[t].first_block = P.blocks;
         P.blocks += (unsigned int)std::max(1ll, std::min((long long)kMaxParts, want));
     }
-    cudaLaunchAttributeValue val = {};
     if constexpr (N == 1) {
         if (P.blocks <= kSmallParts) {
             unsigned int grid = 1;
             while (grid < P.blocks) grid *= 2;
-            val.clusterDim.x = grid;
-            val.clusterDim.y = val.clusterDim.z = 1;
-            return launch_with(sgd_update_kernel<N, true>, grid, cudaLaunchAttributeClusterDimension, val, s, P, ws);
+            return launch_cluster(sgd_update_kernel<N, true>, grid, s, P, ws);
         }
     }
-    val.cooperative = 1;
-    return launch_with(sgd_update_kernel<N, false>, std::min(P.blocks, (unsigned int)(dev.sm_count * kSweepBlocksPerSm)),
-                       cudaLaunchAttributeCooperative, val, s, P, ws);
+    return launch_cooperative(sgd_update_kernel<N, false>, std::min(P.blocks, (unsigned int)(dev.sm_count * kSweepBlocksPerSm)), s, P, ws);
 }
 
 }  // namespace
