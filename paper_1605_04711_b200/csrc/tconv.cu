@@ -784,10 +784,6 @@ int launch_conv(const Geometry &g, const void *X, const uint32_t *T, const twn_s
     const EpilogueArgs ea = epilogue_args(stats, epi, out_dtype_default);
     // problems that do not fill the GPU: small tiles, the reduction split over a cluster
     const SplitPlan split = plan_conv_split(g, dev.sm_count / (g.beside > 1 ? g.beside : 1), ea.in_order);
-    // narrow layers: the kernel that decodes the layer's codes once per block
-    bool handled = false;
-    rc = launch_conv_resident(g, X, T, ea, Y, dev_status, dev, s, split.us, &handled);
-    if (rc != TWN_OK || handled) return rc;
     ConvParams P;
     memset(&P, 0, sizeof P);
     P.n_tiles = (g.Cout + kChan - 1) / kChan;
@@ -796,21 +792,6 @@ int launch_conv(const Geometry &g, const void *X, const uint32_t *T, const twn_s
     P.codes_aligned = 1;
     for (int t = 0; t < g.n_taps; ++t)
         if (g.taps[t].koff % kBlockK != 0) P.codes_aligned = 0;
-    P.T = T;
-    P.wpr = g.ld_codes / (g.code_bits == 1 ? 32 : 16);
-    P.sw = g.sw; P.sh = g.sh;
-    P.Bv = g.Bv; P.Hv = g.Hv; P.Wv = g.Wv;
-    P.OH = g.OH; P.OW = g.OW; P.osh = g.osh; P.osw = g.osw; P.ooh = g.ooh; P.oow = g.oow;
-    P.ldy = g.ldy;
-    P.Cout = g.Cout;
-    P.alpha = ea.alpha; P.scale = ea.scale; P.shift = ea.shift;
-    P.residual = ea.residual; P.res_dtype = ea.res_dtype; P.res_gate = ea.res_gate;
-    P.relu = ea.relu; P.out_dtype = ea.out_dtype;
-    P.Y = Y;
-    P.status = dev_status;
-    P.bn_partial = g.bn_partial;
-    for (int t = 0; t < g.n_taps; ++t) P.taps[t] = g.taps[t];
-
     // Tile shape by a cost model fitted to measured launches (cycles per round of tiles, kb = k-blocks
     // per tile):
     //   128 pixels: max(2000 + 680 kb, 6500), 540 kb with both decode groups: the epilogue overlaps
@@ -839,11 +820,30 @@ int launch_conv(const Geometry &g, const void *X, const uint32_t *T, const twn_s
     if (c192 < (choice ? c256 : c128)) choice = 2;
     // the model counts cycles of the rounds; a launch as a whole takes (fitted to 65 measured launches, mean error 6 %)
     const double us = 3.9 + 0.454e-3 * (double)(choice == 0 ? c128 : choice == 1 ? c256 : c192);
+    // Narrow layers and short reductions: the kernel that decodes its channels' codes once per block.  Up to 64 channels
+    // the general kernel's half-empty tiles lose wherever that kernel runs; above, its own time decides.
+    bool handled = false;
+    rc = launch_conv_resident(g, X, T, ea, Y, dev_status, dev, s, half || split.us < us ? split.us : us, &handled);
+    if (rc != TWN_OK || handled) return rc;
     // The more SMs the general kernel fills by itself, the clearer the gain has to be: beside the weight gradients of a
     // training step a split launch takes SMs that would not have been idle (ResNet-18 at batch 64).
     const long long tiles = choice == 0 ? t128 : choice == 1 ? t256 : t192;
     const double fill = tiles < sms ? (double)tiles / (double)sms : 1.0;
     if (split.us < (1.0 - 0.25 * fill) * us) return launch_conv_split(g, X, T, ea, Y, dev_status, dev, s, split);
+    P.T = T;
+    P.wpr = g.ld_codes / (g.code_bits == 1 ? 32 : 16);
+    P.sw = g.sw; P.sh = g.sh;
+    P.Bv = g.Bv; P.Hv = g.Hv; P.Wv = g.Wv;
+    P.OH = g.OH; P.OW = g.OW; P.osh = g.osh; P.osw = g.osw; P.ooh = g.ooh; P.oow = g.oow;
+    P.ldy = g.ldy;
+    P.Cout = g.Cout;
+    P.alpha = ea.alpha; P.scale = ea.scale; P.shift = ea.shift;
+    P.residual = ea.residual; P.res_dtype = ea.res_dtype; P.res_gate = ea.res_gate;
+    P.relu = ea.relu; P.out_dtype = ea.out_dtype;
+    P.Y = Y;
+    P.status = dev_status;
+    P.bn_partial = g.bn_partial;
+    for (int t = 0; t < g.n_taps; ++t) P.taps[t] = g.taps[t];
     P.dsets = (choice != 1 && two) ? 2 : 1;
     if (g.code_bits == 1) {
         if (choice == 1) return launch_conv_t<256, 1, 1>(g, P, X, dev, enc, s);

@@ -1,10 +1,11 @@
-// Ternary-weight contraction for narrow layers (at most 64 output channels): Eq. 2 forward
+// Ternary-weight contraction for narrow layers and short reductions: Eq. 2 forward
 // block and Algorithm 1 TernaryForward / TernaryBackward, Y = epilogue(alpha * X (*) T), with
 // the layer's decoded weights RESIDENT in shared memory.
 //
 // tconv.cu keeps the weights as the A operand (128 channel rows) and decodes them again for
-// every pixel tile; with 64 or fewer output channels half of every MMA is idle and the decode
-// and the epilogue pace the kernel.  Here the roles are swapped:
+// every pixel tile; with 64 or fewer output channels half of every MMA is idle, with a short
+// reduction there are few MMAs per output, and the decode and the epilogue pace the kernel.
+// Here the roles are swapped:
 //
 //   D[pixel, channel] (+)= A[pixel, k] * B[channel, k]^T      M = 128 pixels, N = Cout (<= 64)
 //
@@ -17,6 +18,14 @@
 //      loads (8+2) x (16+2) pixels per 128 outputs instead of nine 128-pixel tiles.
 //   D  four accumulators of 64 tensor-memory columns: the epilogue of a tile overlaps the
 //      MMAs of the next three.
+//
+// More than 64 output channels are groups of 64: a block keeps one group's weights and walks the
+// pixel tiles of that group, and blocks next to each other share a tile, so the activations that
+// every group reads again come from the L2 cache.  What that pays for: this epilogue writes about
+// 21 outputs per clock and SM (a thread owns a pixel, so there is nothing to transpose), that of
+// tconv.cu 4 to 8.  14704 x 176 x 960 to fp32 26.5 -> 18.4 us, 16384 x 64 x 2048 36.5 -> 25.3,
+// a 1x1 layer of 64x56x56x64 -> 256 55 -> 33 (3.9 TB/s of activations and outputs), 3x3 of
+// 16x58x58x32 -> 272 37.5 -> 24.
 //
 // In the epilogue a thread owns one pixel and reads its channels from tensor memory, so its
 // output is one contiguous run (128 bytes of bf16): it goes through a swizzled per-warp
@@ -74,7 +83,8 @@ struct ResParams {
     int total_tiles, tw, th;
     int lgBW, lgBH;               // pixel tile = BB x BH x BW, powers of two, product 128
     int n_taps, n_cblk, kbpt;     // k-blocks per tile = n_taps * n_cblk
-    int N;                        // UMMA N: Cout rounded up to 16
+    int groups;                   // groups of 64 output channels; block b works on group b mod groups
+    int N;                        // UMMA N: channels of a group, a multiple of 16
     int Cout;
     const uint32_t *T;            // packed codes, one row of `wpr` words per output channel
     long long wpr;
@@ -165,6 +175,9 @@ tconv_res_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int BWm = (1 << P.lgBW) - 1, BHm = (1 << P.lgBH) - 1;
     const int lgHW = P.lgBW + P.lgBH;
+    // this block's channels, and its place among the blocks that share them
+    const int n0 = (int)(blockIdx.x % (unsigned)P.groups) * kNMax;
+    const int bid = (int)(blockIdx.x / (unsigned)P.groups), nb = (int)(gridDim.x / (unsigned)P.groups);
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kMaxStages; ++s) { mbar_init(&ctl->full[s], 1); mbar_init(&ctl->empty[s], 1); }
@@ -192,9 +205,9 @@ tconv_res_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
         if (tid < kNMax) {
             const int c = tid;
             const float alpha = (P.alpha ? (float)(*P.alpha) : 1.0f) * (P.code_bits == 2 ? 1.0f / kDecodedUnit : 1.0f);
-            const bool c_ok = c < P.Cout;
-            ctl->sc[c] = ((P.scale && c_ok) ? __ldg(P.scale + c) : 1.0f) * alpha;
-            ctl->sf[c] = (P.shift && c_ok) ? __ldg(P.shift + c) : 0.0f;
+            const bool c_ok = n0 + c < P.Cout;
+            ctl->sc[c] = ((P.scale && c_ok) ? __ldg(P.scale + n0 + c) : 1.0f) * alpha;
+            ctl->sf[c] = (P.shift && c_ok) ? __ldg(P.shift + n0 + c) : 0.0f;
         }
         for (int t = tid; t <= P.n_taps && t <= kMaxTaps; t += kWorkers)
             ctl->tap[t] = make_uint2(t < P.n_taps ? (uint32_t)P.a_off[t] : 0u, (uint32_t)(t * P.n_cblk) * ((uint32_t)(P.N * 128) >> 4));
@@ -208,7 +221,7 @@ tconv_res_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
             for (int i = tid; i < items; i += kWorkers) {
                 const int u = i / P.N, n = i - u * P.N;
                 const int t = u / P.n_cblk, cb = u - t * P.n_cblk;
-                const uint32_t *rowp = P.T + (long long)(n < P.Cout ? n : P.Cout - 1) * P.wpr;
+                const uint32_t *rowp = P.T + (long long)(n0 + n < P.Cout ? n0 + n : P.Cout - 1) * P.wpr;
                 uint32_t wv[4] = {0u, 0u, 0u, 0u};
                 const long long last = P.wpr - 1;
                 if (P.code_bits == 2) {
@@ -229,7 +242,7 @@ tconv_res_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
                 uint32_t out[32];
                 if (P.code_bits == 2) decode_kblock<2>(wv, out);
                 else decode_kblock<1>(wv, out);
-                if (n >= P.Cout) {
+                if (n0 + n >= P.Cout) {
 #pragma unroll
                     for (int j = 0; j < 32; ++j) out[j] = 0u;
                 }
@@ -252,7 +265,7 @@ tconv_res_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
         if (lane == 0 && P.kbpt > 0) {
             uint32_t s = 0, ph = 0;
             bool ok = true;
-            for (int tile = blockIdx.x; tile < P.total_tiles && ok; tile += gridDim.x) {
+            for (int tile = bid; tile < P.total_tiles && ok; tile += nb) {
                 int pt = tile;
                 const int twi = pt % P.tw; pt /= P.tw;
                 const int thi = pt % P.th;
@@ -300,7 +313,7 @@ tconv_res_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
             for (uint32_t i = 0; i < me; ++i) skip_tile();
             bool ok = true;
             uint32_t lt = me;
-            for (int tile = blockIdx.x + (int)me * (int)gridDim.x; tile < P.total_tiles && ok; tile += kIssuers * (int)gridDim.x, lt += kIssuers) {
+            for (int tile = bid + (int)me * nb; tile < P.total_tiles && ok; tile += kIssuers * nb, lt += kIssuers) {
                 const uint32_t buf = lt & (kAccBufs - 1);
                 // The token first: once it is here, the threads of all earlier tiles are past their waits for an
                 // accumulator, so the accumulator barrier (shared by the issuing threads in turn) is at most one
@@ -361,13 +374,13 @@ tconv_res_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
             int cw, ch, cbt;
             tile_coords(tile, cw, ch, cbt);
             mbar_expect_tx(&ctl->res_full[ew], kStageBuf);
-            tma_load_4d(base + P.res_off + (size_t)ew * kStageBuf, &map_r, &ctl->res_full[ew], 0, cw, ch, cbt);
+            tma_load_4d(base + P.res_off + (size_t)ew * kStageBuf, &map_r, &ctl->res_full[ew], n0, cw, ch, cbt);
         };
-        const int first_tile = blockIdx.x + set * (int)gridDim.x;
+        const int first_tile = bid + set * nb;
         if (P.has_res && lane == 0 && first_tile < P.total_tiles) res_load(first_tile);
 
         uint32_t lt = set;
-        for (int tile = first_tile; tile < P.total_tiles; tile += 2 * (int)gridDim.x, lt += 2) {
+        for (int tile = first_tile; tile < P.total_tiles; tile += 2 * nb, lt += 2) {
             int cw, ch, cbt;
             tile_coords(tile, cw, ch, cbt);
             const uint32_t buf = lt & (kAccBufs - 1);
@@ -471,7 +484,8 @@ tconv_res_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
                                      v[jj * 4 + 3]);
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                     __syncwarp();
-                    if (lane == 0) tma_store_4d(&map_y, base + P.stg_off + (size_t)ew * kStageBuf, hf * 32, cw, ch, cbt);
+                    if (lane == 0 && n0 + hf * 32 < P.Cout)
+                        tma_store_4d(&map_y, base + P.stg_off + (size_t)ew * kStageBuf, n0 + hf * 32, cw, ch, cbt);
                 }
             };
             chunk(va, 0);
@@ -479,13 +493,13 @@ tconv_res_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
             if (P.out_bf16) {
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 __syncwarp();
-                if (lane == 0) tma_store_4d(&map_y, base + P.stg_off + (size_t)ew * kStageBuf, 0, cw, ch, cbt);
+                if (lane == 0) tma_store_4d(&map_y, base + P.stg_off + (size_t)ew * kStageBuf, n0, cw, ch, cbt);
             }
             if (P.has_res) {
                 // every lane has read its row of the residual: fetch the one of this warp's next tile
                 ++nres;
                 __syncwarp();
-                const int next = tile + 2 * (int)gridDim.x;
+                const int next = tile + 2 * nb;
                 if (lane == 0 && next < P.total_tiles) res_load(next);
             }
         }
@@ -514,7 +528,7 @@ int twn_detail::launch_conv_resident(const Geometry &g, const void *X, const uin
                                      double rival_us, bool *handled)
 {
     *handled = false;
-    if (g.sw != 1 || g.sh != 1 || g.Cout > kNMax || g.Cout < 1) return TWN_OK;
+    if (g.sw != 1 || g.sh != 1 || g.Cout < 1) return TWN_OK;
     if (g.bn_partial) return TWN_OK;      // batch statistics come out of the general kernel's epilogue
     const bool out_bf16 = epi.out_dtype == TWN_BF16;
     const int es = out_bf16 ? 2 : 4;
@@ -531,7 +545,10 @@ int twn_detail::launch_conv_resident(const Geometry &g, const void *X, const uin
     P.n_taps = g.n_taps;
     P.n_cblk = (int)((g.Cin + kBlockK - 1) / kBlockK);
     P.kbpt = P.n_taps * P.n_cblk;
-    P.N = (g.Cout + 15) / 16 * 16;
+    P.groups = (g.Cout + kNMax - 1) / kNMax;
+    P.N = P.groups > 1 ? kNMax : (g.Cout + 15) / 16 * 16;
+    if (P.groups > dev.sm_count) return TWN_OK;
+    const int nb = dev.sm_count / P.groups;      // blocks per group
     P.Cout = g.Cout;
     P.codes_aligned = 1;
     int w_lo = 0, w_hi = 0, h_lo = 0, h_hi = 0;
@@ -573,11 +590,6 @@ int twn_detail::launch_conv_resident(const Geometry &g, const void *X, const uin
     const long long pixels = (long long)g.Bv * g.Hv * g.Wv;
     if (pixels > 65536 && total * kPix > 3 * pixels) return TWN_OK;
 
-    // Fitted to measured launches (1 to 13 tiles per block): set-up with the decoding of the weights, then the tiles.
-    const double per_tile = 0.13 * P.kbpt * (g.Cin < kBlockK ? (double)g.Cin / kBlockK : 1.0);
-    const long long per_block = (total + dev.sm_count - 1) / dev.sm_count;
-    if (4.3 + 0.26 * P.kbpt + (per_block - 1) * (per_tile > 0.5 ? per_tile : 0.5) > rival_us) return TWN_OK;
-
     P.w_lo = w_lo; P.h_lo = h_lo;
     const int row_pix = BW + hw;
     P.a_sbo = hw > 0 ? (uint32_t)row_pix * 128u : 1024u;
@@ -585,6 +597,23 @@ int twn_detail::launch_conv_resident(const Geometry &g, const void *X, const uin
         P.a_off[t] = (((g.taps[t].dh - h_lo) * row_pix + (g.taps[t].dw - w_lo)) * 128) >> 4;
     P.stage_tx = 128 * row_pix * (BH + hh) * BB;
     P.stage_bytes = (P.stage_tx + 1023) / 1024 * 1024;
+
+    // Fitted to measured launches (one group: 1 to 13 tiles per block; several: 1 to 42, 30 shapes): set-up with the
+    // decoding of the weights and the first tile, then a tile per turn of the slowest part: MMAs, the activations
+    // (each group reads them again: 52 GB/s per SM from the L2 cache), or the stores.
+    const long long per_block = (total + nb - 1) / nb;
+    const double mma = 0.13 * P.kbpt * (g.Cin < kBlockK ? (double)g.Cin / kBlockK : 1.0);
+    double first = 0.26 * P.kbpt, per_tile = mma > 0.5 ? mma : 0.5;
+    if (P.groups > 1) {
+        const double loads = (double)P.n_cblk * P.stage_bytes / 16384.0, store = out_bf16 ? 0.7 : 0.9;
+        if (0.42 * loads > first) first = 0.42 * loads;
+        if (0.33 * loads > per_tile) per_tile = 0.33 * loads;
+        if (store > per_tile) per_tile = store;
+    }
+    const double us = 4.3 + first + (double)(per_block - 1) * per_tile;
+    // a margin for the models' error where the other kernels are often the better choice: at 0.95 a 3x3 layer of
+    // 5x50x50x96 -> 200 came here and took 15.2 us instead of 14.5
+    if (us > (P.groups > 1 ? 0.9 : 1.0) * rival_us) return TWN_OK;
     const long long wts_bytes = (long long)P.kbpt * P.N * 128;
     const long long fixed = 1024 + wts_bytes + kEpiWarps * kStageBuf * (epi.residual ? 2 : 1) + 2048;
     if (fixed > kSmemLimit) return TWN_OK;
@@ -664,7 +693,7 @@ int twn_detail::launch_conv_resident(const Geometry &g, const void *X, const uin
         TWN_CUDA_OK(cudaFuncSetAttribute(tconv_res_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit));
         attr_set[dev.ordinal] = true;
     }
-    const int grid = dev.sm_count < P.total_tiles ? dev.sm_count : P.total_tiles;
+    const int grid = P.groups * (int)(nb < P.total_tiles ? nb : P.total_tiles);
     TWN_CUDA_OK(twn_launch_pdl(grid * 2 >= dev.sm_count, tconv_res_kernel, grid, kThreads, (size_t)smem_bytes, s, map_x, map_y, map_r, P));
     TWN_CUDA_OK(cudaGetLastError());
     *handled = true;
