@@ -195,20 +195,20 @@ class TernarizeWorkload:
         return self.n * 4, self.ld // 4 + 64
 
     def launches_per_step(self):
-        return 2
+        return 1
 
     def units_per_step(self):
         return self.n * self.bytes_per_unit / 1e9  # GB of algorithmic traffic
 
     def roofline(self, ms_per_step, peaks):
         ach = self.n * self.bytes_per_unit / (ms_per_step * 1e-3) / 1e9
-        return {"bound": "hbm", "kernel": "sum_abs_kernel + code_pack_kernel (one twn_ternarize call)",
+        return {"bound": "hbm", "kernel": "ternarize_kernel (one twn_ternarize call)",
                 "achieved": ach, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                 "frac": ach / peaks["hbm_gbs"], "peak_source": peaks["source"],
                 "frac_of_nominal_8TBs": ach / 8000.0,
-                # dram__bytes_read.sum + dram__bytes_write.sum of the two kernels of one call (ncu capture of
+                # dram__bytes_read.sum + dram__bytes_write.sum of the one kernel of a call (ncu capture of
                 # this workload, summarised under profiles/); algorithmic: 8.25e8
-                "traffic": 819.6e6 if self.n == 100_000_000 else None}
+                "traffic": 729.5e6 if self.n == 100_000_000 else None}
 
     def check(self):
         st = self.twn.stats_to_host(self.stats)
@@ -364,7 +364,7 @@ class SgdTernarizeWorkload(TernarizeWorkload):
 
     def roofline(self, ms_per_step, peaks):
         r = super().roofline(ms_per_step, peaks)
-        r["kernel"] = "sgd_update_kernel + code_pack_kernel (twn_sgd_update, twn_ternarize_codes)"
+        r["kernel"] = "sgd_update_kernel + ternarize_kernel (twn_sgd_update, twn_ternarize_codes)"
         r["traffic"] = None
         return r
 
@@ -586,7 +586,7 @@ class GemmSweepWorkload:
         unit = "TFLOP/s" if worst["bound"] == "tensor" else "GB/s"
         ach = worst["tflops"] if worst["bound"] == "tensor" else worst["gbs"]
         peak = peaks["bf16_tflops"] if worst["bound"] == "tensor" else peaks["hbm_gbs"]
-        return {"bound": worst["bound"], "kernel": "tconv_kernel / tconv_res_kernel (one twn_gemm call per shape); headline = "
+        return {"bound": worst["bound"], "kernel": "tconv_kernel / tconv_res_kernel / tconv_split_kernel (one twn_gemm call per shape); headline = "
                 f"the worst of the five gated shapes: M={worst['M']} K={worst['K']} N={worst['N']}",
                 "achieved": ach, "peak": peak, "unit": unit, "frac": worst["frac"],
                 "peak_source": peaks["source"] + " (bf16 burst / copy bandwidth: every shape is timed alone, cold L2)",
@@ -717,9 +717,24 @@ class LayerWorkload:
             f"oracle conv2d_fwd on {npix} of {total} output pixels ({dt:.1f} s)", oracle.num_threads()
 
 
+def graph_kernels(graph):
+    """Number of kernel launches in a captured graph."""
+    import ctypes
+    rt = ctypes.CDLL("libcudart.so.12")
+    handle, count = ctypes.c_void_p(graph.raw_cuda_graph()), ctypes.c_size_t()
+    assert rt.cudaGraphGetNodes(handle, None, ctypes.byref(count)) == 0
+    nodes = (ctypes.c_void_p * count.value)()
+    assert rt.cudaGraphGetNodes(handle, nodes, ctypes.byref(count)) == 0
+    kernels, kind = 0, ctypes.c_int()
+    for node in nodes:
+        assert rt.cudaGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)) == 0
+        kernels += kind.value == 0                                # cudaGraphNodeTypeKernel
+    return kernels
+
+
 class NetWorkload:
     """A chained network workload: images/s of a forward pass or of a whole training step,
-    replayed from a CUDA graph (the step is a fixed sequence of ~200 launches)."""
+    replayed from a CUDA graph (the step is a fixed sequence of launches)."""
     metric = "images/s"
     unit = "images/s"
     dtype = "bf16"
@@ -799,12 +814,13 @@ class NetWorkload:
             self._eager()
         torch.cuda.synchronize()
         net.check_status()
-        self.graph = torch.cuda.CUDAGraph()
+        self.graph = torch.cuda.CUDAGraph(keep_graph=True)       # kept so that its kernel nodes can be counted
         # The step is captured on a high-priority stream: the forward / backward-for-data chain is the
         # critical path, while the weight gradients and the code re-layouts (streams of default
         # priority forked from it) fill the SMs it leaves free.
         with torch.cuda.graph(self.graph, stream=torch.cuda.Stream(priority=-1)):
             self._eager()
+        self.graph.instantiate()
         # per-kernel device times from one eager pass; a spin keeps the GPU behind the host so
         # that the events bracket kernels only
         net.timed = []
@@ -901,33 +917,8 @@ class NetWorkload:
         return h2d, self.host_logits.numel() * self.host_logits.element_size()
 
     def launches_per_step(self):
-        n = 0
-        net = self.net
-        for op in net.ops:
-            if op[0] == "layer":
-                L = op[1]
-                n += 1 + (1 if L.small_cin else 0)                       # forward (+ im2col or input fold)
-                if self.train:
-                    n += 1 if L.fold else 0                              # folded codes
-                    n += 1 + 1 + (1 if L.fold else 0)                    # act_bwd, dW (+ unfold)
-                    # the reduction of the pixel splits of dW runs only when there is more than one split
-                    if L.fold:
-                        n += 1
-                    else:
-                        d = L.extra["dw_desc"]
-                        splits = self.twn.conv2d_bwd_weight_workspace_bytes(d) // (d.Cout * d.kh * d.kw * d.Cin * 4)
-                        n += 1 if splits > 1 else 0
-                    if L.src != "input":
-                        # backward for data: one launch per residue class of the stride that a tap reaches
-                        # (a 1x1 projection shortcut adds into the dense gradient in place: one class)
-                        shortcut = L.k == 1 and L.stride > 1 and not L.relu and not L.residual
-                        n += 1 if shortcut else L.stride * L.stride
-            elif op[0] in ("maxpool", "avgpool"):
-                n += 2 if self.train else 1
-        if self.train:
-            n += 3 * ((len(net.layers) + 31) // 32)     # batched ternarization (two sweeps) and code transposes
-            # with the update: coding sweep + update instead of the two sweeps, the same count
-        return n
+        """Kernel nodes of the captured step: every kernel of a step is one of this library's."""
+        return graph_kernels(self.graph)
 
     def units_per_step(self):
         return self.net.B
@@ -957,7 +948,7 @@ class NetWorkload:
         peak = peaks["bf16_tflops"]
         tern = self.per_layer_ternarize_us()
         step_flops = 2.0 * self.net.total_macs()
-        out = {"bound": "tensor", "kernel": "tconv_kernel + tconv_res_kernel (every forward and backward-for-data call of a step, each timed alone)",
+        out = {"bound": "tensor", "kernel": "tconv_kernel + tconv_res_kernel + tconv_split_kernel (every forward and backward-for-data call of a step, each timed alone)",
                "achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak,
                "peak_source": peaks["source"] + " (bf16 burst: isolated kernels)", "traffic": self.measured_traffic(),
                "launches": t[3], "us_in_kernel_isolated": round(t[0], 1), "us_at_bound": round(t[2], 1),
