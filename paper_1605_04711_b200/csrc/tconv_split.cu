@@ -34,9 +34,6 @@ using namespace twn_detail;
 
 namespace {
 
-#ifndef PDLMAX
-#define PDLMAX 100000
-#endif
 constexpr int kChan = 128;
 constexpr int kBlockK = 64;
 constexpr int kSets = 2;                 // decode groups, on k-blocks in turn (three or four: no gain, 1 us more set-up)
@@ -429,7 +426,7 @@ int launch_t(const Geometry &g, SplitParams &P, const void *X, int splits, const
     cfg.stream = s;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = tiles*splits < PDLMAX;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
     attr[1].id = cudaLaunchAttributeClusterDimension;
     attr[1].val.clusterDim.x = (unsigned)splits;
     attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
