@@ -121,6 +121,7 @@ struct ConvParams {
     // writes them with a TMA store (box = 32 channels x sbw x sbh x sbb pixels); 0 = per-thread stores
     int tma_store, lg_sbw, lg_sbh;
     int res_tma;                  // 1: the residual (bf16) is staged by per-warp TMA loads, two chunks deep
+    int fragments;                // 1: bf16 in and out by TMA, no batch statistics: chunks are drained as matrix fragments
     Tap taps[kMaxTaps];
 };
 
@@ -139,8 +140,9 @@ struct __align__(1024) SmemLayout {
     // per-warp output staging for TMA stores: [pixels][32 channels].  The stores of the epilogue
     // queue behind the producer's tile loads in the copy engine, so while the main loop of the next
     // tile runs a store takes long to release its buffer: the overlapped tile shapes keep four.
-    alignas(128) uint8_t stage_out[kEpiWarps][Cfg<PIX>::kOutBufs][kStageBytes];
-    alignas(128) __nv_bfloat16 stage_res[kEpiWarps][2][32 * 32];  // per-warp residual staging: [32 pixels][32 channels]
+    // The fragment path swizzles them (64 bytes), hence the alignment.
+    alignas(1024) uint8_t stage_out[kEpiWarps][Cfg<PIX>::kOutBufs][kStageBytes];
+    alignas(1024) __nv_bfloat16 stage_res[kEpiWarps][2][32 * 32];  // per-warp residual staging: [32 pixels][32 channels]
     unsigned long long res_full[kEpiWarps][2];
     uint32_t kword[kWordTab];              // first code word of k-block u in a packed row, u < kWordTab
     uint32_t tmem_base;
@@ -479,7 +481,12 @@ tconv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ 
                 const int c = es + i * kEpiSets;
                 if (kbpt > 0) {
                     if (warp_on) {
-                        tmem_ld32(t_acc + c * 32, v);
+                        if (P.fragments) {
+                            tmem_ld_16x256b_x4(t_acc + c * 32, v);
+                            tmem_ld_16x256b_x4(t_acc + (16u << 16) + c * 32, v + 16);
+                        } else {
+                            tmem_ld32(t_acc + c * 32, v);
+                        }
                         tmem_wait_ld(v);
                     }
                     if (i + 1 == kMine) {
@@ -493,6 +500,75 @@ tconv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ 
                     for (int j = 0; j < 32; ++j) v[j] = 0u;
                 }
                 if (!warp_on) continue;
+                if (P.fragments) {
+                    // The accumulator's rows are channels, the output's rows pixels: the chunk has to be transposed.  The
+                    // 16x256b load leaves a thread two neighbouring pixels of channels g, g + 8, g + 16, g + 24: packed,
+                    // that is the operand of stmatrix.trans.  Four of those store the chunk, four ldmatrix.trans fetch
+                    // its residual; with a channel per thread (below) each takes 32 two-byte accesses.  Layers gain 3-15 %
+                    // (64x14x14x256 3x3 19.2 -> 17.8 us, 100000x640x256 50.8 -> 43.0); fp32 outputs would store as often
+                    // and lose 3 %, and everything else is rare: they keep the path below, whose registers fit in the
+                    // 96 that two decode groups leave (one loop for all cases spilled and lost 3-5 %).
+                    // v[16 h + 4 k + 2 u + e]: channel g + 8 (2 h + u), pixel 8 k + 2 (ln % 4) + e
+                    uint32_t ln;
+                    asm volatile("mov.u32 %0, %%laneid;" : "=r"(ln));      // read here: nothing of it is kept in registers
+                    // this lane's row of the 8x8 matrices: pixel ln % 8 of eight, channels 8 (ln / 8) ...
+                    const uint32_t mat = (ln & 7) * 64 + (((ln >> 3) ^ ((ln >> 1) & 3)) << 4);
+#pragma unroll
+                    for (int m = 0; m < 4; ++m) {
+                        const float scm = __shfl_sync(0xffffffffu, sc, (ln >> 2) + 8 * m);
+                        const float sfm = __shfl_sync(0xffffffffu, sf, (ln >> 2) + 8 * m);
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            const int j = m / 2 * 16 + k * 4 + m % 2 * 2;
+                            fma_f32x2(v[j], v[j + 1], scm, scm, sfm, sfm);
+                        }
+                    }
+                    if (use_res_tma) {
+                        if (!mbar_wait_warp(&my_res_full[nres & 1u], (nres >> 1) & 1u, abort_flag, P.status, 32)) { alive = false; break; }
+                        const uint32_t rs = smem_u32(my_res) + (nres & 1u) * (32 * 32 * 2) + mat;
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            uint32_t rr[4];
+                            ldmatrix_x4_trans(rs + k * 512, rr);
+#pragma unroll
+                            for (int m = 0; m < 4; ++m) {
+                                const int j = m / 2 * 16 + k * 4 + m % 2 * 2;
+                                const float r0 = __uint_as_float(rr[m] << 16), r1 = __uint_as_float(rr[m] & 0xFFFF0000u);
+                                const float y0 = __uint_as_float(v[j]), y1 = __uint_as_float(v[j + 1]);
+                                v[j] = __float_as_uint(P.res_gate ? (r0 > 0.0f ? y0 : 0.0f) : y0 + r0);
+                                v[j + 1] = __float_as_uint(P.res_gate ? (r1 > 0.0f ? y1 : 0.0f) : y1 + r1);
+                            }
+                        }
+                        // the buffer is free again: fetch the residual of the chunk after the next
+                        __syncwarp();
+                        if (lane == 0 && i + 2 < kMine) res_load(c + 2 * kEpiSets, nres & 1u);
+                        ++nres;
+                    }
+                    // the buffer was last read by the store this warp issued kOutBufs chunks ago
+                    if (lane == 0) asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(kOutBufs - 1) : "memory");
+                    __syncwarp();
+                    uint8_t *const sbuf = my_out + (nst % kOutBufs) * kStageBytes;
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        uint32_t w[4];
+#pragma unroll
+                        for (int m = 0; m < 4; ++m) {
+                            const int j = m / 2 * 16 + k * 4 + m % 2 * 2;
+                            w[m] = relu_in_cvt ? pack_bf16x2_relu(__uint_as_float(v[j]), __uint_as_float(v[j + 1]))
+                                               : pack_bf16x2(__uint_as_float(v[j]), __uint_as_float(v[j + 1]));
+                        }
+                        stmatrix_x4_trans(smem_u32(sbuf) + mat + k * 512, w);
+                    }
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                    __syncwarp();
+                    if (lane == 0) {
+                        const int p0 = c * 32;
+                        tma_store_4d(&map_y, sbuf, c_n0, (p_w0 + (p0 & BWm)) * P.osw, (p_h0 + ((p0 >> P.lgBW) & BHm)) * P.osh,
+                                     p_b0 + (p0 >> (P.lgBW + P.lgBH)));
+                    }
+                    ++nst;
+                    continue;
+                }
                 // output offset of pixel `lane` of this chunk (per-thread stores and residual loads
                 // exchange them by shuffle), ~0 = outside the output
                 uint32_t my_off = 0xFFFFFFFFu;
@@ -705,6 +781,10 @@ int launch_conv_t(const Geometry &g, ConvParams &P, const void *X, const twn_dev
     const int es = P.out_dtype == TWN_BF16 ? 2 : 4;
     P.tma_store = 0;
     P.res_tma = 0;
+    // a bf16 residual is as addressable as a bf16 output of the same pitch, but for its base
+    P.fragments = es == 2 && !P.bn_partial &&
+                  (!P.residual || (P.res_dtype == TWN_BF16 && reinterpret_cast<uintptr_t>(P.residual) % 16 == 0));
+    const CUtensorMapSwizzle swz = P.fragments ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_NONE;
     const long long base_pix = (long long)g.ooh * g.OW + g.oow;
     if ((g.ldy * es) % 16 == 0 && ((long long)g.Cout * es) % 16 == 0 && (reinterpret_cast<uintptr_t>(P.Y) % 16) == 0 &&
         g.OW > g.oow && g.OH > g.ooh) {
@@ -727,7 +807,7 @@ int launch_conv_t(const Geometry &g, ConvParams &P, const void *X, const twn_dev
             cuuint64_t strides[3] = {(cuuint64_t)g.ldy * es, (cuuint64_t)g.OW * g.ldy * es, (cuuint64_t)g.OH * g.OW * g.ldy * es};
             void *ybase = static_cast<char *>(P.Y) + base_pix * g.ldy * es;
             if (enc(&map_y, es == 2 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, ybase, dims,
-                    strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                    strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swz,
                     CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS)
                 P.tma_store = 1;
             // a bf16 residual of the same geometry is staged the same way
@@ -736,12 +816,14 @@ int launch_conv_t(const Geometry &g, ConvParams &P, const void *X, const twn_dev
                 cuuint64_t rstrides[3] = {(cuuint64_t)g.ldy * 2, (cuuint64_t)g.OW * g.ldy * 2, (cuuint64_t)g.OH * g.OW * g.ldy * 2};
                 void *rbase = const_cast<char *>(static_cast<const char *>(P.residual)) + base_pix * g.ldy * 2;
                 if (enc(&map_r, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, rbase, dims, rstrides, rbox, estr,
-                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                        CU_TENSOR_MAP_INTERLEAVE_NONE, swz, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS)
                     P.res_tma = 1;
             }
         }
     }
+    P.fragments = P.fragments && P.tma_store;
+    if (P.fragments && P.residual && !P.res_tma) return TWN_ERR_CUDA;      // the same geometry could be encoded for Y
     const int grid = dev.sm_count < P.total_tiles ? dev.sm_count : P.total_tiles;
     // Programmatic dependent launch pays when the blocks cover the GPU (set-up and launch latency hide behind the
     // previous kernel's last tiles); a launch of a few blocks measured slower with it (an inner product of 8 blocks
