@@ -79,8 +79,8 @@ typedef struct {
  * the lower layer's dZ directly (Algorithm 1, TernaryBackward, followed by the chain rule
  * through y = relu(z * scale + shift)).
  * TWN_SUM_IN_ORDER, or-ed in, keeps a launch that would not fill the GPU from splitting the reduction over several
- * thread blocks: every sum then runs over the taps and channels in order, and an output has the same bits whatever
- * the batch and the launch shape.  Forward passes of a training step want that: a ReLU gate that a differently rounded
+ * thread blocks, and from kernels that take the taps in another order: every sum then runs over the taps and, within
+ * a tap, over the channels, and an output has the same bits whatever the batch and the launch shape.  Forward passes of a training step want that: a ReLU gate that a differently rounded
  * sum flips changes the gradient there by all of its value, not by a rounding. */
 enum { TWN_RESIDUAL_ADD = 0, TWN_RESIDUAL_GATE = 1, TWN_SUM_IN_ORDER = 2 };
 typedef struct {

@@ -94,13 +94,14 @@ struct EpilogueArgs {
     const float *scale, *shift;
     const void *residual;
     int res_dtype, res_gate, relu, out_dtype;
-    bool in_order;                // the reduction is not split (TWN_SUM_IN_ORDER)
+    bool in_order;                // every sum runs over the taps, then the channels (TWN_SUM_IN_ORDER): no split
 };
 
 // Contraction with the layer's decoded weights resident in shared memory (tconv_res.cu).  Launches
-// and returns TWN_OK with *handled = true when the launch fits that kernel (at most 64 output
-// channels, unit input stride, decoded weights that fit in shared memory, outputs that TMA can
-// store) and should not take longer than `rival_us`; otherwise *handled = false and nothing has been launched.
+// and returns TWN_OK with *handled = true when the launch fits that kernel (unit input stride, decoded
+// weights of 64 output channels that fit in shared memory, outputs that TMA can store; not several taps
+// of several channel blocks whose sums must stay in order) and should not take longer than `rival_us`;
+// otherwise *handled = false and nothing has been launched.
 int launch_conv_resident(const Geometry &g, const void *X, const uint32_t *T, const EpilogueArgs &epi, void *Y,
                          int32_t *dev_status, const twn_device_info &dev, cudaStream_t s, double rival_us, bool *handled);
 

@@ -545,6 +545,10 @@ int twn_detail::launch_conv_resident(const Geometry &g, const void *X, const uin
     P.n_taps = g.n_taps;
     P.n_cblk = (int)((g.Cin + kBlockK - 1) / kBlockK);
     P.kbpt = P.n_taps * P.n_cblk;
+    // A tile's channel blocks arrive one after the other and every tap reads a block while it is there, so the sums run
+    // over channel blocks outside and taps inside, in the other kernels the other way round.  With several of both, sums
+    // that were asked for in order are not the same bits here.
+    if (epi.in_order && P.n_taps > 1 && P.n_cblk > 1) return TWN_OK;
     P.groups = (g.Cout + kNMax - 1) / kNMax;
     P.N = P.groups > 1 ? kNMax : (g.Cout + 15) / 16 * 16;
     if (P.groups > dev.sm_count) return TWN_OK;
