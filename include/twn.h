@@ -70,7 +70,7 @@ typedef struct {
 
 /* What follows the contraction, per output element with channel n:
  *   y = acc * alpha;  y = y * scale[n] + shift[n];  y += residual;  y = max(y, 0)
- * each step only if its field is set.  (Eq. 2 puts alpha on the input; a scalar
+ * each step only if its field is set; a NaN stays a NaN through the ReLU.  (Eq. 2 puts alpha on the input; a scalar
  * commutes with the sum, so it is applied once per output here.)
  * With residual_op = TWN_RESIDUAL_GATE the tensor given as `residual` is not added but gates
  * the result: y is kept where residual > 0 and is 0 elsewhere.  This is the backward pass of

@@ -287,6 +287,13 @@ __device__ __forceinline__ uint32_t pack_bf16x2_relu(float lo, float hi)
     asm("cvt.rn.relu.bf16x2.f32 %0, %1, %2;" : "=r"(pk) : "f"(hi), "f"(lo));
     return pk;
 }
+// The ReLU of a result that stays fp32.  As in the conversion above and in y < 0 ? 0 : y, a NaN stays a NaN.
+__device__ __forceinline__ float relu_f32(float x)
+{
+    float y;
+    asm("max.NaN.f32 %0, %1, 0f00000000;" : "=f"(y) : "f"(x));
+    return y;
+}
 // (x0, x1) <- (x0 * a0 + b0, x1 * a1 + b1), both lanes in one instruction.
 __device__ __forceinline__ void fma_f32x2(uint32_t &x0, uint32_t &x1, float a0, float a1, float b0, float b1)
 {

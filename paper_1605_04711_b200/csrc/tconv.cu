@@ -424,7 +424,7 @@ tconv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ 
         const int BWm = (1 << P.lgBW) - 1, BHm = (1 << P.lgBH) - 1;
         const bool out_bf16 = P.out_dtype == TWN_BF16, res_bf16 = P.res_dtype == TWN_BF16;
         const bool need_off = !P.tma_store || (P.residual && !P.res_tma);
-        // the ReLU of a bf16 output rides on the conversion (a NaN stays a NaN); every other path clamps explicitly
+        // the ReLU of a bf16 output rides on the conversion; every other path clamps explicitly (a NaN stays a NaN in both)
         const bool relu_in_cvt = P.relu && out_bf16 && P.tma_store;
         const bool relu_here = P.relu && !relu_in_cvt;
         constexpr int kChunks = PIX / 32;
@@ -635,7 +635,7 @@ tconv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ 
                 }
                 if (relu_here) {
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(fmaxf(__uint_as_float(v[j]), 0.0f));
+                    for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(relu_f32(__uint_as_float(v[j])));
                 }
                 if (P.tma_store) {
                     // a staging buffer holds 32 pixels of bf16 or 16 of fp32: one or two rounds per chunk

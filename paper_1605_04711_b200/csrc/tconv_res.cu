@@ -476,7 +476,7 @@ tconv_res_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
                     __syncwarp();
                     if (P.relu) {
 #pragma unroll
-                        for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(fmaxf(__uint_as_float(v[j]), 0.0f));
+                        for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(relu_f32(__uint_as_float(v[j])));
                     }
 #pragma unroll
                     for (int jj = 0; jj < 8; ++jj)

@@ -127,7 +127,7 @@ __device__ __forceinline__ void finish(const SplitParams &P, size_t off, int lef
     }
     if (P.relu) {
 #pragma unroll
-        for (int x = 0; x < 4; ++x) y[x] = y[x] < 0.0f ? 0.0f : y[x];      // a NaN stays a NaN
+        for (int x = 0; x < 4; ++x) y[x] = relu_f32(y[x]);
     }
     if (P.out_dtype == TWN_BF16) {
         __nv_bfloat16 *yp = reinterpret_cast<__nv_bfloat16 *>(P.Y) + off;
