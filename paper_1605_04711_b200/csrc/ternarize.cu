@@ -74,6 +74,7 @@ struct Item {
     long long rows, cols, wpr;
     unsigned int wpr_used;           // words of a row that hold codes
     unsigned int wpr_magic;          // floor(2^32 / wpr_used) + 1, 0 for one word per row
+    unsigned int last_valid;         // weights of a row's last word; every other word holds 16
     unsigned int parts, part_words;
     unsigned int first_part;         // of this tensor, among the parts of the launch
     unsigned int first_pass;         // weights of a part that phase 1 reads without keeping them in L2
@@ -144,10 +145,11 @@ __device__ __forceinline__ Place place_word(const Item &it, const PartRange &r, 
         // jj / wpr_used: the multiplication is at most one too high
         unsigned int ro = it.wpr_magic ? __umulhi(jj, it.wpr_magic) : jj;
         if (ro * it.wpr_used > jj) --ro;
-        const unsigned int j = jj - ro * it.wpr_used, cols = (unsigned int)it.cols;
+        const unsigned int j = jj - ro * it.wpr_used;
         p.out = r.out0 + (unsigned long long)ro * (unsigned long long)it.wpr + j;
-        p.f = ro * cols + 16 * j - 16 * r.j0;
-        p.valid = min(16u, cols - 16 * j);
+        // the low halves do: the difference is inside the part, which holds fewer than 2^32 weights
+        p.f = ro * (unsigned int)it.cols + 16 * j - 16 * r.j0;
+        p.valid = j + 1 == it.wpr_used ? it.last_valid : 16u;
     }
     return p;
 }
@@ -1044,6 +1046,7 @@ bool make_item(const float *W, int64_t rows, int64_t cols, twn_stats_t *stats, u
     if (used > 0xFFFFFFFFull || part > 0x08000000ull) return false;
     it->wpr_used = (unsigned int)used;
     it->wpr_magic = used > 1 ? (unsigned int)((1ull << 32) / used + 1) : 0;
+    it->last_valid = used > 0 ? (unsigned int)(cols - 16 * (used - 1)) : 0;
     it->part_words = (unsigned int)part;
     it->parts = (unsigned int)std::max(1ull, (it->words + part - 1) / part);
     it->vec4 = rows == 1 || cols % 4 == 0;

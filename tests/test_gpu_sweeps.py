@@ -75,3 +75,23 @@ def test_signs(rows, cols, offset):
     st, (ref, codes) = twn.stats_to_host(stats), oracle.binarize(W)
     assert st["status"] == 0 and abs(st["alpha"] - ref.alpha) <= 1e-12 * ref.alpha and st["n_neg"] == int((W < 0).sum())
     assert np.array_equal(host_u32(packed), oracle.pack1(codes.reshape(rows, cols), ld))
+
+
+@pytest.mark.parametrize("cols", [2 ** 32 + 1, 2 ** 32 + 4])
+def test_rows_of_more_than_2_to_the_32_weights(cols):
+    """Rows whose position does not fit in 32 bits and that are no whole number of words (34 GB of weights, all kept)."""
+    if torch.cuda.mem_get_info()[0] < 45e9:
+        pytest.skip("needs 45 GB of device memory")
+    rows, used, ld = 2, (cols + 15) // 16, twn.ld_for(cols)
+    W = torch.ones((rows, cols), dtype=torch.float32, device="cuda")
+    stats = twn.new_stats()
+    packed = torch.full((rows, ld // 16), -1, dtype=torch.int32, device="cuda")
+    twn.ternarize(W, 0.7, stats, packed, ld, None, workspace(twn.ternarize_workspace_bytes()))
+    st = twn.stats_to_host(stats)
+    del W
+    assert st["status"] == 0 and st["alpha"] == 1.0 and (st["n_neg"], st["n_zero"], st["n_pos"]) == (0, 0, rows * cols)
+    whole, last = (int(oracle.pack(np.ones((1, n), dtype=np.int8), 64).view(np.int32)[0, 0]) for n in (16, cols % 16))
+    assert bool((packed[:, :used - 1] == whole).all()) and bool((packed[:, used - 1] == last).all())
+    assert not bool(packed[:, used:].any())
+    del packed
+    torch.cuda.empty_cache()
