@@ -108,7 +108,7 @@ im2col_tile_kernel(const __nv_bfloat16 *__restrict__ X, twn_conv_desc_t d, int H
                 const int o0 = tab[ch * 8 + 2 * e], o1 = tab[ch * 8 + 2 * e + 1];
                 v[e] = (uint32_t)win[o0 < 0 ? zero_at : base + o0] | ((uint32_t)win[o1 < 0 ? zero_at : base + o1] << 16);
             }
-            *reinterpret_cast<uint4 *>(out + ((size_t)(b * Ho + ho0) * Wo + p) * ldk + ch * 8) = make_uint4(v[0], v[1], v[2], v[3]);
+            *reinterpret_cast<uint4 *>(out + (((size_t)b * Ho + ho0) * Wo + p) * ldk + ch * 8) = make_uint4(v[0], v[1], v[2], v[3]);
         }
         return;
     }
@@ -119,7 +119,7 @@ im2col_tile_kernel(const __nv_bfloat16 *__restrict__ X, twn_conv_desc_t d, int H
     for (int e = 0; e < 8; ++e) o[e] = tab[ch * 8 + e];
     const int n_pix = min(rows, Ho - ho0) * Wo;
     int p = threadIdx.x / chunks, ho = p / Wo, wo = p - ho * Wo;
-    __nv_bfloat16 *dst = out + ((size_t)(b * Ho + ho0) * Wo + p) * ldk + ch * 8;
+    __nv_bfloat16 *dst = out + (((size_t)b * Ho + ho0) * Wo + p) * ldk + ch * 8;
     for (; p < n_pix; p += step, dst += (size_t)step * ldk) {
         const int base = ho * d.stride_h * row_el + wo * d.stride_w * Cin;
         uint32_t v[4];

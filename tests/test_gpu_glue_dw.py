@@ -94,6 +94,21 @@ def test_im2col_then_gemm_is_the_small_channel_conv(case):
     assert np.all(host_bf16_bits(Xcol)[:, K:] == 0)
 
 
+def test_patch_matrix_of_more_than_2_to_the_31_rows():
+    """Small images, many of them: the rows of the patch matrix are counted in 64 bits (39 GB)."""
+    if torch.cuda.mem_get_info()[0] < 50e9:
+        pytest.skip("needs 50 GB of device memory")
+    B, H = 2 ** 23 + 1, 256
+    d = twn.conv_desc(B, H, 1, 1, 8, 1, 1, 0)
+    X = torch.randint(1, 2 ** 14, (B * H,), dtype=torch.int16, device="cuda", generator=torch.Generator(device="cuda").manual_seed(7))
+    Xcol = torch.full((B * H, 8), -1, dtype=torch.int16, device="cuda")
+    twn.im2col(d, X.view(torch.bfloat16), Xcol.view(torch.bfloat16), 8)
+    for i in range(0, B * H, 2 ** 28):
+        assert torch.equal(Xcol[i:i + 2 ** 28, 0], X[i:i + 2 ** 28]) and not bool(Xcol[i:i + 2 ** 28, 1:].any())
+    del X, Xcol
+    torch.cuda.empty_cache()
+
+
 FOLD_CASES = [
     # B, H, W, Cin, Cout, k, pad  (stride 2)
     (2, 30, 30, 3, 32, 7, 3),      # the ResNet stem shape in small
