@@ -62,6 +62,7 @@ im2col_kernel(const __nv_bfloat16 *__restrict__ X, twn_conv_desc_t d, I Ho, I Wo
 // (With one block per 64 pixels of a row and a warp per patch row, 28x28x1 at batch 100 left 28 of 32 lanes idle: 11.7 us.)
 constexpr int kTileMaxElems = 24 * 1024;   // window elements (48 KB)
 constexpr int kTileMaxCols = 1024;         // ldk
+static_assert(kTileMaxCols / 8 <= kT, "a thread has one column chunk");
 
 __global__ void __launch_bounds__(kT)
 im2col_tile_kernel(const __nv_bfloat16 *__restrict__ X, twn_conv_desc_t d, int Ho, int Wo, int rows, int row_groups,
@@ -96,22 +97,6 @@ im2col_tile_kernel(const __nv_bfloat16 *__restrict__ X, twn_conv_desc_t d, int H
     }
     __syncthreads();
     const int chunks = ldk >> 3, lanes = kT / chunks * chunks;      // threads that work: whole pixels' worth
-    if (chunks > kT) {
-        // wider than the block: the chunks go round
-        const int n = min(rows, Ho - ho0) * Wo * chunks;
-        for (int i = threadIdx.x; i < n; i += kT) {
-            const int p = i / chunks, ch = i - p * chunks, ho = p / Wo, wo = p - ho * Wo;
-            const int base = ho * d.stride_h * row_el + wo * d.stride_w * Cin;
-            uint32_t v[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const int o0 = tab[ch * 8 + 2 * e], o1 = tab[ch * 8 + 2 * e + 1];
-                v[e] = (uint32_t)win[o0 < 0 ? zero_at : base + o0] | ((uint32_t)win[o1 < 0 ? zero_at : base + o1] << 16);
-            }
-            *reinterpret_cast<uint4 *>(out + (((size_t)b * Ho + ho0) * Wo + p) * ldk + ch * 8) = make_uint4(v[0], v[1], v[2], v[3]);
-        }
-        return;
-    }
     if (threadIdx.x >= lanes) return;
     const int ch = threadIdx.x % chunks, step = lanes / chunks;     // this thread's chunk; pixels between its items
     int o[8];
