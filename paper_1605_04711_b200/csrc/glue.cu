@@ -56,7 +56,8 @@ im2col_kernel(const __nv_bfloat16 *__restrict__ X, twn_conv_desc_t d, I Ho, I Wo
 }
 
 // Tile variant (small Cin, where the kernel above is bound by its index arithmetic and its 2-byte loads): a block
-// takes several whole output rows of an image.  The input rows they read are copied to shared memory with zeros outside
+// takes several whole output rows of an image, or `cols` pixels of one row where the input rows of a whole one do not
+// fit in its shared memory.  The input rows they read are copied to shared memory with zeros outside
 // the image and the shared-memory offset of every patch column is tabulated; a thread then keeps one 16-byte column chunk
 // and steps over the pixels, so it holds its eight offsets in registers and consecutive threads store consecutive chunks.
 // (With one block per 64 pixels of a row and a warp per patch row, 28x28x1 at batch 100 left 28 of 32 lanes idle: 11.7 us.)
@@ -64,21 +65,23 @@ constexpr int kTileMaxElems = 24 * 1024;   // window elements (48 KB)
 constexpr int kTileMaxCols = 1024;         // ldk
 static_assert(kTileMaxCols / 8 <= kT, "a thread has one column chunk");
 
+template <bool PIECES>      // of rows; false: cols = Wo, pieces = 1 (told apart at run time, whole rows of 580 pixels lose 7 %)
 __global__ void __launch_bounds__(kT)
-im2col_tile_kernel(const __nv_bfloat16 *__restrict__ X, twn_conv_desc_t d, int Ho, int Wo, int rows, int row_groups,
-                   __nv_bfloat16 *__restrict__ out, int ldk)
+im2col_tile_kernel(const __nv_bfloat16 *__restrict__ X, twn_conv_desc_t d, int Ho, int Wo, int rows, int row_groups, int cols,
+                   int pieces, __nv_bfloat16 *__restrict__ out, int ldk)
 {
     pdl_begin();
     extern __shared__ __align__(16) unsigned char smem_tile[];
     const int Cin = (int)d.Cin, K = d.kh * d.kw * Cin, H = (int)d.H, W = (int)d.W;
-    const int win_w = (Wo - 1) * d.stride_w + d.kw, row_el = win_w * Cin;
+    const int win_w = ((PIECES ? cols : Wo) - 1) * d.stride_w + d.kw, row_el = win_w * Cin;
     const int win_h = (rows - 1) * d.stride_h + d.kh, zero_at = win_h * row_el;
     int *tab = reinterpret_cast<int *>(smem_tile);                               // [ldk]
     uint16_t *win = reinterpret_cast<uint16_t *>(smem_tile + (size_t)ldk * 4);   // [win_h][row_el], then a zero
-    const int b = blockIdx.x / row_groups, ho0 = (blockIdx.x - b * row_groups) * rows;
+    const int blk = PIECES ? blockIdx.x / pieces : blockIdx.x, wo0 = PIECES ? (blockIdx.x - blk * pieces) * cols : 0;
+    const int b = blk / row_groups, ho0 = (blk - b * row_groups) * rows;
     const int h0 = ho0 * d.stride_h - d.pad_h;
     const uint16_t *src = reinterpret_cast<const uint16_t *>(X) + (size_t)b * H * W * Cin;
-    const int in_el = W * Cin, lead = d.pad_w * Cin;       // elements of an input row; the window starts `lead` before it
+    const int in_el = W * Cin, lead = (d.pad_w - wo0 * d.stride_w) * Cin;       // elements of an input row; the window starts `lead` before it
     for (int r = threadIdx.x >> 5; r < win_h; r += kT / 32) {
         const int h = h0 + r;
         for (int j = threadIdx.x & 31; j < row_el; j += 32) {
@@ -102,9 +105,9 @@ im2col_tile_kernel(const __nv_bfloat16 *__restrict__ X, twn_conv_desc_t d, int H
     int o[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) o[e] = tab[ch * 8 + e];
-    const int n_pix = min(rows, Ho - ho0) * Wo;
+    const int n_pix = PIECES ? min(cols, Wo - wo0) : min(rows, Ho - ho0) * Wo;     // consecutive
     int p = threadIdx.x / chunks, ho = p / Wo, wo = p - ho * Wo;
-    __nv_bfloat16 *dst = out + (((size_t)b * Ho + ho0) * Wo + p) * ldk + ch * 8;
+    __nv_bfloat16 *dst = out + (((size_t)b * Ho + ho0) * Wo + wo0 + p) * ldk + ch * 8;
     for (; p < n_pix; p += step, dst += (size_t)step * ldk) {
         const int base = ho * d.stride_h * row_el + wo * d.stride_w * Cin;
         uint32_t v[4];
@@ -735,21 +738,30 @@ extern "C" int twn_im2col(const twn_conv_desc_t *d, const void *X, void *Xcol, i
     TWN_REQUIRE(Ho > 0 && Wo > 0, TWN_ERR_INVALID_ARG);
     const long long items = d->B * Ho * Wo * (ldk / 8);
     const bool small = items * 8 < 0x7fffffffLL && d->B * d->H * d->W * d->Cin < 0x7fffffffLL;
-    // output rows per block: about 256 pixels, fewer while that leaves SMs without a block, and what fits in shared memory
-    const long long row_el = ((Wo - 1) * d->stride_w + d->kw) * d->Cin;
-    long long rows = std::min(Ho, std::max(1ll, 256 / Wo));
-    while (rows > 1 && (d->B * ((Ho + rows - 1) / rows) < 2 * dev.sm_count || ((rows - 1) * d->stride_h + d->kh) * row_el > kTileMaxElems)) --rows;
-    const long long elems = ((rows - 1) * d->stride_h + d->kh) * row_el, groups = (Ho + rows - 1) / rows;
-    if (elems <= kTileMaxElems && ldk <= kTileMaxCols && d->B * groups < 0x7fffffffLL && d->H * d->W * d->Cin < 0x7fffffffLL) {
+    // Output rows per block: about 256 pixels, fewer while that leaves SMs without a block, and what fits in shared memory.
+    // Pieces of a row where the input rows of one output row do not fit: as many pixels as do, at most 256, so that several
+    // blocks share an SM (600x1300x3, 7x7 stride 2: 128 pixels 23.2 us, 256 23.4, 512 32.1, the kernel above 51.6; 512x2800x3,
+    // 3x3: 59.0, 47.7, 45.2 and 78.2).  Where 64 do not fit, the kernel above takes the layer.
+    const auto elems_of = [&](long long r, long long c) { return ((r - 1) * d->stride_h + d->kh) * ((c - 1) * d->stride_w + d->kw) * d->Cin; };
+    long long rows = std::min(Ho, std::max(1ll, 256 / Wo)), cols = Wo;
+    while (rows > 1 && (d->B * ((Ho + rows - 1) / rows) < 2 * dev.sm_count || elems_of(rows, Wo) > kTileMaxElems)) --rows;
+    if (elems_of(1, Wo) > kTileMaxElems) {
+        cols = 256;
+        while (cols >= 64 && elems_of(1, cols) > kTileMaxElems) cols -= 32;
+    }
+    const long long elems = elems_of(rows, cols), groups = (Ho + rows - 1) / rows, pieces = (Wo + cols - 1) / cols;
+    if (elems <= kTileMaxElems && (cols == Wo || cols >= 64) && ldk <= kTileMaxCols && d->B * groups * pieces < 0x7fffffffLL &&
+        d->H * d->W * d->Cin < 0x7fffffffLL && (d->W + 2LL * d->pad_w) * d->Cin < 0x7fffffffLL - kTileMaxElems) {
         const size_t smem = (size_t)ldk * 4 + (size_t)(elems + 1) * 2;
-        static bool attr_set[64] = {false};
-        if (!attr_set[dev.ordinal]) {
-            TWN_CUDA_OK(cudaFuncSetAttribute(im2col_tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTileMaxCols * 4 + (kTileMaxElems + 1) * 2));
-            attr_set[dev.ordinal] = true;
+        auto kernel = pieces > 1 ? im2col_tile_kernel<true> : im2col_tile_kernel<false>;
+        static bool attr_set[2][64] = {};
+        if (!attr_set[pieces > 1][dev.ordinal]) {
+            TWN_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTileMaxCols * 4 + (kTileMaxElems + 1) * 2));
+            attr_set[pieces > 1][dev.ordinal] = true;
         }
-        TWN_CUDA_OK(twn_launch_small(im2col_tile_kernel, (int)(d->B * groups), kT, smem, twn_cu(stream),
-                                     static_cast<const __nv_bfloat16 *>(X), *d, (int)Ho, (int)Wo, (int)rows, (int)groups,
-                                     static_cast<__nv_bfloat16 *>(Xcol), (int)ldk));
+        TWN_CUDA_OK(twn_launch_small(kernel, (int)(d->B * groups * pieces), kT, smem, twn_cu(stream),
+                                     static_cast<const __nv_bfloat16 *>(X), *d, (int)Ho, (int)Wo, (int)rows, (int)groups, (int)cols,
+                                     (int)pieces, static_cast<__nv_bfloat16 *>(Xcol), (int)ldk));
     } else if (small)
         im2col_kernel<int><<<blocks_for(items, dev.sm_count), kT, 0, twn_cu(stream)>>>(
             static_cast<const __nv_bfloat16 *>(X), *d, (int)Ho, (int)Wo, static_cast<__nv_bfloat16 *>(Xcol), (int)ldk);

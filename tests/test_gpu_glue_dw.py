@@ -94,6 +94,26 @@ def test_im2col_then_gemm_is_the_small_channel_conv(case):
     assert np.all(host_bf16_bits(Xcol)[:, K:] == 0)
 
 
+@pytest.mark.parametrize("case", [
+    # B, H, W, Cin, (kh, kw), stride, pad: the widest image whose rows go whole, the next one, a last piece of one pixel,
+    # a shorter piece, strides, padding beyond the image, and a filter of which 64 pixels do not fit
+    (1, 4, 2728, 3, (3, 3), 1, 1), (2, 4, 2733, 3, (3, 3), 1, 1), (1, 3, 8449, 1, (3, 3), 1, 1), (1, 11, 1173, 3, (7, 7), 2, 3),
+    (1, 2, 4001, 5, (5, 5), 1, 4), (1, 3, 9000, 4, (1, 9), 2, 0), (1, 20, 600, 8, (11, 11), 1, 5), (1, 2, 300, 40, (5, 5), 1, 2)])
+def test_patch_matrix_of_wide_images(case):
+    B, H, W, Cin, k, s, p = case
+    d = twn.conv_desc(B, H, W, Cin, 8, k, s, p)
+    K = k[0] * k[1] * Cin
+    ldk = (K + 7) // 8 * 8 + 8
+    X = dg.draw_bf16(8, f"wide{case}", B * H * W * Cin, "normal").reshape(B, H, W, Cin)
+    Xcol = torch.full((B * d.Ho * d.Wo, ldk), 7.0, dtype=torch.bfloat16, device="cuda")
+    twn.im2col(d, dev_bf16(X), Xcol, ldk)
+    Xp = np.pad(X, ((0, 0), (p, p), (p, p), (0, 0)))
+    taps = [Xp[:, r:r + (d.Ho - 1) * s + 1:s, c:c + (d.Wo - 1) * s + 1:s] for r in range(k[0]) for c in range(k[1])]
+    want = np.concatenate(taps, axis=-1).reshape(-1, K)
+    got = host_bf16_bits(Xcol).reshape(-1, ldk)
+    assert np.array_equal(got[:, :K], want) and not got[:, K:].any()
+
+
 def test_patch_matrix_of_more_than_2_to_the_31_rows():
     """Small images, many of them: the rows of the patch matrix are counted in 64 bits (39 GB)."""
     if torch.cuda.mem_get_info()[0] < 50e9:
