@@ -27,8 +27,50 @@ def _bf16(bits: np.ndarray) -> torch.Tensor:
     return torch.from_numpy(np.ascontiguousarray(bits).view(np.int16)).cuda().view(torch.bfloat16)
 
 
+class _Changes:
+    """Counts the assignments to the buffers and parameters of a network: a pass's prepared list of calls holds what they
+    were, and is made again when the count has moved.  (An object of its own, so that the dicts that report to it form no
+    cycle with the network and its memory goes when the last reference does.)"""
+    n = 0
+
+
+class _Buffers(dict):
+    """A dict that counts the changes to its entries."""
+
+    def __init__(self, entries, changes):
+        super().__init__(entries)
+        self._changes = changes
+
+    def _counted(method):
+        def call(self, *args, **kwargs):
+            self._changes.n += 1
+            return method(self, *args, **kwargs)
+        return call
+
+    __setitem__, __delitem__, __ior__ = _counted(dict.__setitem__), _counted(dict.__delitem__), _counted(dict.__ior__)
+    clear, pop, popitem = _counted(dict.clear), _counted(dict.pop), _counted(dict.popitem)
+    setdefault, update = _counted(dict.setdefault), _counted(dict.update)
+
+    def __reduce__(self):
+        return dict, (dict(self),)       # a copy, or a saved one, is a plain dict
+
+
+class _Counted:
+    """Assignments to attributes count as changes, dicts among them report theirs."""
+
+    def __setattr__(self, name, value):
+        changes = self.__dict__.get("_changes")
+        if changes is not None and name not in self._uncounted:
+            changes.n += 1
+            if type(value) is dict:
+                value = _Buffers(value, changes)
+        object.__setattr__(self, name, value)
+
+    _uncounted = frozenset(["_changes"])
+
+
 @dataclass
-class Layer:
+class Layer(_Counted):
     name: str
     Cin: int
     Cout: int
@@ -64,29 +106,38 @@ class Layer:
         return self.B * self.Ho * self.Wo * self.K * self.Cout
 
 
-class TernaryNet:
-    """A chain of ternary conv / FC layers with pooling glue, all buffers preallocated."""
+class TernaryNet(_Counted):
+    """A chain of ternary conv / FC layers with pooling glue, all buffers preallocated.  A buffer or parameter may be
+    replaced between two passes (act, aux, grad, a layer's extra, ...); the next pass uses the new one."""
+    # what a pass itself assigns, and what its list of calls does not hold
+    _uncounted = frozenset(["_changes", "_made", "_built", "_fwd", "_bwd", "_delta_ready", "_pending_join", "_dz_ready", "last_grads", "timed",
+                            "side_streams", "dw_stream"])
 
     def __init__(self, name: str, batch: int, in_shape, ops, seed: int = 0, delta_factor: float = 0.7,
                  train: bool = False, optimizer: dict | None = None):
         """optimizer: None (the step ends with the weight gradients) or dict(lr, momentum, weight_decay):
         the step then ends with the SGD update of the master weights (Algorithm 1, UpdateParameters), which
         also leaves the next iteration's thresholds behind, so that later steps run only the coding sweep."""
+        self._changes = _Changes()
         self.name, self.B, self.in_shape, self.ops = name, batch, in_shape, ops
         self.seed, self.delta_factor, self.train = seed, delta_factor, train
         self.optimizer = optimizer if train else None
         self._delta_ready = False
         self.layers: dict[str, Layer] = {op[1].name: op[1] for op in ops if op[0] == "layer"}
+        for L in self.layers.values():
+            L._changes = self._changes
+            L.extra = dict(L.extra)
         self.act: dict[str, torch.Tensor] = {}
         self.aux: dict[str, torch.Tensor] = {}
         self.grad: dict[str, torch.Tensor] = {}
+        self._made: dict[str, object] = {}       # epilogues and views as this class made them, by layer or activation
         self.status = torch.zeros(1, dtype=torch.int32, device="cuda")
         # the code re-layouts for the backward pass run on a side stream beside the forward pass
         self.side_streams = [torch.cuda.Stream()]
         self.dw_stream = torch.cuda.Stream()     # weight gradients run beside the backward-for-data chain
         self.timed = None          # when a list: (kind, name, flops, start event, end event)
-        self._fwd = None           # calls of a forward pass, made on first use
-        self._bwd = None           # order and fusions of a backward pass, made on first use
+        self._fwd = None           # (changes so far, calls of a forward pass), made on first use
+        self._bwd = None           # (changes so far, order and fusions of a backward pass), made on first use
         self._pending_join = False
         self._codes_ready = torch.cuda.Event()
         self._dz_ready: dict[str, torch.cuda.Event] = {}
@@ -130,11 +181,7 @@ class TernaryNet:
                     e["xcol"] = torch.zeros((M, L.ldk), dtype=torch.bfloat16, device="cuda")
                 out_dtype = torch.float32 if L.out_f32 else torch.bfloat16
                 self.act[L.name] = torch.zeros((B, L.Ho, L.Wo, L.Cout), dtype=out_dtype, device="cuda")
-                res = self.act[L.residual] if L.residual else None
-                e["epi"] = twn.epilogue(e["scale"], e["shift"], res, relu=L.relu,
-                                        out_dtype=twn.F32 if L.out_f32 else twn.BF16,
-                                        # the backward pass goes through the gates of these very bits
-                                        residual_op=twn.SUM_IN_ORDER if self.train else twn.RESIDUAL_ADD)
+                self._make_epilogue(L)
                 if self.optimizer:
                     if L.small_cin and not L.fold:
                         raise NotImplementedError("the update needs a weight gradient in the layout of the weights")
@@ -170,8 +217,7 @@ class TernaryNet:
                 self.act[name] = torch.zeros((Bx, 1, 1, C), dtype=torch.bfloat16, device="cuda")
             elif kind == "flatten":
                 _, name, src = op
-                a = self.act[src]
-                self.act[name] = a.view(a.shape[0], 1, 1, -1)
+                self._make_view(name, src)
         self.ws_tern = torch.empty(twn.ternarize_batch_workspace_bytes(min(len(self.layers), 32)),
                                    dtype=torch.uint8, device="cuda")
         if self.train:
@@ -179,6 +225,29 @@ class TernaryNet:
                 if name != "input" and a.dtype == torch.bfloat16:
                     self.grad[name] = torch.zeros_like(a)
             self.ws_dw = torch.empty(max(ws_dw, 16), dtype=torch.uint8, device="cuda")
+        self._built = self._changes.n
+
+    def _make_epilogue(self, L):
+        """The layer's epilogue, which holds the addresses of its affine and its residual; after the first time, the one
+        that is there gets the addresses of the tensors that are there now, unless it is the caller's own."""
+        e = L.extra
+        tensors = (e["scale"], e["shift"], self.act[L.residual] if L.residual else None)
+        made = self._made.get(L.name)
+        if made is not None and (e["epi"] is not made[0] or all(a is b for a, b in zip(tensors, made[1]))):
+            return
+        epi = twn.epilogue(*tensors, relu=L.relu, out_dtype=twn.F32 if L.out_f32 else twn.BF16,
+                           # the backward pass goes through the gates of these very bits
+                           residual_op=twn.SUM_IN_ORDER if self.train else twn.RESIDUAL_ADD)
+        if made is None:
+            e["epi"] = epi
+        else:
+            old = e["epi"]
+            old.scale, old.shift, old.residual, old.residual_dtype = epi.scale, epi.shift, epi.residual, epi.residual_dtype
+        self._made[L.name] = (e["epi"], tensors)
+
+    def _make_view(self, name, src):
+        a = self.act[src]
+        self.act[name] = self._made[name] = a.view(a.shape[0], 1, 1, -1)
 
     def set_input(self, bits: np.ndarray):
         self.act["input"].copy_(_bf16(bits).view(self.act["input"].shape))
@@ -269,8 +338,15 @@ class TernaryNet:
         return calls
 
     def forward(self):
-        if self._fwd is None or self._fwd[0] is not self.act["input"]:
-            self._fwd = (self.act["input"], self._forward_calls())
+        if self._fwd is None or self._fwd[0] != self._changes.n:
+            if self._changes.n != self._built:
+                for op in self.ops:
+                    if op[0] == "layer":
+                        self._make_epilogue(op[1])
+                    elif op[0] == "flatten" and self.act[op[1]] is self._made[op[1]]:
+                        self._make_view(op[1], op[2])
+            calls = self._forward_calls()
+            self._fwd = (self._changes.n, calls)
         for call in self._fwd[1]:
             self._call(*call)
         return self.act[self.ops[-1][1].name]
@@ -396,8 +472,9 @@ class TernaryNet:
         every layer.  An activation with two consumers (the input of a residual block) gets its
         second contribution added through the residual input of the backward-for-data epilogue."""
         assert self.train
-        if self._bwd is None or self._bwd[0] is not self.act["input"]:
-            self._bwd = (self.act["input"], *self._backward_steps())
+        if self._bwd is None or self._bwd[0] != self._changes.n:
+            steps, acc = self._backward_steps()
+            self._bwd = (self._changes.n, steps, acc)
         _, steps, acc = self._bwd
         last: Layer = self.ops[-1][1]
         dY = dlogits.view(self.act[last.name].shape)
