@@ -852,8 +852,10 @@ EpilogueArgs epilogue_args(const twn_stats_t *stats, const twn_epilogue_t *epi, 
     return ea;
 }
 
+// With `us_only`, nothing is launched: it receives what the launch that the same call would make should take.
 int launch_conv(const Geometry &g, const void *X, const uint32_t *T, const twn_stats_t *stats,
-                const twn_epilogue_t *epi, void *Y, int out_dtype_default, int32_t *dev_status, cudaStream_t s)
+                const twn_epilogue_t *epi, void *Y, int out_dtype_default, int32_t *dev_status, cudaStream_t s,
+                double *us_only = nullptr)
 {
     twn_device_info dev;
     int rc = twn_current_device(&dev);
@@ -905,13 +907,18 @@ int launch_conv(const Geometry &g, const void *X, const uint32_t *T, const twn_s
     // Narrow layers and short reductions: the kernel that decodes its channels' codes once per block.  Up to 64 channels
     // the general kernel's half-empty tiles lose wherever that kernel runs; above, its own time decides.
     bool handled = false;
-    rc = launch_conv_resident(g, X, T, ea, Y, dev_status, dev, s, half || split.us < us ? split.us : us, &handled);
+    rc = launch_conv_resident(g, X, T, ea, Y, dev_status, dev, s, half || split.us < us ? split.us : us, &handled, us_only);
     if (rc != TWN_OK || handled) return rc;
     // The more SMs the general kernel fills by itself, the clearer the gain has to be: beside the weight gradients of a
     // training step a split launch takes SMs that would not have been idle (ResNet-18 at batch 64).
     const long long tiles = choice == 0 ? t128 : choice == 1 ? t256 : t192;
     const double fill = tiles < sms ? (double)tiles / (double)sms : 1.0;
-    if (split.us < (1.0 - 0.25 * fill) * us) return launch_conv_split(g, X, T, ea, Y, dev_status, dev, s, split);
+    const bool take_split = split.us < (1.0 - 0.25 * fill) * us;
+    if (us_only) {
+        *us_only = take_split ? split.us : us;
+        return TWN_OK;
+    }
+    if (take_split) return launch_conv_split(g, X, T, ea, Y, dev_status, dev, s, split);
     P.T = T;
     P.wpr = g.ld_codes / (g.code_bits == 1 ? 32 : 16);
     P.sw = g.sw; P.sh = g.sh;
@@ -1249,15 +1256,23 @@ int conv_bwd_data_impl(const twn_conv_desc_t *d, const void *dZ, const uint32_t 
         g.Hv = cls[0].Hv; g.Wv = cls[0].Wv;
         g.n_classes = n_cls;
         for (int c = 0; c < n_cls; ++c) g.cls[c] = cls[c];
-        // The launches of the classes share the SMs, so together they take what the longest takes on its share.
-        // Narrow gradients of many pixels stay with them: the kernel of narrow layers is the faster one there (64 images
-        // of 56x56x64 <- 128: 27 us, 40 us in one launch; 20 images 21 and 18 us).
+        // Apart, the launches follow one another as far as each fills the SMs, and overlap at their ends: the sum of what the
+        // kernels that they would run should take, less 1.2 us for each after the first.  Measured both ways on 180 shapes (1 to
+        // 256 images of 7 to 112 pixels, 32 to 768 channels, 1x1 to 5x5), half of them not used in the fit, the way it takes is
+        // 1.4 % behind the better one on average; at most 23 %, where classes of a few blocks each run side by side after all.
+        // 64 images of 56x56x64 <- 128 take 30 us apart and 44 in one launch, 20 images 24 and 21, 5 of 76x76x640 <- 32 30 and 42,
+        // 8 of 31x31x512 <- 192 (5x5) 30 and 19.
         const EpilogueArgs ea = epilogue_args(stats, epi, TWN_F32);
         const SplitPlan plan = plan_conv_split(g, dev.sm_count, ea.in_order);
-        double apart = 0.0;
-        for (int c = 0; c < n_cls; ++c) apart = std::max(apart, 1.5 + plan_conv_split(one_class(cls[c], 1), dev.sm_count / n_cls, ea.in_order).us);
-        const long long pixels = (long long)all.Bv * all.OH * all.OW;
-        if (plan.pix && plan.us < apart && !(all.Cout <= 96 && pixels > 1000 * 128))
+        constexpr double kLeast = 2.9;           // no model goes below: the sum ends when the answer is known (2 us of host time)
+        double apart = kLeast * n_cls - 1.2 * (n_cls - 1);
+        for (int c = 0; c < n_cls && apart <= plan.us; ++c) {
+            double us = 0.0;
+            rc = launch_conv(one_class(cls[c], n_cls), dZ, T_bwd, stats, epi, dX, TWN_F32, dev_status, user, &us);
+            if (rc != TWN_OK) return rc;
+            apart += us - kLeast;
+        }
+        if (plan.pix && plan.us < apart)
             return launch_conv_split(g, dZ, T_bwd, ea, dX, dev_status, dev, user, plan);
     }
     // A launch per class, side by side on helper streams.

@@ -101,9 +101,11 @@ struct EpilogueArgs {
 // and returns TWN_OK with *handled = true when the launch fits that kernel (unit input stride, decoded
 // weights of 64 output channels that fit in shared memory, outputs that TMA can store; not several taps
 // of several channel blocks whose sums must stay in order) and should not take longer than `rival_us`;
-// otherwise *handled = false and nothing has been launched.
+// otherwise *handled = false and nothing has been launched.  With `us_only` nothing is launched in either
+// case: *handled says whether it would be, *us_only then what it should take.
 int launch_conv_resident(const Geometry &g, const void *X, const uint32_t *T, const EpilogueArgs &epi, void *Y,
-                         int32_t *dev_status, const twn_device_info &dev, cudaStream_t s, double rival_us, bool *handled);
+                         int32_t *dev_status, const twn_device_info &dev, cudaStream_t s, double rival_us, bool *handled,
+                         double *us_only);
 
 // Contraction for problems that do not fill the GPU (tconv_split.cu): tiles of 128 channels x `pix` pixels (32, 64, 128
 // or 256), the reduction of each split over a cluster of `splits` blocks (1, 2, 4 or 8; 256 pixels: 1 or 2).  Takes every

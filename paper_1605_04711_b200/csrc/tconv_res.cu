@@ -525,7 +525,7 @@ tconv_res_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
 
 int twn_detail::launch_conv_resident(const Geometry &g, const void *X, const uint32_t *T, const EpilogueArgs &epi,
                                      void *Y, int32_t *dev_status, const twn_device_info &dev, cudaStream_t s,
-                                     double rival_us, bool *handled)
+                                     double rival_us, bool *handled, double *us_only)
 {
     *handled = false;
     if (g.sw != 1 || g.sh != 1 || g.Cout < 1) return TWN_OK;
@@ -624,6 +624,11 @@ int twn_detail::launch_conv_resident(const Geometry &g, const void *X, const uin
     int n_stages = P.kbpt > 0 ? (int)((kSmemLimit - fixed) / P.stage_bytes) : 0;
     if (n_stages > kMaxStages) n_stages = kMaxStages;
     if (P.kbpt > 0 && n_stages < 2) return TWN_OK;
+    if (us_only) {
+        *us_only = us;
+        *handled = true;
+        return TWN_OK;
+    }
     P.n_stages = n_stages;
     P.wts_off = (uint32_t)(n_stages * P.stage_bytes);
     P.stg_off = P.wts_off + (uint32_t)wts_bytes;
