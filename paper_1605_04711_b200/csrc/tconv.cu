@@ -909,8 +909,11 @@ int launch_conv(const Geometry &g, const void *X, const uint32_t *T, const twn_s
     bool handled = false;
     rc = launch_conv_resident(g, X, T, ea, Y, dev_status, dev, s, half || split.us < us ? split.us : us, &handled, us_only);
     if (rc != TWN_OK || handled) return rc;
-    // The more SMs the general kernel fills by itself, the clearer the gain has to be: beside the weight gradients of a
-    // training step a split launch takes SMs that would not have been idle (ResNet-18 at batch 64).
+    // The more SMs the general kernel fills by itself, the clearer the modelled gain has to be: near the line the split
+    // kernel's model is the optimistic one.  Of 81 drawn calls that this margin alone keeps here, timed alone, 44 are more than
+    // 3 % slower split and 18 faster: convolutions lose 9 % on average, inner products to fp32 gain 3 % (4001x4608x512 25.9 us
+    // split, 25.3 here).  Without it a forward pass of ResNet-18 at 64 images takes 438 us instead of 415, of VGG-7 at 128
+    // 203 instead of 198, a training step of ResNet-18 at 64, with the weight gradients beside it, 1306 instead of 1270.
     const long long tiles = choice == 0 ? t128 : choice == 1 ? t256 : t192;
     const double fill = tiles < sms ? (double)tiles / (double)sms : 1.0;
     const bool take_split = split.us < (1.0 - 0.25 * fill) * us;
