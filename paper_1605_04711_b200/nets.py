@@ -7,6 +7,13 @@ layer, forward through the ternary weights, backward for data through the same c
 straight-through weight gradients for the fp32 master weights).
 
 Activations and gradients are NHWC bf16; logits and weight gradients are fp32.
+
+Sums of a training step's forward pass are taken in order (twn.SUM_IN_ORDER): the backward pass goes through the ReLU gates
+of these very bits, and an image has them in every batch.  Inference and the backward-for-data calls let the library split
+the sums as the batch suggests.  That moves the weight gradients of a small batch, by up to 6e-3 of their norm, but not away
+from the truth: against a 64-bit backward pass over the same activations their error (root mean square over the layers of
+both ResNet-18s, 1, 4 and 16 images) is 2.7e-3 to 4.3e-3 either way, within 5 % of each other and larger on neither side; it
+is the rounding of each data gradient to bf16.
 """
 from __future__ import annotations
 
@@ -269,7 +276,7 @@ class TernaryNet(_Counted):
     # ------------------------------------------------------------------ Algorithm 1, first loop
     def ternarize_all(self, join: bool = True):
         """Algorithm 1, first loop: every layer's threshold, codes and scale, all layers in one
-        batched call (two launches per 32 layers) on the current stream.  The re-layouts of the codes
+        batched call (one launch per 32 layers) on the current stream.  The re-layouts of the codes
         for the backward pass follow as one batched launch on a side stream, beside the forward pass;
         the backward pass waits for its event."""
         layers = list(self.layers.values())

@@ -252,7 +252,10 @@ SUM_IN_ORDER = 2          # or-ed into residual_op
 
 
 def epilogue(scale=None, shift=None, residual=None, relu=False, out_dtype=F32, residual_op=RESIDUAL_ADD):
-    """Builds a twn_epilogue_t; keeps no reference, the caller keeps the tensors alive."""
+    """Builds a twn_epilogue_t; keeps no reference, the caller keeps the tensors alive.
+
+    The sums of a contraction may be split over blocks as its sizes suggest, so an image's outputs can be rounded
+    differently in batches of different size; SUM_IN_ORDER in residual_op makes them the same bits in every batch."""
     e = Epilogue(_ptr(scale).value, _ptr(shift).value, _ptr(residual).value,
                  BF16 if (residual is not None and residual.dtype == torch.bfloat16) else F32,
                  int(bool(relu)), out_dtype, residual_op)
