@@ -951,7 +951,7 @@ class NetWorkload:
         out = {"bound": "tensor", "kernel": "tconv_kernel + tconv_res_kernel + tconv_split_kernel (every forward and backward-for-data call of a step, each timed alone)",
                "achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak,
                "peak_source": peaks["source"] + " (bf16 burst: isolated kernels)", "traffic": self.measured_traffic(),
-               "launches": t[3], "us_in_kernel_isolated": round(t[0], 1), "us_at_bound": round(t[2], 1),
+               "calls": t[3], "us_in_kernel_isolated": round(t[0], 1), "us_at_bound": round(t[2], 1),
                "frac_of_own_bounds": (t[2] / t[0]) if t[0] > 0 else None,
                "isolated_sums_us": {kk: round(v[0], 1) for kk, v in sums.items()},
                "isolated_tflops": {kk: round(v[1] / v[0] / 1e6, 1) for kk, v in sums.items() if v[0] > 0},
@@ -970,7 +970,7 @@ class NetWorkload:
 
     def measured_traffic(self):
         """DRAM bytes per step of the ternary contractions of the ResNet-18 step: sum over the launches of
-        dram__bytes_read.sum + dram__bytes_write.sum over the 50 forward and backward-for-data launches of one step,
+        dram__bytes_read.sum + dram__bytes_write.sum over the 44 launches of the 41 forward and backward-for-data calls of one step,
         from one ncu capture of this workload at its full size (profiles/tconv_resnet18_step_dram.md); None for the
         other workloads."""
         return TRAFFIC_RESNET18_STEP if self.kind in ("resnet18_train", "resnet18_train_sgd") else None
@@ -1052,7 +1052,7 @@ class NetWorkload:
                              f"scaled to batch {B} ({spent:.1f} s of CPU; oracle step time {total_s:.1f} s)"), oracle.num_threads()
 
 # From the ncu capture summarised in profiles/tconv_resnet18_step_dram.md (see NetWorkload.measured_traffic).
-TRAFFIC_RESNET18_STEP = 873.2e6
+TRAFFIC_RESNET18_STEP = 843.7e6
 
 WORKLOADS = {"ternarize": lambda: TernarizeWorkload(), "binarize": lambda: BinarizeWorkload(), "sgd_ternarize": lambda: SgdTernarizeWorkload(), "ternarize_rows": lambda: TernarizeRowsWorkload(), "resnet18_train": lambda: NetWorkload("resnet18_train"),
              "gemm_16384": lambda: GemmWorkload(16384), "gemm_4096": lambda: GemmWorkload(4096),
