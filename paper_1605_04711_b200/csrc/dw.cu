@@ -90,10 +90,6 @@ __device__ __forceinline__ void dw_mma(uint32_t d_tmem, uint64_t a_desc, uint64_
         ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(acc)
         : "memory");
 }
-__device__ __forceinline__ void dw_commit(void *bar)
-{
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
 
 __global__ void __launch_bounds__(kDwThreads, 1)
 dw_kernel(const __grid_constant__ CUtensorMap map_dz, const __grid_constant__ CUtensorMap map_x,
@@ -214,7 +210,7 @@ dw_kernel(const __grid_constant__ CUtensorMap map_dz, const __grid_constant__ CU
         // idles unless another thread has work queued.  The threads take alternate k-blocks and the epilogue
         // adds the two accumulators; the ring has an even number of stages, so a stage always belongs to the
         // same thread and each full barrier has one waiter that sees every phase in turn.
-        if (lane == 0) {
+        if (elect_one()) {
             const uint32_t me = warp == 1 ? 0u : 1u;
             uint32_t it = 0, lu = 0;     // lu counts the units that accumulate something
             bool ok = true;
@@ -260,11 +256,11 @@ dw_kernel(const __grid_constant__ CUtensorMap map_dz, const __grid_constant__ CU
                             dw_mma(d_tmem, adesc0 + so + 896, bd[7] + so, idesc, 1u);
                         }
                         acc = 1u;
-                        dw_commit(&sm->empty[s]);
+                        tc_commit(&sm->empty[s]);
                     }
                     if (++s == (uint32_t)P.stages) { s = 0; ph ^= 1u; }
                 }
-                if (ok) dw_commit(&sm->acc_full);
+                if (ok) tc_commit(&sm->acc_full);
                 ++lu;
             }
         }

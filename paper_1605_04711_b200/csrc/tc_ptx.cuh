@@ -122,41 +122,48 @@ __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence:
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
 
-// The MMA warp runs its loops converged; tcgen05.mma and tcgen05.commit are issued by the
-// lane that elect.sync picks, with the predicate applied inside the asm block (measured to be
-// the cheapest way to issue: no divergent region around the instruction).
-// D[tmem] (+)= A[tmem] * B[smem]^T, bf16 x bf16 -> fp32.
+// True in one lane of a converged warp, the same one every time: how a role of one thread (copies, MMAs) picks it.  With
+// elect.sync the compiler knows that one thread runs the branch and keeps descriptors and addresses in uniform registers;
+// behind `lane == 0` it does not, and every tcgen05.mma is set up lane by lane (see tc_mma_ts).
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t r;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r));
+    return r != 0;
+}
+
+// D[tmem] (+)= A[tmem] * B[smem]^T, bf16 x bf16 -> fp32, issued by one elected thread.  The tensor core accepts an
+// instruction when the one before it is nearly done, so whatever the thread executes between two of them is time the
+// tensor core may idle.  4001 x 4608 x 512 (128 x 128 tiles, 256 cycles of MMA a k-block): 377 cycles a k-block when a
+// converged warp elected a lane for every MMA and waited by votes, 320 with one elected thread (260 with no decoding and
+// no activation loads beside it), above 400 with a thread picked by its lane number.  The accumulate flag is a compile-time
+// constant, and a descriptor advances by a 32-bit addition to its lower word (the start address field does not overflow).
 template <bool ACC>
-__device__ __forceinline__ void tc_mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc)
+__device__ __forceinline__ void tc_mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t b_hi, uint32_t idesc)
 {
     asm volatile(
-        "{\n\t.reg .pred p, pe;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "elect.sync _|pe, 0xffffffff;\n\t"
-        "@pe tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "n"(ACC ? 1 : 0)
+        "{\n\t.reg .pred p;\n\t.reg .b64 db;\n\t"
+        "setp.ne.b32 p, %5, 0;\n\t"
+        "mov.b64 db, {%2, %3};\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %4, p;\n\t}"
+        ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(b_hi), "r"(idesc), "n"(ACC ? 1 : 0)
         : "memory");
 }
 
+// The calling thread's MMAs so far: the barrier gets one arrival when they are done.
 __device__ __forceinline__ void tc_commit(void *bar)
 {
-    asm volatile(
-        "{\n\t.reg .pred pe;\n\t"
-        "elect.sync _|pe, 0xffffffff;\n\t"
-        "@pe tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}"
-        ::"r"(smem_u32(bar)) : "memory");
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
-// One k-block: four K=16 MMAs.  FIRST clears the accumulator with the first of them.  The
-// accumulate flag is a compile-time constant so that no predicate has to be built at run time:
-// whatever the issuing thread executes between two MMAs is time the tensor core may sit idle.
+// One k-block: four K=16 MMAs.  FIRST clears the accumulator with the first of them.
 template <bool FIRST>
-__device__ __forceinline__ void tc_mma_block(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc)
+__device__ __forceinline__ void tc_mma_block(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t b_hi, uint32_t idesc)
 {
-    tc_mma_ts<!FIRST>(d_tmem, a_tmem, b_desc, idesc);
-    tc_mma_ts<true>(d_tmem, a_tmem + 8, b_desc + 2, idesc);
-    tc_mma_ts<true>(d_tmem, a_tmem + 16, b_desc + 4, idesc);
-    tc_mma_ts<true>(d_tmem, a_tmem + 24, b_desc + 6, idesc);
+    tc_mma_ts<!FIRST>(d_tmem, a_tmem, b_lo, b_hi, idesc);
+    tc_mma_ts<true>(d_tmem, a_tmem + 8, b_lo + 2, b_hi, idesc);
+    tc_mma_ts<true>(d_tmem, a_tmem + 16, b_lo + 4, b_hi, idesc);
+    tc_mma_ts<true>(d_tmem, a_tmem + 24, b_lo + 6, b_hi, idesc);
 }
 
 // Read-only global loads that the compiler neither moves nor wraps in control flow.
@@ -342,21 +349,6 @@ __device__ __forceinline__ void decode_kblock(const uint32_t (&wv)[4], uint32_t 
 }
 // what a decoded +1 is worth: taken out again with the scale of the epilogue
 template <int BITS> __host__ __device__ constexpr float decoded_unit() { return BITS == 2 ? kDecodedUnit : 1.0f; }
-
-// ---------------------------------------------------------------- the kernel
-
-// D[tmem] (+)= A[smem] * B[smem]^T, both operands through shared-memory descriptors.
-template <bool ACC>
-__device__ __forceinline__ void tc_mma_ss(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc)
-{
-    asm volatile(
-        "{\n\t.reg .pred p, pe;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "elect.sync _|pe, 0xffffffff;\n\t"
-        "@pe tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "n"(ACC ? 1 : 0)
-        : "memory");
-}
 
 // MN-major, 128-byte swizzled operand: the MN index runs along 128-byte rows (64 bf16), eight
 // K rows form a 1024-byte group, `mn_block_bytes` separates consecutive 64-element MN blocks.

@@ -214,7 +214,7 @@ tconv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ 
 
     if (warp == 0) {
         // ------------------------------------------------ TMA producer
-        if (lane == 0) {
+        if (elect_one()) {
             uint32_t it = 0;
             bool ok = true;
             const uint32_t block_bytes = kXBytes;
@@ -242,36 +242,38 @@ tconv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ 
             }
         }
     } else if (warp == 1) {
-        // ------------------------------------------------ MMA issuer (whole warp, converged)
+        // ------------------------------------------------ MMA issuer: one thread (see tc_mma_ts)
         // One wait and one commit per stage, constant accumulate flags.  With no taps at all
         // (kbpt == 0) nothing is accumulated and the epilogue does not wait.
-        if (kbpt > 0) {
+        if (kbpt > 0 && elect_one()) {
             constexpr uint32_t idesc = make_idesc(kChan, PIX);
             const uint64_t bdesc0 = smem_desc_sw128(smem_u32(sm->x[0][0]));
+            const uint32_t b_lo0 = (uint32_t)bdesc0, b_hi = (uint32_t)(bdesc0 >> 32);
             uint32_t it = 0, lt = 0;
             bool ok = true;
             for (int tile = blockIdx.x; tile < P.total_tiles && ok; tile += gridDim.x, ++lt) {
                 const int buf = lt % kAccBufs;
                 const uint32_t aph = (lt / kAccBufs) & 1u;
-                if (!mbar_wait_warp(&sm->acc_empty[buf], aph ^ 1u, abort_flag, P.status, 0)) break;
+                if (!mbar_wait(&sm->acc_empty[buf], aph ^ 1u, abort_flag, P.status, 0)) break;
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_acc + buf * PIX;
                 for (int st = 0; st < spt; ++st, ++it) {
                     const int s = it % kStages;
                     const uint32_t ph = (it / kStages) & 1u;
-                    if (!mbar_wait_warp(&sm->full[s], ph, abort_flag, P.status, 0)) { ok = false; break; }
+                    if (!mbar_wait(&sm->full[s], ph, abort_flag, P.status, 0)) { ok = false; break; }
                     tc_fence_after();
-                    const uint64_t bdesc = bdesc0 + (uint64_t)(s * ((kSub * kXBytes) >> 4));
+                    const uint32_t b_lo = b_lo0 + (uint32_t)(s * ((kSub * kXBytes) >> 4));
                     const uint32_t a_tmem = tmem_a + s * kAColsPerStage;
-                    if (st == 0) tc_mma_block<true>(d_tmem, a_tmem, bdesc, idesc);
-                    else tc_mma_block<false>(d_tmem, a_tmem, bdesc, idesc);
+                    if (st == 0) tc_mma_block<true>(d_tmem, a_tmem, b_lo, b_hi, idesc);
+                    else tc_mma_block<false>(d_tmem, a_tmem, b_lo, b_hi, idesc);
                     if (kSub > 1 && kbpt - st * kSub > 1)
-                        tc_mma_block<false>(d_tmem, a_tmem + kAColsPerBlock, bdesc + (kXBytes >> 4), idesc);
+                        tc_mma_block<false>(d_tmem, a_tmem + kAColsPerBlock, b_lo + (kXBytes >> 4), b_hi, idesc);
                     tc_commit(&sm->empty[s]);
                 }
                 if (ok) tc_commit(&sm->acc_full[buf]);
             }
         }
+        __syncwarp();
     } else if (warp < kFirstEpiWarp) {
         // ------------------------------------------------ decode: codes -> bf16 -> tensor memory
         // Two groups of four warps; a group handles every other stage.  Each thread owns one

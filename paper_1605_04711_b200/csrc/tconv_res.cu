@@ -142,11 +142,6 @@ __device__ __forceinline__ void tc_mma_tap(uint32_t d_tmem, uint32_t a_lo, uint3
     tc_mma_ss_1t<true>(d_tmem, a_lo + 4, a_hi, b_lo + 4, b_hi, idesc);
     tc_mma_ss_1t<true>(d_tmem, a_lo + 6, a_hi, b_lo + 6, b_hi, idesc);
 }
-__device__ __forceinline__ void tc_commit_1t(void *bar)
-{
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-
 __device__ __forceinline__ void st_shared_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
 {
     asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
@@ -262,7 +257,7 @@ tconv_res_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
 
     if (warp == 0) {
         // ------------------------------------------------ TMA producer
-        if (lane == 0 && P.kbpt > 0) {
+        if (P.kbpt > 0 && elect_one()) {
             uint32_t s = 0, ph = 0;
             bool ok = true;
             for (int tile = bid; tile < P.total_tiles && ok; tile += nb) {
@@ -294,7 +289,7 @@ tconv_res_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
         // its neighbours: a thread may wait for "stage s, parity p" only once every earlier phase of that
         // barrier is known to be over.  So the threads pass a token: after seeing the last stage of its tile
         // land, a thread lets the next one start waiting for the stages of the next tile.
-        if (lane == 0 && P.kbpt > 0) {
+        if (P.kbpt > 0 && elect_one()) {
             const uint32_t me = warp == 1 ? 0u : (uint32_t)(warp - kIssuerB + 1);
             const uint32_t idesc = make_idesc(kPix, P.N);
             const uint64_t adesc0 = smem_desc_k_sw128(base_u32, P.a_sbo);
@@ -337,11 +332,11 @@ tconv_res_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
                         nxt = ctl->tap[t + 1];
                         tc_mma_tap<false>(d_tmem, a_s + cur.x, a_hi, b_s + cur.y, b_hi, idesc);
                     }
-                    tc_commit_1t(&ctl->empty[s]);
+                    tc_commit(&ctl->empty[s]);
                     if (++s == (uint32_t)P.n_stages) { s = 0; ph ^= 1u; }
                 }
                 if (ok) {
-                    tc_commit_1t(&ctl->acc_full[buf]);
+                    tc_commit(&ctl->acc_full[buf]);
                     for (int i = 1; i < kIssuers; ++i) skip_tile();
                 }
             }

@@ -243,7 +243,7 @@ tconv_split_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
     const uint32_t tmem = sm->tmem_base, tmem_a = tmem + PIX;
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (elect_one()) {
             int t = k0 / P.n_cblk, cb = k0 - t * P.n_cblk;
             for (int i = 0; i < n_kb; ++i) {
                 const int s = i % kStages;
@@ -256,19 +256,23 @@ tconv_split_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
         }
         __syncwarp();
     } else if (warp == 1) {
-        constexpr uint32_t idesc = make_idesc(kChan, PIX);
-        const uint64_t bdesc0 = smem_desc_sw128(smem_u32(sm->x[0]));
-        bool ok = true;
-        for (int i = 0; i < n_kb; ++i) {
-            const int s = i % kStages;
-            if (!mbar_wait_warp(&sm->full[s], (i / kStages) & 1, abort_flag, P.status, 0)) { ok = false; break; }
-            tc_fence_after();
-            const uint64_t bdesc = bdesc0 + (uint64_t)(s * (L::kXBytes >> 4));
-            if (i == 0) tc_mma_block<true>(tmem, tmem_a + s * kAColsPerBlock, bdesc, idesc);
-            else tc_mma_block<false>(tmem, tmem_a + s * kAColsPerBlock, bdesc, idesc);
-            tc_commit(&sm->empty[s]);
+        if (elect_one()) {                               // see tc_mma_ts
+            constexpr uint32_t idesc = make_idesc(kChan, PIX);
+            const uint64_t bdesc0 = smem_desc_sw128(smem_u32(sm->x[0]));
+            const uint32_t b_lo0 = (uint32_t)bdesc0, b_hi = (uint32_t)(bdesc0 >> 32);
+            bool ok = true;
+            for (int i = 0; i < n_kb; ++i) {
+                const int s = i % kStages;
+                if (!mbar_wait(&sm->full[s], (i / kStages) & 1, abort_flag, P.status, 0)) { ok = false; break; }
+                tc_fence_after();
+                const uint32_t b_lo = b_lo0 + (uint32_t)(s * (L::kXBytes >> 4));
+                if (i == 0) tc_mma_block<true>(tmem, tmem_a + s * kAColsPerBlock, b_lo, b_hi, idesc);
+                else tc_mma_block<false>(tmem, tmem_a + s * kAColsPerBlock, b_lo, b_hi, idesc);
+                tc_commit(&sm->empty[s]);
+            }
+            if (ok && n_kb > 0) tc_commit(&sm->acc_full);
         }
-        if (ok && n_kb > 0) tc_commit(&sm->acc_full);
+        __syncwarp();
     } else {
         const int q = warp & 3, set = (warp - 2) >> 2;
         const uint32_t lane_base = ((uint32_t)(q * 32) << 16);
