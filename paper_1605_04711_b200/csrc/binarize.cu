@@ -291,7 +291,7 @@ extern "C" int twn_binarize(const float *W, int64_t rows, int64_t cols, twn_stat
         while (grid < P.parts) grid *= 2;
         return launch_cluster(binarize_kernel<true>, grid, twn_cu(stream), P);
     }
-    return launch_cooperative(binarize_kernel<false>, std::min(P.parts, (unsigned int)(dev.sm_count * kSweepBlocksPerSm)), twn_cu(stream), P);
+    return launch_cooperative(binarize_kernel<false>, std::min(P.parts, (unsigned int)(dev.sm_count * kSweepBlocksPerSm)), twn_cu(stream), 0, P);
 }
 
 extern "C" int twn_unpack_b1(const uint32_t *packed, int64_t rows, int64_t cols, int64_t ld_codes, int8_t *codes,

@@ -106,7 +106,7 @@ int launch_cluster(K kernel, unsigned int grid, cudaStream_t s, const A &...args
 }
 // A grid whose blocks all run at once and may wait for one another.
 template <typename K, typename... A>
-int launch_cooperative(K kernel, unsigned int grid, cudaStream_t s, const A &...args)
+int launch_cooperative(K kernel, unsigned int grid, cudaStream_t s, size_t smem, const A &...args)
 {
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;
@@ -115,6 +115,7 @@ int launch_cooperative(K kernel, unsigned int grid, cudaStream_t s, const A &...
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(kSweepThreads);
     cfg.stream = s;
+    cfg.dynamicSmemBytes = smem;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     TWN_CUDA_OK(cudaLaunchKernelEx(&cfg, kernel, args...));

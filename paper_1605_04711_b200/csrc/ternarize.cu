@@ -6,6 +6,7 @@
 //   phase 1  S = sum |W_i| in fp64  ->  delta = factor * S / n
 //   phase 2  codes by Eq. 3, packed 16 per word; sum and count of the kept set
 //            ->  alpha (Eq. 5)
+// (tensors much larger than L2 in one phase against an estimate, with corrections: ternarize_once_kernel)
 // with a barrier of all blocks between them (grid-wide in a cooperative launch, a cluster's for small tensors).
 // Phase 2 walks every block's share back to front, so that what phase 1 read last comes from L1 and L2.
 //
@@ -81,6 +82,7 @@ struct Item {
     bool small;
     bool vec4;                       // every word starts on a 16-byte boundary
     bool dense;                      // word w of the packed matrix holds weights 16 w ..
+    bool linear;                     // word w of those that hold codes does: no row ends inside a word
 };
 
 template <int N>
@@ -445,6 +447,29 @@ __device__ __forceinline__ double fold_parts(const double *p, unsigned int parts
     return sweep_sum(s, red, turn);
 }
 
+// The last block's part: the second sums of a tensor's parts, in a fixed order.
+__device__ __forceinline__ void fold_kept(const Item &it, const Workspace &ws, Reduce &red, unsigned long long (&cnt)[2][kSweepWarps], unsigned int &turn)
+{
+    double s = 0.0;
+    unsigned long long pos = 0, neg = 0;
+    for (unsigned int i = threadIdx.x; i < it.parts; i += kSweepThreads) {
+        s += __ldcg(ws.part_kept + i);
+        const unsigned long long c = __ldcg(ws.part_cnt + i);
+        pos += c & 0xFFFFFFFFull;
+        neg += c >> 32;
+    }
+    const double kept = sweep_sum(s, red, turn);
+    pos = warp_sum(pos);
+    neg = warp_sum(neg);
+    if ((threadIdx.x & 31) == 0) { cnt[0][threadIdx.x >> 5] = pos; cnt[1][threadIdx.x >> 5] = neg; }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        pos = neg = 0;
+        for (int w = 0; w < kSweepWarps; ++w) { pos += cnt[0][w]; neg += cnt[1][w]; }
+        write_kept(it, kept, pos, neg);
+    }
+}
+
 // The warps' sums of up to kRun parts of a block.  Nothing joins the warps between the parts, so a warp's loads of its
 // next part are not held up by a slower warp's reduction: with a block-wide sum per part, 1400 parts of the 21 tensors of
 // ResNet-18 took 50 us.
@@ -565,26 +590,343 @@ ternarize_kernel(const __grid_constant__ Launch<N> P, void *ws_raw)
         const int ti = __ffs(mask) - 1;
         const Item &it = P.item[ti];
         const Workspace ws = carve(ws_raw, ti);
-        double s = 0.0;
-        unsigned long long pos = 0, neg = 0;
-        for (unsigned int i = tid; i < it.parts; i += kSweepThreads) {
-            s += __ldcg(ws.part_kept + i);
-            const unsigned long long c = __ldcg(ws.part_cnt + i);
-            pos += c & 0xFFFFFFFFull;
-            neg += c >> 32;
-        }
-        const double kept = sweep_sum(s, red, turn);
-        pos = warp_sum(pos);
-        neg = warp_sum(neg);
-        if ((tid & 31) == 0) { red_cnt64[0][tid >> 5] = pos; red_cnt64[1][tid >> 5] = neg; }
-        __syncthreads();
-        if (tid == 0) {
-            pos = neg = 0;
-            for (int w = 0; w < kSweepWarps; ++w) { pos += red_cnt64[0][w]; neg += red_cnt64[1][w]; }
-            write_kept(it, kept, pos, neg);
-        }
+        fold_kept(it, ws, red, red_cnt64, turn);
         __syncthreads();
     }
+}
+
+// ---- large tensors: one read ------------------------------------------------------
+// A tensor that does not stay in L2 would cross HBM twice, because the threshold needs every weight before the first code.
+// Here it crosses once: a sample (16 runs of 512 weights from every part) gives an estimate `mid` of the threshold and how far
+// off it may be, the one sweep adds up |W|, codes against `mid` and marks the half-words with a weight within `half` of it; when
+// the threshold is known, the weights of marked half-words that lie between it and `mid` get their other code, and sums and
+// counts are put right.  Of normal weights 1.4 % of the half-words are marked; most are kept in shared memory, the others read
+// again.  A threshold further than `half` from the estimate (an order of weights that the sample does not see, a NaN) costs a
+// second sweep.  The codes and counts are the same in any case; the kept sum is that of the sweep plus the corrections, in a
+// fixed order.
+// The sweep costs nearly as many issue slots as memory time, so a thread takes whole words (no exchange among lanes), their
+// kept bits are collected by the fp32 adders (as sums of powers of two) and their signs two at a time.
+//   12288 x 8192 (three tensors in turn) 137.7 -> 88.3 us, 66 at the copy rate.
+// Where one read pays: 9.2 million weights in rows of 2301, cold, 28.9 us so, 27.0 in two sweeps; 14.2 million 24.9 / 26.7; 18.9 million 28.9 / 33.0
+// (27.3 / 26.9 where they are in L2 from the call before); 33.6 million 39.1 / 51.5; rows of 8001 weights 145 / 192.
+constexpr unsigned long long kOnceWeights = 16ull << 20;
+constexpr unsigned int kOnceGroups = 128;        // groups of 512 words in a part (310 million weights in all)
+constexpr unsigned int kOnceKept = 64;           // marked half-words that a warp keeps beside their marks
+constexpr int kSampleRun = 512;                  // weights of a warp's sample
+
+// In shared memory: the weights of each warp's first marks; of warp w in group g, for each half of a thread's word, the lanes
+// with a weight near `mid`; how many of the warp's marks come before those.
+struct Once {
+    float4 (*kept)[kOnceKept][2];
+    uint2 *mark;
+    unsigned int *before;
+};
+__host__ __device__ constexpr unsigned int once_smem(unsigned int groups)
+{
+    return kSweepWarps * (kOnceKept * 2 * (unsigned int)sizeof(float4) + groups * (unsigned int)(sizeof(uint2) + 4));
+}
+
+__device__ __forceinline__ void ld_eight(float (&v)[8], const float *p, bool wide, unsigned long long policy)
+{
+    if (wide) {
+        asm("ld.global.nc.L2::cache_hint.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8], %9;"
+            : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]) : "l"(p), "l"(policy));
+    } else {
+        const float4 x = ld_stream(reinterpret_cast<const float4 *>(p), policy), y = ld_stream(reinterpret_cast<const float4 *>(p) + 1, policy);
+        v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+        v[4] = y.x; v[5] = y.y; v[6] = y.z; v[7] = y.w;
+    }
+}
+// Half `h` of word `wl` of a part, zeros where there is no weight: aligned vectors, shifted into place.
+__device__ __forceinline__ void load_eight(const Item &it, const PartRange &r, unsigned int wl, int h, float (&v)[8])
+{
+#pragma unroll
+    for (int x = 0; x < 8; ++x) v[x] = 0.0f;
+    if (wl >= r.words) return;
+    const Place p = place_word(it, r, wl);
+    const unsigned int left = p.valid > 8u * h ? p.valid - 8u * h : 0;
+    if (left == 0) return;
+    const unsigned long long at = r.f0 + p.f + 8 * h;
+    if (at + 12 > it.n) {
+        for (int x = 0; x < 8; ++x)
+            if ((unsigned)x < left) v[x] = __ldg(it.W + at + x);
+        return;
+    }
+    const float4 *p4 = reinterpret_cast<const float4 *>(it.W + (at & ~3ull));
+    const unsigned int mis = (unsigned int)at & 3;
+    const float4 q0 = __ldg(p4), q1 = __ldg(p4 + 1), q2 = __ldg(p4 + 2);
+    const float s[12] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w, q2.x, q2.y, q2.z, q2.w};
+    const bool one = mis & 1, two = mis & 2;
+    float t[10];
+#pragma unroll
+    for (int x = 0; x < 10; ++x) t[x] = one ? s[x + 1] : s[x];
+#pragma unroll
+    for (int x = 0; x < 8; ++x) v[x] = (unsigned)x < left ? (two ? t[x + 2] : t[x]) : 0.0f;
+}
+
+// The codes of a word: bit 0 of the kept weights' fields, and the signs in the place of bit 1.
+struct Word {
+    float even = 8388608.0f, odd = 8388608.0f;       // 2^23 plus a sum of distinct powers of two below 2^15: exact
+    uint32_t signs = 0;
+    __device__ __forceinline__ uint32_t kept() const { return __byte_perm(__float_as_uint(even), __float_as_uint(odd), 0x5410) & 0x7FFF7FFFu; }
+};
+
+// Half `h` of a word: the sums, the codes against `mid`; whether a weight lies within `half` of `mid`.
+template <bool SUMS>
+__device__ __forceinline__ bool sweep_eight(const float (&v)[8], int h, float mid, float half, double (&a)[2], double (&k)[2], Word &w)
+{
+    float near[8];
+#pragma unroll
+    for (int x = 0; x < 8; ++x) {
+        const float m = fabsf(v[x]);
+        const double d = (double)m;
+        if (SUMS) a[x & 1] += d;
+        if (m > mid) {
+            k[x & 1] += d;
+            (x & 1 ? w.odd : w.even) += (float)(1 << (14 - 8 * h - (x & ~1)));
+        }
+        near[x] = fabsf(__fsub_rn(m, mid));
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const int down = 2 * (4 * h + j);
+        w.signs |= (__byte_perm(__float_as_uint(v[2 * j]), __float_as_uint(v[2 * j + 1]), 0x7632) >> down) & (0x80008000u >> down);
+    }
+    auto min3 = [](float x, float y, float z) {
+        float r;
+        asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(x), "f"(y), "f"(z));
+        return r;
+    };
+    return SUMS && min3(min3(near[0], near[1], near[2]), min3(near[3], near[4], near[5]), fminf(near[6], near[7])) <= half;
+}
+
+// A word's codes to memory, and its counts.
+__device__ __forceinline__ void finish_word(const Item &it, const PartRange &r, unsigned int wl, const Word &w, unsigned int &pos, unsigned int &neg)
+{
+    const uint32_t kept = w.kept(), minus = w.signs & (kept << 1);
+    const unsigned int n_neg = __popc(minus);
+    neg += n_neg;
+    pos += __popc(kept) - n_neg;
+    if (wl >= r.words) return;
+    if (it.dense && !it.codes_i8) {
+        it.packed[r.w0 + wl] = kept | minus;
+        return;
+    }
+    const Place p = place_word(it, r, wl);
+    it.packed[p.out] = kept | minus;
+    if (it.codes_i8)
+#pragma unroll 1
+        for (unsigned int e = 0; e < p.valid; ++e) {
+            const uint32_t f = ((kept | minus) >> field_pos((int)e)) & 3u;
+            it.codes_i8[r.f0 + p.f + e] = (int8_t)(f == 0 ? 0 : f == 1 ? 1 : -1);
+        }
+}
+
+// A marked half-word coded against `mid`, now that the threshold is known.
+__device__ __forceinline__ void correct(const Item &it, const PartRange &r, unsigned int wl, int h, const float (&v)[8], float mid, float thr,
+                                        double &kept, unsigned int &pos, unsigned int &neg)
+{
+    uint32_t flip = 0;
+#pragma unroll
+    for (int x = 0; x < 8; ++x) {
+        const float mag = fabsf(v[x]);
+        const bool now = mag > thr, minus = v[x] < 0.0f;
+        if (now == (mag > mid)) continue;
+        kept += now ? (double)mag : -(double)mag;
+        const unsigned int one = now ? 1u : 0xFFFFFFFFu;
+        if (minus) neg += one; else pos += one;
+        flip |= (minus ? 3u : 1u) << field_pos(x);
+    }
+    if (!flip) return;
+    const Place p = place_word(it, r, wl);
+    atomicXor(it.packed + p.out, flip >> (8 * h));   // field_pos(8 + x) = field_pos(x) - 8; nobody waits for the word
+    if (it.codes_i8)
+        for (int x = 0; x < 8; ++x)
+            if ((flip >> field_pos(x)) & 1u) it.codes_i8[r.f0 + p.f + 8 * h + x] = fabsf(v[x]) > thr ? (v[x] < 0.0f ? -1 : 1) : 0;
+}
+
+// sum |W| over a warp's run of the sample, 0 where the part is too short for one
+__device__ __forceinline__ float sample_run(const Item &it, const PartRange &r)
+{
+    const unsigned int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (r.len < 2 * kSampleRun) return 0.0f;
+    // the run starts on a 16-byte boundary of the tensor
+    const unsigned long long at = (r.f0 + (unsigned long long)(r.len - kSampleRun - 4) * (2 * warp + 1) / (2 * kSweepWarps) + 3) & ~3ull;
+    const float4 *p = reinterpret_cast<const float4 *>(it.W + at) + lane;
+    float4 v[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] = __ldg(p + 32 * k);
+    float s = 0.0f;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) s += (fabsf(v[k].x) + fabsf(v[k].y)) + (fabsf(v[k].z) + fabsf(v[k].w));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    return s;
+}
+
+__global__ void __launch_bounds__(kSweepThreads, kSweepBlocksPerSm)
+ternarize_once_kernel(const __grid_constant__ Launch<1> P, void *ws_raw)
+{
+    __shared__ Reduce red;
+    __shared__ unsigned long long red_cnt64[2][kSweepWarps];
+    __shared__ float run_s[kSweepWarps];
+    __shared__ unsigned int last_s;
+    extern __shared__ float4 once_raw[];
+    const Item &it = P.item[0];
+    const Workspace ws = carve(ws_raw, 0);
+    const unsigned int b = blockIdx.x, G = gridDim.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    unsigned int turn = 0;
+    if (b == 0 && tid == 0) *ws.done = 0u;
+    const PartRange r = part_range(it, b);          // a block has one part
+    const unsigned int groups = (r.words + 511) >> 9, most = it.part_words >> 9;
+    uint2 *const mark0 = reinterpret_cast<uint2 *>(once_raw + kSweepWarps * kOnceKept * 2);
+    const Once marks = {reinterpret_cast<float4 (*)[kOnceKept][2]>(once_raw), mark0, reinterpret_cast<unsigned int *>(mark0 + kSweepWarps * most)};
+
+
+    // ---- the sample: per part its sum and the squared deviations of its runs (in the arrays of the final sums).  Loads of the
+    // sweep that are issued before its barrier hold the barrier up by more than they gain (88 -> 94 us, the first 128 KB of every
+    // part fetched into L2 88 -> 97).
+    {
+        const float s = sample_run(it, r);
+        if (lane == 0) run_s[warp] = s;
+        __syncthreads();
+        if (tid == 0) {
+            double sum = 0.0, dev = 0.0;
+            for (int w = 0; w < kSweepWarps; ++w) sum += (double)run_s[w];
+            for (int w = 0; w < kSweepWarps; ++w) {
+                const double d = (double)run_s[w] - sum / kSweepWarps;
+                dev += d * d;
+            }
+            ws.part_kept[b] = sum;
+            ws.part_cnt[b] = (unsigned long long)__double_as_longlong(dev);
+        }
+    }
+    cooperative_groups::this_grid().sync();
+    float mid, half;
+    {
+        double sum = 0.0, dev = 0.0;
+        unsigned int n = 0, unused = 0;
+        for (unsigned int i = tid; i < it.parts; i += kSweepThreads) {
+            sum += __ldcg(ws.part_kept + i);
+            dev += __longlong_as_double((long long)__ldcg(ws.part_cnt + i));
+            n += part_range(it, i).len >= 2 * kSampleRun ? kSweepWarps : 0;
+        }
+        sum = sweep_sum(sum, n, unused, red, turn);
+        dev = sweep_sum(dev, red, turn);
+        // 4.5 standard errors of a mean of n runs drawn from strata, and what the rounding of the runs' sums may be
+        const double mean = sum / ((double)n * kSampleRun), se = sqrt(dev * (kSweepWarps / (kSweepWarps - 1.0))) / ((double)n * kSampleRun);
+        mid = (float)(P.factor * mean);
+        half = fminf((float)(P.factor * (4.5 * se + 2e-5 * mean)), 3.0e38f);
+    }
+
+    // ---- the sweep.  The registers of half a word take the next group's as soon as they are coded: a thread's loads never pause.
+    double a[2] = {0.0, 0.0}, k[2] = {0.0, 0.0};
+    unsigned int pos = 0, neg = 0;
+    float v[2][8];
+    {
+        const unsigned int whole = it.linear ? r.len >> 13 : 0;        // groups of 512 words of 16 weights, in memory order
+        const unsigned long long pol = evict_first_policy();
+        const bool wide = (reinterpret_cast<uintptr_t>(it.W) & 31) == 0;
+        const float *p = it.W + r.f0 + 16 * tid;
+        unsigned int n_marks = 0;                                      // of this warp
+        if (whole > 0) {
+            ld_eight(v[0], p, wide, pol);
+            ld_eight(v[1], p + 8, wide, pol);
+        }
+#pragma unroll 1
+        for (unsigned int g = 0; g < groups; ++g) {
+            p += 16 * kSweepThreads;
+            if (g >= whole) {
+                load_eight(it, r, (g << 9) + tid, 0, v[0]);
+                load_eight(it, r, (g << 9) + tid, 1, v[1]);
+            }
+            Word w;
+            unsigned int near[2];
+            if (lane == 0) marks.before[g * kSweepWarps + warp] = n_marks;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const bool mine = sweep_eight<true>(v[h], h, mid, half, a, k, w);
+                near[h] = __ballot_sync(0xffffffffu, mine);
+                if (near[h]) {
+                    const unsigned int slot = n_marks + __popc(near[h] & ((1u << lane) - 1));
+                    if (mine && slot < kOnceKept) {
+                        marks.kept[warp][slot][0] = make_float4(v[h][0], v[h][1], v[h][2], v[h][3]);
+                        marks.kept[warp][slot][1] = make_float4(v[h][4], v[h][5], v[h][6], v[h][7]);
+                    }
+                    n_marks += __popc(near[h]);
+                }
+                if (g + 1 < whole) ld_eight(v[h], p + 8 * h, wide, pol);
+            }
+            if (lane == 0) marks.mark[g * kSweepWarps + warp] = make_uint2(near[0], near[1]);
+            finish_word(it, r, (g << 9) + tid, w, pos, neg);
+        }
+    }
+    write_padding(it, b, G);
+    double kept = k[0] + k[1];
+    {
+        const double s = sweep_sum(a[0] + a[1], red, turn);
+        if (tid == 0) ws.part_sum[b] = s;
+    }
+    cooperative_groups::this_grid().sync();
+    const double s = fold_parts(ws.part_sum, it.parts, red, turn);
+    const double delta = threshold(it, s, P.factor);
+    if (b == 0 && tid == 0) write_threshold(it, s, delta);
+    const float thr = __double2float_rd(delta);
+
+    if (fabsf(__fsub_rn(thr, mid)) <= half) {
+        // ---- put right what lies between.  x -> |x - mid| as computed here and in the sweep is monotonic on either side of
+        // mid, so a weight between mid and thr is no further from mid than thr is: its half-word is marked.  A warp takes its own
+        // marks, a lane every 32nd.
+        const unsigned int last = (groups - 1) * kSweepWarps + warp;
+        const unsigned int total = groups ? marks.before[last] + __popc(marks.mark[last].x) + __popc(marks.mark[last].y) : 0;
+#pragma unroll 1
+        for (unsigned int m = lane; m < total; m += 32) {
+            unsigned int g = 0;                                        // the last group with no more than m marks before it
+            for (unsigned int hi = groups; hi - g > 1;) {
+                const unsigned int c = (g + hi) >> 1;
+                if (marks.before[c * kSweepWarps + warp] <= m) g = c; else hi = c;
+            }
+            const uint2 mk = marks.mark[g * kSweepWarps + warp];
+            unsigned int skip = m - marks.before[g * kSweepWarps + warp], lanes = mk.x;
+            const int h = skip >= __popc(mk.x);
+            if (h) { skip -= __popc(mk.x); lanes = mk.y; }
+            for (; skip > 0; --skip) lanes &= lanes - 1;
+            const unsigned int wl = (g << 9) + warp * 32 + __ffs(lanes) - 1;
+            float m8[8];
+            if (m < kOnceKept) {
+                const float4 x = marks.kept[warp][m][0], y = marks.kept[warp][m][1];
+                m8[0] = x.x; m8[1] = x.y; m8[2] = x.z; m8[3] = x.w;
+                m8[4] = y.x; m8[5] = y.y; m8[6] = y.z; m8[7] = y.w;
+            } else {
+                load_eight(it, r, wl, h, m8);
+            }
+            correct(it, r, wl, h, m8, mid, thr, kept, pos, neg);
+        }
+    } else {
+        k[0] = k[1] = 0.0;
+        pos = neg = 0;
+#pragma unroll 1
+        for (unsigned int g = groups; g-- > 0;) {
+            Word w;
+            load_eight(it, r, (g << 9) + tid, 0, v[0]);
+            load_eight(it, r, (g << 9) + tid, 1, v[1]);
+            sweep_eight<false>(v[0], 0, thr, 0.0f, a, k, w);
+            sweep_eight<false>(v[1], 1, thr, 0.0f, a, k, w);
+            finish_word(it, r, (g << 9) + tid, w, pos, neg);
+        }
+        kept = k[0] + k[1];
+    }
+    // pos and neg of a thread may be below zero after corrections: their sums over the block are counts again
+    kept = sweep_sum(kept, pos, neg, red, turn);
+    if (tid == 0) {
+        ws.part_kept[b] = kept;
+        ws.part_cnt[b] = ((unsigned long long)neg << 32) + pos;
+        unsigned int old;
+        asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(old) : "l"(ws.done) : "memory");
+        last_s = old == it.parts - 1;
+    }
+    __syncthreads();
+    if (last_s) fold_kept(it, ws, red, red_cnt64, turn);
 }
 
 // ---- parameter update fused with the sums of the next iteration ----------------
@@ -1051,10 +1393,31 @@ bool make_item(const float *W, int64_t rows, int64_t cols, twn_stats_t *stats, u
     it->parts = (unsigned int)std::max(1ull, (it->words + part - 1) / part);
     it->vec4 = rows == 1 || cols % 4 == 0;
     it->dense = rows == 1 || ld_codes == cols;
+    it->linear = rows == 1 || cols % 16 == 0;
     it->first_pass = 4ull * n > kKeptBytes ? (unsigned int)(16 * part - 16 * part * kKeptBytes / (4ull * n)) : 0;
     it->first_part = 0;
     *rc = TWN_OK;
     return true;
+}
+
+// Whether a tensor's codes and sums come from one read (ternarize_once_kernel): it is large enough for that to pay, every
+// block has one part, and the marks of a part fit.  Alone and in a batch alike, so that the sums are the same bits.
+bool read_once(const Item &it, const twn_device_info &dev)
+{
+    return it.n >= kOnceWeights && it.parts <= (unsigned int)(dev.sm_count * kSweepBlocksPerSm) && it.part_words <= kOnceGroups * 512;
+}
+
+int launch_once(Launch<1> &P, double factor, void *ws, const twn_device_info &dev, cudaStream_t s)
+{
+    P.factor = factor;
+    P.parts = P.item[0].parts;
+    P.item[0].first_part = 0;
+    static bool attr_set[64] = {false};
+    if (!attr_set[dev.ordinal]) {
+        TWN_CUDA_OK(cudaFuncSetAttribute(ternarize_once_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)once_smem(kOnceGroups)));
+        attr_set[dev.ordinal] = true;
+    }
+    return launch_cooperative(ternarize_once_kernel, P.parts, s, once_smem(P.item[0].part_words >> 9), P, ws);
 }
 
 template <int N, bool SUMS>
@@ -1078,8 +1441,9 @@ int launch_sweeps(Launch<N> &P, double factor, void *ws, cudaStream_t s)
                         : q <= 4 ? ternarize_small_kernel<4, SUMS> : ternarize_small_kernel<8, SUMS>;
             return launch_cluster(kernel, grid, s, P);
         }
+        if (SUMS && read_once(P.item[0], dev)) return launch_once(P, factor, ws, dev, s);
     }
-    return launch_cooperative(ternarize_kernel<N, SUMS>, std::min(P.parts, (unsigned int)(dev.sm_count * kSweepBlocksPerSm)), s, P, ws);
+    return launch_cooperative(ternarize_kernel<N, SUMS>, std::min(P.parts, (unsigned int)(dev.sm_count * kSweepBlocksPerSm)), s, 0, P, ws);
 }
 
 bool batch_items(const twn_ternarize_item_t *items, int count, Launch<kMaxBatch> &P, int *rc)
@@ -1112,7 +1476,7 @@ int launch_sgd(SgdLaunch<N> &P, void *ws, cudaStream_t s)
             return launch_cluster(sgd_update_kernel<N, true>, grid, s, P, ws);
         }
     }
-    return launch_cooperative(sgd_update_kernel<N, false>, std::min(P.blocks, (unsigned int)(dev.sm_count * kSweepBlocksPerSm)), s, P, ws);
+    return launch_cooperative(sgd_update_kernel<N, false>, std::min(P.blocks, (unsigned int)(dev.sm_count * kSweepBlocksPerSm)), s, 0, P, ws);
 }
 
 }  // namespace
@@ -1162,6 +1526,25 @@ extern "C" int twn_ternarize_batch(const twn_ternarize_item_t *items, int count,
     int rc;
     Launch<kMaxBatch> P;
     if (!batch_items(items, count, P, &rc)) return rc;
+    twn_device_info dev;
+    rc = twn_current_device(&dev);
+    if (rc != TWN_OK) return rc;
+    // tensors that are read once have launches of their own
+    int rest = 0;
+    for (int t = 0; t < count; ++t) {
+        if (!read_once(P.item[t], dev)) {
+            if (rest != t) P.item[rest] = P.item[t];
+            ++rest;
+            continue;
+        }
+        Launch<1> one;
+        one.count = 1;
+        one.item[0] = P.item[t];
+        rc = launch_once(one, delta_factor, static_cast<char *>(workspace) + (size_t)t * kWorkspaceBytes, dev, twn_cu(stream));
+        if (rc != TWN_OK) return rc;
+    }
+    if (rest == 0) return TWN_OK;
+    P.count = rest;
     return launch_sweeps<kMaxBatch, true>(P, delta_factor, workspace, twn_cu(stream));
 }
 
