@@ -10,7 +10,7 @@
 // whole word.  (A warp vote per word of 32 costs a 4-byte load, a vote and a select per weight of a lane, and rows that
 // are no whole words were voted one word at a time.)
 // sum |W| has a fixed order: per-thread fp64 sums, the trees of sweep.cuh, one part per block.  The blocks meet through
-// the workspace and a grid-wide barrier, those of a small tensor as one cluster through distributed shared memory.
+// the workspace and a launch that folds them, those of a small tensor as one cluster through distributed shared memory.
 #include <algorithm>
 
 #include "sweep.cuh"
@@ -70,6 +70,19 @@ __device__ __forceinline__ uint32_t exchange_nibbles(uint32_t x)
     return (lane & 1) ? ((x & 0xF0F0F0F0u) | ((y >> 4) & 0x0F0F0F0Fu)) : ((x & 0x0F0F0F0Fu) | ((y << 4) & 0xF0F0F0F0u));
 }
 
+__device__ __forceinline__ void write_binary(const BinParams &P, double s, unsigned long long n_neg)
+{
+    P.stats->delta = 0.0;
+    P.stats->alpha = P.n > 0 ? s / (double)P.n : 0.0;
+    P.stats->sum_abs = s;
+    P.stats->sum_abs_kept = s;
+    P.stats->n_neg = n_neg;
+    P.stats->n_zero = 0;
+    P.stats->n_pos = P.n - n_neg;
+    P.stats->status = isfinite(s) ? TWN_OK : TWN_ERR_NONFINITE;
+    P.stats->reserved = 0;
+}
+
 template <bool CLUSTER>
 __global__ void __launch_bounds__(kSweepThreads, kSweepBlocksPerSm)
 binarize_kernel(const __grid_constant__ BinParams P)
@@ -83,6 +96,8 @@ binarize_kernel(const __grid_constant__ BinParams P)
         if (tid < kSmallParts) { sum_s[tid] = 0.0; neg_s[tid] = 0ull; }
         pdl_begin();
         cluster_arrive();
+    } else {
+        early_start();
     }
     // padding words of the rows
     const unsigned int pad = (unsigned int)(P.wpr - P.wpr_used);
@@ -170,8 +185,6 @@ binarize_kernel(const __grid_constant__ BinParams P)
             P.part_neg[part] = neg;
         }
     }
-    double s = 0.0;
-    unsigned long long c = 0;
     if (CLUSTER) {
         cluster_wait();
         if (tid == 0) {
@@ -180,35 +193,31 @@ binarize_kernel(const __grid_constant__ BinParams P)
         }
         cluster_arrive();
         cluster_wait();
-        if (b != 0) return;
-        s = tree8(sum_s);
+        if (b != 0 || tid != 0) return;
+        unsigned long long c = 0;
         for (int i = 0; i < kSmallParts; ++i) c += neg_s[i];
-    } else {
-        cooperative_groups::this_grid().sync();
-        if (b != 0) return;
-        unsigned int lo = 0, hi = 0;     // of at most kMaxParts counts below 2^32: no carry gets lost
-        for (unsigned int i = tid; i < P.parts; i += kSweepThreads) {
-            s += __ldcg(P.part_sum + i);
-            const unsigned long long k = __ldcg(P.part_neg + i);
-            lo += (unsigned int)(k & 0xFFFFFull);
-            hi += (unsigned int)(k >> 20);
-        }
-        s = sweep_sum(s, lo, hi, red, turn);
-        c = lo + ((unsigned long long)hi << 20);
-    }
-    if (tid == 0) {
-        P.stats->delta = 0.0;
-        P.stats->alpha = P.n > 0 ? s / (double)P.n : 0.0;
-        P.stats->sum_abs = s;
-        P.stats->sum_abs_kept = s;
-        P.stats->n_neg = c;
-        P.stats->n_zero = 0;
-        P.stats->n_pos = P.n - c;
-        P.stats->status = isfinite(s) ? TWN_OK : TWN_ERR_NONFINITE;
-        P.stats->reserved = 0;
+        write_binary(P, tree8(sum_s), c);
     }
 }
-
+// The parts' sums of a larger tensor: a launch of its own that is there when the sweep ends (in one cooperative launch with a
+// grid-wide barrier 663 thousand weights took 8.3 us, 6.4 now).
+__global__ void __launch_bounds__(kSweepThreads)
+binarize_fold_kernel(const BinParams P)
+{
+    __shared__ Reduce red;
+    unsigned int turn = 0;
+    early_start();
+    double s = 0.0;
+    unsigned int lo = 0, hi = 0;         // of at most kMaxParts counts below 2^32: no carry gets lost
+    for (unsigned int i = threadIdx.x; i < P.parts; i += kSweepThreads) {
+        s += __ldcg(P.part_sum + i);
+        const unsigned long long k = __ldcg(P.part_neg + i);
+        lo += (unsigned int)(k & 0xFFFFFull);
+        hi += (unsigned int)(k >> 20);
+    }
+    s = sweep_sum(s, lo, hi, red, turn);
+    if (threadIdx.x == 0) write_binary(P, s, lo + ((unsigned long long)hi << 20));
+}
 
 __global__ void __launch_bounds__(kThreads)
 unpack_b1_kernel(const uint32_t *__restrict__ packed, long long rows, long long cols, long long ld_codes,
@@ -291,7 +300,10 @@ extern "C" int twn_binarize(const float *W, int64_t rows, int64_t cols, twn_stat
         while (grid < P.parts) grid *= 2;
         return launch_cluster(binarize_kernel<true>, grid, twn_cu(stream), P);
     }
-    return launch_cooperative(binarize_kernel<false>, std::min(P.parts, (unsigned int)(dev.sm_count * kSweepBlocksPerSm)), twn_cu(stream), 0, P);
+    TWN_CUDA_OK(twn_launch_pdl(true, binarize_kernel<false>, (int)std::min(P.parts, (unsigned int)(dev.sm_count * kSweepBlocksPerSm)),
+                               kSweepThreads, 0, twn_cu(stream), P));
+    TWN_CUDA_OK(twn_launch_pdl(true, binarize_fold_kernel, 1, kSweepThreads, 0, twn_cu(stream), P));
+    return TWN_OK;
 }
 
 extern "C" int twn_unpack_b1(const uint32_t *packed, int64_t rows, int64_t cols, int64_t ld_codes, int8_t *codes,

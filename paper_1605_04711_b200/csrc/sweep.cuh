@@ -104,6 +104,15 @@ int launch_cluster(K kernel, unsigned int grid, cudaStream_t s, const A &...args
     TWN_CUDA_OK(cudaLaunchKernelEx(&cfg, kernel, args...));
     return TWN_OK;
 }
+// A kernel that follows another in a chain of launches: it may become resident while the one before it drains, and lets the one
+// after it do so; from here on what was written before is visible.
+#ifdef __CUDACC__
+__device__ __forceinline__ void early_start()
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+#endif
 // A grid whose blocks all run at once and may wait for one another.
 template <typename K, typename... A>
 int launch_cooperative(K kernel, unsigned int grid, cudaStream_t s, size_t smem, const A &...args)

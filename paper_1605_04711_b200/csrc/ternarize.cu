@@ -2,12 +2,12 @@
 // threshold rule; Algorithm 1, first loop), the parameter update, plus the standalone pack / unpack /
 // re-layout kernels.
 //
-// Ternarization is one launch of two phases, bound by HBM bandwidth:
+// Ternarization is two phases, bound by HBM bandwidth:
 //   phase 1  S = sum |W_i| in fp64  ->  delta = factor * S / n
 //   phase 2  codes by Eq. 3, packed 16 per word; sum and count of the kept set
 //            ->  alpha (Eq. 5)
-// (tensors much larger than L2 in one phase against an estimate, with corrections: ternarize_once_kernel)
-// with a barrier of all blocks between them (grid-wide in a cooperative launch, a cluster's for small tensors).
+// (and for tensors much larger than L2 one phase against an estimate, with corrections: ternarize_once_kernel).
+// one launch each and one for the last fold, or, for small tensors, one launch of one cluster with its barrier in between
 // Phase 2 walks every block's share back to front, so that what phase 1 read last comes from L1 and L2.
 //
 // All sums have a fixed order that depends on the shape of the tensor alone: a tensor is cut into at most
@@ -311,6 +311,20 @@ __device__ __forceinline__ void write_kept(const Item &it, double kept, unsigned
     it.stats->n_zero = it.n - n_kept;
 }
 
+// The codes of a part against a threshold, back to front: what was read last comes from L2.  (A thread per word, as in
+// ternarize_once_kernel, needs no exchange among lanes but more registers than two blocks leave: 8.4 million weights 12.6 us
+// instead of 12.1, 28.7 million 40.8 instead of 38.3.)
+__device__ __forceinline__ Coder code_part(const Item &it, const PartRange &r, float thr)
+{
+    Coder c;
+    for (unsigned int grp = (r.words + 511) >> 9; grp-- > 0;) {
+        float4 v[4];
+        load_group(it, r, grp << 9, v);
+        c.group(it, r, grp << 9, v, thr);
+    }
+    return c;
+}
+
 // padding words of the rows
 __device__ __forceinline__ void write_padding(const Item &it, unsigned int b, unsigned int G)
 {
@@ -386,7 +400,7 @@ ternarize_small_kernel(const __grid_constant__ Launch<1> P)
     }
 }
 
-// ---- any tensor: a cooperative launch -------------------------------------------
+// ---- any tensor: a launch per phase ---------------------------------------------
 // The tensor of part g, from the one of an earlier part (up) or of a later part (down) on.
 template <int N> __device__ __forceinline__ int item_up(const Launch<N> &P, unsigned int g, int t)
 {
@@ -479,75 +493,11 @@ struct PartRun {
     uint2 cnt[kRun][kSweepWarps];
 };
 
-// N: tensors of the launch (1, or up to kMaxBatch).  SUMS: false for the coding sweep alone, against the
-// threshold that is in the stats.
-template <int N, bool SUMS>
-__global__ void __launch_bounds__(kSweepThreads, kSweepBlocksPerSm)
-ternarize_kernel(const __grid_constant__ Launch<N> P, void *ws_raw)
+// The codes of a block's parts b, b + G, ..., back to front, and their sums into the workspace.
+template <int N>
+__device__ __forceinline__ void code_parts(const Launch<N> &P, void *ws_raw, unsigned int mine, const float *thr_s, PartRun &run)
 {
-    __shared__ Reduce red;
-    __shared__ unsigned long long red_cnt64[2][kSweepWarps];
-    __shared__ PartRun run;
-    __shared__ float thr_s[N];
-    __shared__ unsigned int last_mask;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const unsigned int b = blockIdx.x, G = gridDim.x;
-    unsigned int turn = 0;
-
-    if (tid == 0) last_mask = 0;
-    if (b == 0 && tid < P.count) *carve(ws_raw, tid).done = 0u;
-
-    // this block's parts: b, b + G, ...
-    const unsigned int mine = b < P.parts ? (P.parts - 1 - b) / G + 1 : 0;
-
-    // ---- phase 1
-    if (SUMS) {
-        int ti = 0;
-        for (unsigned int i0 = 0; i0 < mine; i0 += kRun) {
-            const unsigned int n = min(mine - i0, (unsigned int)kRun);
-            for (unsigned int i = 0; i < n; ++i) {
-                const unsigned int g = b + (i0 + i) * G;
-                ti = item_up(P, g, ti);
-                const Item &it = P.item[ti];
-                const double v = warp_sum(part_abs_sum(it, part_range(it, g - it.first_part)));
-                if (lane == 0) run.sum[i][warp] = v;
-            }
-            __syncthreads();
-            if (tid < n) {
-                const unsigned int g = b + (i0 + tid) * G;
-                const int t = item_down(P, g, ti);
-                carve(ws_raw, t).part_sum[g - P.item[t].first_part] = tree16(run.sum[tid]);
-            }
-            __syncthreads();
-        }
-    }
-#pragma unroll 1
-    for (int t = 0; t < P.count; ++t) write_padding(P.item[t], b, G);
-
-    cooperative_groups::this_grid().sync();
-
-    double delta = 0.0;
-    if (SUMS) {
-        if (N == 1) {
-            // every block folds for itself
-            const double s = fold_parts(carve(ws_raw, 0).part_sum, P.item[0].parts, red, turn);
-            delta = threshold(P.item[0], s, P.factor);
-            if (b == 0 && tid == 0) write_threshold(P.item[0], s, delta);
-        } else {
-            for (int t = (int)b; t < P.count; t += (int)G) {
-                const double s = fold_parts(carve(ws_raw, t).part_sum, P.item[t].parts, red, turn);
-                if (tid == 0) write_threshold(P.item[t], s, threshold(P.item[t], s, P.factor));
-            }
-            cooperative_groups::this_grid().sync();
-        }
-    }
-
-    // delta rounded toward -inf: for any float w,  w > delta  <=>  w > thr
-    if (N == 1) thr_s[0] = __double2float_rd(SUMS ? delta : __ldcg(&P.item[0].stats->delta));
-    else if (tid < P.count) thr_s[tid] = __double2float_rd(__ldcg(&P.item[tid].stats->delta));
-    __syncthreads();
-
-    // ---- phase 2, back to front
+    const unsigned int b = blockIdx.x, G = gridDim.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     int ti = P.count - 1;
     for (unsigned int left = mine; left > 0;) {
         const unsigned int n = min(left, (unsigned int)kRun);
@@ -555,14 +505,7 @@ ternarize_kernel(const __grid_constant__ Launch<N> P, void *ws_raw)
             const unsigned int g = b + (left - 1 - i) * G;
             ti = item_down(P, g, ti);
             const Item &it = P.item[ti];
-            const PartRange r = part_range(it, g - it.first_part);
-            const float thr = thr_s[N == 1 ? 0 : ti];
-            Coder c;
-            for (unsigned int grp = (r.words + 511) >> 9; grp-- > 0;) {
-                float4 v[4];
-                load_group(it, r, grp << 9, v);
-                c.group(it, r, grp << 9, v, thr);
-            }
+            const Coder c = code_part(it, part_range(it, g - it.first_part), thr_s[N == 1 ? 0 : ti]);
             const double kept = warp_sum(c.kept());
             const unsigned int p = __reduce_add_sync(0xffffffffu, c.pos), q = __reduce_add_sync(0xffffffffu, c.neg);
             if (lane == 0) { run.sum[i][warp] = kept; run.cnt[i][warp] = make_uint2(p, q); }
@@ -578,21 +521,92 @@ ternarize_kernel(const __grid_constant__ Launch<N> P, void *ws_raw)
             for (int w = 0; w < kSweepWarps; ++w) { p += run.cnt[tid][w].x; q += run.cnt[tid][w].y; }
             ws.part_kept[g - it.first_part] = tree16(run.sum[tid]);
             ws.part_cnt[g - it.first_part] = ((unsigned long long)q << 32) + p;
-            unsigned int old;
-            asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(old) : "l"(ws.done) : "memory");
-            if (old == it.parts - 1) atomicOr(&last_mask, 1u << t);
         }
         __syncthreads();
         left -= n;
     }
-    // the block that wrote the last part of a tensor folds its second sums
-    for (unsigned int mask = last_mask; mask; mask &= mask - 1) {
-        const int ti = __ffs(mask) - 1;
-        const Item &it = P.item[ti];
-        const Workspace ws = carve(ws_raw, ti);
-        fold_kept(it, ws, red, red_cnt64, turn);
+}
+
+// Sums, codes, and the folds of both are launches of their own, each there when the one before it ends (programmatic launches):
+// no block waits for another.  In a cooperative launch with grid-wide barriers a stream of calls came in steps of 2 us: 147
+// thousand to 590 thousand weights 10.3 us so, 7.9 to 8.6 in three launches; the coding sweep of 590 thousand 8.3 and 5.2; the 21
+// tensors of ResNet-18 39.1 and 35.7, their coding sweeps 28.0 and 20.1.
+// N: tensors of the launch (1, or up to kMaxBatch).
+template <int N>
+__global__ void __launch_bounds__(kSweepThreads, kSweepBlocksPerSm)
+sums_kernel(const __grid_constant__ Launch<N> P, void *ws_raw)
+{
+    __shared__ PartRun run;
+    const unsigned int b = blockIdx.x, G = gridDim.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const unsigned int mine = b < P.parts ? (P.parts - 1 - b) / G + 1 : 0;     // this block's parts: b, b + G, ...
+    early_start();
+    int ti = 0;
+    for (unsigned int i0 = 0; i0 < mine; i0 += kRun) {
+        const unsigned int n = min(mine - i0, (unsigned int)kRun);
+        for (unsigned int i = 0; i < n; ++i) {
+            const unsigned int g = b + (i0 + i) * G;
+            ti = item_up(P, g, ti);
+            const Item &it = P.item[ti];
+            const double v = warp_sum(part_abs_sum(it, part_range(it, g - it.first_part)));
+            if (lane == 0) run.sum[i][warp] = v;
+        }
+        __syncthreads();
+        if (tid < n) {
+            const unsigned int g = b + (i0 + tid) * G;
+            const int t = item_down(P, g, ti);
+            carve(ws_raw, t).part_sum[g - P.item[t].first_part] = tree16(run.sum[tid]);
+        }
         __syncthreads();
     }
+}
+// the thresholds of a batch, one block per tensor
+template <int N>
+__global__ void __launch_bounds__(kSweepThreads)
+sums_fold_kernel(const __grid_constant__ Launch<N> P, void *ws_raw)
+{
+    __shared__ Reduce red;
+    unsigned int turn = 0;
+    early_start();
+    const Item &it = P.item[blockIdx.x];
+    const double s = fold_parts(carve(ws_raw, (int)blockIdx.x).part_sum, it.parts, red, turn);
+    if (threadIdx.x == 0) write_threshold(it, s, threshold(it, s, P.factor));
+}
+
+// The coding sweep, against the threshold that is in the stats, or (FOLD, one tensor) that every block folds for itself.
+template <int N, bool FOLD>
+__global__ void __launch_bounds__(kSweepThreads, kSweepBlocksPerSm)
+codes_kernel(const __grid_constant__ Launch<N> P, void *ws_raw)
+{
+    static_assert(!FOLD || N == 1, "the thresholds of a batch have a launch");
+    __shared__ Reduce red;
+    __shared__ PartRun run;
+    __shared__ float thr_s[N];
+    const unsigned int b = blockIdx.x, G = gridDim.x;
+    unsigned int turn = 0;
+    early_start();
+    // delta rounded toward -inf: for any float w,  w > delta  <=>  w > thr
+    if (FOLD) {
+        const double s = fold_parts(carve(ws_raw, 0).part_sum, P.item[0].parts, red, turn);
+        const double delta = threshold(P.item[0], s, P.factor);
+        if (b == 0 && threadIdx.x == 0) write_threshold(P.item[0], s, delta);
+        if (threadIdx.x == 0) thr_s[0] = __double2float_rd(delta);
+    } else if (threadIdx.x < (unsigned)P.count) {
+        thr_s[threadIdx.x] = __double2float_rd(__ldcg(&P.item[threadIdx.x].stats->delta));
+    }
+    __syncthreads();
+    code_parts(P, ws_raw, b < P.parts ? (P.parts - 1 - b) / G + 1 : 0, thr_s, run);
+#pragma unroll 1
+    for (int t = 0; t < P.count; ++t) write_padding(P.item[t], b, G);
+}
+template <int N>
+__global__ void __launch_bounds__(kSweepThreads)
+codes_fold_kernel(const __grid_constant__ Launch<N> P, void *ws_raw)
+{
+    __shared__ Reduce red;
+    __shared__ unsigned long long red_cnt64[2][kSweepWarps];
+    unsigned int turn = 0;
+    early_start();
+    fold_kept(P.item[blockIdx.x], carve(ws_raw, (int)blockIdx.x), red, red_cnt64, turn);
 }
 
 // ---- large tensors: one read ------------------------------------------------------
@@ -672,7 +686,6 @@ struct Word {
 };
 
 // Half `h` of a word: the sums, the codes against `mid`; whether a weight lies within `half` of `mid`.
-template <bool SUMS>
 __device__ __forceinline__ bool sweep_eight(const float (&v)[8], int h, float mid, float half, double (&a)[2], double (&k)[2], Word &w)
 {
     float near[8];
@@ -680,7 +693,7 @@ __device__ __forceinline__ bool sweep_eight(const float (&v)[8], int h, float mi
     for (int x = 0; x < 8; ++x) {
         const float m = fabsf(v[x]);
         const double d = (double)m;
-        if (SUMS) a[x & 1] += d;
+        a[x & 1] += d;
         if (m > mid) {
             k[x & 1] += d;
             (x & 1 ? w.odd : w.even) += (float)(1 << (14 - 8 * h - (x & ~1)));
@@ -697,7 +710,7 @@ __device__ __forceinline__ bool sweep_eight(const float (&v)[8], int h, float mi
         asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(x), "f"(y), "f"(z));
         return r;
     };
-    return SUMS && min3(min3(near[0], near[1], near[2]), min3(near[3], near[4], near[5]), fminf(near[6], near[7])) <= half;
+    return min3(min3(near[0], near[1], near[2]), min3(near[3], near[4], near[5]), fminf(near[6], near[7])) <= half;
 }
 
 // A word's codes to memory, and its counts.
@@ -845,7 +858,7 @@ ternarize_once_kernel(const __grid_constant__ Launch<1> P, void *ws_raw)
             if (lane == 0) marks.before[g * kSweepWarps + warp] = n_marks;
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-                const bool mine = sweep_eight<true>(v[h], h, mid, half, a, k, w);
+                const bool mine = sweep_eight(v[h], h, mid, half, a, k, w);
                 near[h] = __ballot_sync(0xffffffffu, mine);
                 if (near[h]) {
                     const unsigned int slot = n_marks + __popc(near[h] & ((1u << lane) - 1));
@@ -903,18 +916,8 @@ ternarize_once_kernel(const __grid_constant__ Launch<1> P, void *ws_raw)
             correct(it, r, wl, h, m8, mid, thr, kept, pos, neg);
         }
     } else {
-        k[0] = k[1] = 0.0;
-        pos = neg = 0;
-#pragma unroll 1
-        for (unsigned int g = groups; g-- > 0;) {
-            Word w;
-            load_eight(it, r, (g << 9) + tid, 0, v[0]);
-            load_eight(it, r, (g << 9) + tid, 1, v[1]);
-            sweep_eight<false>(v[0], 0, thr, 0.0f, a, k, w);
-            sweep_eight<false>(v[1], 1, thr, 0.0f, a, k, w);
-            finish_word(it, r, (g << 9) + tid, w, pos, neg);
-        }
-        kept = k[0] + k[1];
+        const Coder c = code_part(it, r, thr);
+        kept = c.kept(); pos = c.pos; neg = c.neg;
     }
     // pos and neg of a thread may be below zero after corrections: their sums over the block are counts again
     kept = sweep_sum(kept, pos, neg, red, turn);
@@ -970,9 +973,17 @@ __device__ __forceinline__ void sgd_four(float4 &w, const float4 g, float4 &v, f
     a0 += (double)fabsf(w.x); a1 += (double)fabsf(w.y); a0 += (double)fabsf(w.z); a1 += (double)fabsf(w.w);
 }
 
-// The blocks' sums meet as in the ternarization kernels: through distributed shared memory where one cluster of at
-// most eight blocks does, else through the workspace and a grid-wide barrier (1.2 us; a ticket in the workspace has to
-// be cleared first, by a memset that costs its own launch: 3 us).
+__device__ __forceinline__ void write_next(const SgdItem &it, double factor, double s)
+{
+    it.stats->sum_abs = s;
+    it.stats->delta = it.n > 0 ? factor * (s / (double)it.n) : 0.0;
+    it.stats->status = isfinite(s) ? TWN_OK : TWN_ERR_NONFINITE;
+    it.stats->reserved = 0;
+}
+
+// The blocks' sums meet through distributed shared memory where one cluster of at most eight blocks does, else in the
+// workspace, where a launch of their own folds them, one block per tensor, that is there when this one ends (in a cooperative
+// launch with a barrier 590 thousand weights took 6.2 us, 4.4 now, 8.4 million 32.4 and 30.3).
 template <int N, bool CLUSTER>
 __global__ void __launch_bounds__(kSweepThreads, kSweepBlocksPerSm)
 sgd_update_kernel(const __grid_constant__ SgdLaunch<N> P, void *ws_raw)
@@ -986,6 +997,8 @@ sgd_update_kernel(const __grid_constant__ SgdLaunch<N> P, void *ws_raw)
         if (threadIdx.x < kSmallParts) sum_s[threadIdx.x] = 0.0;
         pdl_begin();
         cluster_arrive();
+    } else {
+        early_start();
     }
     for (unsigned int g = blockIdx.x; g < P.blocks; g += gridDim.x) {
         int t = 0;
@@ -1032,29 +1045,28 @@ sgd_update_kernel(const __grid_constant__ SgdLaunch<N> P, void *ws_raw)
         if (CLUSTER) own = s;
         else if (threadIdx.x == 0) carve(ws_raw, t).part_sum[vb] = s;
     }
-    auto finish = [&](const SgdItem &it, double s) {
-        it.stats->sum_abs = s;
-        it.stats->delta = it.n > 0 ? P.factor * (s / (double)it.n) : 0.0;
-        it.stats->status = isfinite(s) ? TWN_OK : TWN_ERR_NONFINITE;
-        it.stats->reserved = 0;
-    };
     if (CLUSTER) {
         // a block has at most one share
         cluster_wait();
         if (threadIdx.x == 0) st_peer(peer_smem(&sum_s[blockIdx.x], 0), __double_as_longlong(own));
         cluster_arrive();
         cluster_wait();
-        if (blockIdx.x == 0 && threadIdx.x == 0 && P.item[0].stats) finish(P.item[0], tree8(sum_s));
-    } else {
-        cooperative_groups::this_grid().sync();
-        for (int t = (int)blockIdx.x; t < P.count; t += (int)gridDim.x) {
-            const SgdItem &it = P.item[t];
-            if (!it.stats) continue;
-            const unsigned int vg = (t + 1 < P.count ? P.item[t + 1 < N ? t + 1 : 0].first_block : P.blocks) - it.first_block;
-            const double s = fold_parts(carve(ws_raw, t).part_sum, vg, red, turn);
-            if (threadIdx.x == 0) finish(it, s);
-        }
+        if (blockIdx.x == 0 && threadIdx.x == 0 && P.item[0].stats) write_next(P.item[0], P.factor, tree8(sum_s));
     }
+}
+template <int N>
+__global__ void __launch_bounds__(kSweepThreads)
+sgd_fold_kernel(const __grid_constant__ SgdLaunch<N> P, void *ws_raw)
+{
+    __shared__ Reduce red;
+    unsigned int turn = 0;
+    early_start();
+    const int t = (int)blockIdx.x;
+    const SgdItem &it = P.item[t];
+    if (!it.stats) return;
+    const unsigned int vg = (t + 1 < P.count ? P.item[t + 1 < N ? t + 1 : 0].first_block : P.blocks) - it.first_block;
+    const double s = fold_parts(carve(ws_raw, t).part_sum, vg, red, turn);
+    if (threadIdx.x == 0) write_next(it, P.factor, s);
 }
 
 // ---- standalone pack / unpack / re-layout ----------------------------------
@@ -1443,7 +1455,12 @@ int launch_sweeps(Launch<N> &P, double factor, void *ws, cudaStream_t s)
         }
         if (SUMS && read_once(P.item[0], dev)) return launch_once(P, factor, ws, dev, s);
     }
-    return launch_cooperative(ternarize_kernel<N, SUMS>, std::min(P.parts, (unsigned int)(dev.sm_count * kSweepBlocksPerSm)), s, 0, P, ws);
+    const unsigned int grid = std::min(P.parts, (unsigned int)(dev.sm_count * kSweepBlocksPerSm));
+    if (SUMS) TWN_CUDA_OK(twn_launch_pdl(true, sums_kernel<N>, (int)grid, kSweepThreads, 0, s, P, ws));
+    if (SUMS && N > 1) TWN_CUDA_OK(twn_launch_pdl(true, sums_fold_kernel<N>, P.count, kSweepThreads, 0, s, P, ws));
+    TWN_CUDA_OK(twn_launch_pdl(true, codes_kernel<N, SUMS && N == 1>, (int)grid, kSweepThreads, 0, s, P, ws));
+    TWN_CUDA_OK(twn_launch_pdl(true, codes_fold_kernel<N>, P.count, kSweepThreads, 0, s, P, ws));
+    return TWN_OK;
 }
 
 bool batch_items(const twn_ternarize_item_t *items, int count, Launch<kMaxBatch> &P, int *rc)
@@ -1476,7 +1493,10 @@ int launch_sgd(SgdLaunch<N> &P, void *ws, cudaStream_t s)
             return launch_cluster(sgd_update_kernel<N, true>, grid, s, P, ws);
         }
     }
-    return launch_cooperative(sgd_update_kernel<N, false>, std::min(P.blocks, (unsigned int)(dev.sm_count * kSweepBlocksPerSm)), s, 0, P, ws);
+    TWN_CUDA_OK(twn_launch_pdl(true, sgd_update_kernel<N, false>, (int)std::min(P.blocks, (unsigned int)(dev.sm_count * kSweepBlocksPerSm)),
+                               kSweepThreads, 0, s, P, ws));
+    TWN_CUDA_OK(twn_launch_pdl(true, sgd_fold_kernel<N>, P.count, kSweepThreads, 0, s, P, ws));
+    return TWN_OK;
 }
 
 }  // namespace
