@@ -97,7 +97,7 @@ binarize_kernel(const __grid_constant__ BinParams P)
         pdl_begin();
         cluster_arrive();
     } else {
-        early_start();
+        chain_wait();
     }
     // padding words of the rows
     const unsigned int pad = (unsigned int)(P.wpr - P.wpr_used);
@@ -206,7 +206,7 @@ binarize_fold_kernel(const BinParams P)
 {
     __shared__ Reduce red;
     unsigned int turn = 0;
-    early_start();
+    chain_wait();
     double s = 0.0;
     unsigned int lo = 0, hi = 0;         // of at most kMaxParts counts below 2^32: no carry gets lost
     for (unsigned int i = threadIdx.x; i < P.parts; i += kSweepThreads) {

@@ -104,14 +104,12 @@ int launch_cluster(K kernel, unsigned int grid, cudaStream_t s, const A &...args
     TWN_CUDA_OK(cudaLaunchKernelEx(&cfg, kernel, args...));
     return TWN_OK;
 }
-// A kernel that follows another in a chain of launches: it may become resident while the one before it drains, and lets the one
-// after it do so; from here on what was written before is visible.
+// A kernel of a chain of launches: launched programmatically, it is there when the one before it ends, and from here on what that
+// wrote is visible.  It lets its own successor start by ending, not earlier: with a trigger at the start of every kernel the
+// successors' blocks were resident and waiting three launches ahead, and a training layer of one 83x83x224 image (96 channels)
+// took 59.6 us instead of 52.4, the 21 tensors of ResNet-18 35.6 instead of 31.1.
 #ifdef __CUDACC__
-__device__ __forceinline__ void early_start()
-{
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-}
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 #endif
 // A grid whose blocks all run at once and may wait for one another.
 template <typename K, typename... A>

@@ -6,8 +6,8 @@
 //   phase 1  S = sum |W_i| in fp64  ->  delta = factor * S / n
 //   phase 2  codes by Eq. 3, packed 16 per word; sum and count of the kept set
 //            ->  alpha (Eq. 5)
-// (and for tensors much larger than L2 one phase against an estimate, with corrections: ternarize_once_kernel).
-// one launch each and one for the last fold, or, for small tensors, one launch of one cluster with its barrier in between
+// one launch each and one for the last fold, or, for small tensors, one launch of a cluster with its barrier in between; for
+// tensors much larger than L2 one phase against an estimate of the threshold, with corrections (ternarize_once_kernel).
 // Phase 2 walks every block's share back to front, so that what phase 1 read last comes from L1 and L2.
 //
 // All sums have a fixed order that depends on the shape of the tensor alone: a tensor is cut into at most
@@ -539,7 +539,7 @@ sums_kernel(const __grid_constant__ Launch<N> P, void *ws_raw)
     __shared__ PartRun run;
     const unsigned int b = blockIdx.x, G = gridDim.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const unsigned int mine = b < P.parts ? (P.parts - 1 - b) / G + 1 : 0;     // this block's parts: b, b + G, ...
-    early_start();
+    chain_wait();
     int ti = 0;
     for (unsigned int i0 = 0; i0 < mine; i0 += kRun) {
         const unsigned int n = min(mine - i0, (unsigned int)kRun);
@@ -566,7 +566,7 @@ sums_fold_kernel(const __grid_constant__ Launch<N> P, void *ws_raw)
 {
     __shared__ Reduce red;
     unsigned int turn = 0;
-    early_start();
+    chain_wait();
     const Item &it = P.item[blockIdx.x];
     const double s = fold_parts(carve(ws_raw, (int)blockIdx.x).part_sum, it.parts, red, turn);
     if (threadIdx.x == 0) write_threshold(it, s, threshold(it, s, P.factor));
@@ -583,7 +583,7 @@ codes_kernel(const __grid_constant__ Launch<N> P, void *ws_raw)
     __shared__ float thr_s[N];
     const unsigned int b = blockIdx.x, G = gridDim.x;
     unsigned int turn = 0;
-    early_start();
+    chain_wait();
     // delta rounded toward -inf: for any float w,  w > delta  <=>  w > thr
     if (FOLD) {
         const double s = fold_parts(carve(ws_raw, 0).part_sum, P.item[0].parts, red, turn);
@@ -605,7 +605,7 @@ codes_fold_kernel(const __grid_constant__ Launch<N> P, void *ws_raw)
     __shared__ Reduce red;
     __shared__ unsigned long long red_cnt64[2][kSweepWarps];
     unsigned int turn = 0;
-    early_start();
+    chain_wait();
     fold_kept(P.item[blockIdx.x], carve(ws_raw, (int)blockIdx.x), red, red_cnt64, turn);
 }
 
@@ -998,7 +998,7 @@ sgd_update_kernel(const __grid_constant__ SgdLaunch<N> P, void *ws_raw)
         pdl_begin();
         cluster_arrive();
     } else {
-        early_start();
+        chain_wait();
     }
     for (unsigned int g = blockIdx.x; g < P.blocks; g += gridDim.x) {
         int t = 0;
@@ -1060,7 +1060,7 @@ sgd_fold_kernel(const __grid_constant__ SgdLaunch<N> P, void *ws_raw)
 {
     __shared__ Reduce red;
     unsigned int turn = 0;
-    early_start();
+    chain_wait();
     const int t = (int)blockIdx.x;
     const SgdItem &it = P.item[t];
     if (!it.stats) return;
