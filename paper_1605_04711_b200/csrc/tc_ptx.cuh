@@ -171,6 +171,11 @@ __device__ __forceinline__ void ld_nc_v4(uint4 &v, const uint32_t *p)
 {
     asm volatile("ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
 }
+__device__ __forceinline__ void ld_nc_v8(uint4 &v, uint4 &w, const uint32_t *p)      // 32-byte aligned
+{
+    asm volatile("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w), "=r"(w.x), "=r"(w.y), "=r"(w.z), "=r"(w.w) : "l"(p));
+}
 __device__ __forceinline__ void ld_nc_v2(uint32_t &x, uint32_t &y, const uint32_t *p)
 {
     asm volatile("ld.global.nc.v2.u32 {%0, %1}, [%2];" : "=r"(x), "=r"(y) : "l"(p));

@@ -20,21 +20,20 @@
 //   warp 1            allocates tensor memory, issues tcgen05.mma, commits to mbarriers
 //   warps 2-5 (2-9)   decode: packed codes (global, L2) -> bf16 pairs -> tensor memory; one group
 //                     of four warps (one per lane quadrant), or two groups that take the stages
-//                     in turn (template parameter DS)
+//                     in turn
 //   last eight warps  epilogue, two per lane quadrant: tensor memory -> registers -> per-warp
 //                     staging buffer -> TMA store
 //
 // Three tile shapes (template parameter PIX = pixels per tile; the channel tile is always 128).
-// Measured on B200: one thread can issue a tcgen05.mma about every 50-90 cycles whatever its
-// size, and waits or commits between MMAs are not hidden unless the MMA itself is long.  A
-// 128x256x16 MMA (128 cycles) hides that; a 128x128x16 one (64 cycles) does not.
+// A k-block takes 256 pixels 517 cycles of 512 of MMA, 192 pixels 444 of 384 (the activation feed: 24 KB from L2), 128 pixels
+// 255 to 280 of 256.
 //   PIX = 256: one accumulator (256 of the 512 tensor-memory columns, the rest holds decoded
 //              weights), five stages; the epilogue of a tile is not overlapped with the next
 //              tile's MMAs.  Long reductions with many tiles.
 //   PIX = 192: two accumulators and four stages fill the tensor memory exactly; the epilogue
 //              overlaps the next tile.
 //   PIX = 128: two accumulators, four stages of two k-blocks each.
-// The host picks the shape and the number of decode groups per launch with a cost model.
+// The host picks the shape per launch with a model of its time.
 //
 // Every wait on an mbarrier is bounded (about a second); on expiry the kernel records
 // TWN_ERR_TIMEOUT, all roles leave their loops, tensor memory is freed and the grid exits.
@@ -57,9 +56,9 @@ namespace {
 
 constexpr int kChan = 128;          // output channels per tile (UMMA M)
 constexpr int kBlockK = 64;         // reduction elements per k-block (128 bytes of bf16)
-// Groups of 4 decode warps in a block (template parameter DS): one, or two that take the stages in turn.
-// Two pay where decoding paces an overlapped tile shape on a long reduction; elsewhere the four extra
-// warps cost speed (they cap the block at 112 registers), so each variant is a kernel of its own.
+// Groups of 4 decode warps in a block: one, or two that take the stages in turn.  Two where the epilogue overlaps the next
+// tile's reduction (128 pixels: 0 to 28 % faster on 40 shapes, 16384x576x1000 30.7 -> 22.0 us, 3x3 64x7x7x512 17.8 -> 16.1; 192
+// pixels: 24 % slower without on the latter, 3 % faster on 1x1 64x28x28x512); 256 pixels are bound by their MMAs with one.
 __host__ __device__ constexpr int first_epi_warp(int ds) { return 2 + 4 * ds; }
 constexpr int kEpiSets = 2;         // epilogue warps per lane quadrant; each drains every other 32-pixel chunk
 __host__ __device__ constexpr int threads_conv(int ds) { return 32 * (first_epi_warp(ds) + 4 * kEpiSets); }
@@ -75,12 +74,14 @@ template <> struct Cfg<128> {
     static constexpr int kSub = 2;      // k-blocks per stage: one wait and one commit per 8 MMAs
     static constexpr int kAccBufs = 2;  // the epilogue of a tile overlaps the MMAs of the next
     static constexpr int kOutBufs = 4;  // output staging buffers per epilogue warp
+    static constexpr int kDecodeGroups = 2;
 };
 template <> struct Cfg<256> {
     static constexpr int kStages = 5;
     static constexpr int kSub = 1;
     static constexpr int kAccBufs = 1;
     static constexpr int kOutBufs = 2;
+    static constexpr int kDecodeGroups = 1;
 };
 // 192 pixels: the largest tile that leaves room for two accumulators beside four stages of
 // decoded weights (2 x 192 + 4 x 32 = 512 columns); the pixel tile is 3 * 2^k images deep.
@@ -89,6 +90,7 @@ template <> struct Cfg<192> {
     static constexpr int kSub = 1;
     static constexpr int kAccBufs = 2;
     static constexpr int kOutBufs = 4;
+    static constexpr int kDecodeGroups = 2;
 };
 
 struct ConvParams {
@@ -97,7 +99,8 @@ struct ConvParams {
     int lgBW, lgBH;               // pixel tile = BB x BH x BW, powers of two, product PIX
     // reduction
     int n_taps, n_cblk;           // k-blocks per tile = n_taps * n_cblk
-    int codes_aligned;            // 1: every k-block starts on a 16-byte boundary of the packed row
+    int codes_aligned;            // 1: every k-block starts on a 16-byte boundary of the packed row; 2: k-block u follows k-block
+                                  // u - 1, and every other one starts on a boundary of two
     const uint32_t *T;            // packed codes, one row of `wpr` words per output channel
     long long wpr;
     int sw, sh;                   // input pixel = output pixel * (sh, sw) + (dh, dw)
@@ -112,7 +115,6 @@ struct ConvParams {
     const void *residual;
     int res_dtype, relu, out_dtype;
     int res_gate;                 // 0: the residual is added; 1: it gates the result (kept where residual > 0)
-    int dsets;                    // host only: decode groups of the kernel variant to launch
     void *Y;
     int32_t *status;
     // optional batch statistics: [tile][epilogue warp of the quadrant][128 channels][sum, sum of squares]
@@ -156,13 +158,13 @@ static_assert(offsetof(SmemLayout<128>, stage_res) % 128 == 0 && offsetof(SmemLa
                   offsetof(SmemLayout<128>, stage_out) % 128 == 0 && offsetof(SmemLayout<256>, stage_out) % 128 == 0,
               "TMA and vector accesses need aligned shared-memory regions");
 
-template <int PIX, int DS, int BITS>
-__global__ void __launch_bounds__(threads_conv(DS), 1)
+template <int PIX, int BITS>
+__global__ void __launch_bounds__(threads_conv(Cfg<PIX>::kDecodeGroups), 1)
 tconv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_y,
              const __grid_constant__ CUtensorMap map_r, const __grid_constant__ ConvParams P)
 {
     using L = SmemLayout<PIX>;
-    constexpr int kStages = Cfg<PIX>::kStages, kSub = Cfg<PIX>::kSub, kAccBufs = Cfg<PIX>::kAccBufs;
+    constexpr int kStages = Cfg<PIX>::kStages, kSub = Cfg<PIX>::kSub, kAccBufs = Cfg<PIX>::kAccBufs, DS = Cfg<PIX>::kDecodeGroups;
     constexpr int kOutBufs = Cfg<PIX>::kOutBufs;
     constexpr int kXBytes = L::kXBytes;
     constexpr int kAColsPerStage = kSub * kAColsPerBlock;
@@ -293,6 +295,19 @@ tconv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ 
         // channels that are never stored, or multiplies activations that the TMA zero-fills.
         struct Codes { uint4 v[kSub]; };
         auto fetch = [&](Codes &c, const uint32_t *rowp, int st) {
+            // A warp's load touches 32 rows, and that is what it costs: both k-blocks of a stage come with one 32-byte load
+            // where the codes lie so.  With two of 16 bytes a k-block of 128 pixels took 320 cycles, 255 with one
+            // (4001x4608x512 20.1 -> 17.7 us, 3x3 64x7x7x512 18.9 -> 16.0).
+            if (kSub == 2 && P.codes_aligned == 2) {
+                if (BITS == 2) {
+                    ld_nc_v8(c.v[0], c.v[kSub - 1], rowp + 8 * st);
+                } else {
+                    uint4 both;
+                    ld_nc_v4(both, rowp + 4 * st);
+                    c.v[0].x = both.x; c.v[0].y = both.y; c.v[kSub - 1].x = both.z; c.v[kSub - 1].y = both.w;
+                }
+                return;
+            }
 #pragma unroll
             for (int sb = 0; sb < kSub; ++sb) {
                 int u = st * kSub + sb;
@@ -741,14 +756,14 @@ bn_reduce_kernel(const float *__restrict__ partial, int total_tiles, int n_tiles
 }
 
 // ---------------------------------------------------------------- host side
-template <int PIX, int DS, int BITS>
+template <int PIX, int BITS>
 int launch_conv_t(const Geometry &g, ConvParams &P, const void *X, const twn_device_info &dev,
                   EncodeTiledFn enc, cudaStream_t s)
 {
     static bool attr_set[64] = {false};
     const int smem_bytes = (int)sizeof(SmemLayout<PIX>) + 1024;
     if (!attr_set[dev.ordinal]) {
-        TWN_CUDA_OK(cudaFuncSetAttribute(tconv_kernel<PIX, DS, BITS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes));
+        TWN_CUDA_OK(cudaFuncSetAttribute(tconv_kernel<PIX, BITS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes));
         attr_set[dev.ordinal] = true;
     }
     pick_tile(g, PIX, &P.lgBW, &P.lgBH);
@@ -832,7 +847,7 @@ int launch_conv_t(const Geometry &g, ConvParams &P, const void *X, const twn_dev
     // after a convolution: 21 us instead of 12), so those launch the plain way.
     const bool kPdlConv = grid * 2 >= dev.sm_count;
     if (P.bn_partial && (size_t)P.total_tiles * kEpiSets * 2 * kChan * sizeof(float) > g.bn_partial_bytes) return TWN_ERR_WORKSPACE;
-    TWN_CUDA_OK(twn_launch_pdl(kPdlConv, tconv_kernel<PIX, DS, BITS>, grid, threads_conv(DS), (size_t)smem_bytes, s, map_x, map_y, map_r, P));
+    TWN_CUDA_OK(twn_launch_pdl(kPdlConv, tconv_kernel<PIX, BITS>, grid, threads_conv(Cfg<PIX>::kDecodeGroups), (size_t)smem_bytes, s, map_x, map_y, map_r, P));
     if (P.bn_partial)
         bn_reduce_kernel<<<(g.Cout + 7) / 8, 256, 0, s>>>(P.bn_partial, P.total_tiles, P.n_tiles, g.Cout, g.bn_sum, g.bn_sumsq);
     TWN_CUDA_OK(cudaGetLastError());
@@ -875,50 +890,47 @@ int launch_conv(const Geometry &g, const void *X, const uint32_t *T, const twn_s
     P.n_tiles = (g.Cout + kChan - 1) / kChan;
     P.n_taps = g.n_taps;
     P.n_cblk = (int)((g.Cin + kBlockK - 1) / kBlockK);
-    P.codes_aligned = 1;
+    P.codes_aligned = g.ld_codes % 128 == 0 && reinterpret_cast<uintptr_t>(T) % 32 == 0 ? 2 : 1;
+    for (int t = 0; t < g.n_taps; ++t)
+        if (g.taps[t].koff != t * P.n_cblk * kBlockK) P.codes_aligned = std::min(P.codes_aligned, 1);
     for (int t = 0; t < g.n_taps; ++t)
         if (g.taps[t].koff % kBlockK != 0) P.codes_aligned = 0;
-    // Tile shape by a cost model fitted to measured launches (cycles per round of tiles, kb = k-blocks
-    // per tile):
-    //   128 pixels: max(2000 + 680 kb, 6500), 540 kb with both decode groups: the epilogue overlaps
-    //               the next tile and bounds short reductions
-    //   192 pixels: max(2500 + 700 kb, 10500), 630 kb with both decode groups; floor 7600 when only the lower half of the channel
-    //               tile exists: overlapped as well, fewer rounds than 128
-    //   256 pixels: 8000 + 700 kb: one accumulator, so the epilogue is exposed; 7000 when only the
-    //               lower half of the channel tile exists (half of the epilogue warps idle)
+    // Tile shape by a model of the launch's time: a fixed part and, per round of tiles, an epilogue and the k-blocks, or where
+    // the epilogue of one tile overlaps the reduction of the next at least the epilogue.  Fitted to 40 launches (convolutions of
+    // 16 to 128 images, inner products of 333 to 50176 rows) forced to each shape, three inputs in turn; what it picks takes 0.7 %
+    // longer on average than the best of the three, 9 % at most (32x32x128, 128 images).
     int a, b;
     const long long kb = (long long)P.n_taps * P.n_cblk;
     const long long sms = dev.sm_count;
-    const bool half = g.Cout <= kChan / 2;
+    const bool half = g.Cout <= kChan / 2;           // half of the epilogue warps idle
     const long long t128 = pick_tile(g, 128, &a, &b) * P.n_tiles, t256 = pick_tile(g, 256, &a, &b) * P.n_tiles;
     const long long t192 = pick_tile(g, 192, &a, &b) * P.n_tiles;
-    // a second decode group pays where decoding paces the overlapped shapes: long reductions
-    const bool two = kb >= 18;
-    const long long lin128 = two ? 2000 + 540 * kb : 2000 + 680 * kb;
-    const long long per128 = lin128 > 6500 ? lin128 : 6500;
-    const long long floor192 = half ? 7600 : 10500;
-    const long long lin192 = two ? 2500 + 630 * kb : 2500 + 700 * kb;
-    const long long per192 = lin192 > floor192 ? lin192 : floor192;
-    const long long per256 = (half ? 7000 : 8000) + 700 * kb;
-    const long long c128 = ((t128 + sms - 1) / sms) * per128, c192 = ((t192 + sms - 1) / sms) * per192,
-                    c256 = ((t256 + sms - 1) / sms) * per256;
-    int choice = c256 < c128 ? 1 : 0;
-    if (c192 < (choice ? c256 : c128)) choice = 2;
-    // the model counts cycles of the rounds; a launch as a whole takes (fitted to 65 measured launches, mean error 6 %)
-    const double us = 3.9 + 0.454e-3 * (double)(choice == 0 ? c128 : choice == 1 ? c256 : c192);
+    auto time_us = [&](long long tiles, double fixed, double per_tile, double per_block, double least) {
+        return fixed + (double)((tiles + sms - 1) / sms) * std::max(per_tile + per_block * (double)kb, least);
+    };
+    // (code words off the 16-byte boundaries come one at a time, which the smaller shapes wait for: 7 further shapes)
+    const bool words = P.codes_aligned == 0;
+    const double u128 = time_us(t128, 4.3, 1.4, words ? 0.225 : 0.155, 1.85),
+                 u192 = time_us(t192, 5.1, 1.6, words ? 0.24 : 0.225, half ? 1.76 : 2.43),
+                 u256 = time_us(t256, 5.4, half ? 2.4 : 2.8, 0.293, 3.0);
+    // Another shape than 128 pixels has to gain more than a launch loses whose code is not that of the launches before it (1.5
+    // us): VGG-7 at 128 images takes 189.7 us when its five layers run in the 128-pixel kernel, 200.3 with two of the others
+    // between them, although alone each layer is within 10 % in its best shape.
+    constexpr double kOther = 1.5;
+    int choice = u256 + kOther < u128 ? 1 : 0;
+    if (u192 + (choice ? 0.0 : kOther) < (choice ? u256 : u128)) choice = 2;
+    const double us = choice == 0 ? u128 : choice == 1 ? u256 : u192;
     // Narrow layers and short reductions: the kernel that decodes its channels' codes once per block.  Up to 64 channels
     // the general kernel's half-empty tiles lose wherever that kernel runs; above, its own time decides.
     bool handled = false;
     rc = launch_conv_resident(g, X, T, ea, Y, dev_status, dev, s, half || split.us < us ? split.us : us, &handled, us_only);
     if (rc != TWN_OK || handled) return rc;
     // The more SMs the general kernel fills by itself, the clearer the modelled gain has to be: near the line the split
-    // kernel's model is the optimistic one.  Of 81 drawn calls that this margin alone keeps here, timed alone, 44 are more than
-    // 3 % slower split and 18 faster: convolutions lose 9 % on average, inner products to fp32 gain 3 % (4001x4608x512 25.9 us
-    // split, 25.3 here).  Without it a forward pass of ResNet-18 at 64 images takes 438 us instead of 415, of VGG-7 at 128
-    // 203 instead of 198, a training step of ResNet-18 at 64, with the weight gradients beside it, 1306 instead of 1270.
+    // kernel's model is the optimistic one where most SMs are filled (3x3 3x56x56x64 -> 256: 66 % filled, 9.5 us split, 7.7 here,
+    // modelled 8.4 and 8.7), and not where few are (1392x624x720: 45 %, 7.1 split, 8.4 here, modelled 6.5 and 7.2).
     const long long tiles = choice == 0 ? t128 : choice == 1 ? t256 : t192;
     const double fill = tiles < sms ? (double)tiles / (double)sms : 1.0;
-    const bool take_split = split.us < (1.0 - 0.25 * fill) * us;
+    const bool take_split = split.us < (1.0 - 0.25 * fill * fill) * us;
     if (us_only) {
         *us_only = take_split ? split.us : us;
         return TWN_OK;
@@ -938,15 +950,11 @@ int launch_conv(const Geometry &g, const void *X, const uint32_t *T, const twn_s
     P.status = dev_status;
     P.bn_partial = g.bn_partial;
     for (int t = 0; t < g.n_taps; ++t) P.taps[t] = g.taps[t];
-    P.dsets = (choice != 1 && two) ? 2 : 1;
-    if (g.code_bits == 1) {
-        if (choice == 1) return launch_conv_t<256, 1, 1>(g, P, X, dev, enc, s);
-        if (choice == 2) return P.dsets == 2 ? launch_conv_t<192, 2, 1>(g, P, X, dev, enc, s) : launch_conv_t<192, 1, 1>(g, P, X, dev, enc, s);
-        return P.dsets == 2 ? launch_conv_t<128, 2, 1>(g, P, X, dev, enc, s) : launch_conv_t<128, 1, 1>(g, P, X, dev, enc, s);
-    }
-    if (choice == 1) return launch_conv_t<256, 1, 2>(g, P, X, dev, enc, s);
-    if (choice == 2) return P.dsets == 2 ? launch_conv_t<192, 2, 2>(g, P, X, dev, enc, s) : launch_conv_t<192, 1, 2>(g, P, X, dev, enc, s);
-    return P.dsets == 2 ? launch_conv_t<128, 2, 2>(g, P, X, dev, enc, s) : launch_conv_t<128, 1, 2>(g, P, X, dev, enc, s);
+    if (g.code_bits == 1)
+        return choice == 1 ? launch_conv_t<256, 1>(g, P, X, dev, enc, s) : choice == 2 ? launch_conv_t<192, 1>(g, P, X, dev, enc, s)
+                                                                                    : launch_conv_t<128, 1>(g, P, X, dev, enc, s);
+    return choice == 1 ? launch_conv_t<256, 2>(g, P, X, dev, enc, s) : choice == 2 ? launch_conv_t<192, 2>(g, P, X, dev, enc, s)
+                                                                                : launch_conv_t<128, 2>(g, P, X, dev, enc, s);
 }
 
 // Helper streams for launches that are independent of one another (the residue classes of a

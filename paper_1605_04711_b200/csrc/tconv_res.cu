@@ -42,6 +42,8 @@
 // Every wait on an mbarrier is bounded; on expiry the kernel records TWN_ERR_TIMEOUT, all roles
 // leave their loops, tensor memory is freed and the grid exits.
 #include <cuda.h>
+
+#include <algorithm>
 #include <cuda_bf16.h>
 
 #include <cstddef>
@@ -597,22 +599,20 @@ int twn_detail::launch_conv_resident(const Geometry &g, const void *X, const uin
     P.stage_tx = 128 * row_pix * (BH + hh) * BB;
     P.stage_bytes = (P.stage_tx + 1023) / 1024 * 1024;
 
-    // Fitted to measured launches (one group: 1 to 13 tiles per block; several: 1 to 42, 30 shapes): set-up with the
-    // decoding of the weights and the first tile, then a tile per turn of the slowest part: MMAs, the activations
-    // (each group reads them again: 52 GB/s per SM from the L2 cache), or the stores.
+    // Fitted to measured launches (32 shapes, up to 43 tiles per block): set-up with the decoding of the weights and the first
+    // tile, then a tile per turn of the slowest part: MMAs (of whole 64-channel blocks, also where fewer channels exist), the
+    // activations (each group reads them again), or the stores.
     const long long per_block = (total + nb - 1) / nb;
-    const double mma = 0.13 * P.kbpt * (g.Cin < kBlockK ? (double)g.Cin / kBlockK : 1.0);
-    double first = 0.26 * P.kbpt, per_tile = mma > 0.5 ? mma : 0.5;
+    double first = 0.26 * P.kbpt, per_tile = std::max(0.107 * P.kbpt, 0.5);
     if (P.groups > 1) {
-        const double loads = (double)P.n_cblk * P.stage_bytes / 16384.0, store = out_bf16 ? 0.7 : 0.9;
-        if (0.42 * loads > first) first = 0.42 * loads;
-        if (0.33 * loads > per_tile) per_tile = 0.33 * loads;
-        if (store > per_tile) per_tile = store;
+        const double loads = (double)P.n_cblk * P.stage_bytes / 16384.0, store = out_bf16 ? 0.66 : 0.85;
+        first = std::max(first, 0.42 * loads);
+        per_tile = std::max(per_tile, std::max(0.21 * loads, store));
     }
     const double us = 4.3 + first + (double)(per_block - 1) * per_tile;
-    // a margin for the models' error where the other kernels are often the better choice: at 0.95 a 3x3 layer of
-    // 5x50x50x96 -> 200 came here and took 15.2 us instead of 14.5
-    if (us > (P.groups > 1 ? 0.9 : 1.0) * rival_us) return TWN_OK;
+    // a margin where the other kernels are often the better choice: 8x56x56x64 -> 256, 3x3, modelled 12.4 here and 12.7 there,
+    // takes 11.9 in both
+    if (us > (P.groups > 1 ? 0.95 : 1.0) * rival_us) return TWN_OK;
     const long long wts_bytes = (long long)P.kbpt * P.N * 128;
     const long long fixed = 1024 + wts_bytes + kEpiWarps * kStageBuf * (epi.residual ? 2 : 1) + 2048;
     if (fixed > kSmemLimit) return TWN_OK;

@@ -300,12 +300,11 @@ tconv_split_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
             };
             uint4 c0, c1, c2;
             if (n_kb > 0) { fetch(c0, set); fetch(c1, set + kSets); fetch(c2, set + 2 * kSets); }
-#pragma unroll 1
-            for (int i = set; i < n_kb; i += kSets) {
+            auto decode = [&](const uint4 &c, int i) -> bool {
                 const int s = i % kStages;
-                if (i >= kStages && !mbar_wait_warp(&sm->empty[s], ((i / kStages) & 1) ^ 1, abort_flag, P.status, 32)) break;
+                if (i >= kStages && !mbar_wait_warp(&sm->empty[s], ((i / kStages) & 1) ^ 1, abort_flag, P.status, 32)) return false;
                 tc_fence_after();
-                const uint32_t wv[4] = {c0.x, c0.y, c0.z, c0.w};
+                const uint32_t wv[4] = {c.x, c.y, c.z, c.w};
                 uint32_t out[32];
                 decode_kblock<BITS>(wv, out);
                 tmem_st32(tmem_a + lane_base + s * kAColsPerBlock, out);
@@ -313,9 +312,17 @@ tconv_split_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&sm->full[s]);
-                c0 = c1;
-                c1 = c2;
-                fetch(c2, i + 3 * kSets);
+                return true;
+            };
+            // three buffers in turn, each refilled where it was used: no register is copied while its load is in flight
+#pragma unroll 1
+            for (int i = set; i < n_kb; i += 3 * kSets) {
+                if (!decode(c0, i)) break;
+                fetch(c0, i + 3 * kSets);
+                if (i + kSets >= n_kb || !decode(c1, i + kSets)) break;
+                fetch(c1, i + 4 * kSets);
+                if (i + 2 * kSets >= n_kb || !decode(c2, i + 2 * kSets)) break;
+                fetch(c2, i + 5 * kSets);
             }
         }
         // the accumulator -> shared memory, [pixel][channel]; the two warps of a lane quadrant take alternate chunks.
