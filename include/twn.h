@@ -349,6 +349,18 @@ int twn_conv2d_fwd(const twn_conv_desc_t *desc, const void *X, const uint32_t *T
                    int32_t *dev_status, twn_stream_t stream);
 
 /*
+ * twn_conv2d_fwd and the 2x2 max pooling (stride 2, no padding) of its output:
+ *   Yp     bf16 NHWC [B, Ho / 2, Wo / 2, Cout], what twn_maxpool2d_fwd makes of Y with k = stride = 2 (no
+ *          argmax: for inference), 4-byte aligned.
+ * epi is needed, with out_dtype = TWN_BF16, and Ho, Wo >= 2.  One launch where the layer's size suits it
+ * (the windows are taken from the output while it is on chip), two otherwise; Y and Yp are the same
+ * either way, but for sums that one kernel splits and another does not (see TWN_SUM_IN_ORDER).
+ */
+int twn_conv2d_fwd_maxpool(const twn_conv_desc_t *desc, const void *X, const uint32_t *T_fwd, int64_t ld_codes,
+                           const twn_stats_t *stats, const twn_epilogue_t *epi, void *Y, void *Yp,
+                           int32_t *dev_status, twn_stream_t stream);
+
+/*
  * twn_conv2d_fwd that also returns the batch statistics of its output, for the batch normalisation
  * that follows every ternary convolution while the network is trained (Sec. 2.4; the block of Fig. 1):
  *   bn_sum[o]   = sum over (b, ho, wo) of z[b,ho,wo,o]

@@ -245,6 +245,24 @@ __device__ __forceinline__ void ldmatrix_x4_trans(uint32_t saddr, uint32_t (&w)[
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
                  : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]) : "r"(saddr) : "memory");
 }
+__device__ __forceinline__ uint4 ld_shared_v4(uint32_t saddr)
+{
+    uint4 v;
+    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(saddr) : "memory");
+    return v;
+}
+// The maximum of a pooling window, two channels per word: as the pooling kernels take it (the first of equals, a NaN never wins).
+__device__ __forceinline__ uint32_t max_first_bf16x2(uint32_t best, uint32_t x)
+{
+    const uint32_t m = __hgt2_mask(*reinterpret_cast<const __nv_bfloat162 *>(&x), *reinterpret_cast<const __nv_bfloat162 *>(&best));
+    return (x & m) | (best & ~m);
+}
+// A maximum that is still at -inf is written as zero.
+__device__ __forceinline__ uint32_t no_max_to_zero(uint32_t best)
+{
+    const uint32_t low = 0xFF80FF80u;
+    return best & ~__heq2_mask(*reinterpret_cast<const __nv_bfloat162 *>(&best), *reinterpret_cast<const __nv_bfloat162 *>(&low));
+}
 __device__ __forceinline__ void st_shared_b32(uint32_t saddr, uint32_t v)
 {
     asm volatile("st.shared.b32 [%0], %1;" ::"r"(saddr), "r"(v) : "memory");

@@ -121,7 +121,10 @@ struct ConvParams {
     float *bn_partial;
     // output path: 1 = each epilogue warp stages its 32 channels x 32 pixels in shared memory and
     // writes them with a TMA store (box = 32 channels x sbw x sbh x sbb pixels); 0 = per-thread stores
-    int tma_store, lg_sbw, lg_sbh;
+    int tma_store;
+    // optional 2x2 max pooling of the output (with `fragments`): a chunk of 32 pixels is 2^lg_sbw x 2^lg_sbh x the rest images
+    __nv_bfloat16 *pool;
+    int PH, PW, lg_sbw, lg_sbh;
     int res_tma;                  // 1: the residual (bf16) is staged by per-warp TMA loads, two chunks deep
     int fragments;                // 1: bf16 in and out by TMA, no batch statistics: chunks are drained as matrix fragments
     Tap taps[kMaxTaps];
@@ -583,6 +586,28 @@ tconv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ 
                         tma_store_4d(&map_y, sbuf, c_n0, (p_w0 + (p0 & BWm)) * P.osw, (p_h0 + ((p0 >> P.lgBW) & BHm)) * P.osh,
                                      p_b0 + (p0 >> (P.lgBW + P.lgBH)));
                     }
+                    if (P.pool) {
+                        // The chunk's eight windows from the staged output: a lane takes one, eight channels of it.  A sweep of
+                        // its own reads the whole output again: 12.5 us for 128x32x32x128, 8.8 for 128x16x16x256, 5.7 for
+                        // 128x8x8x512; here 1.7, 1.5 and 0.7.
+                        const int o = (int)ln >> 2, cg = (int)ln & 3;
+                        const int ox = o & ((1 << (P.lg_sbw - 1)) - 1), oy = (o >> (P.lg_sbw - 1)) & ((1 << (P.lg_sbh - 1)) - 1),
+                                  ob = o >> (P.lg_sbw + P.lg_sbh - 2);
+                        const int q0 = (((ob << P.lg_sbh) + 2 * oy) << P.lg_sbw) + 2 * ox, p0 = c * 32;
+                        uint32_t best[4] = {0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u};
+#pragma unroll
+                        for (int t = 0; t < 4; ++t) {
+                            const int q = q0 + (t & 1) + ((t >> 1) << P.lg_sbw);
+                            const uint4 x = ld_shared_v4(smem_u32(sbuf) + q * 64 + ((cg ^ ((q >> 1) & 3)) << 4));
+                            best[0] = max_first_bf16x2(best[0], x.x); best[1] = max_first_bf16x2(best[1], x.y);
+                            best[2] = max_first_bf16x2(best[2], x.z); best[3] = max_first_bf16x2(best[3], x.w);
+                        }
+                        const int gx = ((p_w0 + (p0 & BWm)) >> 1) + ox, gy = ((p_h0 + ((p0 >> P.lgBW) & BHm)) >> 1) + oy,
+                                  gb = p_b0 + (p0 >> (P.lgBW + P.lgBH)) + ob, gc = c_n0 + 8 * cg;
+                        if (gx < P.PW && gy < P.PH && gb < P.Bv && gc < P.Cout)
+                            *reinterpret_cast<uint4 *>(P.pool + (((size_t)gb * P.PH + gy) * P.PW + gx) * P.Cout + gc) =
+                                make_uint4(no_max_to_zero(best[0]), no_max_to_zero(best[1]), no_max_to_zero(best[2]), no_max_to_zero(best[3]));
+                    }
                     ++nst;
                     continue;
                 }
@@ -840,6 +865,13 @@ int launch_conv_t(const Geometry &g, ConvParams &P, const void *X, const twn_dev
         }
     }
     P.fragments = P.fragments && P.tma_store;
+    if (g.pool) {
+        if (!P.fragments) return TWN_ERR_CUDA;       // the caller has looked at everything that could be in the way
+        P.pool = static_cast<__nv_bfloat16 *>(g.pool);
+        P.PH = g.Hv / 2; P.PW = g.Wv / 2;
+        P.lg_sbw = P.lgBW;
+        P.lg_sbh = std::min(P.lgBH, 5 - P.lgBW);
+    }
     if (P.fragments && P.residual && !P.res_tma) return TWN_ERR_CUDA;      // the same geometry could be encoded for Y
     const int grid = dev.sm_count < P.total_tiles ? dev.sm_count : P.total_tiles;
     // Programmatic dependent launch pays when the blocks cover the GPU (set-up and launch latency hide behind the
@@ -884,7 +916,7 @@ int launch_conv(const Geometry &g, const void *X, const uint32_t *T, const twn_s
     if ((long long)g.Bv * g.OH * g.OW * g.ldy >= 0xFFFFFFFFLL) return TWN_ERR_INVALID_ARG;
     const EpilogueArgs ea = epilogue_args(stats, epi, out_dtype_default);
     // problems that do not fill the GPU: small tiles, the reduction split over a cluster
-    const SplitPlan split = plan_conv_split(g, dev.sm_count / (g.beside > 1 ? g.beside : 1), ea.in_order);
+    const SplitPlan split = g.pool ? SplitPlan{0, 0, 1e30} : plan_conv_split(g, dev.sm_count / (g.beside > 1 ? g.beside : 1), ea.in_order);
     ConvParams P;
     memset(&P, 0, sizeof P);
     P.n_tiles = (g.Cout + kChan - 1) / kChan;
@@ -923,7 +955,7 @@ int launch_conv(const Geometry &g, const void *X, const uint32_t *T, const twn_s
     // Narrow layers and short reductions: the kernel that decodes its channels' codes once per block.  Up to 64 channels
     // the general kernel's half-empty tiles lose wherever that kernel runs; above, its own time decides.
     bool handled = false;
-    rc = launch_conv_resident(g, X, T, ea, Y, dev_status, dev, s, half || split.us < us ? split.us : us, &handled, us_only);
+    if (!g.pool) rc = launch_conv_resident(g, X, T, ea, Y, dev_status, dev, s, half || split.us < us ? split.us : us, &handled, us_only);
     if (rc != TWN_OK || handled) return rc;
     // The more SMs the general kernel fills by itself, the clearer the modelled gain has to be: near the line the split
     // kernel's model is the optimistic one where most SMs are filled (3x3 3x56x56x64 -> 256: 66 % filled, 9.5 us split, 7.7 here,
@@ -1068,10 +1100,11 @@ int conv_common_checks(const twn_conv_desc_t *d)
 namespace {
 
 struct BnArgs { double *sum, *sumsq; void *ws; size_t ws_bytes; };
+struct PoolArgs { void *Yp; bool *done; };
 
 int conv_fwd_impl(const twn_conv_desc_t *d, const void *X, const uint32_t *T_fwd, int64_t ld_codes,
                   const twn_stats_t *stats, const twn_epilogue_t *epi, void *Y,
-                  int32_t *dev_status, twn_stream_t stream, int bits, const BnArgs *bn = nullptr)
+                  int32_t *dev_status, twn_stream_t stream, int bits, const BnArgs *bn = nullptr, const PoolArgs *pool = nullptr)
 {
     int rc = conv_common_checks(d);
     if (rc != TWN_OK) return rc;
@@ -1106,6 +1139,27 @@ int conv_fwd_impl(const twn_conv_desc_t *d, const void *X, const uint32_t *T_fwd
         g.bn_partial = static_cast<float *>(bn->ws);
         g.bn_partial_bytes = bn->ws_bytes;
         g.bn_sum = bn->sum; g.bn_sumsq = bn->sumsq;
+    }
+    if (pool) {
+        // Pooled in the epilogue of the general kernel, if that and no sweep should take less time than the kernel that the layer
+        // would get by itself and a sweep (modelled as 2 us and 4.2 TB/s; 2.1 us for 100x8x8x64).  What TMA cannot store or the
+        // fragments do not hold stays with the sweep.
+        *pool->done = false;
+        const double bytes = 2.5 * (double)g.Bv * g.Hv * g.Wv * g.Cout;
+        if (epi && epi->out_dtype == TWN_BF16 && g.Cout % 8 == 0 && twn_aligned(Y, 16) && twn_aligned(pool->Yp, 16) &&
+            (!epi->residual || (epi->residual_dtype == TWN_BF16 && twn_aligned(epi->residual, 16)))) {
+            double apart = 0.0, here = 0.0;
+            rc = launch_conv(g, X, T_fwd, stats, epi, Y, TWN_F32, dev_status, twn_cu(stream), &apart);
+            if (rc != TWN_OK) return rc;
+            Geometry p = g;
+            p.pool = pool->Yp;
+            rc = launch_conv(p, X, T_fwd, stats, epi, Y, TWN_F32, dev_status, twn_cu(stream), &here);
+            if (rc != TWN_OK) return rc;
+            if (here < apart + 2.0 + bytes / 4.2e6) {
+                *pool->done = true;
+                return launch_conv(p, X, T_fwd, stats, epi, Y, TWN_F32, dev_status, twn_cu(stream));
+            }
+        }
     }
     return launch_conv(g, X, T_fwd, stats, epi, Y, TWN_F32, dev_status, twn_cu(stream));
 }
@@ -1144,6 +1198,22 @@ extern "C" int twn_conv2d_fwd(const twn_conv_desc_t *d, const void *X, const uin
                               int32_t *dev_status, twn_stream_t stream)
 {
     return conv_fwd_impl(d, X, T_fwd, ld_codes, stats, epi, Y, dev_status, stream, 2);
+}
+
+extern "C" int twn_conv2d_fwd_maxpool(const twn_conv_desc_t *d, const void *X, const uint32_t *T_fwd, int64_t ld_codes,
+                                      const twn_stats_t *stats, const twn_epilogue_t *epi, void *Y, void *Yp,
+                                      int32_t *dev_status, twn_stream_t stream)
+{
+    const int rc0 = conv_common_checks(d);
+    if (rc0 != TWN_OK) return rc0;
+    TWN_REQUIRE(Yp && epi && epi->out_dtype == TWN_BF16, TWN_ERR_INVALID_ARG);
+    const int64_t Ho = (d->H + 2 * d->pad_h - d->kh) / d->stride_h + 1, Wo = (d->W + 2 * d->pad_w - d->kw) / d->stride_w + 1;
+    TWN_REQUIRE(Ho >= 2 && Wo >= 2, TWN_ERR_INVALID_ARG);
+    TWN_REQUIRE(twn_aligned(Yp, 4), TWN_ERR_MISALIGNED);
+    bool done = false;
+    const PoolArgs pool = {Yp, &done};
+    const int rc = conv_fwd_impl(d, X, T_fwd, ld_codes, stats, epi, Y, dev_status, stream, 2, nullptr, &pool);
+    return rc != TWN_OK || done ? rc : twn_maxpool2d_fwd(Y, d->B, Ho, Wo, d->Cout, 2, 2, 0, Yp, nullptr, stream);
 }
 
 extern "C" int twn_conv2d_fwd_b1(const twn_conv_desc_t *d, const void *X, const uint32_t *B_fwd, int64_t ld_codes,

@@ -55,6 +55,8 @@ struct Geometry {
     int Cout;
     long long ld_codes, code_cols;  // packed row pitch and used columns
     int code_bits;   // 2: ternary codes, 16 per word; 1: binary codes, 32 per word
+    // 2x2 max pooling of the output, written beside it (optional): bf16 [Bv, Hv / 2, Wv / 2, Cout]
+    void *pool;
     // batch statistics of the pre-activation output (optional): per-tile partial sums, then the totals
     float *bn_partial;
     size_t bn_partial_bytes;
@@ -80,6 +82,8 @@ inline long long pick_tile(const Geometry &g, int pix, int *lgBW, int *lgBH)
         for (int b = 0; a + b <= lg; ++b) {
             const int BW = 1 << a, BH = 1 << b, BB = pix >> (a + b);
             if (BW * g.sw > 256 || BH * g.sh > 256 || BB > 256) continue;
+            // pooled from chunks of 32 pixels of a tile: those have to hold whole windows
+            if (g.pool && (a < 1 || a > 4 || b < 1)) continue;
             const long long tiles = ((g.Wv + BW - 1) / BW) * (long long)((g.Hv + BH - 1) / BH) * ((g.Bv + BB - 1) / BB);
             // prefer fewer tiles, then wider rows
             if (best < 0 || tiles < best || (tiles == best && a > bw)) { best = tiles; bw = a; bh = b; }

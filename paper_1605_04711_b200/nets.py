@@ -314,7 +314,8 @@ class TernaryNet(_Counted):
     def _forward_calls(self):
         """The calls of a forward pass, (kind, name, flops, entry point, arguments) each: a pass walks this list."""
         calls = []
-        for op in self.ops:
+        pooled = None            # the pooling that its layer's call has done
+        for op, after in zip(self.ops, [*self.ops[1:], ("end",)]):
             kind = op[0]
             if kind == "layer":
                 L: Layer = op[1]
@@ -330,10 +331,16 @@ class TernaryNet(_Counted):
                     calls.append((None, "", 0, "im2col", (L.desc, x, e["xcol"], L.ldk)))
                     calls.append((*row, "gemm", (e["xcol"], L.ldk, e["packed"], e["ld"], e["stats"], M, L.Cout, L.K, e["epi"],
                                                  y, L.Cout, self.status)))
+                elif not self.train and after[0] == "maxpool" and after[2:] == (L.name, 2, 2, 0) and after[1] not in self.aux:
+                    pooled = after[1]
+                    calls.append((*row, "conv2d_fwd_maxpool", (L.desc, x, e["packed"], e["ld"], e["stats"], e["epi"], y,
+                                                               self.act[pooled], self.status)))
                 else:
                     calls.append((*row, "conv2d_fwd", (L.desc, x, e["packed"], e["ld"], e["stats"], e["epi"], y, self.status)))
             elif kind == "maxpool":
                 _, name, src, k, s, p = op
+                if name == pooled:
+                    continue
                 x = self.act[src]
                 Bx, H, W, C = x.shape
                 calls.append((None, "", 0, "maxpool2d_fwd", (x, Bx, H, W, C, k, s, p, self.act[name], self.aux.get(name))))

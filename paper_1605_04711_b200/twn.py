@@ -272,6 +272,12 @@ def conv2d_fwd(desc: ConvDesc, X: torch.Tensor, T_fwd: torch.Tensor, ld_codes: i
     _check(_C.conv2d_fwd(desc, X, T_fwd, ld_codes, stats, epi, Y, dev_status, stream), "twn_conv2d_fwd")
 
 
+def conv2d_fwd_maxpool(desc: ConvDesc, X: torch.Tensor, T_fwd: torch.Tensor, ld_codes: int, stats, epi,
+                       Y: torch.Tensor, Yp: torch.Tensor, dev_status=None, stream=None) -> None:
+    """conv2d_fwd, and the 2x2 max pooling of its output into Yp (inference)."""
+    _check(_C.conv2d_fwd_maxpool(desc, X, T_fwd, ld_codes, stats, epi, Y, Yp, dev_status, stream), "twn_conv2d_fwd_maxpool")
+
+
 def conv2d_fwd_bn_workspace_bytes(desc: ConvDesc) -> int:
     return int(lib().twn_conv2d_fwd_bn_workspace_bytes(C.byref(desc)))
 
