@@ -586,7 +586,7 @@ tconv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ 
                         tma_store_4d(&map_y, sbuf, c_n0, (p_w0 + (p0 & BWm)) * P.osw, (p_h0 + ((p0 >> P.lgBW) & BHm)) * P.osh,
                                      p_b0 + (p0 >> (P.lgBW + P.lgBH)));
                     }
-                    if (P.pool) {
+                    if (PIX == 128 && P.pool) {
                         // The chunk's eight windows from the staged output: a lane takes one, eight channels of it.  A sweep of
                         // its own reads the whole output again: 12.5 us for 128x32x32x128, 8.8 for 128x16x16x256, 5.7 for
                         // 128x8x8x512; here 1.7, 1.5 and 0.7.
@@ -951,6 +951,9 @@ int launch_conv(const Geometry &g, const void *X, const uint32_t *T, const twn_s
     constexpr double kOther = 1.5;
     int choice = u256 + kOther < u128 ? 1 : 0;
     if (u192 + (choice ? 0.0 : kOther) < (choice ? u256 : u128)) choice = 2;
+    // Pooling is in that kernel alone: the others, whose epilogue is longer with it, lost 0.6 % on 16384x4096x4096 to code that
+    // they do not run.
+    if (g.pool) choice = 0;
     const double us = choice == 0 ? u128 : choice == 1 ? u256 : u192;
     // Narrow layers and short reductions: the kernel that decodes its channels' codes once per block.  Up to 64 channels
     // the general kernel's half-empty tiles lose wherever that kernel runs; above, its own time decides.

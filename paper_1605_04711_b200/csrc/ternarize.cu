@@ -13,7 +13,8 @@
 // All sums have a fixed order that depends on the shape of the tensor alone: a tensor is cut into at most
 // kMaxParts parts, every part is summed by one block in a fixed way (per-thread strided sums, shuffle tree per
 // warp, warps in order) and the parts are folded in a fixed way.  Which block takes a part does not matter, so a
-// tensor gets the same bits alone and in a batch, on any number of SMs.  No floating-point atomics.
+// tensor gets the same bits alone and in a batch, on any number of SMs (the kept sum of a tensor read once: an order that
+// depends on its values too, ternarize_once_kernel).  No floating-point atomics.
 #include <algorithm>
 
 #include "sweep.cuh"
