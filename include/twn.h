@@ -137,9 +137,13 @@ size_t twn_ternarize_workspace_bytes(void);
  * workspace/workspace_bytes  scratch of at least twn_ternarize_workspace_bytes(),
  *          256-byte aligned; contents need not be preserved or initialised.
  *          Two calls that overlap on the device must not share it.
- * The sums are fp64 with a fixed reduction order.  The comparison is done in
- * fp32 against delta rounded toward -inf, which decides exactly as the fp64
- * comparison does.  n = 0 gives delta = alpha = 0.
+ * The sums are fp64.  sum_abs (and with it delta) is added up in an order that rows,
+ * cols and delta_factor fix; sum_abs_kept and alpha are the bits that
+ * twn_ternarize_codes gives for the same weights and threshold.  (From 2^24 weights on
+ * a tensor may be read once, and its kept sum then has another order, but only where
+ * fp64 holds every partial sum without rounding: n <= 2^28 * delta_factor.)
+ * The comparison is done in fp32 against delta rounded toward -inf, which decides
+ * exactly as the fp64 comparison does.  n = 0 gives delta = alpha = 0.
  * Device status: TWN_ERR_NONFINITE if any W_i is NaN/Inf (other outputs
  * are then unspecified).
  */

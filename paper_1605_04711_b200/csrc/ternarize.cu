@@ -13,8 +13,8 @@
 // All sums have a fixed order that depends on the shape of the tensor alone: a tensor is cut into at most
 // kMaxParts parts, every part is summed by one block in a fixed way (per-thread strided sums, shuffle tree per
 // warp, warps in order) and the parts are folded in a fixed way.  Which block takes a part does not matter, so a
-// tensor gets the same bits alone and in a batch, on any number of SMs (the kept sum of a tensor read once: an order that
-// depends on its values too, ternarize_once_kernel).  No floating-point atomics.
+// tensor gets the same bits alone and in a batch.  The kept sum of a tensor that is read once has an order of its own, but no
+// rounding in it (read_once), so alpha is the same bits whichever call wrote it.  No floating-point atomics.
 #include <algorithm>
 
 #include "sweep.cuh"
@@ -617,8 +617,8 @@ codes_fold_kernel(const __grid_constant__ Launch<N> P, void *ws_raw)
 // the threshold is known, the weights of marked half-words that lie between it and `mid` get their other code, and sums and
 // counts are put right.  Of normal weights 1.4 % of the half-words are marked; most are kept in shared memory, the others read
 // again.  A threshold further than `half` from the estimate (an order of weights that the sample does not see, a NaN) costs a
-// second sweep.  The codes and counts are the same in any case; the kept sum is that of the sweep plus the corrections, in a
-// fixed order.
+// second sweep.  Codes, counts and kept sum are the same bits in any case: the kernel is not taken where the kept sum could be
+// rounded (read_once).
 // The sweep costs nearly as many issue slots as memory time, so a thread takes whole words (no exchange among lanes), their
 // kept bits are collected by the fp32 adders (as sums of powers of two) and their signs two at a time.
 //   12288 x 8192 (three tensors in turn) 137.7 -> 88.3 us, 66 at the copy rate.
@@ -887,7 +887,7 @@ ternarize_once_kernel(const __grid_constant__ Launch<1> P, void *ws_raw)
     if (b == 0 && tid == 0) write_threshold(it, s, delta);
     const float thr = __double2float_rd(delta);
 
-    if (fabsf(__fsub_rn(thr, mid)) <= half) {
+    if (fabsf(__fsub_rn(thr, mid)) <= half && thr <= 2.0f * mid) {     // (the second: read_once)
         // ---- put right what lies between.  x -> |x - mid| as computed here and in the sweep is monotonic on either side of
         // mid, so a weight between mid and thr is no further from mid than thr is: its half-word is marked.  A warp takes its own
         // marks, a lane every 32nd.
@@ -1414,10 +1414,18 @@ bool make_item(const float *W, int64_t rows, int64_t cols, twn_stats_t *stats, u
 }
 
 // Whether a tensor's codes and sums come from one read (ternarize_once_kernel): it is large enough for that to pay, every
-// block has one part, and the marks of a part fit.  Alone and in a batch alike, so that the sums are the same bits.
-bool read_once(const Item &it, const twn_device_info &dev)
+// block has one part, the marks of a part fit, and the kept sum is exact.  Alone and in a batch alike, so that the sums are the
+// same bits.
+// Exact: the sweep adds up what lies above the estimate and the corrections take it to the threshold, another order than that of
+// the coding sweep, which twn_ternarize_codes would put in its place for the same weights.  With the threshold in [2^e, 2^(e+1))
+// every fp32 magnitude above it, and above an estimate no more than a binade below, is a multiple of 2^(e-24), and no partial sum
+// exceeds sum |W| = n * threshold / factor <= 2^(e+1) * n / factor.  So for n <= 2^28 * factor all partial sums are whole
+// multiples of 2^(e-24) below 2^53 of them: fp64 holds each without rounding, and every order gives the same bits.  (Factor 0.7:
+// 188 million weights, factor 0.0625: 2^24.)  An estimate further below than that is a miss, whatever its window.
+bool read_once(const Item &it, double factor, const twn_device_info &dev)
 {
-    return it.n >= kOnceWeights && it.parts <= (unsigned int)(dev.sm_count * kSweepBlocksPerSm) && it.part_words <= kOnceGroups * 512;
+    return it.n >= kOnceWeights && (double)it.n <= 0x1p28 * factor && it.parts <= (unsigned int)(dev.sm_count * kSweepBlocksPerSm) &&
+           it.part_words <= kOnceGroups * 512;
 }
 
 int launch_once(Launch<1> &P, double factor, void *ws, const twn_device_info &dev, cudaStream_t s)
@@ -1454,7 +1462,7 @@ int launch_sweeps(Launch<N> &P, double factor, void *ws, cudaStream_t s)
                         : q <= 4 ? ternarize_small_kernel<4, SUMS> : ternarize_small_kernel<8, SUMS>;
             return launch_cluster(kernel, grid, s, P);
         }
-        if (SUMS && read_once(P.item[0], dev)) return launch_once(P, factor, ws, dev, s);
+        if (SUMS && read_once(P.item[0], factor, dev)) return launch_once(P, factor, ws, dev, s);
     }
     const unsigned int grid = std::min(P.parts, (unsigned int)(dev.sm_count * kSweepBlocksPerSm));
     if (SUMS) TWN_CUDA_OK(twn_launch_pdl(true, sums_kernel<N>, (int)grid, kSweepThreads, 0, s, P, ws));
@@ -1553,7 +1561,7 @@ extern "C" int twn_ternarize_batch(const twn_ternarize_item_t *items, int count,
     // tensors that are read once have launches of their own
     int rest = 0;
     for (int t = 0; t < count; ++t) {
-        if (!read_once(P.item[t], dev)) {
+        if (!read_once(P.item[t], delta_factor, dev)) {
             if (rest != t) P.item[rest] = P.item[t];
             ++rest;
             continue;

@@ -52,6 +52,32 @@ def test_nonfinite_weights_are_reported(bad):
     assert twn.stats_to_host(stats)["status"] == -4
 
 
+@pytest.mark.parametrize("kind,factor", [("normal", 0.7), ("normal", 0.0625), ("tiny", 2.0 ** -45)])
+@pytest.mark.parametrize("rows,cols", [(4096, 4096), (4099, 4111)])
+def test_the_coding_sweep_alone_gives_the_same_bits(rows, cols, kind, factor):
+    """Codes, kept sum and scale of twn_ternarize are those of twn_ternarize_codes against the same threshold.  Where fp64 cannot
+    hold the kept sum: a 1 in every 512 weights, so that a sample sees what there is, and beside it weights of 3 * 2^-52, all kept.
+    A partial sum from 4 on rounds each of them up by 2^-52, so the sum depends on how many a thread adds to which partial sum."""
+    if kind == "normal":
+        W = dev_f32(weights(rows, cols, "normal"))
+    else:
+        W = torch.full((rows * cols,), 3 * 2.0 ** -52, dtype=torch.float32, device="cuda")
+        W[::512] = 1.0
+        W = W.view(rows, cols)
+    ld = twn.ld_for(cols)
+    both = []
+    for call in (twn.ternarize, None):
+        packed = torch.zeros((rows, ld // 16), dtype=torch.int32, device="cuda")
+        if call:
+            stats = twn.new_stats()
+            twn.ternarize(W, factor, stats, packed, ld, None, workspace(twn.ternarize_workspace_bytes()))
+        else:
+            stats = both[0][0].clone()
+            twn.ternarize_codes(W, rows, cols, stats, packed, ld, None, workspace(twn.ternarize_workspace_bytes()))
+        both.append((stats, packed))
+    assert torch.equal(both[0][0], both[1][0]) and torch.equal(both[0][1], both[1][1])
+
+
 def test_weights_off_the_32_byte_boundaries_and_batches():
     """The same bits alone, in a batch beside small tensors, and from a base that is aligned to 16 bytes only."""
     W = dev_f32(weights(4096, 4096, "normal"))
