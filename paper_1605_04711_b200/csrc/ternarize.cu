@@ -624,9 +624,13 @@ codes_fold_kernel(const __grid_constant__ Launch<N> P, void *ws_raw)
 //   12288 x 8192 (three tensors in turn) 137.7 -> 88.3 us, 66 at the copy rate.
 // Where one read pays: 9.2 million weights in rows of 2301, cold, 28.9 us so, 27.0 in two sweeps; 14.2 million 24.9 / 26.7; 18.9 million 28.9 / 33.0
 // (27.3 / 26.9 where they are in L2 from the call before); 33.6 million 39.1 / 51.5; rows of 8001 weights 145 / 192.
+// Where it loses: a threshold outside the window (sorted weights, large ones that no run of the sample sees) 151 to 154 us against
+// 136 in two sweeps, 33.6 million weights 60 / 49; every weight at the threshold 156 / 136.  Normal, Laplace, uniform, sparse
+// weights, rows of different scale, outliers 84 to 92, Cauchy 99.
 constexpr unsigned long long kOnceWeights = 16ull << 20;
 constexpr unsigned int kOnceGroups = 128;        // groups of 512 words in a part (310 million weights in all)
 constexpr unsigned int kOnceKept = 64;           // marked half-words that a warp keeps beside their marks
+constexpr unsigned int kOnceDense = 20;          // of a warp's 64 half-words in a group, marked ones from which its part is swept again
 constexpr int kSampleRun = 512;                  // weights of a warp's sample
 
 // In shared memory: the weights of each warp's first marks; of warp w in group g, for each half of a thread's word, the lanes
@@ -887,12 +891,19 @@ ternarize_once_kernel(const __grid_constant__ Launch<1> P, void *ws_raw)
     if (b == 0 && tid == 0) write_threshold(it, s, delta);
     const float thr = __double2float_rd(delta);
 
-    if (fabsf(__fsub_rn(thr, mid)) <= half && thr <= 2.0f * mid) {     // (the second: read_once)
+    // This warp's marks, none if the estimate was the threshold; a block with a warp that has too many sweeps its part again.
+    // (12288 x 8192 with half of the half-words marked: 181 us by the list of marks, 133 with such blocks swept again; all marked
+    // 260 and 156; all weights zero, so marked but none to correct, 246 and 87.  From about 20 of 64 on the second sweep is shorter.)
+    unsigned int total = 0;
+    if (groups && thr != mid) {
+        const unsigned int last = (groups - 1) * kSweepWarps + warp;
+        total = marks.before[last] + __popc(marks.mark[last].x) + __popc(marks.mark[last].y);
+    }
+    const bool dense = __syncthreads_or(total > kOnceDense * groups);
+    if (!dense && fabsf(__fsub_rn(thr, mid)) <= half && thr <= 2.0f * mid) {     // (the last: read_once)
         // ---- put right what lies between.  x -> |x - mid| as computed here and in the sweep is monotonic on either side of
         // mid, so a weight between mid and thr is no further from mid than thr is: its half-word is marked.  A warp takes its own
         // marks, a lane every 32nd.
-        const unsigned int last = (groups - 1) * kSweepWarps + warp;
-        const unsigned int total = groups ? marks.before[last] + __popc(marks.mark[last].x) + __popc(marks.mark[last].y) : 0;
 #pragma unroll 1
         for (unsigned int m = lane; m < total; m += 32) {
             unsigned int g = 0;                                        // the last group with no more than m marks before it

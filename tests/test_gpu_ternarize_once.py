@@ -18,6 +18,12 @@ def weights(rows, cols, kind):
         W = (W.reshape(rows, cols) * np.linspace(0.1, 2.0, rows, dtype=np.float32)[:, None]).reshape(-1)
     elif kind == "near":         # half of the weights within 1e-4 of the threshold, 0.7 times the mean magnitude
         W = np.where(np.arange(W.size) % 2 == 0, 0.7, 1.3).astype(np.float32) * (1 + np.float32(1e-4) * W) * np.where(W < 0, -1, 1).astype(np.float32)
+    elif kind == "some":         # every weight of the middle third that near, normal weights around it
+        lo, hi = W.size // 3, 2 * W.size // 3
+        rest = np.abs(W[:lo], dtype=np.float64).sum() + np.abs(W[hi:], dtype=np.float64).sum()
+        W[lo:hi] = rest * 0.7 / (W.size - 0.7 * (hi - lo)) * (1 + 1e-4 * W[lo:hi]) * np.where(W[lo:hi] < 0, -1, 1)
+    elif kind == "zeros":
+        W[:] = 0.0
     elif kind == "unseen":       # large weights where no part is sampled: the estimate misses
         W[::8192] = 500.0
     return np.ascontiguousarray(W, dtype=np.float32).reshape(rows, cols)
@@ -25,7 +31,8 @@ def weights(rows, cols, kind):
 
 @pytest.mark.parametrize("rows,cols,kind,extra,i8", [
     (4096, 4096, "normal", 0, False), (1, 2 ** 24 + 5, "normal", 64, True), (4099, 4111, "normal", 64, True), (4096, 4112, "rows", 0, True),
-    (4096, 4100, "near", 0, False), (4096, 4096, "near", 0, True), (4097, 4099, "unseen", 0, False), (4096, 4096, "unseen", 0, True)])
+    (4096, 4100, "near", 0, False), (4096, 4096, "near", 0, True),
+    (4096, 4096, "some", 0, True), (4099, 4111, "some", 0, False), (4096, 4096, "zeros", 0, True), (4097, 4099, "unseen", 0, False), (4096, 4096, "unseen", 0, True)])
 def test_codes_and_sums(rows, cols, kind, extra, i8):
     W = weights(rows, cols, kind)
     ld = twn.ld_for(cols) + extra
