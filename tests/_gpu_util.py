@@ -1,4 +1,6 @@
 """Helpers shared by the GPU parity tests: move numpy arrays to the device and back."""
+import ctypes
+
 import numpy as np
 import torch
 
@@ -26,3 +28,23 @@ def host_bf16_bits(t):
 
 def workspace(nbytes):
     return torch.empty((nbytes + 255) // 256 * 256, dtype=torch.uint8, device="cuda")
+
+
+def kernel_launches(call):
+    """Number of kernels that one call launches, counted in a graph that captures it."""
+    call()                                       # what is set up at a first call is not captured
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph, stream=torch.cuda.Stream()):
+        call()
+    rt, count = ctypes.CDLL("libcudart.so.12"), ctypes.c_size_t()
+    handle = ctypes.c_void_p(graph.raw_cuda_graph())
+    assert rt.cudaGraphGetNodes(handle, None, ctypes.byref(count)) == 0
+    nodes = (ctypes.c_void_p * count.value)()
+    assert rt.cudaGraphGetNodes(handle, nodes, ctypes.byref(count)) == 0
+    kinds = []
+    for node in nodes:
+        kind = ctypes.c_int()
+        assert rt.cudaGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)) == 0
+        kinds.append(kind.value)
+    return kinds.count(0)                        # cudaGraphNodeTypeKernel

@@ -7,7 +7,7 @@ import torch
 import oracle
 from paper_1605_04711_b200 import datagen as dg
 from paper_1605_04711_b200 import twn
-from _gpu_util import dev_f32, host_u32, workspace
+from _gpu_util import dev_f32, host_u32, kernel_launches, workspace
 
 pytestmark = pytest.mark.gpu
 
@@ -83,6 +83,9 @@ def test_the_coding_sweep_alone_gives_the_same_bits(rows, cols, kind, factor):
             twn.ternarize_codes(W, rows, cols, stats, packed, ld, None, workspace(twn.ternarize_workspace_bytes()))
         both.append((stats, packed))
     assert torch.equal(both[0][0], both[1][0]) and torch.equal(both[0][1], both[1][1])
+    ws = workspace(twn.ternarize_workspace_bytes())
+    launches = kernel_launches(lambda: twn.ternarize(W, factor, both[0][0], both[0][1], ld, None, ws))
+    assert launches == (1 if rows * cols <= factor * 2 ** 28 else 3)
 
 
 def test_weights_off_the_32_byte_boundaries_and_batches():
