@@ -154,8 +154,9 @@ int twn_ternarize(const float *W, int64_t rows, int64_t cols, double delta_facto
 
 /*
  * The first loop of Algorithm 1 for a whole network: ternarizes up to 32 tensors (layers) with one
- * launch per sweep instead of one per tensor.  Every tensor gets its own per-layer threshold,
- * codes and scale exactly as from a twn_ternarize call of its own (same reduction order, same bits).
+ * launch per sweep instead of one per tensor (a tensor that is read once, from 2^24 weights on, has
+ * a launch of its own).  Every tensor gets its own per-layer threshold, codes and scale exactly as
+ * from a twn_ternarize call of its own (same reduction order, same bits).
  *   items     HOST array of `count` descriptors; the fields have the meaning and the alignment
  *             rules of the twn_ternarize arguments of the same name (device pointers inside).
  *             Read during the call only.

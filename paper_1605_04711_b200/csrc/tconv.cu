@@ -281,10 +281,11 @@ tconv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ 
         __syncwarp();
     } else if (warp < kFirstEpiWarp) {
         // ------------------------------------------------ decode: codes -> bf16 -> tensor memory
-        // Two groups of four warps; a group handles every other stage.  Each thread owns one
-        // channel row: it reads the row's 16 bytes of codes per k-block straight from global
-        // memory (L2-resident, fetched two of its stages ahead), so decoding depends only on a
-        // free tensor-memory slot, not on the activation pipeline.
+        // One group of four warps, or two on alternate stages.  Each thread owns one channel row: it
+        // reads the row's codes of a stage (16 bytes per k-block of ternary codes, a stage's two
+        // k-blocks at once where they lie so) straight from global memory (L2-resident, fetched two
+        // or three of its stages ahead), so decoding depends only on a free tensor-memory slot, not
+        // on the activation pipeline.
         const int q = warp & 3;                 // tensor-memory lane quadrant of this warp
         const int set = (warp - 2) >> 2;
         constexpr int dsets = DS;               // groups of this kernel; the loops below are stepped by it
@@ -947,7 +948,10 @@ int launch_conv(const Geometry &g, const void *X, const uint32_t *T, const twn_s
                  u256 = time_us(t256, 5.4, half ? 2.4 : 2.8, 0.293, 3.0);
     // Another shape than 128 pixels has to gain more than a launch loses whose code is not that of the launches before it (1.5
     // us): VGG-7 at 128 images takes 189.7 us when its five layers run in the 128-pixel kernel, 200.3 with two of the others
-    // between them, although alone each layer is within 10 % in its best shape.
+    // between them, although alone each layer is within 10 % in its best shape.  What a call loses with it whose neighbours are
+    // of its own kind: of 140 calls of all sizes, each alone in a graph of twelve, it decides ten, where the three models are
+    // close, and those are 3 % faster with it on average (81x81x384, 5x5: 48.4 us, 64.7 without; 6 of the ten between -2 and
+    // -6 %); at worst 6 % slower (16384x4608x512: 63.8 / 60.1).
     constexpr double kOther = 1.5;
     int choice = u256 + kOther < u128 ? 1 : 0;
     if (u192 + (choice ? 0.0 : kOther) < (choice ? u256 : u128)) choice = 2;

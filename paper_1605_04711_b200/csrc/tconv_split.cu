@@ -2,8 +2,9 @@
 // TernaryBackward): one tile per block, the reduction split over the blocks of a cluster.
 //
 // What bounds such a problem is latency, not a pipe: in tconv_kernel a block walks the whole reduction of its tile
-// alone (430-540 cycles per 64-element k-block), and the first tile of its long straight-line epilogue costs 4400
-// cycles of cold instruction fetch.  1x1024x512 took 10.9 us on 4 blocks, 14x14x256 at batch 8 14.2 us on 26.  Here
+// alone (255-280 cycles per 64-element k-block of 128 pixels), and the first tile of its long straight-line epilogue
+// costs 4400 cycles of cold instruction fetch.  1x1024x512 took 10.9 us there on 4 blocks, 14x14x256 at batch 8 14.2 us
+// on 26 (both with k-blocks of 430-540 cycles; the second 10.9 now).  Here
 //   - a tile is 128 output channels x PIX pixels with PIX = 32 ... 256, so that small problems still make blocks;
 //   - a cluster of S = 1 ... 8 blocks shares a tile, every block reduces a contiguous share of the k-blocks;
 //   - every block leaves its fp32 accumulator in shared memory as [pixel][channel] and finishes PIX / S of the pixels:
@@ -458,6 +459,10 @@ namespace twn_detail {
 // for blocks that have an SM to themselves the number of rounds, where clusters do not fill every SM; E and R what a
 // block and a k-block take (few pixels make a k-block hardly cheaper: its decoding and its issue stay); X the exchange.
 // What it picks takes 3 % longer on average than the best of what was measured, and a third less than without this kernel.
+// The constants are those of the kernel before one elected thread issued and its code buffers rotated (0.5 us of a call of 36
+// k-blocks); on 140 calls of all sizes forced into the kernel as it is, the model is 0.2 % high on average, half of its errors
+// are under 7 % and a tenth over 18 % (calls of 10 to 20 us 5 % low), and what the three kernels' models pick together is 1.1 %
+// behind the best of the four on average (26 % at worst: 80x19x19x96 -> 48, 3x3 stride 2, 10.0 us split, 7.9 in the general kernel).
 SplitPlan plan_conv_split(const Geometry &g, int sm_count, bool in_order)
 {
     static const int pixels[4] = {32, 64, 128, 256};

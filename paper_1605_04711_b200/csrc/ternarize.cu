@@ -628,7 +628,7 @@ codes_fold_kernel(const __grid_constant__ Launch<N> P, void *ws_raw)
 // 136 in two sweeps, 33.6 million weights 60 / 49; every weight at the threshold 156 / 136.  Normal, Laplace, uniform, sparse
 // weights, rows of different scale, outliers 84 to 92, Cauchy 99.
 constexpr unsigned long long kOnceWeights = 16ull << 20;
-constexpr unsigned int kOnceGroups = 128;        // groups of 512 words in a part (310 million weights in all)
+constexpr unsigned int kOnceGroups = 128;        // groups of 512 words in a part (310 million weights in all; see read_once, too)
 constexpr unsigned int kOnceKept = 64;           // marked half-words that a warp keeps beside their marks
 constexpr unsigned int kOnceDense = 20;          // of a warp's 64 half-words in a group, marked ones from which its part is swept again
 constexpr int kSampleRun = 512;                  // weights of a warp's sample
@@ -1378,7 +1378,10 @@ int grid_for(long long items_per_thread_units, int sm_count)
 
 // What phase 1 reads last and phase 2 first is marked to stay in L2, the rest of a tensor larger than this to go first:
 // of 134 MB (8192 x 4096 weights, three tensors in turn) 53.4 us without marks, 50.3 / 49.3 / 50.0 / 50.7 / 51.4 us with 1 /
-// 40 / 60 / 80 / 100 MB kept; of 403 MB 136.9 us without, 131.4 us with 40 MB.
+// 40 / 60 / 80 / 100 MB kept; of 403 MB 136.9 us without, 131.4 us with 40 MB.  (Tensors of these sizes are read once now, at the
+// usual factors.  What goes this way are tensors of 40 to 67 MB, the coding sweep alone, and what read_once leaves here:
+// 44, 52 and 66 MB, three in turn, 21.6, 24.5 and 27.7 us without marks, 19.8, 22.8 and 26.5 with; the coding sweep of 134 MB 30.1 and
+// 28.3.  One tensor again and again is no faster with them, 66 MB 21.2 and 22.1; 864 MB neither.)
 constexpr unsigned long long kKeptBytes = 40000000ull;
 
 int transpose_blocks(int Cout, int Cin, int taps, long long words, int sm_count)
