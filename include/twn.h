@@ -154,8 +154,8 @@ int twn_ternarize(const float *W, int64_t rows, int64_t cols, double delta_facto
 
 /*
  * The first loop of Algorithm 1 for a whole network: ternarizes up to 32 tensors (layers) with one
- * launch per sweep instead of one per tensor (a tensor that is read once, from 2^24 weights on, has
- * a launch of its own).  Every tensor gets its own per-layer threshold, codes and scale exactly as
+ * launch per sweep, and one for its sums, instead of as many per tensor (a tensor that is read once,
+ * from 2^24 weights on, has a launch of its own).  Every tensor gets its own per-layer threshold, codes and scale exactly as
  * from a twn_ternarize call of its own (same reduction order, same bits).
  *   items     HOST array of `count` descriptors; the fields have the meaning and the alignment
  *             rules of the twn_ternarize arguments of the same name (device pointers inside).
@@ -237,7 +237,7 @@ int twn_ternarize_codes(const float *W, int64_t rows, int64_t cols, twn_stats_t 
                         void *workspace, size_t workspace_bytes, twn_stream_t stream);
 
 /* twn_sgd_update and twn_ternarize_codes for up to 32 tensors (the layers of a network) in one
- * launch each; every tensor gets the bits of a call of its own.  items: HOST arrays, read during
+ * sweep each, a launch and one that folds its sums; every tensor gets the bits of a call of its own.  items: HOST arrays, read during
  * the call only; fields as the arguments of the single-tensor calls.  workspace: at least
  * twn_ternarize_batch_workspace_bytes(count), 256-byte aligned. */
 typedef struct {
