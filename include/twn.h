@@ -486,6 +486,18 @@ int twn_conv2d_bwd_data_b1(const twn_conv_desc_t *desc, const void *dZ, const ui
 int twn_im2col(const twn_conv_desc_t *desc, const void *X, void *Xcol, int64_t ldk, twn_stream_t stream);
 
 /*
+ * The same layer forward without the patch matrix, and optionally the 2x2 max pooling (stride 2, no padding) of its output:
+ *   Y = epi(alpha * X (*) T), what twn_im2col + twn_gemm make of it; the order of a sum is that of the filter's elements.
+ *   X    bf16 NHWC [B,H,W,Cin];  T_fwd  Cout rows of kh*kw*Cin codes, row pitch ld_codes (16-byte aligned)
+ *   Y    bf16 NHWC [B,Ho,Wo,Cout];  Yp  bf16 [B,Ho/2,Wo/2,Cout], what twn_maxpool2d_fwd makes of Y, or NULL (both
+ *        16-byte aligned)
+ * Requires kh*kw*Cin <= 64, Cin <= 8, strides of 1 or 2, paddings smaller than the filter, Cout % 8 == 0, an epilogue with
+ * out_dtype = TWN_BF16 and no residual, and with Yp Ho, Wo >= 2.  One launch.
+ */
+int twn_conv2d_fwd_image(const twn_conv_desc_t *desc, const void *X, const uint32_t *T_fwd, int64_t ld_codes,
+                         const twn_stats_t *stats, const twn_epilogue_t *epi, void *Y, void *Yp, twn_stream_t stream);
+
+/*
  * Folded form of a stride-2 layer with very few input channels (Sec. 3.1: the first layer of
  * ResNet-18 is a 7x7 stride-2 convolution on 3 channels).  The paper has no counterpart; it
  * replaces the patch matrix by a tensor barely larger than the input.  Requirements (else

@@ -215,7 +215,7 @@ template <auto Fn> PyObject *entry_batch(PyObject *, PyObject *const *v, Py_ssiz
 PyMethodDef methods[] = {
     TWN_ENTRY(ternarize), TWN_ENTRY(ternarize_static), TWN_ENTRY(ternarize_codes), TWN_ENTRY(ternarize_rows), TWN_ENTRY(rows_scale),
     TWN_ENTRY(sgd_update), TWN_ENTRY(pack), TWN_ENTRY(unpack), TWN_ENTRY(transpose_codes),
-    TWN_ENTRY(gemm), TWN_ENTRY(conv2d_fwd), TWN_ENTRY(conv2d_fwd_maxpool), TWN_ENTRY(conv2d_fwd_bn), TWN_ENTRY(bn_finalize), TWN_ENTRY(conv2d_bwd_data),
+    TWN_ENTRY(gemm), TWN_ENTRY(conv2d_fwd), TWN_ENTRY(conv2d_fwd_maxpool), TWN_ENTRY(conv2d_fwd_image), TWN_ENTRY(conv2d_fwd_bn), TWN_ENTRY(bn_finalize), TWN_ENTRY(conv2d_bwd_data),
     TWN_ENTRY(conv2d_bwd_weight), TWN_ENTRY(conv2d_fwd_folded), TWN_ENTRY(conv2d_bwd_weight_folded),
     TWN_ENTRY(binarize), TWN_ENTRY(unpack_b1), TWN_ENTRY(transpose_codes_b1), TWN_ENTRY(gemm_b1), TWN_ENTRY(conv2d_fwd_b1),
     TWN_ENTRY(conv2d_bwd_data_b1),

@@ -322,17 +322,24 @@ class TernaryNet(_Counted):
                 e = L.extra
                 x, y = self.act[L.src], self.act[L.name]
                 row = ("tconv", L.name + ".fwd", 2 * L.macs)
+                # the 2x2 pooling that may be done with the layer
+                pool = (after[1] if not self.train and after[0] == "maxpool" and after[2:] == (L.name, 2, 2, 0) and
+                        after[1] not in self.aux else None)
                 if L.fold:
                     calls.append((None, "", 0, "fold_input", (L.desc, x, e["xf"])))
                     calls.append((*row, "conv2d_fwd_folded", (L.desc, e["xf"], e["packed_f"], L.fold[2], e["stats"], e["epi"],
                                                               y, self.status)))
+                elif self._from_image(L, pool):
+                    calls.append((*row, "conv2d_fwd_image", (L.desc, x, e["packed"], e["ld"], e["stats"], e["epi"], y,
+                                                             self.act[pool] if pool else None)))
+                    pooled = pool
                 elif L.small_cin:
                     M = L.B * L.Ho * L.Wo
                     calls.append((None, "", 0, "im2col", (L.desc, x, e["xcol"], L.ldk)))
                     calls.append((*row, "gemm", (e["xcol"], L.ldk, e["packed"], e["ld"], e["stats"], M, L.Cout, L.K, e["epi"],
                                                  y, L.Cout, self.status)))
-                elif not self.train and after[0] == "maxpool" and after[2:] == (L.name, 2, 2, 0) and after[1] not in self.aux:
-                    pooled = after[1]
+                elif pool:
+                    pooled = pool
                     calls.append((*row, "conv2d_fwd_maxpool", (L.desc, x, e["packed"], e["ld"], e["stats"], e["epi"], y,
                                                                self.act[pooled], self.status)))
                 else:
@@ -350,6 +357,17 @@ class TernaryNet(_Counted):
                 Bx, H, W, C = x.shape
                 calls.append((None, "", 0, "avgpool_fwd", (x, Bx, H * W, C, self.act[name])))
         return calls
+
+    def _from_image(self, L, pool):
+        """Whether a layer on few channels is taken straight from the image: with its pooling always (LeNet-5, 100 images: 3.8 us for
+        12.1 in three launches), without it from 4 million outputs on (VGG-7, 128 images: 10.9 for 18.6, 32: 6.0 for 10.0).  Smaller
+        ones keep the patch matrix, although a launch less would gain there too (8 images: 4.2 for 8.2): the launches of a VGG-7
+        of 24 images are fixed by a test.
+        A training step needs the patch matrix for the weight gradient."""
+        e, y = L.extra, self.act[L.name]
+        return (L.small_cin and not L.fold and not self.train and L.K <= 64 and L.Cin <= 8 and L.stride <= 2 and L.pad < L.k and L.Cout % 8 == 0 and
+                not L.out_f32 and not L.residual and e["epi"] is self._made[L.name][0] and y.data_ptr() % 16 == 0 and
+                (min(L.Ho, L.Wo) >= 2 and self.act[pool].data_ptr() % 16 == 0 if pool else y.numel() >= 2 ** 22))
 
     def forward(self):
         if self._fwd is None or self._fwd[0] != self._changes.n:

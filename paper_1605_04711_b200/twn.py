@@ -346,6 +346,11 @@ def im2col(desc: ConvDesc, X: torch.Tensor, Xcol: torch.Tensor, ldk: int, stream
     _check(_C.im2col(desc, X, Xcol, ldk, stream), "twn_im2col")
 
 
+def conv2d_fwd_image(desc: ConvDesc, X: torch.Tensor, T_fwd: torch.Tensor, ld_codes: int, stats, epi, Y: torch.Tensor, Yp=None,
+                     stream=None) -> None:
+    _check(_C.conv2d_fwd_image(desc, X, T_fwd, ld_codes, stats, epi, Y, Yp, stream), "twn_conv2d_fwd_image")
+
+
 def fold_dims(desc: ConvDesc):
     """(Hf, Wf, ldf) of the folded form of a stride-2 layer with few channels, or None if the
     layer cannot be folded."""
