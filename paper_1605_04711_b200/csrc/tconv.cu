@@ -917,7 +917,7 @@ int launch_conv(const Geometry &g, const void *X, const uint32_t *T, const twn_s
     if ((long long)g.Bv * g.OH * g.OW * g.ldy >= 0xFFFFFFFFLL) return TWN_ERR_INVALID_ARG;
     const EpilogueArgs ea = epilogue_args(stats, epi, out_dtype_default);
     // problems that do not fill the GPU: small tiles, the reduction split over a cluster
-    const SplitPlan split = g.pool ? SplitPlan{0, 0, 1e30} : plan_conv_split(g, dev.sm_count / (g.beside > 1 ? g.beside : 1), ea.in_order);
+    const SplitPlan split = plan_conv_split(g, dev.sm_count / (g.beside > 1 ? g.beside : 1), ea.in_order);
     ConvParams P;
     memset(&P, 0, sizeof P);
     P.n_tiles = (g.Cout + kChan - 1) / kChan;

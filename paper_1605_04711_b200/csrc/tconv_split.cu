@@ -70,6 +70,8 @@ struct SplitParams {
     int res_dtype, res_gate, relu, out_dtype;
     int vec;                          // four channels at a time are aligned in Y and the residual
     void *Y;
+    __nv_bfloat16 *pool;              // 2x2 max pooling of the output [Bv, PH, PW, Cout]: whole windows in every block's share
+    int PH, PW;
     int32_t *status;
     Tap taps[kMaxTaps];
 };
@@ -102,8 +104,8 @@ __device__ __forceinline__ uint32_t peer(uint32_t addr, int rank)
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.aligned;" ::: "memory"); }
 
-// Four channels of a pixel: affine, residual, ReLU, store.
-__device__ __forceinline__ void finish(const SplitParams &P, size_t off, int left, const float4 a, const float (&sc)[4], const float (&sf)[4])
+// Four channels of a pixel: affine, residual, ReLU, store.  Returns them as stored where that is bf16, four at a time.
+__device__ __forceinline__ uint2 finish(const SplitParams &P, size_t off, int left, const float4 a, const float (&sc)[4], const float (&sf)[4])
 {
     float y[4] = {fmaf(a.x, sc[0], sf[0]), fmaf(a.y, sc[1], sf[1]), fmaf(a.z, sc[2], sf[2]), fmaf(a.w, sc[3], sf[3])};
     if (P.residual) {
@@ -133,7 +135,9 @@ __device__ __forceinline__ void finish(const SplitParams &P, size_t off, int lef
     if (P.out_dtype == TWN_BF16) {
         __nv_bfloat16 *yp = reinterpret_cast<__nv_bfloat16 *>(P.Y) + off;
         if (P.vec) {
-            *reinterpret_cast<uint2 *>(yp) = make_uint2(pack_bf16x2(y[0], y[1]), pack_bf16x2(y[2], y[3]));
+            const uint2 packed = make_uint2(pack_bf16x2(y[0], y[1]), pack_bf16x2(y[2], y[3]));
+            *reinterpret_cast<uint2 *>(yp) = packed;
+            return packed;
         } else {
 #pragma unroll
             for (int x = 0; x < 4; ++x) if (x < left) yp[x] = __float2bfloat16_rn(y[x]);
@@ -147,6 +151,7 @@ __device__ __forceinline__ void finish(const SplitParams &P, size_t off, int lef
             for (int x = 0; x < 4; ++x) if (x < left) yp[x] = y[x];
         }
     }
+    return make_uint2(0u, 0u);
 }
 
 // Adds the S partial sums of a block's pixels, in rank order, and finishes them.  A warp takes every tenth pixel, 32
@@ -183,7 +188,53 @@ __device__ __forceinline__ void final_sums(const SplitParams &P, const Sums &m, 
     }
 }
 
-template <int PIX, int BITS>
+// The same for a pooled output: a warp takes every tenth window of the block's pixels, its four pixels one after the other.
+// `p0` is the block's first pixel, which starts a row pair of the tile.
+template <int S>
+__device__ __forceinline__ void final_sums_pool(const SplitParams &P, const Sums &m, const float (&sc)[4], const float (&sf)[4], int p0, int h0, int w0, int b0)
+{
+#pragma unroll 1
+    for (int win = threadIdx.x >> 5; win < m.per / 4; win += kThreads / 32) {
+        const int x = win & ((1 << (P.lgBW - 1)) - 1), y = win >> (P.lgBW - 1);
+        const int first = (y << (P.lgBW + 1)) + 2 * x;              // in the block's share
+        uint2 best = make_uint2(0xFF80FF80u, 0xFF80FF80u);
+        bool whole = false;
+        constexpr int kPix = S <= 4 ? 4 : 1;                         // pixels whose partial sums are in registers at once
+#pragma unroll 1
+        for (int q0 = 0; q0 < 4; q0 += kPix) {
+            float4 v[kPix][S];
+#pragma unroll
+            for (int u = 0; u < kPix; ++u)
+#pragma unroll
+                for (int r = 0; r < S; ++r) {
+                    const int q = q0 + u;
+                    const float *src = r == m.rank ? m.own : m.recv + (r < m.rank ? r : r - 1) * m.per * kPitch;
+                    v[u][r] = *reinterpret_cast<const float4 *>(src + (first + (q & 1) + ((q >> 1) << P.lgBW)) * kPitch);
+                }
+#pragma unroll
+            for (int u = 0; u < kPix; ++u) {
+                const int q = q0 + u;
+                float4 a = v[u][0];
+#pragma unroll
+                for (int r = 1; r < S; ++r) { a.x += v[u][r].x; a.y += v[u][r].y; a.z += v[u][r].z; a.w += v[u][r].w; }
+                const uint32_t off = m.off[first + (q & 1) + ((q >> 1) << P.lgBW)];
+                whole = off != 0xFFFFFFFFu;                              // of the last pixel: the tile starts on a window
+                if (!whole) continue;
+                const uint2 z = finish(P, (size_t)off + m.n0, m.left, a, sc, sf);
+                best.x = max_first_bf16x2(best.x, z.x);
+                best.y = max_first_bf16x2(best.y, z.y);
+            }
+        }
+        if (whole) {
+            const int p = p0 + first, lgHW = P.lgBW + P.lgBH;
+            const int gw = (w0 + (p & ((1 << P.lgBW) - 1))) >> 1, gh = (h0 + ((p >> P.lgBW) & ((1 << P.lgBH) - 1))) >> 1, gb = b0 + (p >> lgHW);
+            *reinterpret_cast<uint2 *>(P.pool + (((size_t)gb * P.PH + gh) * P.PW + gw) * P.Cout + m.n0) =
+                make_uint2(no_max_to_zero(best.x), no_max_to_zero(best.y));
+        }
+    }
+}
+
+template <int PIX, int BITS, bool POOL>
 __global__ void __launch_bounds__(kThreads, PIX <= 128 ? 2 : 1)
 tconv_split_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ SplitParams P, int splits)
 {
@@ -383,7 +434,12 @@ tconv_split_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
     }
     if (n0 < P.Cout) {
         const Sums sums = {sm->acc + (rank * per) * kPitch + lane * 4, sm->recv + lane * 4, sm->off + rank * per, per, rank, n0, P.Cout - n0};
-        if (splits == 1) final_sums<1>(P, sums, sc, sf);
+        if (POOL) {
+            if (splits == 1) final_sums_pool<1>(P, sums, sc, sf, rank * per, h0, w0, b0);
+            else if (splits == 2) final_sums_pool<2>(P, sums, sc, sf, rank * per, h0, w0, b0);
+            else if (splits == 4) final_sums_pool<4>(P, sums, sc, sf, rank * per, h0, w0, b0);
+            else final_sums_pool<8>(P, sums, sc, sf, rank * per, h0, w0, b0);
+        } else if (splits == 1) final_sums<1>(P, sums, sc, sf);
         else if (splits == 2) final_sums<2>(P, sums, sc, sf);
         else if (splits == 4) final_sums<4>(P, sums, sc, sf);
         else final_sums<8>(P, sums, sc, sf);
@@ -394,11 +450,11 @@ tconv_split_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
         for (int i = 0; i < 64; ++i) __nanosleep(1000);      // copies still in flight land before the memory is released
 }
 
-template <int PIX, int BITS>
+template <int PIX, int BITS, bool POOL>
 int launch_t(const Geometry &g, SplitParams &P, const void *X, int splits, const twn_device_info &dev, cudaStream_t s)
 {
     static bool attr_set[64] = {false};
-    auto kernel = tconv_split_kernel<PIX, BITS>;
+    auto kernel = tconv_split_kernel<PIX, BITS, POOL>;
     // At most two blocks on an SM, as many as its tensor memory holds: a block that waits for tensor memory in one
     // cluster while its peers wait for it must never be possible.
     constexpr int kFloor = 78 * 1024, kMost = std::max(kFloor, PIX == 256 ? smem_bytes<PIX>(2) : smem_bytes<PIX>(8));
@@ -468,7 +524,10 @@ SplitPlan plan_conv_split(const Geometry &g, int sm_count, bool in_order)
     static const int pixels[4] = {32, 64, 128, 256};
     static const double E[4] = {3.89, 4.47, 5.51, 7.73}, R[4] = {0.241, 0.249, 0.255, 0.275};
     SplitPlan best = {0, 0, 1e30};
-    if (g.bn_partial) return best;
+    // A pooled output: up to 64 channels, where half of a tile of the general kernel is idle (14x14x64, 3x3 on 64: 16 images 7.2 us, 5.3 here, 64 images 7.8 and
+    // 6.6; 12x12x64, 5x5 on 32: 32 images 8.7 and 7.4, 100 images 10.7 and 10.5, in LeNet-5 behind its first layer 2.2 us less); the sums of
+    // wider pooled layers stay in order, as those of callers who ask for that do, in the general kernel.
+    if (g.bn_partial || (g.pool && (in_order || g.code_bits != 2 || g.Cout > 64))) return best;
     // with classes: as many tiles as the largest has each (it comes first), the longest reduction and the mean one
     const int classes = g.n_classes > 0 ? g.n_classes : 1;
     const long long cblk = (g.Cin + kBlockK - 1) / kBlockK;
@@ -483,6 +542,7 @@ SplitPlan plan_conv_split(const Geometry &g, int sm_count, bool in_order)
         for (int splits = 1; splits <= (in_order ? 1 : pix == 256 ? 2 : 8); splits *= 2) {
             const long long n = (kb + splits - 1) / splits;
             if ((splits > 1 && splits > kb) || n > kMaxBlocks) continue;
+            if (g.pool && pix / splits < 2 << a) continue;
             const double ctas = (double)tiles * classes * splits, L = ctas / sm_count;
             const bool alone = pix == 256 || (pix == 128 && splits >= 4);
             // clusters of 4 and 8 fill 128 and 112 of 148 SMs
@@ -529,14 +589,23 @@ int launch_conv_split(const Geometry &g, const void *X, const uint32_t *T, const
     P.vec = g.Cout % 4 == 0 && g.ldy % 4 == 0 && reinterpret_cast<uintptr_t>(Y) % (4 * es) == 0 &&
             (!epi.residual || reinterpret_cast<uintptr_t>(epi.residual) % 8 == 0);
     P.Y = Y;
+    P.pool = static_cast<__nv_bfloat16 *>(g.pool);
+    P.PH = g.Hv / 2; P.PW = g.Wv / 2;
+    if (g.pool && !P.vec) return TWN_ERR_CUDA;       // the caller has looked at the alignment
     P.status = dev_status;
     const bool b1 = g.code_bits == 1;
     const int splits = plan.splits;
+    if (g.pool) switch (plan.pix) {
+        case 32: return launch_t<32, 2, true>(g, P, X, splits, dev, s);
+        case 64: return launch_t<64, 2, true>(g, P, X, splits, dev, s);
+        case 128: return launch_t<128, 2, true>(g, P, X, splits, dev, s);
+        default: return launch_t<256, 2, true>(g, P, X, splits, dev, s);
+    }
     switch (plan.pix) {
-        case 32: return b1 ? launch_t<32, 1>(g, P, X, splits, dev, s) : launch_t<32, 2>(g, P, X, splits, dev, s);
-        case 64: return b1 ? launch_t<64, 1>(g, P, X, splits, dev, s) : launch_t<64, 2>(g, P, X, splits, dev, s);
-        case 128: return b1 ? launch_t<128, 1>(g, P, X, splits, dev, s) : launch_t<128, 2>(g, P, X, splits, dev, s);
-        default: return b1 ? launch_t<256, 1>(g, P, X, splits, dev, s) : launch_t<256, 2>(g, P, X, splits, dev, s);
+        case 32: return b1 ? launch_t<32, 1, false>(g, P, X, splits, dev, s) : launch_t<32, 2, false>(g, P, X, splits, dev, s);
+        case 64: return b1 ? launch_t<64, 1, false>(g, P, X, splits, dev, s) : launch_t<64, 2, false>(g, P, X, splits, dev, s);
+        case 128: return b1 ? launch_t<128, 1, false>(g, P, X, splits, dev, s) : launch_t<128, 2, false>(g, P, X, splits, dev, s);
+        default: return b1 ? launch_t<256, 1, false>(g, P, X, splits, dev, s) : launch_t<256, 2, false>(g, P, X, splits, dev, s);
     }
 }
 
