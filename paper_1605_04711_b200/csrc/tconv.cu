@@ -99,8 +99,8 @@ struct ConvParams {
     int lgBW, lgBH;               // pixel tile = BB x BH x BW, powers of two, product PIX
     // reduction
     int n_taps, n_cblk;           // k-blocks per tile = n_taps * n_cblk
-    int codes_aligned;            // 1: every k-block starts on a 16-byte boundary of the packed row; 2: k-block u follows k-block
-                                  // u - 1, and every other one starts on a boundary of two
+    int code_run;                 // words of the packed row on whose boundaries every k-block starts: 1, 2, 4; 8: k-block u follows
+                                  // k-block u - 1, and every other one starts on such a boundary
     const uint32_t *T;            // packed codes, one row of `wpr` words per output channel
     long long wpr;
     int sw, sh;                   // input pixel = output pixel * (sh, sw) + (dh, dw)
@@ -302,7 +302,7 @@ tconv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ 
             // A warp's load touches 32 rows, and that is what it costs: both k-blocks of a stage come with one 32-byte load
             // where the codes lie so.  With two of 16 bytes a k-block of 128 pixels took 320 cycles, 255 with one
             // (4001x4608x512 20.1 -> 17.7 us, 3x3 64x7x7x512 18.9 -> 16.0).
-            if (kSub == 2 && P.codes_aligned == 2) {
+            if (kSub == 2 && P.code_run == 8) {
                 if (BITS == 2) {
                     ld_nc_v8(c.v[0], c.v[kSub - 1], rowp + 8 * st);
                 } else {
@@ -324,8 +324,11 @@ tconv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ 
                     word = (P.taps[t].koff / kCodesPerWord) + cb * kWordsPerBlock;
                 }
                 if (BITS == 2) {
-                    if (P.codes_aligned) {
+                    if (P.code_run >= 4) {
                         ld_nc_v4(c.v[sb], rowp + word);
+                    } else if (P.code_run == 2) {
+                        ld_nc_v2(c.v[sb].x, c.v[sb].y, rowp + word);
+                        ld_nc_v2(c.v[sb].z, c.v[sb].w, rowp + (word + 2 < P.wpr ? word + 2 : word));
                     } else {
                         const long long last = P.wpr - 1;
                         ld_nc_u32(c.v[sb].x, rowp + (word + 0 < last ? word + 0 : last));
@@ -334,7 +337,7 @@ tconv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ 
                         ld_nc_u32(c.v[sb].w, rowp + (word + 3 < last ? word + 3 : last));
                     }
                 } else {
-                    if (P.codes_aligned) {
+                    if (P.code_run >= 2) {
                         ld_nc_v2(c.v[sb].x, c.v[sb].y, rowp + word);
                     } else {
                         const long long last = P.wpr - 1;
@@ -923,11 +926,13 @@ int launch_conv(const Geometry &g, const void *X, const uint32_t *T, const twn_s
     P.n_tiles = (g.Cout + kChan - 1) / kChan;
     P.n_taps = g.n_taps;
     P.n_cblk = (int)((g.Cin + kBlockK - 1) / kBlockK);
-    P.codes_aligned = g.ld_codes % 128 == 0 && reinterpret_cast<uintptr_t>(T) % 32 == 0 ? 2 : 1;
-    for (int t = 0; t < g.n_taps; ++t)
-        if (g.taps[t].koff != t * P.n_cblk * kBlockK) P.codes_aligned = std::min(P.codes_aligned, 1);
-    for (int t = 0; t < g.n_taps; ++t)
-        if (g.taps[t].koff % kBlockK != 0) P.codes_aligned = 0;
+    P.code_run = code_run(g);
+    // (a pair of k-blocks: 8 words of ternary codes, 4 of binary ones)
+    if (P.code_run * (g.code_bits == 1 ? 2 : 1) == 4 && g.ld_codes % 128 == 0 && reinterpret_cast<uintptr_t>(T) % 32 == 0) {
+        bool follow = true;
+        for (int t = 0; t < g.n_taps; ++t) follow &= g.taps[t].koff == t * P.n_cblk * kBlockK;
+        if (follow) P.code_run = 8;
+    }
     // Tile shape by a model of the launch's time: a fixed part and, per round of tiles, an epilogue and the k-blocks, or where
     // the epilogue of one tile overlaps the reduction of the next at least the epilogue.  Fitted to 40 launches (convolutions of
     // 16 to 128 images, inner products of 333 to 50176 rows) forced to each shape, three inputs in turn; what it picks takes 0.7 %
@@ -942,7 +947,7 @@ int launch_conv(const Geometry &g, const void *X, const uint32_t *T, const twn_s
         return fixed + (double)((tiles + sms - 1) / sms) * std::max(per_tile + per_block * (double)kb, least);
     };
     // (code words off the 16-byte boundaries come one at a time, which the smaller shapes wait for: 7 further shapes)
-    const bool words = P.codes_aligned == 0;
+    const bool words = P.code_run * (g.code_bits == 1 ? 2 : 1) < 4;
     const double u128 = time_us(t128, 4.3, 1.4, words ? 0.225 : 0.155, 1.85),
                  u192 = time_us(t192, 5.1, 1.6, words ? 0.24 : 0.225, half ? 1.76 : 2.43),
                  u256 = time_us(t256, 5.4, half ? 2.4 : 2.8, 0.293, 3.0);

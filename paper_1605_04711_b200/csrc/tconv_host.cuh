@@ -70,6 +70,19 @@ struct Geometry {
     TapClass cls[kMaxClasses];
 };
 
+// Words of a packed row on whose boundaries every k-block of 64 codes starts: 4, 2 or 1 (binary codes: 2 or 1).  A k-block's
+// codes come with as many loads, and a warp's load costs the 32 rows that it touches, not their bytes.  Layers of 32 (mod 64)
+// channels, two loads instead of four: 16x14x14x224 -> 256, 3x3, 20.9 -> 14.4 us (split kernel), 64x14x14x608 -> 512 63.9 -> 61.1,
+// 100x14x14x288 -> 688, 5x5, 179.8 -> 173.1 (general kernel), 4x14x14x96 -> 96 5.7 -> 5.2.
+inline int code_run(const Geometry &g)
+{
+    const int word = g.code_bits == 1 ? 32 : 16;
+    int run = 64 / word;
+    for (int t = 0; t < g.n_taps; ++t)
+        while (g.taps[t].koff % (run * word) != 0) run /= 2;
+    return run;
+}
+
 // Picks the pixel-tile shape BW x BH x BB (BW and BH powers of two, product `pix`) that needs the
 // fewest tiles.
 inline long long pick_tile(const Geometry &g, int pix, int *lgBW, int *lgBH)
