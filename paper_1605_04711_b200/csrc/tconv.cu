@@ -130,6 +130,14 @@ struct ConvParams {
     Tap taps[kMaxTaps];
 };
 
+// The classes of a strided backward pass: their tiles follow one another, those without taps last; each class has its own run of
+// taps and place in the output.  (An argument of their own: in the parameters of every launch they cost small layers 0.3 us.)
+struct ClassTable {
+    int n, live_tiles;            // classes; tiles of those with taps
+    struct { int tile0, tw, th, Hv, Wv, ooh, oow, tap0, kb0, kb, stages; } cls[kMaxClasses];
+};
+struct NoClasses {};
+
 template <int PIX>
 struct __align__(1024) SmemLayout {
     static constexpr int kStages = Cfg<PIX>::kStages, kSub = Cfg<PIX>::kSub;
@@ -161,10 +169,14 @@ static_assert(offsetof(SmemLayout<128>, stage_res) % 128 == 0 && offsetof(SmemLa
                   offsetof(SmemLayout<128>, stage_out) % 128 == 0 && offsetof(SmemLayout<256>, stage_out) % 128 == 0,
               "TMA and vector accesses need aligned shared-memory regions");
 
-template <int PIX, int BITS>
+// CLASSES: the residue classes of a strided backward pass in one launch, the longest reductions first; fragments alone.
+// WORDS: the ternary codes come word by word (in a kernel of its own where they do: with the wider loads beside them those layers
+// lost 2 %, 64x28x28x192 <- 272, 3x3, 52.7 -> 54.2 us).
+template <int PIX, int BITS, bool CLASSES, bool WORDS>
 __global__ void __launch_bounds__(threads_conv(Cfg<PIX>::kDecodeGroups), 1)
 tconv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_y,
-             const __grid_constant__ CUtensorMap map_r, const __grid_constant__ ConvParams P)
+             const __grid_constant__ CUtensorMap map_r, const __grid_constant__ ConvParams P,
+             const __grid_constant__ std::conditional_t<CLASSES, ClassTable, NoClasses> K)
 {
     using L = SmemLayout<PIX>;
     constexpr int kStages = Cfg<PIX>::kStages, kSub = Cfg<PIX>::kSub, kAccBufs = Cfg<PIX>::kAccBufs, DS = Cfg<PIX>::kDecodeGroups;
@@ -181,8 +193,14 @@ tconv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ 
     volatile int *abort_flag = &sm->abort_flag;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int kbpt = P.n_taps * P.n_cblk;               // k-blocks per tile
-    const int spt = (kbpt + kSub - 1) / kSub;           // stages per tile (the last may hold fewer k-blocks)
+    const int kb_all = P.n_taps * P.n_cblk;             // k-blocks per tile (of all classes)
+    // the class of a tile, from that of an earlier one
+    auto seek = [&](int &c, int tile) {
+        if constexpr (CLASSES)
+            while (c + 1 < K.n && tile >= K.cls[c + 1].tile0) ++c;
+    };
+    int live_tiles = P.total_tiles;
+    if constexpr (CLASSES) live_tiles = K.live_tiles;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) {
@@ -200,7 +218,7 @@ tconv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ 
     // code-word offset of every k-block, in the order the k-blocks are consumed: taps outer,
     // channel blocks inner
     constexpr int kFirstEpiWarp = first_epi_warp(DS), kThreadsConv = threads_conv(DS);
-    for (int u = threadIdx.x; u < kbpt && u < kWordTab; u += kThreadsConv) {
+    for (int u = threadIdx.x; u < kb_all && u < kWordTab; u += kThreadsConv) {
         const int t = u / P.n_cblk, cb = u - t * P.n_cblk;
         sm->kword[u] = (uint32_t)(P.taps[t].koff / kCodesPerWord) + cb * kWordsPerBlock;
     }
@@ -223,11 +241,18 @@ tconv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ 
             uint32_t it = 0;
             bool ok = true;
             const uint32_t block_bytes = kXBytes;
-            for (int tile = blockIdx.x; tile < P.total_tiles && ok; tile += gridDim.x) {
-                int pt = tile / P.n_tiles;
-                const int twi = pt % P.tw; pt /= P.tw;
-                const int thi = pt % P.th;
-                const int tbi = pt / P.th;
+            int ci = 0;
+            for (int tile = blockIdx.x; tile < live_tiles && ok; tile += gridDim.x) {
+                int tw = P.tw, th = P.th, tap0 = 0, kbpt = kb_all, spt = (kb_all + kSub - 1) / kSub, pt = tile;
+                if constexpr (CLASSES) {
+                    seek(ci, tile);
+                    const auto &C = K.cls[ci];
+                    tw = C.tw; th = C.th; tap0 = C.tap0; kbpt = C.kb; spt = C.stages; pt -= C.tile0;
+                }
+                pt /= P.n_tiles;
+                const int twi = pt % tw; pt /= tw;
+                const int thi = pt % th;
+                const int tbi = pt / th;
                 const int w0 = (twi << P.lgBW) * P.sw;
                 const int h0 = (thi << P.lgBH) * P.sh;
                 const int b0 = tbi * (PIX >> (P.lgBW + P.lgBH));
@@ -239,7 +264,7 @@ tconv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ 
                     if (!mbar_wait(&sm->empty[s], ph ^ 1u, abort_flag, P.status)) { ok = false; break; }
                     mbar_expect_tx(&sm->full[s], nsb * block_bytes);
                     for (int sb = 0; sb < nsb; ++sb) {
-                        const Tap tap = P.taps[t];
+                        const Tap tap = P.taps[tap0 + t];
                         tma_load_4d(sm->x[s][sb], &map_x, &sm->full[s], cb * kBlockK, w0 + tap.dw, h0 + tap.dh, b0);
                         if (++cb == P.n_cblk) { cb = 0; ++t; }
                     }
@@ -249,14 +274,28 @@ tconv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ 
     } else if (warp == 1) {
         // ------------------------------------------------ MMA issuer: one thread (see tc_mma_ts)
         // One wait and one commit per stage, constant accumulate flags.  With no taps at all
-        // (kbpt == 0) nothing is accumulated and the epilogue does not wait.
-        if (kbpt > 0 && elect_one()) {
+        // (no k-blocks) nothing is accumulated and the epilogue does not wait.
+        if (kb_all > 0 && elect_one()) {
             constexpr uint32_t idesc = make_idesc(kChan, PIX);
             const uint64_t bdesc0 = smem_desc_sw128(smem_u32(sm->x[0][0]));
             const uint32_t b_lo0 = (uint32_t)bdesc0, b_hi = (uint32_t)(bdesc0 >> 32);
             uint32_t it = 0, lt = 0;
             bool ok = true;
-            for (int tile = blockIdx.x; tile < P.total_tiles && ok; tile += gridDim.x, ++lt) {
+            // in registers: what this thread waits for between two tiles, the tensor core waits for
+            int first[kMaxClasses], kbs[kMaxClasses];
+            kbs[0] = kb_all;
+            if constexpr (CLASSES)
+                for (int c = 0; c < kMaxClasses; ++c) {
+                    first[c] = c < K.n ? K.cls[c].tile0 : 0x7fffffff;
+                    kbs[c] = K.cls[c].kb;
+                }
+            for (int tile = blockIdx.x; tile < live_tiles && ok; tile += gridDim.x, ++lt) {
+                int kbpt = kbs[0];
+                if (CLASSES) {
+#pragma unroll
+                    for (int c = 1; c < kMaxClasses; ++c) kbpt = tile >= first[c] ? kbs[c] : kbpt;
+                }
+                const int spt = (kbpt + kSub - 1) / kSub;
                 const int buf = lt % kAccBufs;
                 const uint32_t aph = (lt / kAccBufs) & 1u;
                 if (!mbar_wait(&sm->acc_empty[buf], aph ^ 1u, abort_flag, P.status, 0)) break;
@@ -298,16 +337,18 @@ tconv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ 
         // hidden.  What a clamped fetch returns is either never decoded (no such stage) or feeds
         // channels that are never stored, or multiplies activations that the TMA zero-fills.
         struct Codes { uint4 v[kSub]; };
+        int kbpt = kb_all, spt = (kb_all + kSub - 1) / kSub;        // of the tile being decoded
+        int kbpt_f = kbpt, spt_f = spt, kb0_f = 0, tap0_f = 0;      // of the tile being fetched
         auto fetch = [&](Codes &c, const uint32_t *rowp, int st) {
             // A warp's load touches 32 rows, and that is what it costs: both k-blocks of a stage come with one 32-byte load
             // where the codes lie so.  With two of 16 bytes a k-block of 128 pixels took 320 cycles, 255 with one
             // (4001x4608x512 20.1 -> 17.7 us, 3x3 64x7x7x512 18.9 -> 16.0).
-            if (kSub == 2 && P.code_run == 8) {
+            if (kSub == 2 && !WORDS && P.code_run == 8) {
                 if (BITS == 2) {
-                    ld_nc_v8(c.v[0], c.v[kSub - 1], rowp + 8 * st);
+                    ld_nc_v8(c.v[0], c.v[kSub - 1], rowp + (CLASSES ? sm->kword[kb0_f + 2 * st] : 8 * st));
                 } else {
                     uint4 both;
-                    ld_nc_v4(both, rowp + 4 * st);
+                    ld_nc_v4(both, rowp + (CLASSES ? sm->kword[kb0_f + 2 * st] : 4 * st));
                     c.v[0].x = both.x; c.v[0].y = both.y; c.v[kSub - 1].x = both.z; c.v[kSub - 1].y = both.w;
                 }
                 return;
@@ -315,18 +356,18 @@ tconv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ 
 #pragma unroll
             for (int sb = 0; sb < kSub; ++sb) {
                 int u = st * kSub + sb;
-                u = u < kbpt ? u : kbpt - 1;
+                u = u < kbpt_f ? u : kbpt_f - 1;
                 long long word;
-                if (kbpt <= kWordTab) {
-                    word = sm->kword[u];
+                if (kb_all <= kWordTab) {
+                    word = sm->kword[kb0_f + u];
                 } else {
                     const int t = u / P.n_cblk, cb = u - t * P.n_cblk;
-                    word = (P.taps[t].koff / kCodesPerWord) + cb * kWordsPerBlock;
+                    word = (P.taps[tap0_f + t].koff / kCodesPerWord) + cb * kWordsPerBlock;
                 }
                 if (BITS == 2) {
-                    if (P.code_run >= 4) {
+                    if (!WORDS && P.code_run >= 4) {
                         ld_nc_v4(c.v[sb], rowp + word);
-                    } else if (P.code_run == 2) {
+                    } else if (!WORDS && (PIX == 128 || P.code_run == 2)) {
                         ld_nc_v2(c.v[sb].x, c.v[sb].y, rowp + word);
                         ld_nc_v2(c.v[sb].z, c.v[sb].w, rowp + (word + 2 < P.wpr ? word + 2 : word));
                     } else {
@@ -348,9 +389,14 @@ tconv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ 
             }
         };
         // position of this group's next stages: (tile, st), advanced dsets stages at a time
+        int ci_c = 0, ci_f = 0;
         auto advance = [&](int &tile, int &st, int steps) {
             for (int i = 0; i < steps; ++i)
-                if (++st >= spt) { st = 0; tile += gridDim.x; }
+                if (++st >= spt) {
+                    st = 0; tile += gridDim.x;
+                    if constexpr (CLASSES)
+                        if (tile < live_tiles) { seek(ci_c, tile); kbpt = K.cls[ci_c].kb; spt = K.cls[ci_c].stages; }
+                }
         };
         // the fetch position also carries its row of the packed matrix: the channel tile of
         // `tile` is tile mod n_tiles, stepped without a division (one sits in the way of every
@@ -363,19 +409,33 @@ tconv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ 
         };
         auto advance_f = [&](int &tile, int &st, int &nt, const uint32_t *&rowp, int steps) {
             for (int i = 0; i < steps; ++i)
-                if (++st >= spt) {
+                if (++st >= spt_f) {
                     st = 0; tile += gridDim.x;
-                    nt += nt_step; if (nt >= P.n_tiles) nt -= P.n_tiles;
+                    nt += nt_step; if (nt >= P.n_tiles) nt -= P.n_tiles;     // (a class has whole sets of channel tiles)
                     rowp = row_ptr(nt);
+                    if constexpr (CLASSES)
+                        if (tile < live_tiles) {
+                            seek(ci_f, tile);
+                            kbpt_f = K.cls[ci_f].kb; spt_f = K.cls[ci_f].stages; kb0_f = K.cls[ci_f].kb0; tap0_f = K.cls[ci_f].tap0;
+                        }
                 }
         };
-        if (spt > 0) {
+        int tile_c = blockIdx.x, st_c = 0;                   // the stage being decoded
+        if constexpr (CLASSES)
+            if (tile_c < live_tiles) {
+                seek(ci_c, tile_c);
+                kbpt = K.cls[ci_c].kb; spt = K.cls[ci_c].stages;
+            }
+        if (CLASSES ? tile_c < live_tiles : spt > 0) {
             // 256-pixel tiles: three code buffers in rotation, each refilled right after use for the
             // stage three of this group's stages ahead: no register is copied while its load is still
             // in flight.  The other shapes: two buffers, see below.
-            int tile_c = blockIdx.x, st_c = 0;               // the stage being decoded
             advance(tile_c, st_c, set);
             int tile_f = tile_c, st_f = st_c;                // the stage being fetched
+            if constexpr (CLASSES) {
+                ci_f = ci_c;
+                kbpt_f = kbpt; spt_f = spt; kb0_f = K.cls[ci_c].kb0; tap0_f = K.cls[ci_c].tap0;
+            }
             int nt_f = tile_f % P.n_tiles;
             const uint32_t *rowp_f = row_ptr(nt_f);
             Codes c0, c1, c2;
@@ -410,11 +470,11 @@ tconv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ 
             if (PIX == 256) {
                 // long reductions, no slack for a late code word: three buffers in rotation
                 while (true) {
-                    if (tile_c >= P.total_tiles || !decode_stage(c0)) break;
+                    if (tile_c >= live_tiles || !decode_stage(c0)) break;
                     { fetch(c0, rowp_f, st_f); advance_f(tile_f, st_f, nt_f, rowp_f, dsets); }
-                    if (tile_c >= P.total_tiles || !decode_stage(c1)) break;
+                    if (tile_c >= live_tiles || !decode_stage(c1)) break;
                     { fetch(c1, rowp_f, st_f); advance_f(tile_f, st_f, nt_f, rowp_f, dsets); }
-                    if (tile_c >= P.total_tiles || !decode_stage(c2)) break;
+                    if (tile_c >= live_tiles || !decode_stage(c2)) break;
                     { fetch(c2, rowp_f, st_f); advance_f(tile_f, st_f, nt_f, rowp_f, dsets); }
                 }
             } else {
@@ -424,7 +484,7 @@ tconv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ 
                 // unchanged).
 #pragma unroll 1
                 while (true) {
-                    if (tile_c >= P.total_tiles || !decode_stage(c0)) break;
+                    if (tile_c >= live_tiles || !decode_stage(c0)) break;
                     c0 = c1;
                     { fetch(c1, rowp_f, st_f); advance_f(tile_f, st_f, nt_f, rowp_f, dsets); }
                 }
@@ -461,12 +521,20 @@ tconv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ 
         uint32_t nst = 0;      // staging buffers this warp has filled so far (selects the buffer)
         uint32_t nres = 0;     // residual chunks this warp has consumed so far (buffer and phase)
         bool alive = true;
+        int ci = 0;
         for (int tile = blockIdx.x; tile < P.total_tiles && alive; tile += gridDim.x, ++lt) {
             const int nt = tile % P.n_tiles;
-            int pt = tile / P.n_tiles;
-            const int twi = pt % P.tw; pt /= P.tw;
-            const int thi = pt % P.th;
-            const int tbi = pt / P.th;
+            int pt = tile, kbpt = kb_all, tw = P.tw, th = P.th;
+            int sto_w = 0, sto_h = 0;                            // of a store's coordinates; without classes in the tensor map
+            if constexpr (CLASSES) {
+                seek(ci, tile);
+                const auto &C = K.cls[ci];
+                pt -= C.tile0; kbpt = C.kb; tw = C.tw; th = C.th; sto_w = C.oow; sto_h = C.ooh;
+            }
+            pt /= P.n_tiles;
+            const int twi = pt % tw; pt /= tw;
+            const int thi = pt % th;
+            const int tbi = pt / th;
             const int n = nt * kChan + q * 32 + lane;
             const bool n_ok = n < P.Cout;
             // a warp whose 32 channels all lie past Cout hands the accumulator back but loads,
@@ -481,7 +549,7 @@ tconv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ 
                 const int p0 = c * 32;
                 mbar_expect_tx(&my_res_full[slot], 32 * 32 * 2);
                 tma_load_4d(my_res + slot * (32 * 32), &map_r, &my_res_full[slot], c_n0,
-                            (p_w0 + (p0 & BWm)) * P.osw, (p_h0 + ((p0 >> P.lgBW) & BHm)) * P.osh,
+                            (p_w0 + (p0 & BWm)) * P.osw + sto_w, (p_h0 + ((p0 >> P.lgBW) & BHm)) * P.osh + sto_h,
                             p_b0 + (p0 >> (P.lgBW + P.lgBH)));
             };
             // both buffers are free here: the warp has read the last chunk of its previous tile
@@ -505,7 +573,7 @@ tconv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ 
                 const int c = es + i * kEpiSets;
                 if (kbpt > 0) {
                     if (warp_on) {
-                        if (P.fragments) {
+                        if (CLASSES || P.fragments) {
                             tmem_ld_16x256b_x4(t_acc + c * 32, v);
                             tmem_ld_16x256b_x4(t_acc + (16u << 16) + c * 32, v + 16);
                         } else {
@@ -524,7 +592,7 @@ tconv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ 
                     for (int j = 0; j < 32; ++j) v[j] = 0u;
                 }
                 if (!warp_on) continue;
-                if (P.fragments) {
+                if (CLASSES || P.fragments) {
                     // The accumulator's rows are channels, the output's rows pixels: the chunk has to be transposed.  The
                     // 16x256b load leaves a thread two neighbouring pixels of channels g, g + 8, g + 16, g + 24: packed,
                     // that is the operand of stmatrix.trans.  Four of those store the chunk, four ldmatrix.trans fetch
@@ -587,10 +655,10 @@ tconv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ 
                     __syncwarp();
                     if (lane == 0) {
                         const int p0 = c * 32;
-                        tma_store_4d(&map_y, sbuf, c_n0, (p_w0 + (p0 & BWm)) * P.osw, (p_h0 + ((p0 >> P.lgBW) & BHm)) * P.osh,
+                        tma_store_4d(&map_y, sbuf, c_n0, (p_w0 + (p0 & BWm)) * P.osw + sto_w, (p_h0 + ((p0 >> P.lgBW) & BHm)) * P.osh + sto_h,
                                      p_b0 + (p0 >> (P.lgBW + P.lgBH)));
                     }
-                    if (PIX == 128 && P.pool) {
+                    if (PIX == 128 && !CLASSES && P.pool) {
                         // The chunk's eight windows from the staged output: a lane takes one, eight channels of it.  A sweep of
                         // its own reads the whole output again: 12.5 us for 128x32x32x128, 8.8 for 128x16x16x256, 5.7 for
                         // 128x8x8x512; here 1.7, 1.5 and 0.7.
@@ -715,8 +783,8 @@ tconv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ 
                         __syncwarp();
                         if (lane == 0) {
                             const int p0 = c * 32 + h * 16;
-                            tma_store_4d(&map_y, sbuf, c_n0, (p_w0 + (p0 & BWm)) * P.osw,
-                                         (p_h0 + ((p0 >> P.lgBW) & BHm)) * P.osh, p_b0 + (p0 >> (P.lgBW + P.lgBH)));
+                            tma_store_4d(&map_y, sbuf, c_n0, (p_w0 + (p0 & BWm)) * P.osw + sto_w,
+                                         (p_h0 + ((p0 >> P.lgBW) & BHm)) * P.osh + sto_h, p_b0 + (p0 >> (P.lgBW + P.lgBH)));
                         }
                         ++nst;
                     }
@@ -736,7 +804,7 @@ tconv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ 
                     }
                 }
             }
-            if (P.bn_partial && warp_on)
+            if (!CLASSES && P.bn_partial && warp_on)
                 *reinterpret_cast<float2 *>(P.bn_partial + ((size_t)tile * kEpiSets + es) * (2 * kChan) + (q * 32 + lane) * 2) =
                     make_float2(bn_s1, bn_s2);
             __syncwarp();
@@ -785,14 +853,14 @@ bn_reduce_kernel(const float *__restrict__ partial, int total_tiles, int n_tiles
 }
 
 // ---------------------------------------------------------------- host side
-template <int PIX, int BITS>
+template <int PIX, int BITS, bool CLASSES = false, bool WORDS = false>
 int launch_conv_t(const Geometry &g, ConvParams &P, const void *X, const twn_device_info &dev,
-                  EncodeTiledFn enc, cudaStream_t s)
+                  EncodeTiledFn enc, cudaStream_t s, ClassTable *table = nullptr)
 {
     static bool attr_set[64] = {false};
     const int smem_bytes = (int)sizeof(SmemLayout<PIX>) + 1024;
     if (!attr_set[dev.ordinal]) {
-        TWN_CUDA_OK(cudaFuncSetAttribute(tconv_kernel<PIX, BITS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes));
+        TWN_CUDA_OK(cudaFuncSetAttribute(tconv_kernel<PIX, BITS, CLASSES, WORDS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes));
         attr_set[dev.ordinal] = true;
     }
     pick_tile(g, PIX, &P.lgBW, &P.lgBH);
@@ -800,7 +868,19 @@ int launch_conv_t(const Geometry &g, ConvParams &P, const void *X, const twn_dev
     P.tw = (g.Wv + BW - 1) / BW;
     P.th = (g.Hv + BH - 1) / BH;
     P.tb = (g.Bv + BB - 1) / BB;
-    const long long total = (long long)P.n_tiles * P.tw * P.th * P.tb;
+    long long total = (long long)P.n_tiles * P.tw * P.th * P.tb;
+    if (CLASSES) {
+        total = 0;
+        for (int c = 0; c < table->n; ++c) {
+            auto &C = table->cls[c];
+            if (total > 0x7fffffffLL) return TWN_ERR_INVALID_ARG;
+            C.tile0 = (int)total;
+            C.tw = (C.Wv + BW - 1) / BW;
+            C.th = (C.Hv + BH - 1) / BH;
+            total += (long long)P.n_tiles * C.tw * C.th * P.tb;
+            if (C.kb > 0) table->live_tiles = (int)std::min(total, 0x7fffffffLL);
+        }
+    }
     if (total <= 0 || total > 0x7fffffffLL) return TWN_ERR_INVALID_ARG;
     P.total_tiles = (int)total;
 
@@ -876,6 +956,7 @@ int launch_conv_t(const Geometry &g, ConvParams &P, const void *X, const twn_dev
         P.lg_sbw = P.lgBW;
         P.lg_sbh = std::min(P.lgBH, 5 - P.lgBW);
     }
+    if (CLASSES && !P.fragments) return TWN_ERR_CUDA;       // the caller has looked at what fragments need
     if (P.fragments && P.residual && !P.res_tma) return TWN_ERR_CUDA;      // the same geometry could be encoded for Y
     const int grid = dev.sm_count < P.total_tiles ? dev.sm_count : P.total_tiles;
     // Programmatic dependent launch pays when the blocks cover the GPU (set-up and launch latency hide behind the
@@ -883,7 +964,10 @@ int launch_conv_t(const Geometry &g, ConvParams &P, const void *X, const twn_dev
     // after a convolution: 21 us instead of 12), so those launch the plain way.
     const bool kPdlConv = grid * 2 >= dev.sm_count;
     if (P.bn_partial && (size_t)P.total_tiles * kEpiSets * 2 * kChan * sizeof(float) > g.bn_partial_bytes) return TWN_ERR_WORKSPACE;
-    TWN_CUDA_OK(twn_launch_pdl(kPdlConv, tconv_kernel<PIX, BITS>, grid, threads_conv(Cfg<PIX>::kDecodeGroups), (size_t)smem_bytes, s, map_x, map_y, map_r, P));
+    std::conditional_t<CLASSES, ClassTable, NoClasses> classes;
+    if constexpr (CLASSES) classes = *table;
+    TWN_CUDA_OK(twn_launch_pdl(kPdlConv, tconv_kernel<PIX, BITS, CLASSES, WORDS>, grid, threads_conv(Cfg<PIX>::kDecodeGroups), (size_t)smem_bytes, s,
+                               map_x, map_y, map_r, P, classes));
     if (P.bn_partial)
         bn_reduce_kernel<<<(g.Cout + 7) / 8, 256, 0, s>>>(P.bn_partial, P.total_tiles, P.n_tiles, g.Cout, g.bn_sum, g.bn_sumsq);
     TWN_CUDA_OK(cudaGetLastError());
@@ -920,7 +1004,8 @@ int launch_conv(const Geometry &g, const void *X, const uint32_t *T, const twn_s
     if ((long long)g.Bv * g.OH * g.OW * g.ldy >= 0xFFFFFFFFLL) return TWN_ERR_INVALID_ARG;
     const EpilogueArgs ea = epilogue_args(stats, epi, out_dtype_default);
     // problems that do not fill the GPU: small tiles, the reduction split over a cluster
-    const SplitPlan split = plan_conv_split(g, dev.sm_count / (g.beside > 1 ? g.beside : 1), ea.in_order);
+    const bool classes = g.n_classes > 0;
+    const SplitPlan split = classes ? SplitPlan{0, 0, 1e30} : plan_conv_split(g, dev.sm_count / (g.beside > 1 ? g.beside : 1), ea.in_order);
     ConvParams P;
     memset(&P, 0, sizeof P);
     P.n_tiles = (g.Cout + kChan - 1) / kChan;
@@ -930,7 +1015,13 @@ int launch_conv(const Geometry &g, const void *X, const uint32_t *T, const twn_s
     // (a pair of k-blocks: 8 words of ternary codes, 4 of binary ones)
     if (P.code_run * (g.code_bits == 1 ? 2 : 1) == 4 && g.ld_codes % 128 == 0 && reinterpret_cast<uintptr_t>(T) % 32 == 0) {
         bool follow = true;
-        for (int t = 0; t < g.n_taps; ++t) follow &= g.taps[t].koff == t * P.n_cblk * kBlockK;
+        if (classes) {
+            // taps in any order: a pair of k-blocks is one of a tap
+            follow = P.n_cblk % 2 == 0 && g.n_taps * P.n_cblk <= kWordTab;
+            for (int t = 0; t < g.n_taps; ++t) follow &= g.taps[t].koff % (2 * kBlockK) == 0;
+        } else {
+            for (int t = 0; t < g.n_taps; ++t) follow &= g.taps[t].koff == t * P.n_cblk * kBlockK;
+        }
         if (follow) P.code_run = 8;
     }
     // Tile shape by a model of the launch's time: a fixed part and, per round of tiles, an epilogue and the k-blocks, or where
@@ -958,16 +1049,43 @@ int launch_conv(const Geometry &g, const void *X, const uint32_t *T, const twn_s
     // close, and those are 3 % faster with it on average (81x81x384, 5x5: 48.4 us, 64.7 without; 6 of the ten between -2 and
     // -6 %); at worst 6 % slower (16384x4608x512: 63.8 / 60.1).
     constexpr double kOther = 1.5;
+    // The classes of a strided backward pass in one launch: their tiles go round the blocks, the longest first, and end with half a
+    // tile's difference.  Fitted to 97 shapes (1 to 128 images of 7 to 110 pixels, 32 to 768 channels, 1x1 to 5x5) forced to it: 7 %
+    // off on average, 22 % at most.
+    double all_classes = 0.0;
+    ClassTable table;
+    if (classes) {
+        table.n = g.n_classes;
+        table.live_tiles = 0;
+        double work = 0.0, longest = 0.0;
+        for (int c = 0; c < g.n_classes; ++c) {
+            const TapClass &k = g.cls[c];
+            table.cls[c].Hv = k.Hv; table.cls[c].Wv = k.Wv; table.cls[c].ooh = k.ooh; table.cls[c].oow = k.oow;
+            table.cls[c].tap0 = k.tap0; table.cls[c].kb0 = k.tap0 * P.n_cblk;
+            table.cls[c].kb = k.n_taps * P.n_cblk; table.cls[c].stages = (table.cls[c].kb + Cfg<128>::kSub - 1) / Cfg<128>::kSub;
+            const double us = 1.24 + (words ? (P.code_run == 1 ? 0.257 : 0.218) : P.code_run == 8 ? 0.149 : 0.219) * (double)(k.n_taps * P.n_cblk);
+            work += us * (double)t128;
+            longest = std::max(longest, us);
+        }
+        all_classes = 4.56 + std::max(longest, work / (double)sms + 0.58 * longest);
+        if (us_only) {
+            // bf16 in and out by TMA, else not at all
+            const bool fits = ea.out_dtype == TWN_BF16 && g.Cout % 8 == 0 && g.ldy % 8 == 0 && twn_aligned(Y, 16) &&
+                              (!ea.residual || (ea.res_dtype == TWN_BF16 && twn_aligned(ea.residual, 16)));
+            *us_only = fits ? all_classes : 1e30;
+            return TWN_OK;
+        }
+    }
     int choice = u256 + kOther < u128 ? 1 : 0;
     if (u192 + (choice ? 0.0 : kOther) < (choice ? u256 : u128)) choice = 2;
     // Pooling is in that kernel alone: the others, whose epilogue is longer with it, lost 0.6 % on 16384x4096x4096 to code that
     // they do not run.
-    if (g.pool) choice = 0;
+    if (g.pool || classes) choice = 0;
     const double us = choice == 0 ? u128 : choice == 1 ? u256 : u192;
     // Narrow layers and short reductions: the kernel that decodes its channels' codes once per block.  Up to 64 channels
     // the general kernel's half-empty tiles lose wherever that kernel runs; above, its own time decides.
     bool handled = false;
-    if (!g.pool) rc = launch_conv_resident(g, X, T, ea, Y, dev_status, dev, s, half || split.us < us ? split.us : us, &handled, us_only);
+    if (!g.pool && !classes) rc = launch_conv_resident(g, X, T, ea, Y, dev_status, dev, s, half || split.us < us ? split.us : us, &handled, us_only);
     if (rc != TWN_OK || handled) return rc;
     // The more SMs the general kernel fills by itself, the clearer the modelled gain has to be: near the line the split
     // kernel's model is the optimistic one where most SMs are filled (3x3 3x56x56x64 -> 256: 66 % filled, 9.5 us split, 7.7 here,
@@ -994,11 +1112,15 @@ int launch_conv(const Geometry &g, const void *X, const uint32_t *T, const twn_s
     P.status = dev_status;
     P.bn_partial = g.bn_partial;
     for (int t = 0; t < g.n_taps; ++t) P.taps[t] = g.taps[t];
-    if (g.code_bits == 1)
+    const bool by_word = P.code_run == 1;
+    if (g.code_bits == 1) {
+        if (classes) return launch_conv_t<128, 1, true>(g, P, X, dev, enc, s, &table);
         return choice == 1 ? launch_conv_t<256, 1>(g, P, X, dev, enc, s) : choice == 2 ? launch_conv_t<192, 1>(g, P, X, dev, enc, s)
                                                                                     : launch_conv_t<128, 1>(g, P, X, dev, enc, s);
-    return choice == 1 ? launch_conv_t<256, 2>(g, P, X, dev, enc, s) : choice == 2 ? launch_conv_t<192, 2>(g, P, X, dev, enc, s)
-                                                                                : launch_conv_t<128, 2>(g, P, X, dev, enc, s);
+    }
+    if (classes) return by_word ? launch_conv_t<128, 2, true, true>(g, P, X, dev, enc, s, &table) : launch_conv_t<128, 2, true>(g, P, X, dev, enc, s, &table);
+    if (choice != 0) return choice == 1 ? launch_conv_t<256, 2>(g, P, X, dev, enc, s) : launch_conv_t<192, 2>(g, P, X, dev, enc, s);
+    return by_word ? launch_conv_t<128, 2, false, true>(g, P, X, dev, enc, s) : launch_conv_t<128, 2>(g, P, X, dev, enc, s);
 }
 
 // Helper streams for launches that are independent of one another (the residue classes of a
@@ -1370,6 +1492,10 @@ int conv_bwd_data_impl(const twn_conv_desc_t *d, const void *dZ, const uint32_t 
         g.Hv = cls[0].Hv; g.Wv = cls[0].Wv;
         g.n_classes = n_cls;
         for (int c = 0; c < n_cls; ++c) g.cls[c] = cls[c];
+        // (the longest reductions first in the general kernel, whose blocks walk the tiles in turn; the split kernel, a block for
+        // each, is 1 to 2 % slower so)
+        Geometry by_length = g;
+        std::stable_sort(by_length.cls, by_length.cls + n_cls, [](const TapClass &a, const TapClass &b) { return a.n_taps > b.n_taps; });
         // Apart, the launches follow one another as far as each fills the SMs, and overlap at their ends: the sum of what the
         // kernels that they would run should take, less 1.2 us for each after the first.  Measured both ways on 180 shapes (1 to
         // 256 images of 7 to 112 pixels, 32 to 768 channels, 1x1 to 5x5), half of them not used in the fit, the way it takes is
@@ -1379,13 +1505,23 @@ int conv_bwd_data_impl(const twn_conv_desc_t *d, const void *dZ, const uint32_t 
         const EpilogueArgs ea = epilogue_args(stats, epi, TWN_F32);
         const SplitPlan plan = plan_conv_split(g, dev.sm_count, ea.in_order);
         constexpr double kLeast = 2.9;           // no model goes below: the sum ends when the answer is known (2 us of host time)
+        // In the general kernel, whose blocks walk tiles of all classes: 50x28x28x192 <- 384 takes 22.1 us so, 28.0 split and 35 apart,
+        // 20 images of 56x56x64 <- 128 12.7, 17.4 and 24, 15x41x41x448 <- 240 28.8, 34.3 and 37.2.  It has to be modelled 5 % below
+        // the split kernel and 10 % below launches apart (35 % where a class has no taps: those take less than their models say).  Of
+        // 97 shapes measured all three ways the choice is 2.4 % behind the best on average, 6.3 % without this way, and on none slower.
+        double together = 0.0;
+        rc = launch_conv(by_length, dZ, T_bwd, stats, epi, dX, TWN_F32, dev_status, user, &together);
+        if (rc != TWN_OK) return rc;
+        const double less = by_length.cls[n_cls - 1].n_taps == 0 ? 0.65 : 0.9;
+        const double one = std::min(plan.us, together / less);
         double apart = kLeast * n_cls - 1.2 * (n_cls - 1);
-        for (int c = 0; c < n_cls && apart <= plan.us; ++c) {
+        for (int c = 0; c < n_cls && apart <= one; ++c) {
             double us = 0.0;
             rc = launch_conv(one_class(cls[c], n_cls), dZ, T_bwd, stats, epi, dX, TWN_F32, dev_status, user, &us);
             if (rc != TWN_OK) return rc;
             apart += us - kLeast;
         }
+        if (together < 0.95 * plan.us && together < less * apart) return launch_conv(by_length, dZ, T_bwd, stats, epi, dX, TWN_F32, dev_status, user);
         if (plan.pix && plan.us < apart)
             return launch_conv_split(g, dZ, T_bwd, ea, dX, dev_status, dev, user, plan);
     }

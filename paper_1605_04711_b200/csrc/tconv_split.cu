@@ -53,7 +53,6 @@ struct SplitParams {
     int n_tiles;                      // channel tiles
     int lgBW, lgBH;                   // pixel tile = BW x BH x BB, product PIX
     int n_cblk;                       // k-blocks per tap
-    int code_run;                     // code words on whose boundaries every k-block starts
     const uint32_t *T;
     long long wpr;
     int sw, sh;
@@ -234,9 +233,9 @@ __device__ __forceinline__ void final_sums_pool(const SplitParams &P, const Sums
     }
 }
 
-// ALIGNED: a k-block's codes are one load.  The other loads are in a kernel of their own: the fetch stands six times in the decode
-// loop, and with two more branches in it layers that never take them lost 1.5 % (3552x1174x72 8.18 -> 8.33 us).
-template <int PIX, int BITS, bool POOL, bool ALIGNED>
+// RUN: code words on whose boundaries every k-block starts.  A kernel for each: the fetch stands six times in the decode loop, and
+// with the loads of other boundaries in it layers that never take them lost 1.5 % (3552x1174x72 8.18 -> 8.33 us).
+template <int PIX, int BITS, bool POOL, int RUN>
 __global__ void __launch_bounds__(kThreads, PIX <= 128 ? 2 : 1)
 tconv_split_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ SplitParams P, int splits)
 {
@@ -337,9 +336,9 @@ tconv_split_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
             auto fetch = [&](uint4 &c, int i) {
                 const long long word = sm->kword[i < n_kb ? i : n_kb - 1], last = P.wpr - 1;
                 if (BITS == 2) {
-                    if (ALIGNED) {
+                    if (RUN == 4) {
                         ld_nc_v4(c, rowp + word);
-                    } else if (P.code_run == 2) {
+                    } else if (RUN == 2) {
                         ld_nc_v2(c.x, c.y, rowp + word);
                         ld_nc_v2(c.z, c.w, rowp + (word + 2 < P.wpr ? word + 2 : word));
                     } else {
@@ -348,7 +347,7 @@ tconv_split_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
                         ld_nc_u32(c.z, rowp + (word + 2 < last ? word + 2 : last));
                         ld_nc_u32(c.w, rowp + (word + 3 < last ? word + 3 : last));
                     }
-                } else if (ALIGNED) {
+                } else if (RUN == 2) {
                     ld_nc_v2(c.x, c.y, rowp + word);
                 } else {
                     ld_nc_u32(c.x, rowp + (word + 0 < last ? word + 0 : last));
@@ -455,11 +454,11 @@ tconv_split_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
         for (int i = 0; i < 64; ++i) __nanosleep(1000);      // copies still in flight land before the memory is released
 }
 
-template <int PIX, int BITS, bool POOL, bool ALIGNED>
+template <int PIX, int BITS, bool POOL, int RUN>
 int launch_t(const Geometry &g, SplitParams &P, const void *X, int splits, const twn_device_info &dev, cudaStream_t s)
 {
     static bool attr_set[64] = {false};
-    auto kernel = tconv_split_kernel<PIX, BITS, POOL, ALIGNED>;
+    auto kernel = tconv_split_kernel<PIX, BITS, POOL, RUN>;
     // At most two blocks on an SM, as many as its tensor memory holds: a block that waits for tensor memory in one
     // cluster while its peers wait for it must never be possible.
     constexpr int kFloor = 78 * 1024, kMost = std::max(kFloor, PIX == 256 ? smem_bytes<PIX>(2) : smem_bytes<PIX>(8));
@@ -509,14 +508,14 @@ int launch_t(const Geometry &g, SplitParams &P, const void *X, int splits, const
     return TWN_OK;
 }
 
-template <int BITS, bool POOL, bool ALIGNED>
+template <int BITS, bool POOL, int RUN>
 int launch_pix(const Geometry &g, SplitParams &P, const void *X, const SplitPlan &plan, const twn_device_info &dev, cudaStream_t s)
 {
     switch (plan.pix) {
-        case 32: return launch_t<32, BITS, POOL, ALIGNED>(g, P, X, plan.splits, dev, s);
-        case 64: return launch_t<64, BITS, POOL, ALIGNED>(g, P, X, plan.splits, dev, s);
-        case 128: return launch_t<128, BITS, POOL, ALIGNED>(g, P, X, plan.splits, dev, s);
-        default: return launch_t<256, BITS, POOL, ALIGNED>(g, P, X, plan.splits, dev, s);
+        case 32: return launch_t<32, BITS, POOL, RUN>(g, P, X, plan.splits, dev, s);
+        case 64: return launch_t<64, BITS, POOL, RUN>(g, P, X, plan.splits, dev, s);
+        case 128: return launch_t<128, BITS, POOL, RUN>(g, P, X, plan.splits, dev, s);
+        default: return launch_t<256, BITS, POOL, RUN>(g, P, X, plan.splits, dev, s);
     }
 }
 
@@ -586,7 +585,7 @@ int launch_conv_split(const Geometry &g, const void *X, const uint32_t *T, const
         P.cls[c].tap0 = k.tap0;
         P.cls[c].kb = k.n_taps * P.n_cblk;
     }
-    P.code_run = code_run(g);
+    const int run = code_run(g);
     for (int t = 0; t < g.n_taps; ++t) P.taps[t] = g.taps[t];
     P.T = T;
     P.wpr = g.ld_codes / (g.code_bits == 1 ? 32 : 16);
@@ -607,10 +606,12 @@ int launch_conv_split(const Geometry &g, const void *X, const uint32_t *T, const
     if (g.pool && !P.vec) return TWN_ERR_CUDA;       // the caller has looked at the alignment
     P.status = dev_status;
     const bool b1 = g.code_bits == 1;
-    const bool aligned = P.code_run == (b1 ? 2 : 4);
-    if (g.pool) return aligned ? launch_pix<2, true, true>(g, P, X, plan, dev, s) : launch_pix<2, true, false>(g, P, X, plan, dev, s);
-    if (b1) return aligned ? launch_pix<1, false, true>(g, P, X, plan, dev, s) : launch_pix<1, false, false>(g, P, X, plan, dev, s);
-    return aligned ? launch_pix<2, false, true>(g, P, X, plan, dev, s) : launch_pix<2, false, false>(g, P, X, plan, dev, s);
+    if (g.pool)
+        return run == 4 ? launch_pix<2, true, 4>(g, P, X, plan, dev, s) : run == 2 ? launch_pix<2, true, 2>(g, P, X, plan, dev, s)
+                                                                      : launch_pix<2, true, 1>(g, P, X, plan, dev, s);
+    if (b1) return run == 2 ? launch_pix<1, false, 2>(g, P, X, plan, dev, s) : launch_pix<1, false, 1>(g, P, X, plan, dev, s);
+    return run == 4 ? launch_pix<2, false, 4>(g, P, X, plan, dev, s) : run == 2 ? launch_pix<2, false, 2>(g, P, X, plan, dev, s)
+                                                                   : launch_pix<2, false, 1>(g, P, X, plan, dev, s);
 }
 
 }  // namespace twn_detail
