@@ -4,27 +4,38 @@
 // its own scale alpha_r = mean of |W_r,i| over |W_r,i| > delta_r (Eq. 5).
 //
 // A team of threads per filter: a warp for filters of up to 1024 weights (12000 filters of 64 weights took 31 us with a
-// block each, most of it blocks starting and joining), a block beyond.  The threshold needs the whole filter before any
+// block each, most of it blocks starting and joining), a block of 128 or 256 threads beyond.  What a block adds to its filter's
+// work is its start, its barriers and the sums across its warps, so smaller teams are faster where they hold a filter in few
+// enough registers (blocks of 256 before and of 128 now, us: 20000 filters of 1152 weights 73.1 and 39.0, 6000 of 2304 26.2 and
+// 18.2, 3000 of 4608 20.6 and 14.4, 4000 of 6912 29.8 and 26.9); few long filters want the more threads (592 of 6912: 5.4, 7.1
+// with 128).  The threshold needs the whole filter before any
 // code can be written, but a filter is small (25 ... 8192 weights in the networks of the paper), so the team keeps it in
 // registers between the two steps, up to sixteen 16-byte vectors per thread: each weight crosses HBM once (4 bytes read,
 // 0.25 bytes written), against two reads for the per-layer rule.  Longer filters are read a second time, back to front
 // (from L2, as a rule).  Filters that start off the 16-byte boundaries are read by two aligned vectors and shifted (with
 // 4-byte loads, twice over, 4000 filters of 5001 weights took 62 us).  Both sums are fp64 with a fixed order (per-thread
 // sums, shuffle tree, warps in order): same inputs, same bits.  No scratch memory.
+#include <type_traits>
+
 #include "sweep.cuh"
 
 namespace {
 
 constexpr int kThreads = 256;
 
-// T threads per filter (32 or kThreads), R vectors of four weights per thread and chunk.
+// T threads per filter (32, 128 or kThreads), R vectors of four weights per thread and chunk.
+template <int T> __host__ __device__ constexpr int block_threads() { return T == 32 ? kThreads : T; }
+template <int T, int R> __host__ __device__ constexpr int blocks_per_sm()
+{
+    return T == 128 ? (R > 10 ? 6 : R > 8 ? 7 : R > 4 ? 8 : 10) : R >= 12 ? 2 : R >= 5 ? 4 : 5;
+}
 template <int T, int R>
-__global__ void __launch_bounds__(kThreads, R >= 12 ? 2 : R >= 6 ? 4 : 5)
+__global__ void __launch_bounds__(block_threads<T>(), blocks_per_sm<T, R>())
 ternarize_rows_kernel(const float *__restrict__ W, long long rows, long long cols, double factor,
                       twn_stats_t *__restrict__ stats, uint32_t *__restrict__ packed, long long wpr,
                       int8_t *__restrict__ codes_i8, int vec4)
 {
-    constexpr int kTeams = kThreads / T, kV = (R + 3) / 4 * 4, kWarps = T / 32;
+    constexpr int kTeams = block_threads<T>() / T, kV = (R + 3) / 4 * 4, kWarps = T / 32;
     __shared__ double part_a[T == 32 ? 1 : kWarps], part_b[T == 32 ? 1 : kWarps];
     __shared__ uint2 part_c[T == 32 ? 1 : kWarps];
     const int t = threadIdx.x % T, lane = threadIdx.x & 31, warp = t >> 5;
@@ -185,25 +196,49 @@ extern "C" int twn_ternarize_rows(const float *W, int64_t rows, int64_t cols, do
     if (rc != TWN_OK) return rc;
     // the smallest team and vector count that hold a filter; longer ones go round in chunks of 8192 weights
     const bool vec = twn_aligned(W, 16) && cols % 4 == 0;
-    auto launch = [&](auto kernel, int teams) -> int {
-        const long long grid = (rows + teams - 1) / teams;
+    auto launch = [&](auto team, auto vectors) -> int {
+        constexpr int T = decltype(team)::value, R = decltype(vectors)::value, kTeams = block_threads<T>() / T;
+        const long long grid = (rows + kTeams - 1) / kTeams;
         TWN_REQUIRE(grid < 0x7fffffffLL, TWN_ERR_TOO_LARGE);
-        TWN_CUDA_OK(twn_launch_pdl(true, kernel, (int)grid, kThreads, 0, twn_cu(stream), W, (long long)rows, (long long)cols, delta_factor,
-                                     stats, packed, (long long)(ld_codes / 16), codes_i8, (int)vec));
+        TWN_CUDA_OK(twn_launch_pdl(true, ternarize_rows_kernel<T, R>, (int)grid, block_threads<T>(), 0, twn_cu(stream), W, (long long)rows,
+                                   (long long)cols, delta_factor, stats, packed, (long long)(ld_codes / 16), codes_i8, (int)vec));
         return TWN_OK;
     };
-    constexpr int kWarpTeams = kThreads / 32;
-    if (cols <= 128) return launch(ternarize_rows_kernel<32, 1>, kWarpTeams);
-    if (cols <= 256) return launch(ternarize_rows_kernel<32, 2>, kWarpTeams);
-    if (cols <= 512) return launch(ternarize_rows_kernel<32, 4>, kWarpTeams);
-    if (cols <= 1024) return launch(ternarize_rows_kernel<32, 8>, kWarpTeams);
-    if (cols <= 2048) return launch(ternarize_rows_kernel<kThreads, 2>, 1);
-    if (cols <= 3072) return launch(ternarize_rows_kernel<kThreads, 3>, 1);
-    if (cols <= 4096) return launch(ternarize_rows_kernel<kThreads, 4>, 1);
-    if (cols <= 6144) return launch(ternarize_rows_kernel<kThreads, 6>, 1);
-    if (cols <= 8192 || cols > 16384) return launch(ternarize_rows_kernel<kThreads, 8>, 1);      // fewer registers: more blocks on an SM
-    if (cols <= 12288) return launch(ternarize_rows_kernel<kThreads, 12>, 1);
-    return launch(ternarize_rows_kernel<kThreads, 16>, 1);
+#define TWN_TEAM(t, r) return launch(std::integral_constant<int, t>(), std::integral_constant<int, r>())
+    if (cols <= 1024) switch ((cols + 127) / 128) {
+        case 0: case 1: TWN_TEAM(32, 1);
+        case 2: TWN_TEAM(32, 2);
+        case 3: TWN_TEAM(32, 3);
+        case 4: TWN_TEAM(32, 4);
+        case 5: TWN_TEAM(32, 5);
+        case 6: TWN_TEAM(32, 6);
+        case 7: TWN_TEAM(32, 7);
+        default: TWN_TEAM(32, 8);
+    }
+    // Blocks of 128: up to ten vectors a thread, and with up to fourteen once every SM has ten filters.  Filters off the 16-byte
+    // boundaries, which cost a thread more, from two on an SM on (100 of 1537: 2.8 us, 3.0 with 128; 3000 of 5001 34.3 and 29.0), and
+    // not beyond ten (3000 of 7001: 42.7 and 47.9).
+    if (cols <= 5120 ? vec || rows >= 2LL * dev.sm_count : cols <= 7168 && vec && rows >= 10LL * dev.sm_count) switch ((cols + 511) / 512) {
+        case 3: TWN_TEAM(128, 3);
+        case 4: TWN_TEAM(128, 4);
+        case 5: TWN_TEAM(128, 5);
+        case 6: TWN_TEAM(128, 6);
+        case 7: TWN_TEAM(128, 7);
+        case 8: TWN_TEAM(128, 8);
+        case 9: TWN_TEAM(128, 9);
+        case 10: TWN_TEAM(128, 10);
+        case 11: case 12: TWN_TEAM(128, 12);
+        default: TWN_TEAM(128, 14);
+    }
+    if (cols <= 2048) TWN_TEAM(kThreads, 2);
+    if (cols <= 3072) TWN_TEAM(kThreads, 3);
+    if (cols <= 4096) TWN_TEAM(kThreads, 4);
+    if (cols <= 6144) TWN_TEAM(kThreads, 6);
+    if (cols <= 7168) TWN_TEAM(kThreads, 7);
+    if (cols <= 8192 || cols > 16384) TWN_TEAM(kThreads, 8);      // fewer registers: more blocks on an SM
+    if (cols <= 12288) TWN_TEAM(kThreads, 12);
+    TWN_TEAM(kThreads, 16);
+#undef TWN_TEAM
 }
 
 extern "C" int twn_rows_scale(const twn_stats_t *stats, int64_t rows, const float *scale_in, float *scale_out,
