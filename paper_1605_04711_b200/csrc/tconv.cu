@@ -131,7 +131,7 @@ struct ConvParams {
 };
 
 // The classes of a strided backward pass: their tiles follow one another, those without taps last; each class has its own run of
-// taps and place in the output.  (An argument of their own: in the parameters of every launch they cost small layers 0.3 us.)
+// taps and place in the output.  (An argument of its own: launches without classes do without it.)
 struct ClassTable {
     int n, live_tiles;            // classes; tiles of those with taps
     struct { int tile0, tw, th, Hv, Wv, ooh, oow, tap0, kb0, kb, stages; } cls[kMaxClasses];
@@ -1276,7 +1276,8 @@ int conv_fwd_impl(const twn_conv_desc_t *d, const void *X, const uint32_t *T_fwd
     }
     // Without padding in w the taps of a filter row read one run of kw * Cin elements, in the order of its codes: a "pixel" of as
     // many channels, Cin elements from the next, and one tap per row.  Where that fills the k-blocks of 64 better and a kernel is
-    // modelled faster with it (5x5 on 32 channels: 15 k-blocks for 25; 100x12x12x32 -> 64, pooled, 9.9 -> 7.5 us).  The order of a sum is the same.
+    // modelled faster with it (5x5 on 32 channels: 15 k-blocks for 25; 100x12x12x32 -> 64, pooled, 10.6 -> 9.4
+    // us; 128x30x30x16 -> 128 31.9 -> 19.5).  The order of a sum is the same.
     const long long run = d->kw * d->Cin;
     double alone = -1.0;             // what the layer takes by itself, where that has been looked up
     if (d->pad_w == 0 && d->kw > 1 && (run + 63) / 64 < d->kw * ((d->Cin + 63) / 64)) {
