@@ -1505,24 +1505,30 @@ int conv_bwd_data_impl(const twn_conv_desc_t *d, const void *dZ, const uint32_t 
         // 8 of 31x31x512 <- 192 (5x5) 30 and 19.
         const EpilogueArgs ea = epilogue_args(stats, epi, TWN_F32);
         const SplitPlan plan = plan_conv_split(g, dev.sm_count, ea.in_order);
-        constexpr double kLeast = 2.9;           // no model goes below: the sum ends when the answer is known (2 us of host time)
+        constexpr double kLeast = 2.8;           // no model goes below: a sum that has passed a limit stays above it (saves 2 us of host time)
         // In the general kernel, whose blocks walk tiles of all classes: 50x28x28x192 <- 384 takes 22.1 us so, 28.0 split and 35 apart,
         // 20 images of 56x56x64 <- 128 12.7, 17.4 and 24, 15x41x41x448 <- 240 28.8, 34.3 and 37.2.  It has to be modelled 5 % below
         // the split kernel and 10 % below launches apart (35 % where a class has no taps: those take less than their models say).  Of
-        // 97 shapes measured all three ways the choice is 2.4 % behind the best on average, 6.3 % without this way, and on none slower.
+        // 97 shapes measured all three ways the choice was 2.4 % behind the best on average, 6.3 % without this way, with a sum that ended
+        // at the split kernel's time and left 4 % of all layers, most of them 1x1, split against this rule: of 34 such shapes 32 are
+        // as fast or faster here, two 1.1 and 1.6 % slower, 12 % faster on average (22x32x32x544 <- 544 15.3 us, 19.8 split, 20.9 apart;
+        // 105x12x12x368 <- 112, 3x3, 13.2, 18.7 and 27.1).
         double together = 0.0;
         rc = launch_conv(by_length, dZ, T_bwd, stats, epi, dX, TWN_F32, dev_status, user, &together);
         if (rc != TWN_OK) return rc;
         const double less = by_length.cls[n_cls - 1].n_taps == 0 ? 0.65 : 0.9;
-        const double one = std::min(plan.us, together / less);
+        // The sum ends where it answers the only question left: whether the general kernel is far enough below launches apart, where
+        // it is below the split kernel, else whether the split kernel is below them.
+        const bool below_split = together < 0.95 * plan.us;
+        const double enough = below_split ? together / less : plan.us;
         double apart = kLeast * n_cls - 1.2 * (n_cls - 1);
-        for (int c = 0; c < n_cls && apart <= one; ++c) {
+        for (int c = 0; c < n_cls && apart <= enough; ++c) {
             double us = 0.0;
             rc = launch_conv(one_class(cls[c], n_cls), dZ, T_bwd, stats, epi, dX, TWN_F32, dev_status, user, &us);
             if (rc != TWN_OK) return rc;
             apart += us - kLeast;
         }
-        if (together < 0.95 * plan.us && together < less * apart) return launch_conv(by_length, dZ, T_bwd, stats, epi, dX, TWN_F32, dev_status, user);
+        if (below_split && apart > enough) return launch_conv(by_length, dZ, T_bwd, stats, epi, dX, TWN_F32, dev_status, user);
         if (plan.pix && plan.us < apart)
             return launch_conv_split(g, dZ, T_bwd, ea, dX, dev_status, dev, user, plan);
     }
