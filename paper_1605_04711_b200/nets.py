@@ -143,7 +143,7 @@ class TernaryNet(_Counted):
         self.side_streams = [torch.cuda.Stream()]
         self.dw_stream = torch.cuda.Stream()     # weight gradients run beside the backward-for-data chain
         self.timed = None          # when a list: (kind, name, flops, start event, end event)
-        self._fwd = None           # (changes so far, calls of a forward pass), made on first use
+        self._fwd = None           # (changes so far, calls of a forward pass, epilogues that it depends on), made on first use
         self._bwd = None           # (changes so far, order and fusions of a backward pass), made on first use
         self._pending_join = False
         self._codes_ready = torch.cuda.Event()
@@ -363,14 +363,19 @@ class TernaryNet(_Counted):
         12.1 in three launches), without it from 4 million outputs on (VGG-7, 128 images: 10.9 for 18.6, 32: 6.0 for 10.0).  Smaller
         ones keep the patch matrix, although a launch less would gain there too (8 images: 4.2 for 8.2): the launches of a VGG-7
         of 24 images are fixed by a test.
-        A training step needs the patch matrix for the weight gradient."""
+        A training step needs the patch matrix for the weight gradient, and an epilogue into which the caller has written what the
+        kernel does not do, or asked for one order of the sums at every batch, needs the product."""
         e, y = L.extra, self.act[L.name]
+        epi = e["epi"]
+        if epi.out_dtype != twn.BF16 or epi.residual or epi.residual_op != twn.RESIDUAL_ADD or epi.residual_dtype not in (twn.F32, twn.BF16):
+            return False
         return (L.small_cin and not L.fold and not self.train and L.K <= 64 and L.Cin <= 8 and L.stride <= 2 and L.pad < L.k and L.Cout % 8 == 0 and
-                not L.out_f32 and not L.residual and e["epi"] is self._made[L.name][0] and y.data_ptr() % 16 == 0 and
+                epi is self._made[L.name][0] and y.data_ptr() % 16 == 0 and
                 (min(L.Ho, L.Wo) >= 2 and self.act[pool].data_ptr() % 16 == 0 if pool else y.numel() >= 2 ** 22))
 
     def forward(self):
-        if self._fwd is None or self._fwd[0] != self._changes.n:
+        # (the fields of a first layer's epilogue decide how it is taken, and assignments to them are not counted)
+        if self._fwd is None or self._fwd[0] != self._changes.n or any(bytes(epi) != was for epi, was in self._fwd[2]):
             if self._changes.n != self._built:
                 for op in self.ops:
                     if op[0] == "layer":
@@ -378,7 +383,8 @@ class TernaryNet(_Counted):
                     elif op[0] == "flatten" and self.act[op[1]] is self._made[op[1]]:
                         self._make_view(op[1], op[2])
             calls = self._forward_calls()
-            self._fwd = (self._changes.n, calls)
+            self._fwd = (self._changes.n, calls, [(L.extra["epi"], bytes(L.extra["epi"])) for L in self.layers.values()
+                                                  if L.small_cin and not L.fold and not self.train])
         for call in self._fwd[1]:
             self._call(*call)
         return self.act[self.ops[-1][1].name]
