@@ -492,7 +492,7 @@ int twn_im2col(const twn_conv_desc_t *desc, const void *X, void *Xcol, int64_t l
  *   Y    bf16 NHWC [B,Ho,Wo,Cout];  Yp  bf16 [B,Ho/2,Wo/2,Cout], what twn_maxpool2d_fwd makes of Y, or NULL (both
  *        16-byte aligned)
  * Requires kh*kw*Cin <= 64, Cin <= 8, strides of 1 or 2, paddings smaller than the filter, Cout % 8 == 0, an epilogue with
- * out_dtype = TWN_BF16 and no residual, and with Yp Ho, Wo >= 2.  One launch.
+ * out_dtype = TWN_BF16 and no residual (its other fields are checked as everywhere), and with Yp Ho, Wo >= 2.  One launch.
  */
 int twn_conv2d_fwd_image(const twn_conv_desc_t *desc, const void *X, const uint32_t *T_fwd, int64_t ld_codes,
                          const twn_stats_t *stats, const twn_epilogue_t *epi, void *Y, void *Yp, twn_stream_t stream);

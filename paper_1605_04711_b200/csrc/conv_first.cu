@@ -21,6 +21,7 @@
 
 #include "common.cuh"
 #include "tc_ptx.cuh"
+#include "tconv_host.cuh"
 
 namespace {
 
@@ -245,9 +246,11 @@ extern "C" int twn_conv2d_fwd_image(const twn_conv_desc_t *d, const void *X, con
                 TWN_ERR_INVALID_ARG);
     TWN_REQUIRE(d->H + 2 * d->pad_h >= d->kh && d->W + 2 * d->pad_w >= d->kw, TWN_ERR_INVALID_ARG);
     TWN_REQUIRE(d->Cout % 8 == 0 && ld_codes % 64 == 0 && ld_codes >= d->kh * d->kw * d->Cin, TWN_ERR_INVALID_ARG);
-    TWN_REQUIRE(epi->out_dtype == TWN_BF16 && !epi->residual && (epi->relu == 0 || epi->relu == 1), TWN_ERR_INVALID_ARG);
-    TWN_REQUIRE(twn_aligned(X, 2) && twn_aligned(T_fwd, 16) && twn_aligned(Y, 16) && twn_aligned(Yp, 16) && twn_aligned(stats, 8) &&
-                    twn_aligned(epi->scale, 4) && twn_aligned(epi->shift, 4), TWN_ERR_MISALIGNED);
+    int rc = twn_detail::check_epilogue(epi);
+    if (rc != TWN_OK) return rc;
+    TWN_REQUIRE(epi->out_dtype == TWN_BF16 && !epi->residual, TWN_ERR_INVALID_ARG);
+    TWN_REQUIRE(twn_aligned(X, 2) && twn_aligned(T_fwd, 16) && twn_aligned(Y, 16) && twn_aligned(Yp, 16) && twn_aligned(stats, 8),
+                TWN_ERR_MISALIGNED);
     FirstParams P;
     memset(&P, 0, sizeof P);
     P.Ho = (int)((d->H + 2 * d->pad_h - d->kh) / d->stride_h + 1);
@@ -255,7 +258,7 @@ extern "C" int twn_conv2d_fwd_image(const twn_conv_desc_t *d, const void *X, con
     P.PH = P.Ho / 2; P.PW = P.Wo / 2;
     TWN_REQUIRE(!Yp || (P.PH > 0 && P.PW > 0), TWN_ERR_INVALID_ARG);
     twn_device_info dev;
-    const int rc = twn_current_device(&dev);
+    rc = twn_current_device(&dev);
     if (rc != TWN_OK) return rc;
     P.X = static_cast<const __nv_bfloat16 *>(X);
     P.T = T_fwd;

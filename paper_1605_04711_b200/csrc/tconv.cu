@@ -1151,21 +1151,6 @@ ForkPool *fork_pool(int ordinal)
     return &p;
 }
 
-int check_epilogue(const twn_epilogue_t *e)
-{
-    if (!e) return TWN_OK;
-    TWN_REQUIRE(e->out_dtype == TWN_F32 || e->out_dtype == TWN_BF16, TWN_ERR_INVALID_ARG);
-    TWN_REQUIRE(e->residual_dtype == TWN_F32 || e->residual_dtype == TWN_BF16, TWN_ERR_INVALID_ARG);
-    TWN_REQUIRE(e->relu == 0 || e->relu == 1, TWN_ERR_INVALID_ARG);
-    TWN_REQUIRE(e->residual_op >= 0 && e->residual_op <= (TWN_RESIDUAL_GATE | TWN_SUM_IN_ORDER), TWN_ERR_INVALID_ARG);
-    TWN_REQUIRE(twn_aligned(e->scale, 4) && twn_aligned(e->shift, 4) && twn_aligned(e->residual, 4), TWN_ERR_MISALIGNED);
-    return TWN_OK;
-}
-
-}  // namespace
-
-namespace {
-
 // Shared by the ternary (bits = 2) and binary (bits = 1) entry points.
 int gemm_impl(const void *X, int64_t ldx, const uint32_t *T_packed, int64_t ld_codes,
               const twn_stats_t *stats, int64_t M, int64_t N, int64_t K,

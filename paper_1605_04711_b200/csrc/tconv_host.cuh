@@ -116,6 +116,18 @@ inline long long pick_tile(const Geometry &g, int pix, int *lgBW, int *lgBH)
     return best;
 }
 
+// What every contraction asks of an epilogue; NULL stands for the default one.
+inline int check_epilogue(const twn_epilogue_t *e)
+{
+    if (!e) return TWN_OK;
+    TWN_REQUIRE(e->out_dtype == TWN_F32 || e->out_dtype == TWN_BF16, TWN_ERR_INVALID_ARG);
+    TWN_REQUIRE(e->residual_dtype == TWN_F32 || e->residual_dtype == TWN_BF16, TWN_ERR_INVALID_ARG);
+    TWN_REQUIRE(e->relu == 0 || e->relu == 1, TWN_ERR_INVALID_ARG);
+    TWN_REQUIRE(e->residual_op >= 0 && e->residual_op <= (TWN_RESIDUAL_GATE | TWN_SUM_IN_ORDER), TWN_ERR_INVALID_ARG);
+    TWN_REQUIRE(twn_aligned(e->scale, 4) && twn_aligned(e->shift, 4) && twn_aligned(e->residual, 4), TWN_ERR_MISALIGNED);
+    return TWN_OK;
+}
+
 // What follows the contraction (twn_epilogue_t with the device scalar alpha resolved).
 struct EpilogueArgs {
     const double *alpha;          // device scalar (twn_stats_t::alpha) or nullptr for 1
