@@ -269,8 +269,9 @@ extern "C" int twn_conv2d_fwd_image(const twn_conv_desc_t *d, const void *X, con
     P.kw = (int)d->kw; P.K = (int)(d->kh * d->kw * d->Cin);
     P.sh = (int)d->stride_h; P.sw = (int)d->stride_w; P.ph = (int)d->pad_h; P.pw = (int)d->pad_w;
     P.wpr = (int)(ld_codes / 16);
-    // offsets of outputs, and of a unit past the last, in 32 bits
-    TWN_REQUIRE((double)d->B * (P.Ho + 16) * (P.Wo + 16) * d->Cout < 4294967296.0, TWN_ERR_TOO_LARGE);
+    // Offsets of outputs in 32 bits, the general kernel's limit.  (Those past an output's edge may wrap: they are not stored to.)
+    // It leaves less than 2^29 units, each of at least one pixel of at least eight channels.
+    TWN_REQUIRE((double)d->B * P.Ho * P.Wo * d->Cout < 4294967295.0, TWN_ERR_TOO_LARGE);
     // A unit: eight windows in the shape that covers the output with the fewest (12 by 12 windows: 18 units of 4 x 2, 24 of 8 x 1),
     // the wider of equals.
     const int wins_x = (P.Wo + 1) / 2, wins_y = (P.Ho + 1) / 2;
@@ -282,7 +283,7 @@ extern "C" int twn_conv2d_fwd_image(const twn_conv_desc_t *d, const void *X, con
         best = nx * ny;
         P.lgUx = lg; P.nx = (int)nx; P.ny = (int)ny; P.rows = rows; P.pitch = pitch;
     }
-    if (P.rows * P.pitch > kMostPiece || best * d->B > 0x3fffffffLL) return TWN_ERR_TOO_LARGE;
+    if (P.rows * P.pitch > kMostPiece) return TWN_ERR_TOO_LARGE;
     P.units = (int)(best * d->B);
     const cudaStream_t s = twn_cu(stream);
     switch ((P.K + 15) / 16) {

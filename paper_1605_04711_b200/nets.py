@@ -370,7 +370,7 @@ class TernaryNet(_Counted):
         if epi.out_dtype != twn.BF16 or epi.residual or epi.residual_op != twn.RESIDUAL_ADD or epi.residual_dtype not in (twn.F32, twn.BF16):
             return False
         return (L.small_cin and not L.fold and not self.train and L.K <= 64 and L.Cin <= 8 and L.stride <= 2 and L.pad < L.k and L.Cout % 8 == 0 and
-                epi is self._made[L.name][0] and y.data_ptr() % 16 == 0 and
+                max(L.H, L.W, L.Cout) < 2 ** 24 and epi is self._made[L.name][0] and y.data_ptr() % 16 == 0 and
                 (min(L.Ho, L.Wo) >= 2 and self.act[pool].data_ptr() % 16 == 0 if pool else y.numel() >= 2 ** 22))
 
     def forward(self):
