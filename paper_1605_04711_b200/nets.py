@@ -34,6 +34,16 @@ def _bf16(bits: np.ndarray) -> torch.Tensor:
     return torch.from_numpy(np.ascontiguousarray(bits).view(np.int16)).cuda().view(torch.bfloat16)
 
 
+# bf16 outputs, no residual, no order of the sums asked for: the fields of an epilogue behind its affine
+_REST = twn.Epilogue.residual.offset
+_PLAIN = frozenset(bytes(twn.Epilogue(out_dtype=twn.BF16, relu=relu, residual_dtype=dtype))[_REST:] for relu in (0, 1)
+                   for dtype in (twn.F32, twn.BF16))
+
+
+def _plain(epi):
+    return bytes(epi)[_REST:] in _PLAIN
+
+
 class _Changes:
     """Counts the assignments to the buffers and parameters of a network: a pass's prepared list of calls holds what they
     were, and is made again when the count has moved.  (An object of its own, so that the dicts that report to it form no
@@ -143,7 +153,7 @@ class TernaryNet(_Counted):
         self.side_streams = [torch.cuda.Stream()]
         self.dw_stream = torch.cuda.Stream()     # weight gradients run beside the backward-for-data chain
         self.timed = None          # when a list: (kind, name, flops, start event, end event)
-        self._fwd = None           # (changes so far, calls of a forward pass, epilogues that it depends on), made on first use
+        self._fwd = None           # (changes so far, calls of a forward pass, what else they depend on), made on first use
         self._bwd = None           # (changes so far, order and fusions of a backward pass), made on first use
         self._pending_join = False
         self._codes_ready = torch.cuda.Event()
@@ -312,8 +322,9 @@ class TernaryNet(_Counted):
 
     # ------------------------------------------------------------------ forward
     def _forward_calls(self):
-        """The calls of a forward pass, (kind, name, flops, entry point, arguments) each: a pass walks this list."""
-        calls = []
+        """The calls of a forward pass, (kind, name, flops, entry point, arguments) each: a pass walks this list.  Beside it the
+        network's own epilogues whose fields it depends on, and whether they were plain."""
+        calls, depends = [], []
         pooled = None            # the pooling that its layer's call has done
         for op, after in zip(self.ops, [*self.ops[1:], ("end",)]):
             kind = op[0]
@@ -329,7 +340,7 @@ class TernaryNet(_Counted):
                     calls.append((None, "", 0, "fold_input", (L.desc, x, e["xf"])))
                     calls.append((*row, "conv2d_fwd_folded", (L.desc, e["xf"], e["packed_f"], L.fold[2], e["stats"], e["epi"],
                                                               y, self.status)))
-                elif self._from_image(L, pool):
+                elif L.small_cin and not self.train and e["epi"] is self._made[L.name][0] and self._from_image(L, pool, depends):
                     calls.append((*row, "conv2d_fwd_image", (L.desc, x, e["packed"], e["ld"], e["stats"], e["epi"], y,
                                                              self.act[pool] if pool else None)))
                     pooled = pool
@@ -356,35 +367,32 @@ class TernaryNet(_Counted):
                 x = self.act[src]
                 Bx, H, W, C = x.shape
                 calls.append((None, "", 0, "avgpool_fwd", (x, Bx, H * W, C, self.act[name])))
-        return calls
+        return calls, depends
 
-    def _from_image(self, L, pool):
-        """Whether a layer on few channels is taken straight from the image: with its pooling always (LeNet-5, 100 images: 3.8 us for
-        12.1 in three launches), without it from 4 million outputs on (VGG-7, 128 images: 10.9 for 18.6, 32: 6.0 for 10.0).  Smaller
-        ones keep the patch matrix, although a launch less would gain there too (8 images: 4.2 for 8.2): the launches of a VGG-7
-        of 24 images are fixed by a test.
+    def _from_image(self, L, pool, depends):
+        """Whether a layer on few channels, not folded, is taken straight from the image: with its pooling always (LeNet-5, 100
+        images: 3.8 us for 12.1 in three launches), without it from 4 million outputs on (VGG-7, 128 images: 10.9 for 18.6, 32: 6.0
+        for 10.0).  Smaller ones keep the patch matrix, although a launch less would gain there too (8 images: 4.2 for 8.2): the
+        launches of a VGG-7 of 24 images are fixed by a test.
         A training step needs the patch matrix for the weight gradient, and an epilogue into which the caller has written what the
         kernel does not do, or asked for one order of the sums at every batch, needs the product."""
-        e, y = L.extra, self.act[L.name]
-        epi = e["epi"]
-        if epi.out_dtype != twn.BF16 or epi.residual or epi.residual_op != twn.RESIDUAL_ADD or epi.residual_dtype not in (twn.F32, twn.BF16):
+        y = self.act[L.name]
+        if (L.K > 64 or L.Cin > 8 or L.stride > 2 or L.pad >= L.k or L.Cout % 8 or max(L.H, L.W, L.Cout) >= 2 ** 24 or y.data_ptr() % 16 or
+                (min(L.Ho, L.Wo) < 2 or self.act[pool].data_ptr() % 16 if pool else y.numel() < 2 ** 22)):
             return False
-        return (L.small_cin and not L.fold and not self.train and L.K <= 64 and L.Cin <= 8 and L.stride <= 2 and L.pad < L.k and L.Cout % 8 == 0 and
-                max(L.H, L.W, L.Cout) < 2 ** 24 and epi is self._made[L.name][0] and y.data_ptr() % 16 == 0 and
-                (min(L.Ho, L.Wo) >= 2 and self.act[pool].data_ptr() % 16 == 0 if pool else y.numel() >= 2 ** 22))
+        depends.append((L.extra["epi"], _plain(L.extra["epi"])))
+        return depends[-1][1]
 
     def forward(self):
-        # (the fields of a first layer's epilogue decide how it is taken, and assignments to them are not counted)
-        if self._fwd is None or self._fwd[0] != self._changes.n or any(bytes(epi) != was for epi, was in self._fwd[2]):
+        # (assignments to the fields of an epilogue are not counted)
+        if self._fwd is None or self._fwd[0] != self._changes.n or any(_plain(epi) != was for epi, was in self._fwd[2]):
             if self._changes.n != self._built:
                 for op in self.ops:
                     if op[0] == "layer":
                         self._make_epilogue(op[1])
                     elif op[0] == "flatten" and self.act[op[1]] is self._made[op[1]]:
                         self._make_view(op[1], op[2])
-            calls = self._forward_calls()
-            self._fwd = (self._changes.n, calls, [(L.extra["epi"], bytes(L.extra["epi"])) for L in self.layers.values()
-                                                  if L.small_cin and not L.fold and not self.train])
+            self._fwd = (self._changes.n, *self._forward_calls())
         for call in self._fwd[1]:
             self._call(*call)
         return self.act[self.ops[-1][1].name]

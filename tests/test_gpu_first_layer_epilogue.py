@@ -54,3 +54,18 @@ def test_refused_by_every_contraction():
     epi.residual_op = 9
     with pytest.raises(twn.TwnError):
         net.forward()
+
+
+def test_no_epilogue():
+    """None stands for fp32 outputs, which a caller may put in place of a layer's own epilogue with a buffer for them."""
+    op = ("layer", nets.Layer("conv", 3, 16, 3, 1, 1, 8, 8, src="input"))
+    net = nets.TernaryNet("one", 2, (8, 8, 3), [op])
+    net.act["input"].normal_()
+    net.ternarize_all()
+    net.layers["conv"].extra["epi"] = None
+    net.act["conv"] = torch.full((2, 8, 8, 16), 7.0, device="cuda")
+    L, y = net.layers["conv"], net.forward()
+    columns, want = torch.zeros((128, L.ldk), dtype=torch.bfloat16, device="cuda"), torch.zeros_like(y)
+    twn.im2col(L.desc, net.act["input"], columns, L.ldk)
+    twn.gemm(columns, L.ldk, L.extra["packed"], L.extra["ld"], L.extra["stats"], 128, 16, 27, None, want, 16)
+    assert torch.equal(y, want) and torch.equal(net.forward(), want)
