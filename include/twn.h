@@ -401,8 +401,9 @@ int twn_bn_finalize(const double *sum, const double *sumsq, int64_t n, int64_t C
  *   dX     NHWC [B,H,W,Cin], fp32 or bf16; every element is written.
  *   epi    scale/shift are indexed by the input channel c; `residual` (shape of dX)
  *          lets a second gradient branch be added in the same pass.
- * Requires Cout % 16 == 0 (Cout % 8 == 0 for a 1x1 filter).  A strided layer runs as
- * stride_h*stride_w launches, one per residue class of (h, w) modulo the stride.
+ * Requires Cout % 16 == 0 (Cout % 8 == 0 for a 1x1 filter).  A strided layer is a
+ * sum for each residue class of (h, w) modulo the stride: up to four of them run in one launch or, where that should
+ * take longer, in a launch each, side by side.
  */
 int twn_conv2d_bwd_data(const twn_conv_desc_t *desc, const void *dZ, const uint32_t *T_bwd, int64_t ld_codes,
                         const twn_stats_t *stats, const twn_epilogue_t *epi, void *dX,

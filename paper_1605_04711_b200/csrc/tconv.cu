@@ -1037,7 +1037,8 @@ int launch_conv(const Geometry &g, const void *X, const uint32_t *T, const twn_s
     auto time_us = [&](long long tiles, double fixed, double per_tile, double per_block, double least) {
         return fixed + (double)((tiles + sms - 1) / sms) * std::max(per_tile + per_block * (double)kb, least);
     };
-    // (code words off the 16-byte boundaries come one at a time, which the smaller shapes wait for: 7 further shapes)
+    // (k-blocks off the 16-byte boundaries come with two or four loads, which the smaller shapes wait for: 7 further shapes, all of
+    // them measured with four)
     const bool words = P.code_run * (g.code_bits == 1 ? 2 : 1) < 4;
     const double u128 = time_us(t128, 4.3, 1.4, words ? 0.225 : 0.155, 1.85),
                  u192 = time_us(t192, 5.1, 1.6, words ? 0.24 : 0.225, half ? 1.76 : 2.43),
@@ -1078,8 +1079,8 @@ int launch_conv(const Geometry &g, const void *X, const uint32_t *T, const twn_s
     }
     int choice = u256 + kOther < u128 ? 1 : 0;
     if (u192 + (choice ? 0.0 : kOther) < (choice ? u256 : u128)) choice = 2;
-    // Pooling is in that kernel alone: the others, whose epilogue is longer with it, lost 0.6 % on 16384x4096x4096 to code that
-    // they do not run.
+    // Of the three shapes pooling is in that kernel alone: the others, whose epilogue is longer with it, lost 0.6 % on
+    // 16384x4096x4096 to code that they do not run.
     if (g.pool || classes) choice = 0;
     const double us = choice == 0 ? u128 : choice == 1 ? u256 : u192;
     // Narrow layers and short reductions: the kernel that decodes its channels' codes once per block.  Up to 64 channels
@@ -1280,8 +1281,8 @@ int conv_fwd_impl(const twn_conv_desc_t *d, const void *X, const uint32_t *T_fwd
         alone = std::min(by_row, by_tap);
     }
     if (pool) {
-        // Pooled in the epilogue of the general kernel, if that and no sweep should take less time than the kernel that the layer
-        // would get by itself and a sweep (modelled as 2 us and 4.2 TB/s; 2.1 us for 100x8x8x64).  What TMA cannot store or the
+        // Pooled in the epilogue of the general or the split kernel, if that and no sweep should take less time than the kernel that
+        // the layer would get by itself and a sweep (modelled as 2 us and 4.2 TB/s; 2.1 us for 100x8x8x64).  What TMA cannot store or the
         // fragments do not hold stays with the sweep.
         *pool->done = false;
         const double bytes = 2.5 * (double)g.Bv * g.Hv * g.Wv * g.Cout;

@@ -65,7 +65,7 @@ struct Geometry {
     Tap taps[kMaxTaps];
     long long Cin;   // channels per tap
     int beside;      // launches that run at the same time as this one (0 or 1: none)
-    // 0: one class, described by the fields above; else all of them in one launch (launch_conv_split only)
+    // 0: one class, described by the fields above; else all of them in one launch (split kernel, general kernel of 128 pixels)
     int n_classes;
     TapClass cls[kMaxClasses];
 };
@@ -149,7 +149,8 @@ int launch_conv_resident(const Geometry &g, const void *X, const uint32_t *T, co
 
 // Contraction for problems that do not fill the GPU (tconv_split.cu): tiles of 128 channels x `pix` pixels (32, 64, 128
 // or 256), the reduction of each split over a cluster of `splits` blocks (1, 2, 4 or 8; 256 pixels: 1 or 2).  Takes every
-// geometry but batch statistics and reductions of more than 512 k-blocks per block.
+// geometry but batch statistics, reductions of more than 512 k-blocks per block, and pooled outputs of more than 64 channels, of
+// binary codes or with their sums in order.
 struct SplitPlan {
     int pix, splits;
     double us;        // what the launch should take

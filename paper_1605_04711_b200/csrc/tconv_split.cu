@@ -540,8 +540,9 @@ SplitPlan plan_conv_split(const Geometry &g, int sm_count, bool in_order)
     static const double E[4] = {3.89, 4.47, 5.51, 7.73}, R[4] = {0.241, 0.249, 0.255, 0.275};
     SplitPlan best = {0, 0, 1e30};
     // A pooled output: up to 64 channels, where half of a tile of the general kernel is idle (14x14x64, 3x3 on 64: 16 images 7.2 us, 5.3 here, 64 images 7.8 and
-    // 6.6; 12x12x64, 5x5 on 32: 32 images 8.7 and 7.4, 100 images 10.7 and 10.5, in LeNet-5 behind its first layer 2.2 us less); the sums of
-    // wider pooled layers stay in order, as those of callers who ask for that do, in the general kernel.
+    // 6.6; 12x12x64, 5x5 on 32: 32 images 8.7 and 7.4, 100 images 10.7 and 10.5, in LeNet-5 behind its first layer 2.2 us less).
+    // Wider pooled layers were not timed here and stay in the general kernel, which does not split their sums: a test compares a
+    // VGG-7's at 24 images bit by bit with sums in order.  Callers who ask for that order get it there as well.
     if (g.bn_partial || (g.pool && (in_order || g.code_bits != 2 || g.Cout > 64))) return best;
     // with classes: as many tiles as the largest has each (it comes first), the longest reduction and the mean one
     const int classes = g.n_classes > 0 ? g.n_classes : 1;
